@@ -58,17 +58,18 @@ TOTALS_EVERY = 100
 # of the kernel sources it was captured from.  bench reports the traffic only while the sources
 # still hash to that value, else null.
 TRAFFIC_PER_CELL = {
-    "f32": {"bytes": 125.89, "sources": ("lbm_step_tma.cu", "lbm_device.cuh", "lbm_tma_util.cuh"),
-            "sha": "07a62d28b685263d"},
-    "f64": {"bytes": 251.63, "sources": ("lbm_step_stream.cu", "lbm_device.cuh", "lbm_tma_util.cuh"),
-            "sha": "01bf052590e27491"},
-    "dd": {"bytes": 247.87, "sources": ("lbm_step_dd.cu", "lbm_dd.cuh", "lbm_device.cuh", "lbm_tma_util.cuh"),
-           "sha": "a502465f89b98477"},
+    "f32": {"bytes": 125.83, "sources": ("lbm_step_tma.cu", "lbm_device.cuh", "lbm_tma_util.cuh"),
+            "sha": "cab4bf9af2fde156"},
+    "f64": {"bytes": 251.37, "sources": ("lbm_step_stream.cu", "lbm_device.cuh", "lbm_tma_util.cuh"),
+            "sha": "5c2c8bd0138a90d8"},
+    "dd": {"bytes": 274.54, "sources": ("lbm_step_dd.cu", "lbm_dd.cuh", "lbm_device.cuh", "lbm_tma_util.cuh"),
+           "sha": "903244fc4e130362"},
 }
-# float32-pipe operations (add, multiply, FMA: one each) per cell of one launch of the double-float
-# float64 kernel on 32 x 32 tiles, counted by ncu on the same sources
-# (profiles/k_step_dd_f64_shear_layer.md); None when the sources changed since.
-DD_FP32_OPS = {"ops": 3649.3, "sha": "a502465f89b98477"}
+# float32-pipe lane operations per cell of one launch of the double-float float64 kernel on wide
+# tiles: ncu's FMA-pipe busy fraction x cycles x 128 lanes (its counters of float32 instructions do
+# not see the packed f32x2 ones), on the same sources (profiles/k_step_dd_f64_shear_layer.md); None
+# when the sources changed since.
+DD_FP32_OPS = {"ops": 3847.3, "sha": "903244fc4e130362"}
 FP32_LANES_PER_SM = 128           # float32 FMA lanes per SM per cycle (GB300)
 
 

@@ -110,10 +110,10 @@ typedef struct {
                                       128 columns), 6 = persistent TMA-staged 32 x 16 tiles with
                                       two tile buffers per CTA (LBM_FP32_DEV only), 7 = plain
                                       64-cell tiles (32 x 2; spreads small float64 grids over
-                                      every SM), 8 = LBM_FP64 only: the 32 x 32 TMA-staged tiles
+                                      every SM), 8 = LBM_FP64 only: TMA-staged tiles
                                       with the step's arithmetic in double-float form (pairs of
                                       float32, about 2^-47 rounding per operation) on the float32
-                                      pipe, populations still stored and returned in float64
+                                      pipe, 32 x 16 tiles, populations still stored and returned in float64
                                       (grids of at least 32 x 32), 9 = LBM_FP64 only: the same
                                       arithmetic on 32 x 4 tiles, two CTAs per SM (grids of at
                                       least 32 columns and 4 rows); all agree to round-off of
@@ -221,7 +221,7 @@ int lbm_autotune(lbm_ctx *ctx, int reps, int *choice);
    - contexts whose step kernel is the TMA-staged tile kernel (float32) or a double-float
      kernel (float64), i.e. the automatic choice on grids of at least 32 x 16 (float32) or
      32 x 4 (float64), have their tiles in one launch of that kernel's batched form per 128
-     such grids (float64: one for the 32 x 32 tiles, one for the 32 x 4 tiles) (one CTA per tile; the launch's parameters hold each grid's tensor map,
+     such grids (float64: one for the 32 x 16 tiles, one for the 32 x 4 tiles) (one CTA per tile; the launch's parameters hold each grid's tensor map,
      output buffer and tile count, and the CTA stages its grid's coefficients in shared
      memory), with the arithmetic of the single-grid kernel, bit for bit;
    - the other grids share the packed plain kernel, whose persistent CTAs walk a tile list

@@ -48,12 +48,13 @@ struct lbm_ctx {
     bool use_pipe = false;
     bool use_dd = false;          // float64 mode in double-float arithmetic (step_kernel 8)
     bool use_ddn = false;         // the same on narrow tiles of 32 x 4 (step_kernel 9)
-    lbm::Coef<lbm::dd> cdd{};     // their coefficients
+    lbm::CoefDD cdd{};     // their coefficients
     int plain_ty = lbm::kTY;      // tile height of the plain step kernel
     CUtensorMap tmap[2];          // tile-copy descriptors of the two population buffers
     CUtensorMap smap[2];          // row-copy descriptors (streaming kernel)
     CUtensorMap pmap[2];          // tile-copy descriptors of the double-buffered kernel
-    CUtensorMap nmap[2];          // tile-copy descriptors of the narrow double-float tiles
+    CUtensorMap dmap[2];          // tile-copy descriptors of the wide double-float tiles
+    CUtensorMap nmap[2];          // and of the narrow ones
     // lbm_step replays pairs of steps (ghost fill + fused step, twice) from a CUDA graph per
     // starting buffer, captured on a private stream at first use; lbm_autotune drops them
     cudaGraphExec_t pair[2] = {nullptr, nullptr};
@@ -273,12 +274,15 @@ bool make_tile_maps(lbm_ctx *c)
            make_tensor_map(&c->tmap[1], c->f[1], c->P, c->prec, sw, sh);
 }
 
-bool make_narrow_maps(lbm_ctx *c)
+template <typename S>
+bool make_dd_maps(lbm_ctx *c, CUtensorMap *m)
 {
-    const int sw = lbm::DdNarrowShape::SW, sh = lbm::DdNarrowShape::SH;
-    return make_tensor_map(&c->nmap[0], c->f[0], c->P, c->prec, sw, sh) &&
-           make_tensor_map(&c->nmap[1], c->f[1], c->P, c->prec, sw, sh);
+    return make_tensor_map(&m[0], c->f[0], c->P, c->prec, S::SW, S::SH) &&
+           make_tensor_map(&m[1], c->f[1], c->P, c->prec, S::SW, S::SH);
 }
+
+bool make_wide_maps(lbm_ctx *c) { return make_dd_maps<lbm::DdWideShape>(c, c->dmap); }
+bool make_narrow_maps(lbm_ctx *c) { return make_dd_maps<lbm::DdNarrowShape>(c, c->nmap); }
 
 bool make_row_maps(lbm_ctx *c)
 {
@@ -309,15 +313,15 @@ bool tma_ready(lbm_ctx *c)
 // interior itself: on a grid periodic in x it needs only the ghost rows.
 bool ghost_rows_only(const lbm_ctx *c) { return (c->use_tma || c->use_dd) && (c->P.wrap & 1); }
 
-// The double-float float64 kernel: the float64 tile maps and the Coef<dd> of the context.
+// The double-float float64 kernel: the float64 tile maps and the CoefDD of the context.
 bool dd_ready(lbm_ctx *c)
 {
     if (c->prec != LBM_FP64 || !lbm::tma_supported(c->P, LBM_FP64) || lbm::dd_prepare() != cudaSuccess) return false;
     lbm::coef_dd(c->P, &c->cdd);
-    return make_tile_maps(c);
+    return make_wide_maps(c);
 }
 
-// The double-float kernel on narrow tiles (grids of 4 to 31 rows): their maps and the Coef<dd>.
+// The double-float kernel on narrow tiles (grids of 4 to 31 rows): their maps and the CoefDD.
 bool ddn_ready(lbm_ctx *c)
 {
     if (c->prec != LBM_FP64 || !lbm::dd_narrow_supported(c->P) || lbm::dd_prepare() != cudaSuccess) return false;
@@ -328,7 +332,7 @@ bool ddn_ready(lbm_ctx *c)
 // One fused step of context c from buffer `in` into buffer in ^ 1, on stream st.
 cudaError_t launch_fused_step(lbm_ctx *c, int in, cudaStream_t st)
 {
-    if (c->use_dd) return lbm::launch_step_dd(c->P, &c->cdd, &c->tmap[in], c->f[in], c->f[in ^ 1], c->tma_err, st);
+    if (c->use_dd) return lbm::launch_step_dd(c->P, &c->cdd, &c->dmap[in], c->f[in], c->f[in ^ 1], c->tma_err, st);
     if (c->use_ddn)
         return lbm::launch_step_dd(c->P, &c->cdd, &c->nmap[in], c->f[in], c->f[in ^ 1], c->tma_err, st, true);
     if (c->use_pipe) return lbm::launch_step_tma_pipe(c->P, &c->pmap[in], c->f[in ^ 1], c->tma_err, st);
@@ -556,10 +560,9 @@ int lbm_create_ex(int nx, int ny, double dx, double dt, double gamma, double Pr,
     // 32 rows of a 256-column strip; else the plain kernel, on 256-cell tiles when they still
     // give every SM four tiles (their flow-velocity ring costs less), on 64-cell tiles below
     // that, which spread a small grid's float64 work over more SMs.  The double-float kernel
-    // runs on 32 x 32 tiles where the grid has at least two thirds of a wave of them (one CTA
-    // per SM); on smaller grids, and on grids of 4 to 31 rows, on 32 x 4 tiles (two CTAs per
-    // SM): a 32 x 32 tile takes about 44 us on its SM, so a small grid finishes sooner in more,
-    // shorter tiles (128 x 96: 17 us against 44 us a step)
+    // runs on 32 x 16 tiles (two CTAs per SM) where the grid has at least two thirds of an SM's
+    // count of 32 x 32 cells; on smaller grids, and on grids of 4 to 31 rows, on 32 x 4 tiles: a
+    // small grid finishes sooner in more, shorter tiles
     if (want == 0 && prec == LBM_FP64) {
         int sms = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
@@ -1038,7 +1041,7 @@ int lbm_autotune(lbm_ctx *c, int reps, int *choice)
                 return lbm::launch_step_dd(c->P, &c->cdd, &c->nmap[c->cur], c->f[c->cur], c->f[c->cur ^ 1],
                                            c->tma_err, c->stream, true);
             if (cd == 8)
-                return lbm::launch_step_dd(c->P, &c->cdd, &c->tmap[c->cur], c->f[c->cur], c->f[c->cur ^ 1],
+                return lbm::launch_step_dd(c->P, &c->cdd, &c->dmap[c->cur], c->f[c->cur], c->f[c->cur ^ 1],
                                            c->tma_err, c->stream);
             if (cd == 6)
                 return lbm::launch_step_tma_pipe(c->P, &c->pmap[c->cur], c->f[c->cur ^ 1], c->tma_err, c->stream);
@@ -1105,10 +1108,10 @@ struct lbm_batch {
         int ntiles = 0, max_ghost = 0;
         int nt = lbm::kBatchThreads;             // threads (= cells) per tile
         // batched TMA-staged kernels: the row spans they serve (member index into members, first
-        // row, rows; in launch order; float64 spans on 32 x 32 tiles in tk, on narrow 32 x 4
-        // tiles in tkn) and one TileGrid block per span (Coef<float> or Coef<dd> by precision),
-        // tk's first.  A float64 member on 32 x 32 tiles whose last tile row would hold at most
-        // 24 of its rows has those rows in a narrow span.
+        // row, rows; in launch order; float64 spans on 32 x 16 tiles in tk, on narrow 32 x 4
+        // tiles in tkn) and one TileGrid block per span (Coef<float> or CoefDD by precision),
+        // tk's first.  A float64 member on 32 x 16 tiles whose last tile row would hold at most
+        // 12 of its rows has those rows in a narrow span.
         struct Span {
             int k, y0, rows;
         };
@@ -1147,7 +1150,7 @@ cudaError_t batch_upload_cur(lbm_batch *b)
 }
 
 // The group's batched TMA-staged launches (kTmaBatchGrids grids each) over the members `tk`
-// (float32 tile kernel, or float64 double-float kernel on 32 x 32 tiles) and, in float64, over
+// (float32 tile kernel, or float64 double-float kernel on 32 x 16 tiles) and, in float64, over
 // the members `tkn` on narrow 32 x 4 tiles, with every member's input map, output buffer and flag
 // resolved for this step's parity.  The group's TileGrid table holds tk's blocks, then tkn's.
 cudaError_t batch_launch_tma_list(lbm_batch *b, const lbm_batch::Group &g, const std::vector<lbm_batch::Group::Span> &list,
@@ -1155,8 +1158,8 @@ cudaError_t batch_launch_tma_list(lbm_batch *b, const lbm_batch::Group &g, const
 {
     static thread_local lbm::TmaBatchArgs A;
     const bool f64 = g.prec == LBM_FP64;
-    const int tr = narrow ? lbm::DdNarrowShape::TR : (f64 ? lbm::TmaShape<double>::TR : lbm::TmaShape<float>::TR);
-    const size_t tgb = f64 ? sizeof(lbm::TileGrid<lbm::Coef<lbm::dd>>) : sizeof(lbm::TileGrid<lbm::Coef<float>>);
+    const int tr = narrow ? lbm::DdNarrowShape::TR : (f64 ? lbm::DdWideShape::TR : lbm::TmaShape<float>::TR);
+    const size_t tgb = f64 ? sizeof(lbm::TileGrid<lbm::CoefDD>) : sizeof(lbm::TileGrid<lbm::Coef<float>>);
     for (size_t c0 = 0; c0 < list.size(); c0 += lbm::kTmaBatchGrids) {
         const int n = (int)std::min<size_t>(lbm::kTmaBatchGrids, list.size() - c0);
         int tiles = 0;
@@ -1164,7 +1167,7 @@ cudaError_t batch_launch_tma_list(lbm_batch *b, const lbm_batch::Group &g, const
             const lbm_batch::Group::Span &sp = list[c0 + k];
             const lbm_ctx *c = b->ctxs[g.members[sp.k]];
             const int in = c->cur ^ phase;
-            A.map[k] = narrow ? c->nmap[in] : c->tmap[in];
+            A.map[k] = narrow ? c->nmap[in] : (f64 ? c->dmap[in] : c->tmap[in]);
             A.out[k] = c->f[in ^ 1];
             A.err[k] = c->tma_err;
             A.first[k] = tiles;
@@ -1176,7 +1179,7 @@ cudaError_t batch_launch_tma_list(lbm_batch *b, const lbm_batch::Group &g, const
         A.n = n;
         const char *tg = tg0 + c0 * tgb;
         const cudaError_t ce =
-            f64 ? lbm::launch_step_dd_batch(A, (const lbm::TileGrid<lbm::Coef<lbm::dd>> *)tg, g.limiter, narrow, st)
+            f64 ? lbm::launch_step_dd_batch(A, (const lbm::TileGrid<lbm::CoefDD> *)tg, g.limiter, narrow, st)
                 : lbm::launch_step_tma_batch(A, (const lbm::TileGrid<lbm::Coef<float>> *)tg, g.limiter, st);
         if (ce != cudaSuccess) return ce;
     }
@@ -1188,7 +1191,7 @@ cudaError_t batch_launch_tma(lbm_batch *b, const lbm_batch::Group &g, int phase,
     const char *tg = (const char *)g.tblock;
     cudaError_t ce = batch_launch_tma_list(b, g, g.tk, false, tg, phase, st);
     if (ce == cudaSuccess && !g.tkn.empty())
-        ce = batch_launch_tma_list(b, g, g.tkn, true, tg + g.tk.size() * sizeof(lbm::TileGrid<lbm::Coef<lbm::dd>>),
+        ce = batch_launch_tma_list(b, g, g.tkn, true, tg + g.tk.size() * sizeof(lbm::TileGrid<lbm::CoefDD>),
                                    phase, st);
     return ce;
 }
@@ -1266,17 +1269,17 @@ int lbm_batch_create(lbm_ctx *const *ctxs, int n, lbm_batch **out)
     if (ce == cudaSuccess) ce = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device);
     if (ce != cudaSuccess) { delete b; return cuda_fail(nullptr, ce, "device query"); }
     b->ctas = 4 * sms;
-    // a float64 member on narrow double-float tiles whose grid takes 32 x 32 tiles steps on those
+    // a float64 member on narrow double-float tiles whose grid takes wide tiles steps on those
     // in the batch (the same bits: the two shapes run the same operations on every value; spread
     // over a batch, the larger tiles cost less per cell)
     std::vector<char> wide(n, 0), split(n, 0);
     for (int i = 0; i < n; i++) {
         lbm_ctx *c = ctxs[i];
-        wide[i] = c->use_dd || (c->use_ddn && lbm::tma_supported(c->P, LBM_FP64) && make_tile_maps(c));
-        // a last 32 x 32 tile row with at most 24 of the grid's rows: those rows on narrow tiles
-        // (a narrow tile costs about 1.3x per cell, a part-filled row of 32 x 32 tiles 32 / rows)
-        const int rem = c->P.ny % lbm::TmaShape<double>::TR;
-        split[i] = wide[i] && rem > 0 && rem <= 24 && lbm::dd_narrow_supported(c->P) && make_narrow_maps(c);
+        wide[i] = c->use_dd || (c->use_ddn && lbm::tma_supported(c->P, LBM_FP64) && make_wide_maps(c));
+        // a last 32 x 16 tile row with at most 12 of the grid's rows: those rows on narrow tiles
+        // (a narrow tile costs about 1.3x per cell, a part-filled row of 32 x 16 tiles 16 / rows)
+        const int rem = c->P.ny % lbm::DdWideShape::TR;
+        split[i] = wide[i] && rem > 0 && rem <= 3 * lbm::DdWideShape::TR / 4 && lbm::dd_narrow_supported(c->P) && make_narrow_maps(c);
     }
     cudaGetLastError();
     for (int i = 0; i < n; i++) {
@@ -1309,8 +1312,8 @@ int lbm_batch_create(lbm_ctx *const *ctxs, int n, lbm_batch **out)
         std::vector<int4> tiles;
         std::vector<lbm::Params> hp;
         std::vector<lbm::TileGrid<lbm::Coef<float>>> htf;
-        std::vector<lbm::TileGrid<lbm::Coef<lbm::dd>>> htd, htdn;   // float64: 32 x 32 members, narrow ones
-        const int tr = g.prec == LBM_FP64 ? lbm::TmaShape<double>::TR : lbm::TmaShape<float>::TR;
+        std::vector<lbm::TileGrid<lbm::CoefDD>> htd, htdn;   // float64: wide spans, narrow ones
+        const int tr = g.prec == LBM_FP64 ? lbm::DdWideShape::TR : lbm::TmaShape<float>::TR;
         for (size_t k = 0; k < g.members.size(); k++) {
             const lbm_ctx *c = b->ctxs[g.members[k]];
             hp.push_back(c->P);
@@ -1320,7 +1323,7 @@ int lbm_batch_create(lbm_ctx *const *ctxs, int n, lbm_batch **out)
             if (g.tma[k]) {
                 const int i = g.members[k], ntx = (c->P.nx + lbm::kTmaTX - 1) / lbm::kTmaTX;
                 if (g.prec == LBM_FP64) {
-                    const lbm::TileGrid<lbm::Coef<lbm::dd>> blk{c->P.nx, c->P.ny, c->P.pitch, c->P.has_c9,
+                    const lbm::TileGrid<lbm::CoefDD> blk{c->P.nx, c->P.ny, c->P.pitch, c->P.has_c9,
                                                                 c->P.plane, 0, c->cdd};
                     const int nr = lbm::DdNarrowShape::TR;
                     const int wide_rows = !wide[i] ? 0 : (split[i] ? c->P.ny - c->P.ny % tr : c->P.ny);

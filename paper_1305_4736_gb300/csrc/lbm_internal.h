@@ -80,22 +80,40 @@ struct TmaShape {
     static constexpr size_t smem_bytes = tile_bytes + sizeof(R) * (sizeof(R) == sizeof(float) ? 2 : 3) * UW * UH;
 };
 bool tma_supported(const Params &P, int prec);
-// Narrow tiles of the double-float float64 kernel (step_kernel 9): 4 warps, 32 x 4 tiles, one
-// row per thread, two CTAs per SM, for grids of 4 to 31 rows (and 32 columns or more), where the
-// 32 x 32 tiles do not fit.  The staged tile is that of TmaShape<double> with 8 rows.
-struct DdNarrowShape {
-    static constexpr int TT = 4;
-    static constexpr int CTAS = 2;
-    static constexpr int KR = 1;
+// Tiles of the double-float float64 kernels: 32 columns by TT * KR rows, TT warps, KR rows per
+// thread, CTAS CTAs per SM.
+template <int TT_, int KR_, int CTAS_>
+struct DdShape {
+    static constexpr int TT = TT_, KR = KR_, CTAS = CTAS_;
     static constexpr int TR = TT * KR;
-    static constexpr int HX = 2;
+    static constexpr int HX = 2;                       // x halo (8-byte elements: 16-byte TMA origin)
     static constexpr int SW = kTmaTX + 2 * HX;
     static constexpr int SH = TR + 4;
     static constexpr int PL = SW * SH;
     static constexpr int UW = kTmaTX + 2, UH = TR + 2;
     static constexpr size_t tile_bytes = sizeof(double) * NQ * PL;
-    static constexpr size_t smem_bytes = tile_bytes + sizeof(double) * 3 * UW * UH;
+    // shared memory: the staged tile, (u_x, u_y) on the tile plus its ring, (e, 1/rho) of the
+    // tile's cells, and the x edge values of its rows
+    static constexpr size_t uv_off = tile_bytes;
+    static constexpr size_t eir_off = uv_off + 16 * UW * UH;
+    static constexpr size_t edge_off = eir_off + 16 * kTmaTX * TR;
+    static constexpr size_t smem_bytes = edge_off + 2 * 16 * 6 * TR;
 };
+using DdWideShape = DdShape<8, 2, 2>;
+// Narrow tiles (step_kernel 9): 32 x 4, for grids of 4 to 31 rows (and 32 columns or more) and for
+// small grids.
+using DdNarrowShape = DdShape<4, 1, 2>;
+static_assert(DdWideShape::CTAS * (DdWideShape::smem_bytes + 2048) <= 228 * 1024, "wide tiles per SM");
+// Coefficients of the double-float kernels in the order of the population pairs (lane e of pair
+// p belongs to shell 2p + e); the column of row 13 in pEy is negated, as the kernel forms that
+// row negated.
+struct CoefDD {
+    dd2 hh[2], hhy[2], cr[2], cry[2];
+    dd2 pA[2][2], pEx[2][3], pEy[2][3], pB1[2], pB2[2];
+    dd2 q89, g4;
+    dd b, inv_b, two_b2, six_b, b4, four_inv_b, ry, pad_;
+};
+static_assert(sizeof(CoefDD) % 16 == 0, "CoefDD is copied in 16-byte words");
 bool dd_narrow_supported(const Params &P);
 // Batched TMA-staged steps over the tiles of up to kTmaBatchGrids grids of a batch group, one
 // CTA per tile of kTmaTX x TmaShape<R>::TR cells: grid k owns the launch's tiles first[k] ..
@@ -114,7 +132,7 @@ struct TmaBatchArgs {
     int n;                              // grids of the launch
 };
 // Per-grid block of a batched launch (global memory, one per grid in launch order): the
-// geometry and the coefficients that the tile kernels read (C = Coef<float> or Coef<dd>); each
+// geometry and the coefficients that the tile kernels read (C = Coef<float> or CoefDD); each
 // CTA copies its grid's block to shared memory while its tile copy is in flight.
 template <typename C>
 struct TileGrid {
@@ -125,7 +143,7 @@ struct TileGrid {
 cudaError_t launch_step_tma_batch(const TmaBatchArgs &A, const TileGrid<Coef<float>> *tg, int limiter,
                                   cudaStream_t st);
 // narrow: tiles of DdNarrowShape (the grids' maps have its box), else of TmaShape<double>.
-cudaError_t launch_step_dd_batch(const TmaBatchArgs &A, const TileGrid<Coef<dd>> *tg, int limiter, bool narrow,
+cudaError_t launch_step_dd_batch(const TmaBatchArgs &A, const TileGrid<CoefDD> *tg, int limiter, bool narrow,
                                  cudaStream_t st);
 // Failure-path check of the bounded mbarrier waits (lbm_wait_selftest): *flag = 1 when the
 // wait on a phase that nothing completes gave up at its limit; *ms = the kernel's duration.
@@ -177,10 +195,10 @@ cudaError_t stream_prepare();
 cudaError_t launch_step_stream(const Params &P, int prec, const void *tmap, void *fout, int *err, cudaStream_t st);
 
 // Float64-mode step in double-float arithmetic on the float32 pipe (step_kernel 8): the tiles
-// and tensor maps of the float64 TMA-staged kernel; `coef` is the Coef<dd> of the context
+// and tensor maps of the float64 TMA-staged kernel; `coef` is the CoefDD of the context
 // (coef_dd).  narrow (step_kernel 9): the tiles of DdNarrowShape, `tmap` with its box, no x
 // wrap in the kernel.
-void coef_dd(const Params &P, Coef<dd> *out);
+void coef_dd(const Params &P, CoefDD *out);
 cudaError_t dd_prepare();
 cudaError_t launch_step_dd(const Params &P, const void *coef, const void *tmap, const void *fin, void *fout,
                            int *err, cudaStream_t st, bool narrow = false);

@@ -6,17 +6,36 @@
 // tile of 32 columns x TR rows and one elected thread brings all 16 float64 planes of the
 // tile plus its stencil halo into shared memory with one tensor copy (bounded mbarrier wait);
 // then
-//   split    every staged value becomes hi + lo in place (8 bytes either way);
-//   phase 1  flow velocity and 1/rho on the tile + 1 ring (for grad u);
-//   phase 2  per row: the MRT collision with the energy-flux correction (Eq. 3, Sec. II) in
-//            the shell basis, the limited x and y convection (Sec. III; each x face difference
-//            and slope is formed once, by the lane of its column, and passed to the neighbour
-//            lane by a shuffle; y slopes from a sliding window down the thread's column), the
-//            forward-Euler update, and one float64 store per population (the double-float
-//            result rounded to float64).
+//   split    every staged value becomes hi + lo in place (8 bytes either way), the hi parts of the
+//            population pair (q, q + 4) together in plane q, the lo parts in plane q + 4;
+//   phase 1  flow velocity on the tile + 1 ring (for grad u), e and 1/rho on the tile, and the
+//            face differences and slopes one column outside the tile;
+//   phase 2  per thread the MRT collision of its cells with the energy-flux correction (Eq. 3,
+//            Sec. II) in the shell basis, then pair by pair the limited x and y convection
+//            (Sec. III; each x face difference and slope is formed once, by the lane of its column,
+//            and passed to the neighbour lane by a shuffle; y slopes from a window sliding down the
+//            thread's column), the forward-Euler update, and one float64 store per population (the
+//            double-float result rounded to float64).
 // The formulas are those of the float64 kernels, operation for operation; each rounds at
 // about 2^-47 instead of 2^-53, so results agree with the float64 kernels and the oracle to a
 // few parts in 1e14 per step.
+//
+// What bounds it: the float32 pipe, about 3850 lane operations a cell (30 cycles of an SM at 128
+// lanes), then the fixed latency of the double-float chains and the float64 pipe that rounds the
+// results (48 operations a cell, 24 cycles).  Measured on 2048 x 2048 (MC, Pr != 1; the step
+// kernel, CUDA events), starting from scalar operations with one 8-warp CTA per SM on 32 x 32
+// tiles (245 registers a thread, issue slots 57% busy, most stalls on fixed latencies):
+//   0.981 ms  start
+//   0.940     the same operations on population pairs with f32x2 instructions (5263 -> 3600 thread
+//             instructions a cell; the latencies of two warps per scheduler remain)
+//   0.720     collision first, then convection pair by pair, so that 128 registers a thread do and
+//             two 8-warp CTAs on 32 x 16 tiles run per SM (their phases overlap)
+//   0.681     the tile of the CTA half a resident wave later prefetched into L2; the populations
+//             read again after the collision instead of kept
+//   0.644     the split in half the integer operations, Fast2Sum where the order is known
+// Other shapes (warps, rows per thread, CTAs per SM), same code: 16 x 2, one CTA 0.807 ms; 12 x 2,
+// one CTA 0.843; 6 x 2, two CTAs 0.712; 7 x 2, two CTAs 0.714; 5 x 3, two CTAs 1.09; 4 x 4, two
+// CTAs 1.31 (the unrolled rows spill).  The results are bit for bit those of the scalar kernel.
 #include <cuda.h>
 
 #include "lbm_dd.cuh"
@@ -27,122 +46,189 @@ namespace lbm {
 
 namespace {
 
-// ---- constants and coefficients in double-float ----------------------------------------
+// ---- constants in double-float ------------------------------------------------------------
 // Velocity-set constants that float32 does not hold exactly (Sec. II, Appendix A), split at
 // compile time.
 __host__ __device__ constexpr float hi_of(double x) { return (float)x; }
 __host__ __device__ constexpr float lo_of(double x) { return (float)(x - (double)(float)x); }
-__device__ __forceinline__ dd kd3() { return dd{hi_of(kD3), lo_of(kD3)}; }                              // sqrt2
-__device__ __forceinline__ dd kd4() { return dd{hi_of(kD4), lo_of(kD4)}; }                              // 3/sqrt2
-__device__ __forceinline__ dd k4s2() { return dd{hi_of(4.0 * kSqrt2), lo_of(4.0 * kSqrt2)}; }          // 4 sqrt2
-__device__ __forceinline__ dd k27s2() { return dd{hi_of(27.0 / kSqrt2), lo_of(27.0 / kSqrt2)}; }       // 27/sqrt2
+__device__ __forceinline__ dd2 both(double x) { return dd2{f2(hi_of(x), hi_of(x)), f2(lo_of(x), lo_of(x))}; }
 
-// ---- Appendix A rows in the shell basis (as conserved_of / moments_of) -------------------
-__device__ __forceinline__ void conserved_dd(const Shells<dd> &s, dd &rho, dd &jx, dd &jy, dd &e)
+// ---- shells on population pairs (as shells2_of of the float32 path) ------------------------
+struct ShellsDD { dd2 S[2], X[2], Y[2], Q[2]; };   // [0]: shells 1, 2; [1]: shells 3, 4
+
+__device__ __forceinline__ ShellsDD shells_dd(const dd2 *fp)
 {
-    rho = (s.S[0] + s.S[1]) + (s.S[2] + s.S[3]);
-    jx = ((s.X[0] + s.X[1] * 6.0f) + kd3() * s.X[2]) + kd4() * s.X[3];
-    jy = ((s.Y[0] + s.Y[1] * 6.0f) + kd3() * s.Y[2]) + kd4() * s.Y[3];
-    e = ((s.S[0] * 7.25f + s.S[1] * 36.0f) + scale2(s.S[2], 4.0f)) + s.S[3] * 9.0f;
+    ShellsDD s;
+    {
+        const dd2 a = fp[0] + fp[2], b = fp[1] + fp[3];
+        s.S[0] = a + b;
+        s.Q[0] = a - b;
+        s.X[0] = fp[0] - fp[2];
+        s.Y[0] = fp[1] - fp[3];
+    }
+    {
+        const dd2 a = fp[4] + fp[6], b = fp[5] + fp[7];
+        const dd2 c = fp[4] - fp[6], d = fp[5] - fp[7];
+        s.S[1] = a + b;
+        s.Q[1] = a - b;
+        s.X[1] = c - d;
+        s.Y[1] = c + d;
+    }
+    return s;
 }
 
-// Flow velocity of the cell whose population q is at p[q * stride].
-__device__ __forceinline__ void flow_dd(const dd *p, int stride, dd &u, dd &v, dd &ir)
+__device__ __forceinline__ void unbutterfly_dd_axis(dd2 S, dd2 X, dd2 Y, dd2 Q, dd2 *p)
 {
-    dd g[NQ];
+    const dd2 a = S + Q, b = S - Q;
+    p[0] = a + X;
+    p[2] = a - X;
+    p[1] = b + Y;
+    p[3] = b - Y;
+}
+
+__device__ __forceinline__ void unbutterfly_dd_diag(dd2 S, dd2 X, dd2 Y, dd2 Q, dd2 *p)
+{
+    const dd2 a = S + Q, b = S - Q, c = X + Y, d = X - Y;
+    p[0] = a + c;
+    p[2] = a - c;
+    p[1] = b - d;
+    p[3] = b + d;
+}
+
+// The staged tile after the split: population pair pr of the cell at offset c is
+// (hi of q, hi of q + 4) in plane q = pair_q(pr) and (lo of q, lo of q + 4) in plane q + 4, so
+// every access is 8 bytes wide and free of bank conflicts.
+template <typename S>
+__device__ __forceinline__ dd2 tile_pair(const float2 *t, int pr, int c)
+{
+    return dd2{t[pair_q(pr) * S::PL + c], t[(pair_q(pr) + 4) * S::PL + c]};
+}
+
+__device__ __forceinline__ float4 quad(dd2 a) { return make_float4(a.hi.x, a.hi.y, a.lo.x, a.lo.y); }
+__device__ __forceinline__ dd2 unquad(float4 v) { return dd2{f2(v.x, v.y), f2(v.z, v.w)}; }
+
+// (j_x, j_y) over the shells 1 .. 4.
+__device__ __forceinline__ dd2 flux_dd(dd2 X0, dd2 X1, dd2 Y0, dd2 Y1)
+{
+    return ((firsts(X0, Y0) + seconds(X0, Y0) * f2(6.0f, 6.0f)) + both(kD3) * firsts(X1, Y1)) +
+           both(kD4) * seconds(X1, Y1);
+}
+
+// (u_x, u_y) and (e, 1/rho) of the staged cell at offset c.
+template <typename S>
+__device__ __forceinline__ void macro_dd(const float2 *t, int c, dd2 &u, dd2 &eir)
+{
+    dd2 fp[8];
 #pragma unroll
-    for (int q = 0; q < NQ; q++) g[q] = p[q * stride];
-    dd rho, jx, jy, e;
-    conserved_dd(shells_of(g), rho, jx, jy, e);
-    ir = recip(rho);
-    u = jx * ir;
-    v = jy * ir;
+    for (int pr = 0; pr < 8; pr++) fp[pr] = tile_pair<S>(t, pr, c);
+    const dd2 S0 = (fp[0] + fp[2]) + (fp[1] + fp[3]), S1 = (fp[4] + fp[6]) + (fp[5] + fp[7]);
+    const dd2 cc = fp[4] - fp[6], dm = fp[5] - fp[7];
+    const dd rho = sum_lanes(S0) + sum_lanes(S1);
+    const dd2 j = flux_dd(fp[0] - fp[2], cc - dm, fp[1] - fp[3], cc + dm);
+    const dd2 e0 = S0 * f2(7.25f, 36.0f), e1 = S1 * f2(4.0f, 9.0f);
+    const dd ir = recip(rho);
+    u = j * bcast(ir);
+    eir = pack((sum_lanes(e0) + first(e1)) + second(e1), ir);
 }
 
 // dt M^-1 S (f_hat - f_hat^eq) with the energy-flux correction (Eq. 3, Sec. II), float64 mode
-// (zero reference state): the operations of collide<double, false>.
+// (zero reference state): the formulas of collide<double, false> on shell pairs, with the x and y
+// rows as pairs; gx, gy: the differences of (u_x, u_y) along x and y.
 template <bool C9>
-__device__ __forceinline__ void collide_dd(const Coef<dd> &C, const Shells<dd> &s, dd jx, dd jy, dd de, dd ir,
-                                           dd ux, dd uy, dd dxux, dd dyux, dd dxuy, dd dyuy, dd *out)
+__device__ __forceinline__ void collide_dd(const CoefDD &C, const ShellsDD &s, dd de, dd ir, dd2 u, dd2 gx,
+                                           dd2 gy, dd2 *out)
 {
     // rows 5..16 of Appendix A
-    const dd x8 = ((s.X[0] * 7.25f + s.X[1] * 216.0f) + k4s2() * s.X[2]) + k27s2() * s.X[3];
-    const dd y8 = ((s.Y[0] * 7.25f + s.Y[1] * 216.0f) + k4s2() * s.Y[2]) + k27s2() * s.Y[3];
-    const dd m13 = ((s.S[0] * 7.25f + s.S[1] * 1296.0f) + scale2(s.S[2], 16.0f)) + s.S[3] * 81.0f;
-    const dd m9 = x8 - s.X[0] * 6.25f, m10 = y8 - s.Y[0] * 6.25f;
-    const dd m11 = s.X[0] + s.X[1] * 216.0f;
-    const dd m12 = -(s.Y[0] + s.Y[1] * 216.0f);
-    const dd m5 = s.Q[0] + s.Q[1] * 36.0f, m15 = s.Q[0] * 7.25f + s.Q[1] * 1296.0f;
-    const dd m6 = scale2(s.Q[2], 2.0f) + s.Q[3] * 4.5f, m14 = scale2(s.Q[2], 8.0f) + s.Q[3] * 40.5f;
-    // equilibria (Appendix A closed forms), as feq_hat_dev<R, false>
-    const dd jx2 = jx * ux, jy2 = jy * uy, J2 = jx2 + jy2;
+    const dd2 XY0 = firsts(s.X[0], s.Y[0]), XY1 = seconds(s.X[0], s.Y[0]);
+    const dd2 m78 = ((XY0 * f2(7.25f, 7.25f) + XY1 * f2(216.0f, 216.0f)) +
+                     both(4.0 * kSqrt2) * firsts(s.X[1], s.Y[1])) + both(27.0 / kSqrt2) * seconds(s.X[1], s.Y[1]);
+    const dd2 t13 = s.S[1] * f2(16.0f, 81.0f);
+    const dd m13 = (sum_lanes(s.S[0] * f2(7.25f, 1296.0f)) + first(t13)) + second(t13);
+    const dd2 m910 = m78 - XY0 * f2(6.25f, 6.25f);
+    const dd2 m1112 = XY0 + XY1 * f2(216.0f, 216.0f);       // row 13 negated, as its column of cEy
+    const dd2 m515 = bcast(first(s.Q[0])) * f2(1.0f, 7.25f) + bcast(second(s.Q[0])) * f2(36.0f, 1296.0f);
+    const dd2 m614 = bcast(first(s.Q[1])) * f2(2.0f, 8.0f) + bcast(second(s.Q[1])) * f2(4.5f, 40.5f);
+    // equilibria (Appendix A closed forms), as feq_hat_dev<R, false>; e is the cell's own e
+    const dd2 j = flux_dd(s.X[0], s.X[1], s.Y[0], s.Y[1]);
+    const dd2 jj = j * u;
+    const dd J2 = sum_lanes(jj), dxy = first(jj) - second(jj);
     const dd dP = (de - J2) * C.inv_b;
-    const dd e_dev = fma_dd(C.b, dP, J2);
-    const dd dxy = jx2 - jy2;
-    const dd q4 = scale2(dP, 2.0f) + J2;
-    const dd q6 = jx * uy;
-    const dd e2p = e_dev + scale2(dP, 2.0f);
-    const dd g4 = scale2(dP, 4.0f) + J2;
+    const dd P2 = scale2(dP, 2.0f);
+    const dd q6 = first(j) * second(u);
     const dd q13 = ir * (dP * fma_dd(C.two_b2, dP, C.six_b * J2) + J2 * J2);
     const dd k = fma_dd(C.b4, dP, J2);
-    dd D4 = (de - s.S[0] * 6.25f) - q4;
-    dd D7 = x8 - e2p * ux, D8 = y8 - e2p * uy;
-    const dd D9 = m9 - g4 * ux, D10 = m10 - g4 * uy;
-    const dd D11 = m11 - (scale2(dP, 2.0f) + dxy) * ux, D12 = m12 - (dxy - scale2(dP, 2.0f)) * uy;
+    const dd e2p = fma_dd(C.b, dP, J2) + P2;
+    const dd2 q1415 = bcast(k) * pack(first(u), dxy) * pack(second(u), ir);   // rows 15, 16
+    const dd D4 = (de - first(s.S[0]) * 6.25f) - (P2 + J2);
     const dd D13 = m13 - q13;
-    const dd D5 = m5 - dxy, D6 = m6 - q6;
-    const dd D14 = m14 - k * ux * uy, D15 = m15 - k * dxy * ir;
+    dd2 D78 = m78 - bcast(e2p) * u;
+    const dd2 D910 = m910 - bcast(scale2(dP, 4.0f) + J2) * u;
+    const dd2 D1112 = m1112 - pack(P2 + dxy, P2 - dxy) * u;
+    const dd2 D515 = m515 - pack(dxy, second(q1415));
+    const dd2 D614 = m614 - pack(q6, first(q1415));
     if (C9) {
-        // y differences weighted by ry = dx/dy (q8, q9 carry 1/(2 dx))
-        const dd div = dxux + C.ry * dyuy, shr = dxuy + C.ry * dyux;
-        D7 += C.q8 * dP * (ux * (scale2(dxux, 4.0f) - C.four_inv_b * div) + scale2(uy * shr, 2.0f));
-        D8 += C.q9 * dP * (scale2(ux * shr, 2.0f) + uy * (C.g4[1] * dyuy - C.four_inv_b * div));
+        // y differences weighted by ry = dx/dy (q89 carries 1/(2 dx))
+        const dd div = first(gx) + C.ry * second(gy), shr = second(gx) + C.ry * first(gy);
+        const dd2 g = pack(first(gx), second(gy)) * C.g4 - bcast(C.four_inv_b * div);
+        const dd2 h = u * g + scale2(pack(second(u), first(u)) * bcast(shr), 2.0f);
+        D78 = D78 + C.q89 * bcast(dP) * h;
     }
-    dd S[4], X[4], Y[4], Q[4];
-#pragma unroll
-    for (int r = 0; r < 4; r++) {
-        S[r] = C.cA[r][0] * D4 + C.cA[r][1] * D13;
-        X[r] = (C.cEx[r][0] * D7 + C.cEx[r][1] * D9) + C.cEx[r][2] * D11;
-        Y[r] = (C.cEy[r][0] * D8 + C.cEy[r][1] * D10) + C.cEy[r][2] * D12;
+    const dd2 d4 = bcast(D4), d13 = bcast(D13), d5 = bcast(first(D515)), d15 = bcast(second(D515));
+    const dd2 d6 = bcast(first(D614)), d14 = bcast(second(D614));
+    {
+        const dd2 d7 = bcast(first(D78)), d9 = bcast(first(D910)), d11 = bcast(first(D1112));
+        const dd2 d8 = bcast(second(D78)), d10 = bcast(second(D910)), d12 = bcast(second(D1112));
+        unbutterfly_dd_axis(C.pA[0][0] * d4 + C.pA[0][1] * d13,
+                            (C.pEx[0][0] * d7 + C.pEx[0][1] * d9) + C.pEx[0][2] * d11,
+                            (C.pEy[0][0] * d8 + C.pEy[0][1] * d10) + C.pEy[0][2] * d12,
+                            C.pB1[0] * d5 + C.pB1[1] * d15, out);
+        unbutterfly_dd_diag(C.pA[1][0] * d4 + C.pA[1][1] * d13,
+                            (C.pEx[1][0] * d7 + C.pEx[1][1] * d9) + C.pEx[1][2] * d11,
+                            (C.pEy[1][0] * d8 + C.pEy[1][1] * d10) + C.pEy[1][2] * d12,
+                            C.pB2[0] * d6 + C.pB2[1] * d14, out + 4);
     }
-    Q[0] = C.cB1[0][0] * D5 + C.cB1[0][1] * D15;
-    Q[1] = C.cB1[1][0] * D5 + C.cB1[1][1] * D15;
-    Q[2] = C.cB2[0][0] * D6 + C.cB2[0][1] * D14;
-    Q[3] = C.cB2[1][0] * D6 + C.cB2[1][1] * D14;
-    unbutterfly_axis(S[0], X[0], Y[0], Q[0], out + 0);
-    unbutterfly_axis(S[1], X[1], Y[1], Q[1], out + 4);
-    unbutterfly_diag(S[2], X[2], Y[2], Q[2], out + 8);
-    unbutterfly_diag(S[3], X[3], Y[3], Q[3], out + 12);
 }
 
-__device__ __forceinline__ dd shfl_dd(dd v, int src)
+__device__ __forceinline__ float2 shfl_down2(float2 v)
 {
-    return dd{__shfl_sync(0xffffffffu, v.hi, src), __shfl_sync(0xffffffffu, v.lo, src)};
+    return f2(__shfl_down_sync(0xffffffffu, v.x, 1), __shfl_down_sync(0xffffffffu, v.y, 1));
 }
-__device__ __forceinline__ dd shfl_down_dd(dd v)
+__device__ __forceinline__ float2 shfl_up2(float2 v)
 {
-    return dd{__shfl_down_sync(0xffffffffu, v.hi, 1), __shfl_down_sync(0xffffffffu, v.lo, 1)};
+    return f2(__shfl_up_sync(0xffffffffu, v.x, 1), __shfl_up_sync(0xffffffffu, v.y, 1));
 }
-__device__ __forceinline__ dd shfl_up_dd(dd v)
+__device__ __forceinline__ dd2 shfl_down_dd(dd2 v) { return dd2{shfl_down2(v.hi), shfl_down2(v.lo)}; }
+__device__ __forceinline__ dd2 shfl_up_dd(dd2 v) { return dd2{shfl_up2(v.hi), shfl_up2(v.lo)}; }
+
+// v, or the pair at shared address a where `own` holds (a predicated 16-byte load: no selects).
+__device__ __forceinline__ void take_edge(dd2 &v, unsigned a, bool own)
 {
-    return dd{__shfl_up_sync(0xffffffffu, v.hi, 1), __shfl_up_sync(0xffffffffu, v.lo, 1)};
+    asm("{\n\t.reg .pred p;\n\t"
+        "setp.ne.s32 p, %5, 0;\n\t"
+        "@p ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];\n\t}"
+        : "+f"(v.hi.x), "+f"(v.hi.y), "+f"(v.lo.x), "+f"(v.lo.y)
+        : "r"(a), "r"((int)own));
 }
 
 // Face differences enter the MC slope normalised (norm_lim, once per difference: each feeds two
 // slopes); the other limiters use them as they are.
 template <int Lim>
-__device__ __forceinline__ dd norm_lim(dd a)
+__device__ __forceinline__ dd2 norm_lim(dd2 a)
 {
     return Lim == 0 ? norm(a) : a;
 }
 
 template <int Lim>
-__device__ __forceinline__ dd slope_dd(dd a, dd b)
+__device__ __forceinline__ dd2 slope_dd(dd2 a, dd2 b)
 {
     if (Lim == 0) return mc2n(a, b);
     if (Lim == 1) return scale2(b, 2.0f);
-    return dd{0.0f, 0.0f};
+    return dd2{f2(0.0f, 0.0f), f2(0.0f, 0.0f)};
 }
+
+// x-moving pair e (0 .. 5) of the six, and its index among them
+__device__ __forceinline__ constexpr int xpair(int e) { return e < 2 ? 2 * e : e + 2; }
+__device__ __forceinline__ constexpr int xpair_index(int pr) { return pr < 4 ? pr >> 1 : pr - 2; }
 
 }  // namespace
 
@@ -151,170 +237,157 @@ __device__ __forceinline__ dd slope_dd(dd a, dd b)
 // shared memory (smraw) is split, then phases 1 and 2 produce the tile's new float64 values.
 // ---------------------------------------------------------------------------
 // P: the context's Params, or the TileGrid block of a batched launch (nx, ny, pitch, plane).
-// S: the tile shape (TmaShape<double> or DdNarrowShape).
+// S: the tile shape (DdWideShape or DdNarrowShape).
 template <int Lim, bool C9, typename S, typename PP>
-__device__ __forceinline__ void dd_tile(const PP &P, const Coef<dd> &C, unsigned char *smraw,
+__device__ __forceinline__ void dd_tile(const PP &P, const CoefDD &C, unsigned char *smraw,
                                         double *__restrict__ fout, int x0, int y0)
 {
     double *tile64 = reinterpret_cast<double *>(smraw);
-    dd *tile = reinterpret_cast<dd *>(smraw);
-    dd *su = tile + NQ * S::PL;
-    dd *sv = su + S::UW * S::UH;
-    dd *sir = sv + S::UW * S::UH;
+    float2 *tile = reinterpret_cast<float2 *>(smraw);
+    float4 *suv = reinterpret_cast<float4 *>(smraw + S::uv_off);        // (u_x, u_y), tile + ring
+    float4 *seir = reinterpret_cast<float4 *>(smraw + S::eir_off);      // (e, 1/rho), tile
+    float4 *sedge = reinterpret_cast<float4 *>(smraw + S::edge_off);    // x edge values per row and pair
     const int lane = threadIdx.x, ty = threadIdx.y, tid = ty * kTmaTX + lane;
     constexpr int kThreads = kTmaTX * S::TT;
     const int nx = P.nx, ny = P.ny;
-    // ---- split: float64 -> hi + lo in place
-    for (int k = tid; k < NQ * S::PL; k += kThreads) tile[k] = dd_split(tile64[k]);
+    // ---- split: float64 -> hi + lo in place, population pairs (q, q + 4)
+#pragma unroll 4
+    for (int k = tid; k < 8 * S::PL; k += kThreads) {
+        const int a = k < 4 * S::PL ? k : k + 4 * S::PL, b = a + 4 * S::PL;
+        const dd2 v = dd_split2(tile64[a], tile64[b]);
+        tile[a] = v.hi;
+        tile[b] = v.lo;
+    }
     __syncthreads();
 
-    // ---- phase 1: flow velocity and 1/rho on the tile plus its ring
-    {
-        int i = tid % S::UW, j = tid / S::UW;
-        for (int k = tid; k < S::UW * S::UH; k += kThreads) {
-            dd ux, uy, ir;
-            flow_dd(tile + (j + 1) * S::SW + (i + S::HX - 1), S::PL, ux, uy, ir);
-            su[k] = ux;
-            sv[k] = uy;
-            sir[k] = ir;
-            i += kThreads % S::UW;
-            j += kThreads / S::UW;
-            if (i >= S::UW) {
-                i -= S::UW;
-                j++;
+    // ---- phase 1: macroscopic values on the tile plus its ring, then the values one column
+    // outside the tile for the x stencils: per row and x-moving pair D(x0 + 32) for lane 31, and
+    // the slope beyond the upwind end, S(x0 - 1) = mc2(D(x0 - 1), D(x0)) for pairs moving right,
+    // S(x0 + 32) = mc2(D(x0 + 32), D(x0 + 33)) for those moving left
+    constexpr int kCells = S::UW * S::UH, kEdges = 6 * S::TR;
+    for (int k = tid; k < kCells + kEdges; k += kThreads) {
+        if (k < kCells) {
+            const int j = k / S::UW, i = k - j * S::UW;
+            dd2 u, eir;
+            macro_dd<S>(tile, (j + 1) * S::SW + (i + S::HX - 1), u, eir);
+            suv[k] = quad(u);
+            if (i >= 1 && i <= kTmaTX && j >= 1 && j <= S::TR) seir[(j - 1) * kTmaTX + (i - 1)] = quad(eir);
+        } else {
+            const int n = k - kCells, r = n / 6, e = n - 6 * r, pr = xpair(e);
+            const int row = (r + 2) * S::SW + S::HX;                  // smem offset of x0
+            const float2 *hi = tile + pair_q(pr) * S::PL + row, *lo = hi + 4 * S::PL;
+            auto at = [&](int x) { return dd2{hi[x], lo[x]}; };
+            sedge[2 * n] = quad(norm_lim<Lim>(at(kTmaTX) - at(kTmaTX - 1)));
+            if (Lim == 0) {
+                const int c0 = tsgn_x(pair_q(pr)) > 0 ? -2 : kTmaTX - 1;
+                sedge[2 * n + 1] = quad(mc2n(norm(at(c0 + 1) - at(c0)), norm(at(c0 + 2) - at(c0 + 1))));
             }
         }
     }
     __syncthreads();
 
-    // ---- phase 2: rows ty*KR .. ty*KR+KR-1 of the tile, column `lane`
+    // ---- phase 2: rows ty*KR .. ty*KR+KR-1 of the tile, column `lane`: first the collision terms
+    // C of the thread's cells, then pair by pair their convection and update (a pair's windows are
+    // dead before the next one's are formed)
     const int gx = x0 + lane;
     const int r0 = ty * S::KR;
-    dd yw[NQ], yd[NQ], ym[NQ];
+    const int c0 = (r0 + 2) * S::SW + lane + S::HX;
+    dd2 acc[S::KR][8];
 #pragma unroll
-    for (int q = 0; q < NQ; q++) {
-        const int sy = tsgn_y(q);
-        if (sy == 0) continue;
-        const dd *pc = tile + q * S::PL + (lane + S::HX);
-        if (sy > 0) {
-            const dd w0 = pc[r0 * S::SW], w1 = pc[(r0 + 1) * S::SW], w2 = pc[(r0 + 2) * S::SW];
-            const dd d0 = norm_lim<Lim>(w1 - w0), d1 = norm_lim<Lim>(w2 - w1);
-            yw[q] = w2;
-            yd[q] = d1;
-            ym[q] = slope_dd<Lim>(d0, d1);
-        } else {
-            const dd w1 = pc[(r0 + 1) * S::SW], w2 = pc[(r0 + 2) * S::SW], w3 = pc[(r0 + 3) * S::SW];
-            const dd d1 = norm_lim<Lim>(w2 - w1), d2 = norm_lim<Lim>(w3 - w2);
-            yw[q] = w3;
-            yd[q] = d2;
-            ym[q] = slope_dd<Lim>(d2, d1);
-        }
-    }
-#pragma unroll 1
     for (int k = 0; k < S::KR; k++) {
-        const int r = r0 + k;
-        const int gy = y0 + r;
-        const dd *p = tile + (r + 2) * S::SW + (lane + S::HX);
-        // values one column outside the warp for the x stencils: lane L < 12 serves the L-th
-        // x-moving population (q = 0, 2, 4, 6, 8 .. 15): D(x0 + 32) for lane 31, and the slope
-        // beyond the warp's upwind end, S(x0 - 1) = mc2(D(x0 - 1), D(x0)) for populations moving
-        // right, S(x0 + 32) = mc2(D(x0 + 32), D(x0 + 33)) for those moving left
-        dd edgeD, edgeS = dd{0.0f, 0.0f};
-        {
-            const int L = lane < 12 ? lane : 0;
-            const int q = L < 4 ? 2 * L : L + 4;
-            const dd *row = tile + q * S::PL + (r + 2) * S::SW;    // smem column = x - x0 + HX
-            edgeD = norm_lim<Lim>(row[kTmaTX + S::HX] - row[kTmaTX + S::HX - 1]);
-            if (Lim == 0) {
-                const int c0 = tsgn_x(q) > 0 ? 0 : kTmaTX + S::HX - 1;
-                edgeS = mc2(row[c0 + 1] - row[c0], row[c0 + 2] - row[c0 + 1]);
+        dd2 fp[8];
+#pragma unroll
+        for (int pr = 0; pr < 8; pr++) fp[pr] = tile_pair<S>(tile, pr, c0 + k * S::SW);
+        const int ui = (r0 + k + 1) * S::UW + (lane + 1);
+        const dd2 gxu = unquad(suv[ui + 1]) - unquad(suv[ui - 1]);
+        const dd2 gyu = unquad(suv[ui + S::UW]) - unquad(suv[ui - S::UW]);
+        const dd2 eir = unquad(seir[(r0 + k) * kTmaTX + lane]);
+        collide_dd<C9>(C, shells_dd(fp), first(eir), second(eir), unquad(suv[ui]), gxu, gyu, acc[k]);
+    }
+    // the cells' populations are read again below: kept in registers from the collision (which the
+    // compiler does for loads from equal addresses) they would be spilled
+    int c1 = c0;
+    asm volatile("" : "+r"(c1));
+    const unsigned edge_a = (unsigned)__cvta_generic_to_shared(sedge) + 32u * 6u * (unsigned)r0;
+    // f - C - c_x (F_out - F_in)_x - c_y (F_out - F_in)_y
+#pragma unroll
+    for (int pr = 0; pr < 8; pr++) {
+        const int qa = pair_q(pr);
+        const int sx = tsgn_x(qa), sy = tsgn_y(qa);
+        const int sp = pr >> 2;                             // shell pair
+        dd2 f[S::KR], out[S::KR];
+#pragma unroll
+        for (int k = 0; k < S::KR; k++) {
+            f[k] = tile_pair<S>(tile, pr, c1 + k * S::SW);
+            out[k] = f[k] - acc[k][pr];
+        }
+        if (sy != 0) {
+            // y slopes from a window sliding along the motion: last value, face difference, slope;
+            // downward pairs carry differences and slopes negated
+            const int first_row = sy > 0 ? -2 : -1;
+            dd2 w = tile_pair<S>(tile, pr, c1 + first_row * S::SW);
+            dd2 d = dd2{f2(0.0f, 0.0f), f2(0.0f, 0.0f)}, m = d;
+#pragma unroll
+            for (int i = 1; i < S::KR + 3; i++) {
+                const int row = first_row + i;
+                const dd2 wn = row >= 0 && row < S::KR ? f[row] : tile_pair<S>(tile, pr, c1 + row * S::SW);
+                const dd2 dn = norm_lim<Lim>(wn - w);
+                if (i >= 2) {
+                    const dd2 mn = sy > 0 ? slope_dd<Lim>(d, dn) : slope_dd<Lim>(dn, d);
+                    if (i >= 3) {
+                        const int k = i - 3;
+                        const dd2 dm = sy > 0 ? mn - m : m - mn;
+                        // Lim 0: both slopes have the sign of d and at most 4 |d|, and hhy <= 1/4
+                        const dd2 t = Lim == 2   ? d
+                                      : Lim == 0 ? add_smaller(d, C.hhy[sp] * dm)
+                                                 : d + C.hhy[sp] * dm;
+                        out[k] = sy > 0 ? out[k] - C.cry[sp] * t : out[k] + C.cry[sp] * t;
+                    }
+                    m = mn;
+                }
+                w = wn;
+                d = dn;
             }
         }
-        dd f[NQ];
 #pragma unroll
-        for (int q = 0; q < NQ; q++) f[q] = p[q * S::PL];
-        const Shells<dd> sh = shells_of(f);
-        dd rho, jx, jy, de;
-        conserved_dd(sh, rho, jx, jy, de);
-        const int ui = (r + 1) * S::UW + (lane + 1);
-        const dd ir = sir[ui];
-        const dd dxux = su[ui + 1] - su[ui - 1];
-        const dd dyux = su[ui + S::UW] - su[ui - S::UW];
-        const dd dxuy = sv[ui + 1] - sv[ui - 1];
-        const dd dyuy = sv[ui + S::UW] - sv[ui - S::UW];
-        dd acc[NQ];
-        collide_dd<C9>(C, sh, jx, jy, de, ir, su[ui], sv[ui], dxux, dyux, dxuy, dyuy, acc);
-        const bool store = gx < nx && gy < ny;
-        const long long cg = (long long)(gy + OY) * P.pitch + (gx + OX);
-#pragma unroll
-        for (int q = 0; q < NQ; q++) {
-            const int sx = tsgn_x(q), sy = tsgn_y(q);
-            const int shell = q >> 2;
-            dd tx = dd{0.0f, 0.0f}, tyv = dd{0.0f, 0.0f};
+        for (int k = 0; k < S::KR; k++) {
             if (sx != 0) {
                 // this lane's face difference D(x) = f(x) - f(x-1) and slope S(x) =
                 // mc2(D(x), D(x+1)); the neighbours' values by shuffles, those one column
-                // outside the warp from the duty lane of this population
-                const int duty = q < 8 ? q >> 1 : q - 4;
-                const dd D = norm_lim<Lim>(f[q] - p[q * S::PL - 1]);
-                dd Dr = shfl_down_dd(D);
-                const dd eD = shfl_dd(edgeD, duty);
-                if (lane == kTmaTX - 1) Dr = eD;
-                if (Lim == 2) {
-                    tx = sx > 0 ? D : -Dr;
-                } else if (Lim == 1) {
-                    tx = sx > 0 ? D + scale2(C.hh[shell], 2.0f) * (Dr - D) : (-Dr) + scale2(C.hh[shell], 2.0f) * ((-D) - (-Dr));
-                } else {
-                    const dd Sx = mc2n(D, Dr);
-                    const dd eS = shfl_dd(edgeS, duty);
-                    if (sx > 0) {
-                        // upwind slope S(x - 1): from lane - 1, at lane 0 from the duty lane
-                        dd Sl = shfl_up_dd(Sx);
-                        if (lane == 0) Sl = eS;
-                        tx = D + C.hh[shell] * (Sx - Sl);
-                    } else {
-                        // moving left: d1 = -D(x+1), slopes -S(x) and -S(x+1) (mc2n is odd and
-                        // symmetric, up to the choice between candidates within 2^-47 of each
-                        // other)
-                        dd Sr = shfl_down_dd(Sx);
-                        if (lane == kTmaTX - 1) Sr = eS;
-                        tx = (-Dr) + C.hh[shell] * ((-Sx) - (-Sr));
-                    }
+                // outside the tile from the edge table
+                const unsigned ea = edge_a + 32u * (unsigned)(6 * k + xpair_index(pr));
+                const dd2 D = norm_lim<Lim>(f[k] - tile_pair<S>(tile, pr, c1 + k * S::SW - 1));
+                dd2 Dr = shfl_down_dd(D);
+                take_edge(Dr, ea, lane == kTmaTX - 1);
+                dd2 t = sx > 0 ? D : Dr;
+                if (Lim == 1) t = t + scale2(C.hh[sp], 2.0f) * (sx > 0 ? Dr - D : D - Dr);
+                if (Lim == 0) {
+                    const dd2 Sx = mc2n(D, Dr);
+                    // upwind slope: S(x - 1) for pairs moving right; moving left, d1 = -D(x+1) with
+                    // slopes -S(x) and -S(x+1) (mc2n is odd and symmetric, up to the choice between
+                    // candidates within 2^-47 of each other)
+                    dd2 Su = sx > 0 ? shfl_up_dd(Sx) : shfl_down_dd(Sx);
+                    take_edge(Su, ea + 16u, lane == (sx > 0 ? 0 : kTmaTX - 1));
+                    t = add_smaller(t, C.hh[sp] * (Sx - Su));   // as for y
                 }
+                out[k] = sx > 0 ? out[k] - C.cr[sp] * t : out[k] + C.cr[sp] * t;
             }
-            if (sy != 0) {
-                const dd *pc = tile + q * S::PL + (lane + S::HX);
-                const dd wn = pc[(r + (sy > 0 ? 3 : 4)) * S::SW];
-                const dd dn = norm_lim<Lim>(wn - yw[q]);
-                if (sy > 0) {
-                    const dd mn = slope_dd<Lim>(yd[q], dn);
-                    tyv = Lim == 2 ? yd[q] : yd[q] + C.hhy[shell] * (mn - ym[q]);
-                    ym[q] = mn;
-                } else {
-                    const dd mn = slope_dd<Lim>(dn, yd[q]);
-                    tyv = Lim == 2 ? yd[q] : yd[q] + C.hhy[shell] * (ym[q] - mn);
-                    ym[q] = mn;
-                }
-                yw[q] = wn;
-                yd[q] = dn;
+            const int gy = y0 + r0 + k;
+            if (gx < nx && gy < ny) {
+                double *o = fout + (long long)(gy + OY) * P.pitch + (gx + OX);
+                o[qa * P.plane] = dd_to_double(first(out[k]));
+                o[(qa + 4) * P.plane] = dd_to_double(second(out[k]));
             }
-            // f - C - c_x (F_out - F_in)_x - c_y (F_out - F_in)_y
-            dd out = f[q] - acc[q];
-            if (sy > 0) out -= C.cry[shell] * tyv;
-            if (sy < 0) out += C.cry[shell] * tyv;
-            if (sx != 0) out -= C.cr[shell] * tx;
-            if (store) fout[q * P.plane + cg] = dd_to_double(out);
         }
     }
 }
 
 // ---------------------------------------------------------------------------
-// The single-grid kernel.  Shape as the float64 TMA-staged kernel: 8 warps, 32 x 32 tiles,
-// 4 rows per thread, one CTA per SM (the staged tile takes 162 KB).
+// The single-grid kernel.
 // ---------------------------------------------------------------------------
-template <int Lim, bool Wrap, bool C9, typename S = TmaShape<double>>
+template <int Lim, bool Wrap, bool C9, typename S = DdWideShape>
 __global__ void __launch_bounds__(kTmaTX * S::TT, S::CTAS)
-k_step_dd(const __grid_constant__ Params P, const __grid_constant__ Coef<dd> C, const __grid_constant__ CUtensorMap tm,
+k_step_dd(const __grid_constant__ Params P, const __grid_constant__ CoefDD C, const __grid_constant__ CUtensorMap tm,
           const double *__restrict__ fin, double *__restrict__ fout, int *err)
 {
     extern __shared__ __align__(128) unsigned char smraw[];
@@ -341,6 +414,15 @@ k_step_dd(const __grid_constant__ Params P, const __grid_constant__ Coef<dd> C, 
                      " [%0], [%1, {%2, %3, %4}], [%5];"
                      ::"r"(dst), "l"(reinterpret_cast<unsigned long long>(&tm)), "r"(x0 + OX - S::HX), "r"(y0),
                      "r"(0), "r"(bar_a) : "memory");
+        // bring the tile of the CTA half a resident wave later into L2
+        unsigned nsm;
+        asm("mov.u32 %0, %%nsmid;" : "=r"(nsm));
+        const long long bn = (long long)blockIdx.y * gridDim.x + blockIdx.x + (long long)S::CTAS * nsm / 2;
+        if (bn < (long long)gridDim.x * gridDim.y) {
+            const int xn = (int)(bn % gridDim.x) * kTmaTX + OX - S::HX, yn = (int)(bn / gridDim.x) * S::TR;
+            asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];"
+                         ::"l"(reinterpret_cast<unsigned long long>(&tm)), "r"(xn), "r"(yn), "r"(0) : "memory");
+        }
     }
     const bool ok = mbar_wait(bar_a, 0);
     if (!__syncthreads_and(ok)) {
@@ -351,7 +433,7 @@ k_step_dd(const __grid_constant__ Params P, const __grid_constant__ Coef<dd> C, 
         return;
     }
     if (Wrap && (x0 < S::HX || x0 + kTmaTX + S::HX > nx)) {
-        wrap_halo<double>(P, fin, tile64, x0, y0, tid, kThreads);
+        wrap_halo<double, S>(P, fin, tile64, x0, y0, tid, kThreads);
         __syncthreads();
     }
     dd_tile<Lim, C9, S>(P, C, smraw, fout, x0, y0);
@@ -365,11 +447,11 @@ k_step_dd(const __grid_constant__ Params P, const __grid_constant__ Coef<dd> C, 
 // correction runs for every grid; its factors are zero where s8 = s5, which leaves the
 // residuals unchanged bit for bit.
 // ---------------------------------------------------------------------------
-template <int Lim, typename S = TmaShape<double>>
+template <int Lim, typename S = DdWideShape>
 __global__ void __launch_bounds__(kTmaTX * S::TT, S::CTAS)
-k_step_dd_batch(const __grid_constant__ TmaBatchArgs A, const TileGrid<Coef<dd>> *__restrict__ TG)
+k_step_dd_batch(const __grid_constant__ TmaBatchArgs A, const TileGrid<CoefDD> *__restrict__ TG)
 {
-    using T = TileGrid<Coef<dd>>;
+    using T = TileGrid<CoefDD>;
     static_assert(sizeof(T) % 16 == 0, "TileGrid copy");
     extern __shared__ __align__(128) unsigned char smraw[];
     __shared__ __align__(16) T Ts;
@@ -381,7 +463,7 @@ k_step_dd_batch(const __grid_constant__ TmaBatchArgs A, const TileGrid<Coef<dd>>
     const unsigned bar_a = (unsigned)__cvta_generic_to_shared(&bar);
     if (tid == 0)
         batch_issue<S::TR, S::HX>(A, g, x0, y0, (unsigned)__cvta_generic_to_shared(smraw), bar_a,
-                                  (unsigned)S::tile_bytes, 0);
+                                  (unsigned)S::tile_bytes, S::CTAS);
     // the grid's block, while the tile copy is in flight
     {
         const int4 *src = reinterpret_cast<const int4 *>(TG + g);
@@ -401,16 +483,41 @@ k_step_dd_batch(const __grid_constant__ TmaBatchArgs A, const TileGrid<Coef<dd>>
 }
 
 // Coefficients in double-float from the float64 tables (host).
-void coef_dd(const Params &P, Coef<dd> *out)
+void coef_dd(const Params &P, CoefDD *out)
 {
-    static_assert(sizeof(Coef<dd>) == sizeof(Coef<double>), "Coef layout");
-    const double *src = reinterpret_cast<const double *>(&P.cd);
-    dd *dst = reinterpret_cast<dd *>(out);
-    for (size_t k = 0; k < sizeof(Coef<double>) / sizeof(double); k++) dst[k] = dd_host(src[k]);
+    const Coef<double> &C = P.cd;
+    auto pair = [](double x, double y) {
+        const dd a = dd_host(x), b = dd_host(y);
+        return dd2{make_float2(a.hi, b.hi), make_float2(a.lo, b.lo)};
+    };
+    for (int p = 0; p < 2; p++) {
+        out->hh[p] = pair(C.hh[2 * p], C.hh[2 * p + 1]);
+        out->hhy[p] = pair(C.hhy[2 * p], C.hhy[2 * p + 1]);
+        out->cr[p] = pair(C.cr[2 * p], C.cr[2 * p + 1]);
+        out->cry[p] = pair(C.cry[2 * p], C.cry[2 * p + 1]);
+        for (int j = 0; j < 2; j++) out->pA[p][j] = pair(C.cA[2 * p][j], C.cA[2 * p + 1][j]);
+        for (int j = 0; j < 3; j++) {
+            const double sg = j == 2 ? -1.0 : 1.0;          // row 13 enters negated
+            out->pEx[p][j] = pair(C.cEx[2 * p][j], C.cEx[2 * p + 1][j]);
+            out->pEy[p][j] = pair(sg * C.cEy[2 * p][j], sg * C.cEy[2 * p + 1][j]);
+        }
+        out->pB1[p] = pair(C.cB1[0][p], C.cB1[1][p]);
+        out->pB2[p] = pair(C.cB2[0][p], C.cB2[1][p]);
+    }
+    out->q89 = pair(C.q8, C.q9);
+    out->g4 = pair(C.g4[0], C.g4[1]);
+    out->b = dd_host(C.b);
+    out->inv_b = dd_host(C.inv_b);
+    out->two_b2 = dd_host(C.two_b2);
+    out->six_b = dd_host(C.six_b);
+    out->b4 = dd_host(C.b4);
+    out->four_inv_b = dd_host(C.four_inv_b);
+    out->ry = dd_host(C.ry);
+    out->pad_ = dd{0.0f, 0.0f};
 }
 
 template <int Lim, bool Wrap, typename S>
-static void launch_dd_lim(const Params &P, const Coef<dd> &C, const CUtensorMap &tm, const double *a, double *b,
+static void launch_dd_lim(const Params &P, const CoefDD &C, const CUtensorMap &tm, const double *a, double *b,
                           int *err, cudaStream_t st)
 {
     const dim3 block(kTmaTX, S::TT);
@@ -428,10 +535,10 @@ bool dd_narrow_supported(const Params &P)
 cudaError_t launch_step_dd(const Params &P, const void *coef, const void *tmap, const void *fin, void *fout,
                            int *err, cudaStream_t st, bool narrow)
 {
-    using W = TmaShape<double>;
+    using W = DdWideShape;
     using N = DdNarrowShape;
     const CUtensorMap &tm = *reinterpret_cast<const CUtensorMap *>(tmap);
-    const Coef<dd> &C = *reinterpret_cast<const Coef<dd> *>(coef);
+    const CoefDD &C = *reinterpret_cast<const CoefDD *>(coef);
     const double *a = (const double *)fin;
     double *b = (double *)fout;
     if (narrow) {
@@ -456,7 +563,7 @@ cudaError_t launch_step_dd(const Params &P, const void *coef, const void *tmap, 
 }
 
 template <typename S>
-static void launch_dd_batch_shape(const TmaBatchArgs &A, const TileGrid<Coef<dd>> *tg, int limiter, int ntiles,
+static void launch_dd_batch_shape(const TmaBatchArgs &A, const TileGrid<CoefDD> *tg, int limiter, int ntiles,
                                   cudaStream_t st)
 {
     const dim3 block(kTmaTX, S::TT);
@@ -465,13 +572,13 @@ static void launch_dd_batch_shape(const TmaBatchArgs &A, const TileGrid<Coef<dd>
     else k_step_dd_batch<2, S><<<ntiles, block, S::smem_bytes, st>>>(A, tg);
 }
 
-cudaError_t launch_step_dd_batch(const TmaBatchArgs &A, const TileGrid<Coef<dd>> *tg, int limiter, bool narrow,
+cudaError_t launch_step_dd_batch(const TmaBatchArgs &A, const TileGrid<CoefDD> *tg, int limiter, bool narrow,
                                  cudaStream_t st)
 {
     const int ntiles = A.first[A.n];
     if (ntiles <= 0) return cudaSuccess;
     if (narrow) launch_dd_batch_shape<DdNarrowShape>(A, tg, limiter, ntiles, st);
-    else launch_dd_batch_shape<TmaShape<double>>(A, tg, limiter, ntiles, st);
+    else launch_dd_batch_shape<DdWideShape>(A, tg, limiter, ntiles, st);
     return cudaGetLastError();
 }
 
@@ -480,7 +587,7 @@ cudaError_t dd_prepare()
     cudaError_t e = cudaSuccess;
     auto set = [&](const void *fn) {
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TmaShape<double>::smem_bytes);
+            e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DdWideShape::smem_bytes);
     };
     set((const void *)k_step_dd<0, false, false>);
     set((const void *)k_step_dd<0, false, true>);

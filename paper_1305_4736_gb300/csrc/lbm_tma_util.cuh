@@ -73,11 +73,10 @@ __device__ __forceinline__ R slope2(R a, R b)
 // the wrapped interior cells of fin, as the periodic ghost fill would have written them.  The
 // ghost rows come from the ghost fill (contiguous rows, cheap to copy); cells outside along
 // both axes are corners of the ring, which the cross stencil of stored cells never reads.
-template <typename R>
+template <typename R, typename S = TmaShape<R>>
 __device__ __noinline__ void wrap_halo(const Params &P, const R *__restrict__ fin, R *tile, int x0, int y0, int tid,
                                        int nthreads)
 {
-    using S = TmaShape<R>;
     for (int k = tid; k < S::SW * S::SH; k += nthreads) {
         const int c = k % S::SW, r = k / S::SW;
         const int x = x0 + c - S::HX, y = y0 + r - 2;
