@@ -92,11 +92,10 @@ struct DdShape {
     static constexpr int PL = SW * SH;
     static constexpr int UW = kTmaTX + 2, UH = TR + 2;
     static constexpr size_t tile_bytes = sizeof(double) * NQ * PL;
-    // shared memory: the staged tile, (u_x, u_y) on the tile plus its ring, (e, 1/rho) of the
-    // tile's cells, and the x edge values of its rows
+    // shared memory: the staged tile, (u_x, u_y) on the tile plus its ring, and the x edge values
+    // of its rows
     static constexpr size_t uv_off = tile_bytes;
-    static constexpr size_t eir_off = uv_off + 16 * UW * UH;
-    static constexpr size_t edge_off = eir_off + 16 * kTmaTX * TR;
+    static constexpr size_t edge_off = uv_off + 16 * UW * UH;
     static constexpr size_t smem_bytes = edge_off + 2 * 16 * 6 * TR;
 };
 using DdWideShape = DdShape<8, 2, 2>;

@@ -8,10 +8,12 @@
 // then
 //   split    every staged value becomes hi + lo in place (8 bytes either way), the hi parts of the
 //            population pair (q, q + 4) together in plane q, the lo parts in plane q + 4;
-//   phase 1  flow velocity on the tile + 1 ring (for grad u), e and 1/rho on the tile, and the
-//            face differences and slopes one column outside the tile;
-//   phase 2  per thread the MRT collision of its cells with the energy-flux correction (Eq. 3,
-//            Sec. II) in the shell basis, then pair by pair the limited x and y convection
+//   phase 1  per thread the residuals f_hat - f_hat^eq of its cells (Eq. 3 in the shell basis:
+//            all of the collision but the energy-flux correction, which needs grad u) and their
+//            flow velocity; the velocity of the ring; the face differences and slopes one column
+//            outside the tile;
+//   phase 2  the correction and the relaxation of the residuals, then pair by pair the limited x
+//            and y convection
 //            (Sec. III; each x face difference and slope is formed once, by the lane of its column,
 //            and passed to the neighbour lane by a shuffle; y slopes from a window sliding down the
 //            thread's column), the forward-Euler update, and one float64 store per population (the
@@ -20,7 +22,7 @@
 // about 2^-47 instead of 2^-53, so results agree with the float64 kernels and the oracle to a
 // few parts in 1e14 per step.
 //
-// What bounds it: the float32 pipe, about 3850 lane operations a cell (30 cycles of an SM at 128
+// What bounds it: the float32 pipe, about 3540 lane operations a cell (28 cycles of an SM at 128
 // lanes), then the fixed latency of the double-float chains and the float64 pipe that rounds the
 // results (48 operations a cell, 24 cycles).  Measured on 2048 x 2048 (MC, Pr != 1; the step
 // kernel, CUDA events), starting from scalar operations with one 8-warp CTA per SM on 32 x 32
@@ -32,10 +34,13 @@
 //             two 8-warp CTAs on 32 x 16 tiles run per SM (their phases overlap)
 //   0.681     the tile of the CTA half a resident wave later prefetched into L2; the populations
 //             read again after the collision instead of kept
-//   0.644     the split in half the integer operations, Fast2Sum where the order is known
-// Other shapes (warps, rows per thread, CTAs per SM), same code: 16 x 2, one CTA 0.807 ms; 12 x 2,
-// one CTA 0.843; 6 x 2, two CTAs 0.712; 7 x 2, two CTAs 0.714; 5 x 3, two CTAs 1.09; 4 x 4, two
-// CTAs 1.31 (the unrolled rows spill).  The results are bit for bit those of the scalar kernel.
+//   0.643     the split in half the integer operations, Fast2Sum where the order is known
+//   0.587     the residuals formed in phase 1 and kept in registers, so that no cell's shells are
+//             formed twice, nothing spills, and the ring is left out where s8 = s5 (3501 -> 3188
+//             thread instructions a cell)
+// Other shapes (warps x rows per thread, CTAs per SM), same code: 16 x 2, one CTA 0.807 ms; 12 x 2,
+// one CTA 0.843; 5 x 3, two CTAs 1.09; 4 x 4, two CTAs 1.31 (the unrolled rows spill), against 0.643;
+// 6 x 2, two CTAs 0.677; 7 x 2, two CTAs 0.665; 10 x 2, one CTA 0.885, against 0.587.  The results are bit for bit those of the scalar kernel.
 #include <cuda.h>
 
 #include "lbm_dd.cuh"
@@ -114,9 +119,9 @@ __device__ __forceinline__ dd2 flux_dd(dd2 X0, dd2 X1, dd2 Y0, dd2 Y1)
            both(kD4) * seconds(X1, Y1);
 }
 
-// (u_x, u_y) and (e, 1/rho) of the staged cell at offset c.
+// (u_x, u_y) of the staged cell at offset c.
 template <typename S>
-__device__ __forceinline__ void macro_dd(const float2 *t, int c, dd2 &u, dd2 &eir)
+__device__ __forceinline__ dd2 velocity_dd(const float2 *t, int c)
 {
     dd2 fp[8];
 #pragma unroll
@@ -124,20 +129,28 @@ __device__ __forceinline__ void macro_dd(const float2 *t, int c, dd2 &u, dd2 &ei
     const dd2 S0 = (fp[0] + fp[2]) + (fp[1] + fp[3]), S1 = (fp[4] + fp[6]) + (fp[5] + fp[7]);
     const dd2 cc = fp[4] - fp[6], dm = fp[5] - fp[7];
     const dd rho = sum_lanes(S0) + sum_lanes(S1);
-    const dd2 j = flux_dd(fp[0] - fp[2], cc - dm, fp[1] - fp[3], cc + dm);
-    const dd2 e0 = S0 * f2(7.25f, 36.0f), e1 = S1 * f2(4.0f, 9.0f);
-    const dd ir = recip(rho);
-    u = j * bcast(ir);
-    eir = pack((sum_lanes(e0) + first(e1)) + second(e1), ir);
+    return flux_dd(fp[0] - fp[2], cc - dm, fp[1] - fp[3], cc + dm) * bcast(recip(rho));
 }
 
-// dt M^-1 S (f_hat - f_hat^eq) with the energy-flux correction (Eq. 3, Sec. II), float64 mode
-// (zero reference state): the formulas of collide<double, false> on shell pairs, with the x and y
-// rows as pairs; gx, gy: the differences of (u_x, u_y) along x and y.
-template <bool C9>
-__device__ __forceinline__ void collide_dd(const CoefDD &C, const ShellsDD &s, dd de, dd ir, dd2 u, dd2 gx,
-                                           dd2 gy, dd2 *out)
+// f_hat - f_hat^eq of a cell (rows 5..16, in the pairs the inverse blocks take), its velocity and
+// pressure: all of the collision that needs the cell's own populations only.
+struct ResidualDD {
+    dd2 d413, d78, d910, d1112, d515, d614, u;
+    dd P;
+};
+
+// Float64 mode (zero reference state): the formulas of collide<double, false> on shell pairs, with
+// the x and y rows as pairs.
+__device__ __forceinline__ ResidualDD residual_dd(const CoefDD &C, const dd2 *fp)
 {
+    const ShellsDD s = shells_dd(fp);
+    ResidualDD r;
+    const dd ir = recip(sum_lanes(s.S[0]) + sum_lanes(s.S[1]));
+    const dd2 j = flux_dd(s.X[0], s.X[1], s.Y[0], s.Y[1]);
+    const dd2 u = j * bcast(ir);
+    r.u = u;
+    const dd2 e0 = s.S[0] * f2(7.25f, 36.0f), e1 = s.S[1] * f2(4.0f, 9.0f);
+    const dd de = (sum_lanes(e0) + first(e1)) + second(e1);
     // rows 5..16 of Appendix A
     const dd2 XY0 = firsts(s.X[0], s.Y[0]), XY1 = seconds(s.X[0], s.Y[0]);
     const dd2 m78 = ((XY0 * f2(7.25f, 7.25f) + XY1 * f2(216.0f, 216.0f)) +
@@ -148,45 +161,52 @@ __device__ __forceinline__ void collide_dd(const CoefDD &C, const ShellsDD &s, d
     const dd2 m1112 = XY0 + XY1 * f2(216.0f, 216.0f);       // row 13 negated, as its column of cEy
     const dd2 m515 = bcast(first(s.Q[0])) * f2(1.0f, 7.25f) + bcast(second(s.Q[0])) * f2(36.0f, 1296.0f);
     const dd2 m614 = bcast(first(s.Q[1])) * f2(2.0f, 8.0f) + bcast(second(s.Q[1])) * f2(4.5f, 40.5f);
-    // equilibria (Appendix A closed forms), as feq_hat_dev<R, false>; e is the cell's own e
-    const dd2 j = flux_dd(s.X[0], s.X[1], s.Y[0], s.Y[1]);
+    // equilibria (Appendix A closed forms), as feq_hat_dev<R, false>
     const dd2 jj = j * u;
     const dd J2 = sum_lanes(jj), dxy = first(jj) - second(jj);
     const dd dP = (de - J2) * C.inv_b;
+    r.P = dP;
     const dd P2 = scale2(dP, 2.0f);
     const dd q6 = first(j) * second(u);
     const dd q13 = ir * (dP * fma_dd(C.two_b2, dP, C.six_b * J2) + J2 * J2);
     const dd k = fma_dd(C.b4, dP, J2);
     const dd e2p = fma_dd(C.b, dP, J2) + P2;
     const dd2 q1415 = bcast(k) * pack(first(u), dxy) * pack(second(u), ir);   // rows 15, 16
-    const dd D4 = (de - first(s.S[0]) * 6.25f) - (P2 + J2);
-    const dd D13 = m13 - q13;
-    dd2 D78 = m78 - bcast(e2p) * u;
-    const dd2 D910 = m910 - bcast(scale2(dP, 4.0f) + J2) * u;
-    const dd2 D1112 = m1112 - pack(P2 + dxy, P2 - dxy) * u;
-    const dd2 D515 = m515 - pack(dxy, second(q1415));
-    const dd2 D614 = m614 - pack(q6, first(q1415));
-    if (C9) {
-        // y differences weighted by ry = dx/dy (q89 carries 1/(2 dx))
-        const dd div = first(gx) + C.ry * second(gy), shr = second(gx) + C.ry * first(gy);
-        const dd2 g = pack(first(gx), second(gy)) * C.g4 - bcast(C.four_inv_b * div);
-        const dd2 h = u * g + scale2(pack(second(u), first(u)) * bcast(shr), 2.0f);
-        D78 = D78 + C.q89 * bcast(dP) * h;
-    }
-    const dd2 d4 = bcast(D4), d13 = bcast(D13), d5 = bcast(first(D515)), d15 = bcast(second(D515));
-    const dd2 d6 = bcast(first(D614)), d14 = bcast(second(D614));
-    {
-        const dd2 d7 = bcast(first(D78)), d9 = bcast(first(D910)), d11 = bcast(first(D1112));
-        const dd2 d8 = bcast(second(D78)), d10 = bcast(second(D910)), d12 = bcast(second(D1112));
-        unbutterfly_dd_axis(C.pA[0][0] * d4 + C.pA[0][1] * d13,
-                            (C.pEx[0][0] * d7 + C.pEx[0][1] * d9) + C.pEx[0][2] * d11,
-                            (C.pEy[0][0] * d8 + C.pEy[0][1] * d10) + C.pEy[0][2] * d12,
-                            C.pB1[0] * d5 + C.pB1[1] * d15, out);
-        unbutterfly_dd_diag(C.pA[1][0] * d4 + C.pA[1][1] * d13,
-                            (C.pEx[1][0] * d7 + C.pEx[1][1] * d9) + C.pEx[1][2] * d11,
-                            (C.pEy[1][0] * d8 + C.pEy[1][1] * d10) + C.pEy[1][2] * d12,
-                            C.pB2[0] * d6 + C.pB2[1] * d14, out + 4);
-    }
+    r.d413 = pack((de - first(s.S[0]) * 6.25f) - (P2 + J2), m13 - q13);
+    r.d78 = m78 - bcast(e2p) * u;
+    r.d910 = m910 - bcast(scale2(dP, 4.0f) + J2) * u;
+    r.d1112 = m1112 - pack(P2 + dxy, P2 - dxy) * u;
+    r.d515 = m515 - pack(dxy, second(q1415));
+    r.d614 = m614 - pack(q6, first(q1415));
+    return r;
+}
+
+// The energy-flux correction (Sec. II) of rows 8, 9; gx, gy: the differences of (u_x, u_y) along x
+// and y, y differences weighted by ry = dx/dy (q89 carries 1/(2 dx)).
+__device__ __forceinline__ void correct_dd(const CoefDD &C, ResidualDD &r, dd2 gx, dd2 gy)
+{
+    const dd div = first(gx) + C.ry * second(gy), shr = second(gx) + C.ry * first(gy);
+    const dd2 g = pack(first(gx), second(gy)) * C.g4 - bcast(C.four_inv_b * div);
+    const dd2 h = r.u * g + scale2(pack(second(r.u), first(r.u)) * bcast(shr), 2.0f);
+    r.d78 = r.d78 + C.q89 * bcast(r.P) * h;
+}
+
+// dt M^-1 S of the residual, per population pair (Eq. 3).
+__device__ __forceinline__ void relax_dd(const CoefDD &C, const ResidualDD &r, dd2 *out)
+{
+    const dd2 d4 = bcast(first(r.d413)), d13 = bcast(second(r.d413));
+    const dd2 d7 = bcast(first(r.d78)), d9 = bcast(first(r.d910)), d11 = bcast(first(r.d1112));
+    const dd2 d8 = bcast(second(r.d78)), d10 = bcast(second(r.d910)), d12 = bcast(second(r.d1112));
+    const dd2 d5 = bcast(first(r.d515)), d15 = bcast(second(r.d515));
+    const dd2 d6 = bcast(first(r.d614)), d14 = bcast(second(r.d614));
+    unbutterfly_dd_axis(C.pA[0][0] * d4 + C.pA[0][1] * d13,
+                        (C.pEx[0][0] * d7 + C.pEx[0][1] * d9) + C.pEx[0][2] * d11,
+                        (C.pEy[0][0] * d8 + C.pEy[0][1] * d10) + C.pEy[0][2] * d12,
+                        C.pB1[0] * d5 + C.pB1[1] * d15, out);
+    unbutterfly_dd_diag(C.pA[1][0] * d4 + C.pA[1][1] * d13,
+                        (C.pEx[1][0] * d7 + C.pEx[1][1] * d9) + C.pEx[1][2] * d11,
+                        (C.pEy[1][0] * d8 + C.pEy[1][1] * d10) + C.pEy[1][2] * d12,
+                        C.pB2[0] * d6 + C.pB2[1] * d14, out + 4);
 }
 
 __device__ __forceinline__ float2 shfl_down2(float2 v)
@@ -238,15 +258,16 @@ __device__ __forceinline__ constexpr int xpair_index(int pr) { return pr < 4 ? p
 // ---------------------------------------------------------------------------
 // P: the context's Params, or the TileGrid block of a batched launch (nx, ny, pitch, plane).
 // S: the tile shape (DdWideShape or DdNarrowShape).
-template <int Lim, bool C9, typename S, typename PP>
+// C9: whether the energy-flux correction runs (0, 1), or 2 to ask P.has_c9.
+template <int Lim, int C9, typename S, typename PP>
 __device__ __forceinline__ void dd_tile(const PP &P, const CoefDD &C, unsigned char *smraw,
                                         double *__restrict__ fout, int x0, int y0)
 {
     double *tile64 = reinterpret_cast<double *>(smraw);
     float2 *tile = reinterpret_cast<float2 *>(smraw);
     float4 *suv = reinterpret_cast<float4 *>(smraw + S::uv_off);        // (u_x, u_y), tile + ring
-    float4 *seir = reinterpret_cast<float4 *>(smraw + S::eir_off);      // (e, 1/rho), tile
     float4 *sedge = reinterpret_cast<float4 *>(smraw + S::edge_off);    // x edge values per row and pair
+    const bool c9 = C9 == 2 ? P.has_c9 != 0 : C9 != 0;
     const int lane = threadIdx.x, ty = threadIdx.y, tid = ty * kTmaTX + lane;
     constexpr int kThreads = kTmaTX * S::TT;
     const int nx = P.nx, ny = P.ny;
@@ -260,49 +281,61 @@ __device__ __forceinline__ void dd_tile(const PP &P, const CoefDD &C, unsigned c
     }
     __syncthreads();
 
-    // ---- phase 1: macroscopic values on the tile plus its ring, then the values one column
-    // outside the tile for the x stencils: per row and x-moving pair D(x0 + 32) for lane 31, and
-    // the slope beyond the upwind end, S(x0 - 1) = mc2(D(x0 - 1), D(x0)) for pairs moving right,
-    // S(x0 + 32) = mc2(D(x0 + 32), D(x0 + 33)) for those moving left
-    constexpr int kCells = S::UW * S::UH, kEdges = 6 * S::TR;
-    for (int k = tid; k < kCells + kEdges; k += kThreads) {
-        if (k < kCells) {
-            const int j = k / S::UW, i = k - j * S::UW;
-            dd2 u, eir;
-            macro_dd<S>(tile, (j + 1) * S::SW + (i + S::HX - 1), u, eir);
-            suv[k] = quad(u);
-            if (i >= 1 && i <= kTmaTX && j >= 1 && j <= S::TR) seir[(j - 1) * kTmaTX + (i - 1)] = quad(eir);
+    // ---- phase 1: flow velocity of the ring (for grad u), then the values one column outside the
+    // tile for the x stencils: per row and x-moving pair D(x0 + 32) for lane 31, and the slope
+    // beyond the upwind end, S(x0 - 1) = mc2(D(x0 - 1), D(x0)) for pairs moving right, S(x0 + 32) =
+    // mc2(D(x0 + 32), D(x0 + 33)) for those moving left
+    constexpr int kRing = 2 * (kTmaTX + S::TR), kEdges = 6 * S::TR;
+    for (int k = tid; k < kRing + kEdges; k += kThreads) {
+        if (k < kRing) {
+            if (!c9) continue;
+            int i, j;                                                 // column, row in the tile + ring
+            if (k < 2 * kTmaTX) {
+                i = (k & (kTmaTX - 1)) + 1;
+                j = k < kTmaTX ? 0 : S::TR + 1;
+            } else {
+                i = k < 2 * kTmaTX + S::TR ? 0 : kTmaTX + 1;
+                j = (k - 2 * kTmaTX) % S::TR + 1;
+            }
+            suv[j * S::UW + i] = quad(velocity_dd<S>(tile, (j + 1) * S::SW + (i + S::HX - 1)));
         } else {
-            const int n = k - kCells, r = n / 6, e = n - 6 * r, pr = xpair(e);
+            const int n = k - kRing, r = n / 6, e = n - 6 * r, pr = xpair(e);
             const int row = (r + 2) * S::SW + S::HX;                  // smem offset of x0
             const float2 *hi = tile + pair_q(pr) * S::PL + row, *lo = hi + 4 * S::PL;
             auto at = [&](int x) { return dd2{hi[x], lo[x]}; };
             sedge[2 * n] = quad(norm_lim<Lim>(at(kTmaTX) - at(kTmaTX - 1)));
             if (Lim == 0) {
-                const int c0 = tsgn_x(pair_q(pr)) > 0 ? -2 : kTmaTX - 1;
-                sedge[2 * n + 1] = quad(mc2n(norm(at(c0 + 1) - at(c0)), norm(at(c0 + 2) - at(c0 + 1))));
+                const int c = tsgn_x(pair_q(pr)) > 0 ? -2 : kTmaTX - 1;
+                sedge[2 * n + 1] = quad(mc2n(norm(at(c + 1) - at(c)), norm(at(c + 2) - at(c + 1))));
             }
         }
     }
-    __syncthreads();
-
-    // ---- phase 2: rows ty*KR .. ty*KR+KR-1 of the tile, column `lane`: first the collision terms
-    // C of the thread's cells, then pair by pair their convection and update (a pair's windows are
-    // dead before the next one's are formed)
+    // the residuals of rows ty*KR .. ty*KR+KR-1 of the tile, column `lane`
     const int gx = x0 + lane;
     const int r0 = ty * S::KR;
     const int c0 = (r0 + 2) * S::SW + lane + S::HX;
-    dd2 acc[S::KR][8];
+    ResidualDD res[S::KR];
 #pragma unroll
     for (int k = 0; k < S::KR; k++) {
         dd2 fp[8];
 #pragma unroll
         for (int pr = 0; pr < 8; pr++) fp[pr] = tile_pair<S>(tile, pr, c0 + k * S::SW);
-        const int ui = (r0 + k + 1) * S::UW + (lane + 1);
-        const dd2 gxu = unquad(suv[ui + 1]) - unquad(suv[ui - 1]);
-        const dd2 gyu = unquad(suv[ui + S::UW]) - unquad(suv[ui - S::UW]);
-        const dd2 eir = unquad(seir[(r0 + k) * kTmaTX + lane]);
-        collide_dd<C9>(C, shells_dd(fp), first(eir), second(eir), unquad(suv[ui]), gxu, gyu, acc[k]);
+        res[k] = residual_dd(C, fp);
+        if (c9) suv[(r0 + k + 1) * S::UW + (lane + 1)] = quad(res[k].u);
+    }
+    __syncthreads();
+
+    // ---- phase 2: the collision terms C of the thread's cells, then pair by pair their
+    // convection and update (a pair's windows are dead before the next one's are formed)
+    dd2 acc[S::KR][8];
+#pragma unroll
+    for (int k = 0; k < S::KR; k++) {
+        if (c9) {
+            const int ui = (r0 + k + 1) * S::UW + (lane + 1);
+            correct_dd(C, res[k], unquad(suv[ui + 1]) - unquad(suv[ui - 1]),
+                       unquad(suv[ui + S::UW]) - unquad(suv[ui - S::UW]));
+        }
+        relax_dd(C, res[k], acc[k]);
     }
     // the cells' populations are read again below: kept in registers from the collision (which the
     // compiler does for loads from equal addresses) they would be spilled
@@ -444,8 +477,7 @@ k_step_dd(const __grid_constant__ Params P, const __grid_constant__ CoefDD C, co
 // tile copy with the grid's tensor map from the parameter block, then the CTA copies the grid's
 // TileGrid block (geometry and double-float coefficients) into shared memory while the copy is
 // in flight.  The ghost cells come from the batched ghost fill, so no x wrap.  The energy-flux
-// correction runs for every grid; its factors are zero where s8 = s5, which leaves the
-// residuals unchanged bit for bit.
+// correction runs where the grid has one.
 // ---------------------------------------------------------------------------
 template <int Lim, typename S = DdWideShape>
 __global__ void __launch_bounds__(kTmaTX * S::TT, S::CTAS)
@@ -479,7 +511,7 @@ k_step_dd_batch(const __grid_constant__ TmaBatchArgs A, const TileGrid<CoefDD> *
         }
         return;
     }
-    dd_tile<Lim, true, S>(Ts, Ts.cf, smraw, static_cast<double *>(A.out[g]), x0, y0);
+    dd_tile<Lim, 2, S>(Ts, Ts.cf, smraw, static_cast<double *>(A.out[g]), x0, y0);
 }
 
 // Coefficients in double-float from the float64 tables (host).
