@@ -60,16 +60,16 @@ TOTALS_EVERY = 100
 TRAFFIC_PER_CELL = {
     "f32": {"bytes": 125.83, "sources": ("lbm_step_tma.cu", "lbm_device.cuh", "lbm_tma_util.cuh"),
             "sha": "cab4bf9af2fde156"},
-    "f64": {"bytes": 251.37, "sources": ("lbm_step_stream.cu", "lbm_device.cuh", "lbm_tma_util.cuh"),
+    "f64": {"bytes": 251.31, "sources": ("lbm_step_stream.cu", "lbm_device.cuh", "lbm_tma_util.cuh"),
             "sha": "5c2c8bd0138a90d8"},
-    "dd": {"bytes": 247.55, "sources": ("lbm_step_dd.cu", "lbm_dd.cuh", "lbm_device.cuh", "lbm_tma_util.cuh"),
-           "sha": "ecf25b108c8b8d74"},
+    "dd": {"bytes": 248.21, "sources": ("lbm_step_dd.cu", "lbm_dd.cuh", "lbm_device.cuh", "lbm_tma_util.cuh"),
+           "sha": "f68aef37ad992747"},
 }
 # float32-pipe lane operations per cell of one launch of the double-float float64 kernel on wide
 # tiles: ncu's FMA-pipe busy fraction x cycles x 128 lanes (its counters of float32 instructions do
 # not see the packed f32x2 ones), on the same sources (profiles/k_step_dd_f64_shear_layer.md); None
 # when the sources changed since.
-DD_FP32_OPS = {"ops": 3542.0, "sha": "ecf25b108c8b8d74"}
+DD_FP32_OPS = {"ops": 3543.9, "sha": "f68aef37ad992747"}
 FP32_LANES_PER_SM = 128           # float32 FMA lanes per SM per cycle (GB300)
 
 
