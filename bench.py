@@ -58,18 +58,18 @@ TOTALS_EVERY = 100
 # of the kernel sources it was captured from.  bench reports the traffic only while the sources
 # still hash to that value, else null.
 TRAFFIC_PER_CELL = {
-    "f32": {"bytes": 125.83, "sources": ("lbm_step_tma.cu", "lbm_device.cuh", "lbm_tma_util.cuh"),
-            "sha": "cab4bf9af2fde156"},
-    "f64": {"bytes": 251.31, "sources": ("lbm_step_stream.cu", "lbm_device.cuh", "lbm_tma_util.cuh"),
-            "sha": "5c2c8bd0138a90d8"},
-    "dd": {"bytes": 248.21, "sources": ("lbm_step_dd.cu", "lbm_dd.cuh", "lbm_device.cuh", "lbm_tma_util.cuh"),
-           "sha": "f68aef37ad992747"},
+    "f32": {"bytes": 125.68, "sources": ("lbm_step_tma.cu", "lbm_device.cuh", "lbm_tma_util.cuh"),
+            "sha": "47657e46462e9076"},
+    "f64": {"bytes": 251.45, "sources": ("lbm_step_stream.cu", "lbm_device.cuh", "lbm_tma_util.cuh"),
+            "sha": "aebba609368ceed7"},
+    "dd": {"bytes": 248.23, "sources": ("lbm_step_dd.cu", "lbm_dd.cuh", "lbm_device.cuh", "lbm_tma_util.cuh"),
+           "sha": "bfccad890b1bf1cf"},
 }
 # float32-pipe lane operations per cell of one launch of the double-float float64 kernel on wide
 # tiles: ncu's FMA-pipe busy fraction x cycles x 128 lanes (its counters of float32 instructions do
 # not see the packed f32x2 ones), on the same sources (profiles/k_step_dd_f64_shear_layer.md); None
 # when the sources changed since.
-DD_FP32_OPS = {"ops": 3543.9, "sha": "f68aef37ad992747"}
+DD_FP32_OPS = {"ops": 3543.9, "sha": "bfccad890b1bf1cf"}
 FP32_LANES_PER_SM = 128           # float32 FMA lanes per SM per cycle (GB300)
 
 
@@ -258,7 +258,6 @@ def run_mode(lbm, p, precision, steps, warmup, device, world, step_kernel=0):
         n = min(TOTALS_EVERY, steps - done)
         s.step(n)
         done += n
-        launches += 2 * n
         s.totals()                                 # float64 reduction of rho, j, e
         launches += 2
     ev1.record(stream)
@@ -267,6 +266,7 @@ def run_mode(lbm, p, precision, steps, warmup, device, world, step_kernel=0):
     barrier(world)
     ms_local = ev0.elapsed_time(ev1)
     ms = reduce_max(ms_local, world, torch.device("cuda", device))
+    launches += int(prof[1] + prof[3])             # fused-step and ghost-fill launches
     step_kernel_ms = prof[0] / max(prof[1], 1)
     ghost_ms = prof[2] / max(prof[3], 1)
     totals_end = s.totals()
@@ -485,7 +485,7 @@ def serving_measure(count, steps, max_nx, max_ny, device, seed=1305):
 
 
 def batch_measure(device, steps=20, warmup=3, seed=1305):
-    """Batched stepping (one lbm_batch: a ghost launch and one batched tile-kernel launch per
+    """Batched stepping (one lbm_batch: one batched tile-kernel launch per
     step over the tiles of all grids) of 24 uneven float32 shear-layer grids whose buffers
     exceed L2, against stepping the same grids one at a time on their automatic kernels."""
     import numpy as np
@@ -531,7 +531,7 @@ def batch_measure(device, steps=20, warmup=3, seed=1305):
             "ms_per_step": ms, "cell_updates_per_s": cells / (ms * 1e-3),
             "roofline": {"bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm,
                          "peak_source": f"{peak_src} hbm_gbs", "traffic": None,
-                         "kernel": "k_ghost_batch, then k_step_tma_batch<MC> over the tiles of all 24 grids "
+                         "kernel": "k_step_tma_batch<MC> over the tiles of all 24 grids "
                                    "(one CTA per 32 x 16 tile), in one CUDA graph"},
             "one_at_a_time_ms_per_step": ms_solo, "speedup_vs_one_at_a_time": ms_solo / ms}
 

@@ -154,8 +154,8 @@ int lbm_create_ex(int nx, int ny, double dx, double dt, double gamma, double Pr,
    device: LBM_ERR_ARG otherwise, and the context is then left uninitialised.  Synchronous. */
 int lbm_init(lbm_ctx *ctx, const double *rho, const double *u, const double *v, const double *T);
 
-/* Enqueue n >= 1 time steps (ghost fill + fused collide/convect per step; Eq. (3) and
-   the update of Sec. III).  Asynchronous on the context's stream.  Runs of 16 steps or more
+/* Enqueue n >= 1 time steps (fused collide/convect per step, preceded by a ghost-fill launch
+   where the step kernel does not read the boundary in place; Eq. (3) and the update of Sec. III).  Asynchronous on the context's stream.  Runs of 16 steps or more
    (outside lbm_profile_begin / lbm_profile_end) replay pairs of steps from a CUDA graph that the
    context captures on a private stream at first use, one per starting buffer (lbm_autotune
    drops them): the same launches, one graph launch per pair.
@@ -193,7 +193,8 @@ int lbm_get_state_rows(lbm_ctx *ctx, int row0, int rows, double *f);
    launch (up to max_steps steps; the events live on the context's stream).
    lbm_profile_end(ctx, out) waits for them and writes out[0] = total fused-step
    kernel time in ms, out[1] = fused-step launches, out[2] = total ghost-fill time
-   in ms, out[3] = ghost-fill launches, then stops recording.
+   in ms, out[3] = ghost-fill launches (both 0 where the steps need none), then stops
+   recording.
    LBM_ERR_STATE if lbm_profile_end is called without lbm_profile_begin. */
 int lbm_profile_begin(lbm_ctx *ctx, int max_steps);
 int lbm_profile_end(lbm_ctx *ctx, double out[4]);
@@ -216,8 +217,8 @@ int lbm_autotune(lbm_ctx *ctx, int reps, int *choice);
    Not part of the paper's method: a throughput tool for many small grids, whose single
    steps are launch-bound.  The contexts must be initialised, share one device and one
    stream, and stay alive while the batch exists.  Each step of lbm_batch_step runs, per
-   group of contexts with the same precision and limiter, one batched ghost-fill launch and
-   fused-step launches over the tiles of the group's grids:
+   group of contexts with the same precision and limiter, one batched ghost-fill launch (for the
+   grids whose step kernel needs one) and fused-step launches over the tiles of the group's grids:
    - contexts whose step kernel is the TMA-staged tile kernel (float32) or a double-float
      kernel (float64), i.e. the automatic choice on grids of at least 32 x 16 (float32) or
      32 x 4 (float64), have their tiles in one launch of that kernel's batched form per 128

@@ -309,9 +309,15 @@ bool tma_ready(lbm_ctx *c)
     return lbm::tma_supported(c->P, c->prec) && lbm::tma_prepare() == cudaSuccess && make_tile_maps(c);
 }
 
-// The TMA-staged tile kernel takes the x halo of tiles at a periodic x edge from the wrapped
-// interior itself: on a grid periodic in x it needs only the ghost rows.
-bool ghost_rows_only(const lbm_ctx *c) { return (c->use_tma || c->use_dd) && (c->P.wrap & 1); }
+// Edges whose ghost cells the ghost launch fills before a step of context c: walls only where the
+// step's tiles fill the others themselves, else every edge.
+int ghost_edges(const lbm_ctx *c)
+{
+    if (!(c->use_tma || c->use_dd || c->use_ddn)) return lbm::kAllEdges;
+    int m = 0;
+    for (int e = 0; e < 4; e++) m |= (c->P.edge[e].kind == LBM_BC_NEQ_WALL) << e;
+    return m;
+}
 
 // The double-float float64 kernel: the float64 tile maps and the CoefDD of the context.
 bool dd_ready(lbm_ctx *c)
@@ -354,7 +360,7 @@ cudaError_t step_pair_graph(lbm_ctx *c, int in)
     if (ce != cudaSuccess) return ce;
     cudaError_t le = cudaSuccess;
     for (int k = 0; k < 2 && le == cudaSuccess; k++) {
-        le = lbm::launch_ghost(c->P, c->prec, c->f[in ^ k], c->cap, ghost_rows_only(c));
+        le = lbm::launch_ghost(c->P, c->prec, c->f[in ^ k], c->cap, ghost_edges(c));
         if (le == cudaSuccess) le = launch_fused_step(c, in ^ k, c->cap);
     }
     ce = cudaStreamEndCapture(c->cap, &graph);
@@ -590,18 +596,8 @@ int lbm_create_ex(int nx, int ny, double dx, double dt, double gamma, double Pr,
     // and then to the plain kernel where the grid or driver does not allow it
     if ((want == 5 || (want == 0 && prec == LBM_FP64)) && stream_ready(c)) c->use_stream = true;
     if ((want == 2 || (want == 0 && !c->use_stream)) && tma_ready(c)) c->use_tma = true;
-    // x halo of periodic edge tiles wrapped inside the TMA-staged tile kernel (P.wrap bit 0), on
-    // grids of at least 32 waves of its tiles (2048 cells per SM a wave): there the kernel's
-    // extra loads in edge tiles cost less than the ghost columns' copy; on smaller grids a
-    // kernel lasts as long as its slowest tiles, which the extra loads lengthen
     if (want == 8 && dd_ready(c)) c->use_dd = true;
     if (want == 9 && ddn_ready(c)) c->use_ddn = true;
-    if ((c->use_tma || c->use_dd) && bc->xlo.kind == LBM_BC_PERIODIC) {
-        int sms = 0;
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-        if (sms < 1) sms = 152;
-        if ((long long)nx * ny >= 32LL * 2048 * sms) c->P.wrap = 1;
-    }
     if (want == 6 && pipe_ready(c)) c->use_pipe = true;
     if ((want == 2 && !c->use_tma) || (want == 5 && !c->use_stream) || (want == 6 && !c->use_pipe) ||
         (want == 8 && !c->use_dd) || (want == 9 && !c->use_ddn)) {
@@ -731,7 +727,7 @@ int lbm_step(lbm_ctx *c, int n)
         cudaEvent_t *ev = nullptr;
         if (c->prof && c->prof_used < c->prof_max) ev = &c->prof_ev[4 * c->prof_used++];
         if (ev) cudaEventRecord(ev[0], c->stream);
-        ce = lbm::launch_ghost(c->P, c->prec, c->f[c->cur], c->stream, ghost_rows_only(c));
+        ce = lbm::launch_ghost(c->P, c->prec, c->f[c->cur], c->stream, ghost_edges(c));
         if (ce != cudaSuccess) return cuda_fail(c, ce, "ghost kernel");
         if (ev) { cudaEventRecord(ev[1], c->stream); cudaEventRecord(ev[2], c->stream); }
         ce = launch_fused_step(c, c->cur, c->stream);
@@ -961,8 +957,9 @@ int lbm_profile_end(lbm_ctx *c, double out[4])
     }
     out[0] = step_ms;
     out[1] = c->prof_used;
-    out[2] = ghost_ms;
-    out[3] = c->prof_used;
+    const bool ghost = ghost_edges(c) != 0;      // no ghost launch where the tiles fill every edge
+    out[2] = ghost ? ghost_ms : 0.0;
+    out[3] = ghost ? c->prof_used : 0;
     for (cudaEvent_t e : c->prof_ev) cudaEventDestroy(e);
     c->prof_ev.clear();
     c->prof = false;
@@ -1168,6 +1165,7 @@ cudaError_t batch_launch_tma_list(lbm_batch *b, const lbm_batch::Group &g, const
             const lbm_ctx *c = b->ctxs[g.members[sp.k]];
             const int in = c->cur ^ phase;
             A.map[k] = narrow ? c->nmap[in] : (f64 ? c->dmap[in] : c->tmap[in]);
+            A.in[k] = c->f[in];
             A.out[k] = c->f[in ^ 1];
             A.err[k] = c->tma_err;
             A.first[k] = tiles;
@@ -1179,8 +1177,8 @@ cudaError_t batch_launch_tma_list(lbm_batch *b, const lbm_batch::Group &g, const
         A.n = n;
         const char *tg = tg0 + c0 * tgb;
         const cudaError_t ce =
-            f64 ? lbm::launch_step_dd_batch(A, (const lbm::TileGrid<lbm::CoefDD> *)tg, g.limiter, narrow, st)
-                : lbm::launch_step_tma_batch(A, (const lbm::TileGrid<lbm::Coef<float>> *)tg, g.limiter, st);
+            f64 ? lbm::launch_step_dd_batch(A, (const lbm::TileGrid<lbm::CoefDD> *)tg, g.dP, g.limiter, narrow, st)
+                : lbm::launch_step_tma_batch(A, (const lbm::TileGrid<lbm::Coef<float>> *)tg, g.dP, g.limiter, st);
         if (ce != cudaSuccess) return ce;
     }
     return cudaSuccess;
@@ -1317,14 +1315,14 @@ int lbm_batch_create(lbm_ctx *const *ctxs, int n, lbm_batch **out)
         for (size_t k = 0; k < g.members.size(); k++) {
             const lbm_ctx *c = b->ctxs[g.members[k]];
             hp.push_back(c->P);
-            hp.back().wrap = 0;                      // the batched ghost fill writes every ghost cell
+            hp.back().ghost = g.tma[k] ? ghost_edges(c) : lbm::kAllEdges;
             g.hG.push_back(lbm::BatchGrid{{c->f[0], c->f[1]}, c->tma_err, c->cur, 0});
-            g.max_ghost = std::max(g.max_ghost, 4 * (c->P.nx + c->P.ny));
+            if (hp.back().ghost) g.max_ghost = std::max(g.max_ghost, 4 * (c->P.nx + c->P.ny));
             if (g.tma[k]) {
                 const int i = g.members[k], ntx = (c->P.nx + lbm::kTmaTX - 1) / lbm::kTmaTX;
                 if (g.prec == LBM_FP64) {
                     const lbm::TileGrid<lbm::CoefDD> blk{c->P.nx, c->P.ny, c->P.pitch, c->P.has_c9,
-                                                                c->P.plane, 0, c->cdd};
+                                                                c->P.plane, (long long)k, c->cdd};
                     const int nr = lbm::DdNarrowShape::TR;
                     const int wide_rows = !wide[i] ? 0 : (split[i] ? c->P.ny - c->P.ny % tr : c->P.ny);
                     if (wide_rows > 0) {
@@ -1342,7 +1340,7 @@ int lbm_batch_create(lbm_ctx *const *ctxs, int n, lbm_batch **out)
                 g.tk.push_back({(int)k, 0, c->P.ny});
                 g.ntt += ntx * ((c->P.ny + tr - 1) / tr);
                 htf.push_back(lbm::TileGrid<lbm::Coef<float>>{c->P.nx, c->P.ny, c->P.pitch, c->P.has_c9,
-                                                              c->P.plane, 0, c->P.cf});
+                                                              c->P.plane, (long long)k, c->P.cf});
                 continue;
             }
             if (g.own[k]) continue;                  // ghost cells only

@@ -80,7 +80,7 @@ struct EdgeDev {
 
 struct Params {
     int nx, ny, pitch, limiter, has_c9;
-    int wrap;                   // bit 0: the tile kernel wraps the x halo of periodic edge tiles
+    int ghost;                  // edges (bit e) whose ghost cells the ghost launch fills
     long long plane;            // elements per population plane
     double dt, T0;
     double feq0[NQ];            // reference populations f^eq(rho0, 0, 0, T0) (deviation mode)

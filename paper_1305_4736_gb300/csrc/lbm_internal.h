@@ -4,6 +4,8 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <utility>
+
 #include "lbm_dd.cuh"
 #include "lbm_device.cuh"
 
@@ -22,8 +24,27 @@ constexpr int kTotalsThreads = 256;
 // addresses of the first of those rows); a bad cell sets *bad.
 cudaError_t launch_init(const Params &P, int prec, void *f, const double *rho, const double *u, const double *v,
                         const double *T, int row0, int rows, int *bad, cudaStream_t st);
-// Ghost cells of every edge, or (y_only) of the y edges only: the ghost rows.
-cudaError_t launch_ghost(const Params &P, int prec, void *f, cudaStream_t st, bool y_only = false);
+// Ghost cells of the edges in `edges` (bit e: x-lo, x-hi, y-lo, y-hi).
+constexpr int kAllEdges = 15;
+cudaError_t launch_ghost(const Params &P, int prec, void *f, cudaStream_t st, int edges = kAllEdges);
+
+// Launch of a kernel that calls grid_dependency_wait before it touches memory: its CTAs may start
+// (barrier initialisation, parameter fetches) while the stream's previous launch drains.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args)
+{
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
 // Plain fused step with tiles of 32 x ty cells (ty = 4, 8 or 16).
 cudaError_t launch_step(const Params &P, int prec, const void *fin, void *fout, cudaStream_t st, int ty = kTY);
 // log2 of the plain kernels' tile width for a grid nx columns wide (5 for nx >= 32, else the
@@ -123,6 +144,7 @@ bool dd_narrow_supported(const Params &P);
 constexpr int kTmaBatchGrids = 128;
 struct TmaBatchArgs {
     CUtensorMap map[kTmaBatchGrids];   // grid k's input buffer (box of TmaShape<R>)
+    const void *in[kTmaBatchGrids];     // grid k's input buffer
     void *out[kTmaBatchGrids];          // grid k's output buffer
     int *err[kTmaBatchGrids];           // grid k's copy-wait flag
     int first[kTmaBatchGrids + 1];      // first[n] = tiles of the launch
@@ -136,21 +158,21 @@ struct TmaBatchArgs {
 template <typename C>
 struct TileGrid {
     int nx, ny, pitch, has_c9;
-    long long plane, pad;
+    long long plane;
+    long long member;           // the grid's index in the group's Params table (its edges)
     C cf;
 };
-cudaError_t launch_step_tma_batch(const TmaBatchArgs &A, const TileGrid<Coef<float>> *tg, int limiter,
+cudaError_t launch_step_tma_batch(const TmaBatchArgs &A, const TileGrid<Coef<float>> *tg, const Params *Pall, int limiter,
                                   cudaStream_t st);
 // narrow: tiles of DdNarrowShape (the grids' maps have its box), else of TmaShape<double>.
-cudaError_t launch_step_dd_batch(const TmaBatchArgs &A, const TileGrid<CoefDD> *tg, int limiter, bool narrow,
+cudaError_t launch_step_dd_batch(const TmaBatchArgs &A, const TileGrid<CoefDD> *tg, const Params *Pall, int limiter, bool narrow,
                                  cudaStream_t st);
 // Failure-path check of the bounded mbarrier waits (lbm_wait_selftest): *flag = 1 when the
 // wait on a phase that nothing completes gave up at its limit; *ms = the kernel's duration.
 cudaError_t wait_selftest(int *flag, float *ms);
 cudaError_t tma_prepare();   // opt the kernels in to their dynamic shared memory (once per device)
-// `tmap` points to the CUtensorMap of the input buffer fin (3-D: pitch x (ny+4) x 16).  Tiles at a
-// periodic x edge take their x halo from the wrapped interior of fin, so on a grid periodic in x
-// the kernel needs only the ghost rows (launch_ghost with y_only).
+// `tmap` points to the CUtensorMap of the input buffer fin (3-D: pitch x (ny+4) x 16).  The tiles fill
+// the ghost cells of every edge but walls themselves, from the interior of fin.
 cudaError_t launch_step_tma(const Params &P, int prec, const void *tmap, const void *fin, void *fout, int *err,
                             cudaStream_t st);
 
@@ -193,10 +215,9 @@ cudaError_t stream_prepare();
 // `tmap` points to the CUtensorMap of the input buffer with box BW x 1 x 16.
 cudaError_t launch_step_stream(const Params &P, int prec, const void *tmap, void *fout, int *err, cudaStream_t st);
 
-// Float64-mode step in double-float arithmetic on the float32 pipe (step_kernel 8): the tiles
-// and tensor maps of the float64 TMA-staged kernel; `coef` is the CoefDD of the context
-// (coef_dd).  narrow (step_kernel 9): the tiles of DdNarrowShape, `tmap` with its box, no x
-// wrap in the kernel.
+// Float64-mode step in double-float arithmetic on the float32 pipe (step_kernel 8), on tiles of
+// DdWideShape, or (narrow, step_kernel 9) of DdNarrowShape, `tmap` with their box; `coef` is the
+// CoefDD of the context (coef_dd).  Ghost cells as in launch_step_tma.
 void coef_dd(const Params &P, CoefDD *out);
 cudaError_t dd_prepare();
 cudaError_t launch_step_dd(const Params &P, const void *coef, const void *tmap, const void *fin, void *fout,

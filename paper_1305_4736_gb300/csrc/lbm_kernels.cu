@@ -14,6 +14,7 @@
 // (x, y) at row y + 2, column x + 4.  R = double stores f in 16 planes; R = float
 // stores g = f - f^eq0 (deviation mode) in 8 planes of population pairs (pidx).
 #include "lbm_internal.h"
+#include "lbm_tma_util.cuh"
 
 namespace lbm {
 
@@ -164,6 +165,8 @@ __global__ void __launch_bounds__(NT)
 k_step(const __grid_constant__ Params P, const R *__restrict__ fin, R *__restrict__ fout, int TX, int log_tx)
 {
     extern __shared__ __align__(16) unsigned char smem_plain[];
+    grid_dependency_wait();
+    grid_launch_dependents();
     const int TY = NT / TX;
     R *su = reinterpret_cast<R *>(smem_plain);
     R *sv = su + (TX + 2) * (TY + 2);
@@ -217,7 +220,7 @@ k_step_batch(const Params *__restrict__ Pall, const BatchGrid *__restrict__ G, c
 // y edges the interior columns (the stencil is a cross; corners are unused).
 // ---------------------------------------------------------------------------
 template <typename R, bool Dev>
-__device__ __forceinline__ void ghost_cell(const Params &P, R *__restrict__ f, int idx)
+__device__ __forceinline__ void ghost_cell(const Params &P, R *__restrict__ f, int idx, int edges)
 {
     const int nx = P.nx, ny = P.ny;
     const long long plane = P.plane;
@@ -226,6 +229,7 @@ __device__ __forceinline__ void ghost_cell(const Params &P, R *__restrict__ f, i
     int edge, gx, gy, sx, sy, mx, my, n, k, along;
     if (idx < n_x) {
         edge = idx / (2 * ny);            // 0 = x-lo, 1 = x-hi
+        if (!(edges >> edge & 1)) return;
         const int r = idx % (2 * ny);
         k = r / ny + 1;                   // ghost layer 1 or 2
         along = r % ny;
@@ -277,6 +281,7 @@ __device__ __forceinline__ void ghost_cell(const Params &P, R *__restrict__ f, i
     } else {
         const int j = idx - n_x;
         edge = 2 + j / (2 * nx);          // 2 = y-lo, 3 = y-hi
+        if (!(edges >> edge & 1)) return;
         const int r = j % (2 * nx);
         k = r / nx + 1;
         along = r % nx;
@@ -332,23 +337,28 @@ __device__ __forceinline__ void ghost_cell(const Params &P, R *__restrict__ f, i
     }
 }
 
-// first: index of the first ghost cell handled (0: every edge; 4 ny: the y edges only)
+// first: index of the first ghost cell handled; edges: those to fill (bit e)
 template <typename R, bool Dev>
-__global__ void k_ghost(const __grid_constant__ Params P, R *__restrict__ f, int first)
+__global__ void k_ghost(const __grid_constant__ Params P, R *__restrict__ f, int first, int edges)
 {
-    ghost_cell<R, Dev>(P, f, first + blockIdx.x * blockDim.x + threadIdx.x);
+    grid_dependency_wait();
+    grid_launch_dependents();
+    ghost_cell<R, Dev>(P, f, first + blockIdx.x * blockDim.x + threadIdx.x, edges);
 }
 
-// Batched ghost fill: blockIdx.y selects the grid of the batch.
+// Batched ghost fill: blockIdx.y selects the grid of the batch, P.ghost its edges.
 template <typename R, bool Dev>
 __global__ void k_ghost_batch(const Params *__restrict__ Pall, const BatchGrid *__restrict__ G, int phase)
 {
+    grid_dependency_wait();
+    grid_launch_dependents();
     const int gi = blockIdx.y;
     const Params &P = Pall[gi];
+    if (P.ghost == 0) return;
     const int n_all = 4 * (P.nx + P.ny);
     const BatchGrid g = G[gi];
     for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n_all; idx += gridDim.x * blockDim.x)
-        ghost_cell<R, Dev>(P, (R *)g.buf[g.cur ^ phase], idx);
+        ghost_cell<R, Dev>(P, (R *)g.buf[g.cur ^ phase], idx, P.ghost);
 }
 
 // ---------------------------------------------------------------------------
@@ -650,13 +660,21 @@ cudaError_t launch_init(const Params &P, int prec, void *f, const double *rho, c
     return cudaGetLastError();
 }
 
-cudaError_t launch_ghost(const Params &P, int prec, void *f, cudaStream_t st, bool y_only)
+// Threads per block of the ghost launches: float64 walls form two equilibria a cell on the float64
+// pipe, so their warps go to as many SMs as there are.
+static int ghost_threads(int prec) { return prec == 0 ? 32 : 128; }
+
+cudaError_t launch_ghost(const Params &P, int prec, void *f, cudaStream_t st, int edges)
 {
-    const int first = y_only ? 4 * P.ny : 0;
-    const int n = 4 * (P.nx + P.ny) - first;
-    if (prec == 0) k_ghost<double, false><<<blocks_for(n, 128), 128, 0, st>>>(P, (double *)f, first);
-    else k_ghost<float, true><<<blocks_for(n, 128), 128, 0, st>>>(P, (float *)f, first);
-    return cudaGetLastError();
+    if (edges == 0) return cudaSuccess;
+    const int bound[5] = {0, 2 * P.ny, 4 * P.ny, 4 * P.ny + 2 * P.nx, 4 * (P.ny + P.nx)};
+    int lo = 0, hi = 4;
+    while (!(edges >> lo & 1)) lo++;
+    while (!(edges >> (hi - 1) & 1)) hi--;
+    const int first = bound[lo], nt = ghost_threads(prec);
+    const dim3 grid(blocks_for(bound[hi] - first, nt));
+    return prec == 0 ? launch_chained(k_ghost<double, false>, grid, dim3(nt), 0, st, P, (double *)f, first, edges)
+                     : launch_chained(k_ghost<float, true>, grid, dim3(nt), 0, st, P, (float *)f, first, edges);
 }
 
 // Tile width of the plain kernels for a grid nx columns wide: 32, or the smallest power of
@@ -669,15 +687,14 @@ int plain_log_tx(int nx)
 }
 
 template <typename R, bool Dev, int NT>
-static void step_launch_nt(const Params &P, const R *a, R *b, cudaStream_t st)
+static cudaError_t step_launch_nt(const Params &P, const R *a, R *b, cudaStream_t st)
 {
     const int log_tx = plain_log_tx(P.nx);
     const int TX = 1 << log_tx, TY = NT / TX;
     const dim3 grid((P.nx + TX - 1) / TX, (P.ny + TY - 1) / TY);
     const size_t smem = 2 * sizeof(R) * (TX + 2) * (TY + 2);
-    if (P.limiter == 0) k_step<R, Dev, 0, NT><<<grid, NT, smem, st>>>(P, a, b, TX, log_tx);
-    else if (P.limiter == 1) k_step<R, Dev, 1, NT><<<grid, NT, smem, st>>>(P, a, b, TX, log_tx);
-    else k_step<R, Dev, 2, NT><<<grid, NT, smem, st>>>(P, a, b, TX, log_tx);
+    const auto fn = P.limiter == 0 ? k_step<R, Dev, 0, NT> : P.limiter == 1 ? k_step<R, Dev, 1, NT> : k_step<R, Dev, 2, NT>;
+    return launch_chained(fn, grid, dim3(NT), smem, st, P, a, b, TX, log_tx);
 }
 
 cudaError_t launch_step(const Params &P, int prec, const void *fin, void *fout, cudaStream_t st, int ty)
@@ -687,30 +704,28 @@ cudaError_t launch_step(const Params &P, int prec, const void *fin, void *fout, 
     if (prec == 0) {
         const double *a = (const double *)fin;
         double *b = (double *)fout;
-        if (ty == 2) step_launch_nt<double, false, kTX * 2>(P, a, b, st);
-        else if (ty == 4) step_launch_nt<double, false, kTX * 4>(P, a, b, st);
-        else if (ty == 16) step_launch_nt<double, false, kTX * 16>(P, a, b, st);
-        else step_launch_nt<double, false, kTX * 8>(P, a, b, st);
-    } else {
-        const float *a = (const float *)fin;
-        float *b = (float *)fout;
-        if (ty == 2) step_launch_nt<float, true, kTX * 2>(P, a, b, st);
-        else if (ty == 4) step_launch_nt<float, true, kTX * 4>(P, a, b, st);
-        else if (ty == 16) step_launch_nt<float, true, kTX * 16>(P, a, b, st);
-        else step_launch_nt<float, true, kTX * 8>(P, a, b, st);
+        if (ty == 2) return step_launch_nt<double, false, kTX * 2>(P, a, b, st);
+        if (ty == 4) return step_launch_nt<double, false, kTX * 4>(P, a, b, st);
+        if (ty == 16) return step_launch_nt<double, false, kTX * 16>(P, a, b, st);
+        return step_launch_nt<double, false, kTX * 8>(P, a, b, st);
     }
-    return cudaGetLastError();
+    const float *a = (const float *)fin;
+    float *b = (float *)fout;
+    if (ty == 2) return step_launch_nt<float, true, kTX * 2>(P, a, b, st);
+    if (ty == 4) return step_launch_nt<float, true, kTX * 4>(P, a, b, st);
+    if (ty == 16) return step_launch_nt<float, true, kTX * 16>(P, a, b, st);
+    return step_launch_nt<float, true, kTX * 8>(P, a, b, st);
 }
 
 cudaError_t launch_ghost_batch(const Params *Pall, const BatchGrid *G, int ngrids, int max_ghost, int prec,
                                int phase, cudaStream_t st)
 {
-    if (ngrids == 0) return cudaSuccess;
-    const int bx = (max_ghost + 127) / 128;
-    const dim3 grid(bx < 1 ? 1 : (bx > 64 ? 64 : bx), ngrids);
-    if (prec == 0) k_ghost_batch<double, false><<<grid, 128, 0, st>>>(Pall, G, phase);
-    else k_ghost_batch<float, true><<<grid, 128, 0, st>>>(Pall, G, phase);
-    return cudaGetLastError();
+    if (ngrids == 0 || max_ghost == 0) return cudaSuccess;
+    const int nt = ghost_threads(prec), most = 64 * 128 / nt;
+    const int bx = (max_ghost + nt - 1) / nt;
+    const dim3 grid(bx > most ? most : bx, ngrids);
+    return prec == 0 ? launch_chained(k_ghost_batch<double, false>, grid, dim3(nt), 0, st, Pall, G, phase)
+                     : launch_chained(k_ghost_batch<float, true>, grid, dim3(nt), 0, st, Pall, G, phase);
 }
 
 cudaError_t launch_step_batch(const Params *Pall, const BatchGrid *G, const int4 *tiles, int ntiles, int prec,

@@ -418,7 +418,7 @@ __device__ __forceinline__ void dd_tile(const PP &P, const CoefDD &C, unsigned c
 // ---------------------------------------------------------------------------
 // The single-grid kernel.
 // ---------------------------------------------------------------------------
-template <int Lim, bool Wrap, bool C9, typename S = DdWideShape>
+template <int Lim, bool C9, typename S = DdWideShape>
 __global__ void __launch_bounds__(kTmaTX * S::TT, S::CTAS)
 k_step_dd(const __grid_constant__ Params P, const __grid_constant__ CoefDD C, const __grid_constant__ CUtensorMap tm,
           const double *__restrict__ fin, double *__restrict__ fout, int *err)
@@ -428,8 +428,6 @@ k_step_dd(const __grid_constant__ Params P, const __grid_constant__ CoefDD C, co
     __shared__ __align__(8) unsigned long long bar;
 
     const int tid = threadIdx.y * kTmaTX + threadIdx.x;
-    constexpr int kThreads = kTmaTX * S::TT;
-    const int nx = P.nx;
     const int x0 = blockIdx.x * kTmaTX, y0 = blockIdx.y * S::TR;
     const unsigned bar_a = (unsigned)__cvta_generic_to_shared(&bar);
     if (tid == 0) {
@@ -437,6 +435,8 @@ k_step_dd(const __grid_constant__ Params P, const __grid_constant__ CoefDD C, co
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    grid_dependency_wait();
+    grid_launch_dependents();
     if (tid == 0) {
         // box origin: interior column x0 - HX = padded column x0 + OX - HX; interior row y0 - 2 =
         // padded row y0
@@ -457,6 +457,9 @@ k_step_dd(const __grid_constant__ Params P, const __grid_constant__ CoefDD C, co
                          ::"l"(reinterpret_cast<unsigned long long>(&tm)), "r"(xn), "r"(yn), "r"(0) : "memory");
         }
     }
+    GhostFill<double, S> ghost;
+    const bool edge = GhostFill<double, S>::edge_tile(P, x0, y0);
+    if (edge) ghost.load(P, P.edge, fin, x0, y0, tid);
     const bool ok = mbar_wait(bar_a, 0);
     if (!__syncthreads_and(ok)) {
         if (tid == 0) {
@@ -465,8 +468,8 @@ k_step_dd(const __grid_constant__ Params P, const __grid_constant__ CoefDD C, co
         }
         return;
     }
-    if (Wrap && (x0 < S::HX || x0 + kTmaTX + S::HX > nx)) {
-        wrap_halo<double, S>(P, fin, tile64, x0, y0, tid, kThreads);
+    if (edge) {
+        ghost.store(tile64);
         __syncthreads();
     }
     dd_tile<Lim, C9, S>(P, C, smraw, fout, x0, y0);
@@ -476,12 +479,13 @@ k_step_dd(const __grid_constant__ Params P, const __grid_constant__ CoefDD C, co
 // Batched form: one CTA per tile of the launch's grids (TmaBatchArgs).  Thread 0 issues the
 // tile copy with the grid's tensor map from the parameter block, then the CTA copies the grid's
 // TileGrid block (geometry and double-float coefficients) into shared memory while the copy is
-// in flight.  The ghost cells come from the batched ghost fill, so no x wrap.  The energy-flux
+// in flight.  The energy-flux
 // correction runs where the grid has one.
 // ---------------------------------------------------------------------------
 template <int Lim, typename S = DdWideShape>
 __global__ void __launch_bounds__(kTmaTX * S::TT, S::CTAS)
-k_step_dd_batch(const __grid_constant__ TmaBatchArgs A, const TileGrid<CoefDD> *__restrict__ TG)
+k_step_dd_batch(const __grid_constant__ TmaBatchArgs A, const TileGrid<CoefDD> *__restrict__ TG,
+                const Params *__restrict__ Pall)
 {
     using T = TileGrid<CoefDD>;
     static_assert(sizeof(T) % 16 == 0, "TileGrid copy");
@@ -493,6 +497,8 @@ k_step_dd_batch(const __grid_constant__ TmaBatchArgs A, const TileGrid<CoefDD> *
     int x0, y0;
     const int g = batch_tile(A, blockIdx.x, S::TR, x0, y0);
     const unsigned bar_a = (unsigned)__cvta_generic_to_shared(&bar);
+    grid_dependency_wait();
+    grid_launch_dependents();
     if (tid == 0)
         batch_issue<S::TR, S::HX>(A, g, x0, y0, (unsigned)__cvta_generic_to_shared(smraw), bar_a,
                                   (unsigned)S::tile_bytes, S::CTAS);
@@ -503,6 +509,9 @@ k_step_dd_batch(const __grid_constant__ TmaBatchArgs A, const TileGrid<CoefDD> *
         for (int k = tid; k < (int)(sizeof(T) / sizeof(int4)); k += kThreads) dst[k] = src[k];
     }
     __syncthreads();                            // the barrier is initialised
+    GhostFill<double, S> ghost;
+    const bool edge = GhostFill<double, S>::edge_tile(Ts, x0, y0);
+    if (edge) ghost.load(Ts, Pall[Ts.member].edge, static_cast<const double *>(A.in[g]), x0, y0, tid);
     const bool ok = mbar_wait(bar_a, 0);
     if (!__syncthreads_and(ok)) {
         if (tid == 0) {
@@ -510,6 +519,10 @@ k_step_dd_batch(const __grid_constant__ TmaBatchArgs A, const TileGrid<CoefDD> *
             mbar_wait(bar_a, 0);               // let a late copy land before the CTA exits (bounded)
         }
         return;
+    }
+    if (edge) {
+        ghost.store(reinterpret_cast<double *>(smraw));
+        __syncthreads();
     }
     dd_tile<Lim, 2, S>(Ts, Ts.cf, smraw, static_cast<double *>(A.out[g]), x0, y0);
 }
@@ -548,14 +561,16 @@ void coef_dd(const Params &P, CoefDD *out)
     out->pad_ = dd{0.0f, 0.0f};
 }
 
-template <int Lim, bool Wrap, typename S>
-static void launch_dd_lim(const Params &P, const CoefDD &C, const CUtensorMap &tm, const double *a, double *b,
-                          int *err, cudaStream_t st)
+template <typename S>
+static cudaError_t launch_dd_shape(const Params &P, const CoefDD &C, const CUtensorMap &tm, const double *a, double *b,
+                                   int *err, cudaStream_t st)
 {
     const dim3 block(kTmaTX, S::TT);
     const dim3 grid((P.nx + kTmaTX - 1) / kTmaTX, (P.ny + S::TR - 1) / S::TR);
-    if (P.has_c9) k_step_dd<Lim, Wrap, true, S><<<grid, block, S::smem_bytes, st>>>(P, C, tm, a, b, err);
-    else k_step_dd<Lim, Wrap, false, S><<<grid, block, S::smem_bytes, st>>>(P, C, tm, a, b, err);
+    const auto fn = P.limiter == 0   ? (P.has_c9 ? k_step_dd<0, true, S> : k_step_dd<0, false, S>)
+                    : P.limiter == 1 ? (P.has_c9 ? k_step_dd<1, true, S> : k_step_dd<1, false, S>)
+                                     : (P.has_c9 ? k_step_dd<2, true, S> : k_step_dd<2, false, S>);
+    return launch_chained(fn, grid, block, S::smem_bytes, st, P, C, tm, a, b, err);
 }
 
 bool dd_narrow_supported(const Params &P)
@@ -567,51 +582,30 @@ bool dd_narrow_supported(const Params &P)
 cudaError_t launch_step_dd(const Params &P, const void *coef, const void *tmap, const void *fin, void *fout,
                            int *err, cudaStream_t st, bool narrow)
 {
-    using W = DdWideShape;
-    using N = DdNarrowShape;
     const CUtensorMap &tm = *reinterpret_cast<const CUtensorMap *>(tmap);
     const CoefDD &C = *reinterpret_cast<const CoefDD *>(coef);
     const double *a = (const double *)fin;
     double *b = (double *)fout;
-    if (narrow) {
-        // the ghost fill writes every ghost cell of a context on narrow tiles: no x wrap
-        if (P.limiter == 0) launch_dd_lim<0, false, N>(P, C, tm, a, b, err, st);
-        else if (P.limiter == 1) launch_dd_lim<1, false, N>(P, C, tm, a, b, err, st);
-        else launch_dd_lim<2, false, N>(P, C, tm, a, b, err, st);
-        return cudaGetLastError();
-    }
-    const bool wrap = (P.wrap & 1) != 0;
-    if (P.limiter == 0) {
-        if (wrap) launch_dd_lim<0, true, W>(P, C, tm, a, b, err, st);
-        else launch_dd_lim<0, false, W>(P, C, tm, a, b, err, st);
-    } else if (P.limiter == 1) {
-        if (wrap) launch_dd_lim<1, true, W>(P, C, tm, a, b, err, st);
-        else launch_dd_lim<1, false, W>(P, C, tm, a, b, err, st);
-    } else {
-        if (wrap) launch_dd_lim<2, true, W>(P, C, tm, a, b, err, st);
-        else launch_dd_lim<2, false, W>(P, C, tm, a, b, err, st);
-    }
-    return cudaGetLastError();
+    return narrow ? launch_dd_shape<DdNarrowShape>(P, C, tm, a, b, err, st)
+                  : launch_dd_shape<DdWideShape>(P, C, tm, a, b, err, st);
 }
 
 template <typename S>
-static void launch_dd_batch_shape(const TmaBatchArgs &A, const TileGrid<CoefDD> *tg, int limiter, int ntiles,
-                                  cudaStream_t st)
+static cudaError_t launch_dd_batch_shape(const TmaBatchArgs &A, const TileGrid<CoefDD> *tg, const Params *Pall,
+                                         int limiter, int ntiles, cudaStream_t st)
 {
     const dim3 block(kTmaTX, S::TT);
-    if (limiter == 0) k_step_dd_batch<0, S><<<ntiles, block, S::smem_bytes, st>>>(A, tg);
-    else if (limiter == 1) k_step_dd_batch<1, S><<<ntiles, block, S::smem_bytes, st>>>(A, tg);
-    else k_step_dd_batch<2, S><<<ntiles, block, S::smem_bytes, st>>>(A, tg);
+    const auto fn = limiter == 0 ? k_step_dd_batch<0, S> : limiter == 1 ? k_step_dd_batch<1, S> : k_step_dd_batch<2, S>;
+    return launch_chained(fn, dim3(ntiles), block, S::smem_bytes, st, A, tg, Pall);
 }
 
-cudaError_t launch_step_dd_batch(const TmaBatchArgs &A, const TileGrid<CoefDD> *tg, int limiter, bool narrow,
-                                 cudaStream_t st)
+cudaError_t launch_step_dd_batch(const TmaBatchArgs &A, const TileGrid<CoefDD> *tg, const Params *Pall, int limiter,
+                                 bool narrow, cudaStream_t st)
 {
     const int ntiles = A.first[A.n];
     if (ntiles <= 0) return cudaSuccess;
-    if (narrow) launch_dd_batch_shape<DdNarrowShape>(A, tg, limiter, ntiles, st);
-    else launch_dd_batch_shape<DdWideShape>(A, tg, limiter, ntiles, st);
-    return cudaGetLastError();
+    return narrow ? launch_dd_batch_shape<DdNarrowShape>(A, tg, Pall, limiter, ntiles, st)
+                  : launch_dd_batch_shape<DdWideShape>(A, tg, Pall, limiter, ntiles, st);
 }
 
 cudaError_t dd_prepare()
@@ -621,18 +615,12 @@ cudaError_t dd_prepare()
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DdWideShape::smem_bytes);
     };
-    set((const void *)k_step_dd<0, false, false>);
-    set((const void *)k_step_dd<0, false, true>);
-    set((const void *)k_step_dd<0, true, false>);
-    set((const void *)k_step_dd<0, true, true>);
-    set((const void *)k_step_dd<1, false, false>);
-    set((const void *)k_step_dd<1, false, true>);
-    set((const void *)k_step_dd<1, true, false>);
-    set((const void *)k_step_dd<1, true, true>);
-    set((const void *)k_step_dd<2, false, false>);
-    set((const void *)k_step_dd<2, false, true>);
-    set((const void *)k_step_dd<2, true, false>);
-    set((const void *)k_step_dd<2, true, true>);
+    set((const void *)k_step_dd<0, false>);
+    set((const void *)k_step_dd<0, true>);
+    set((const void *)k_step_dd<1, false>);
+    set((const void *)k_step_dd<1, true>);
+    set((const void *)k_step_dd<2, false>);
+    set((const void *)k_step_dd<2, true>);
     set((const void *)k_step_dd_batch<0>);
     set((const void *)k_step_dd_batch<1>);
     set((const void *)k_step_dd_batch<2>);

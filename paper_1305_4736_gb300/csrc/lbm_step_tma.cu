@@ -142,9 +142,7 @@ __device__ __forceinline__ void flow_phase(const Coef<R> &C, const R *tile, R *s
     }
 }
 
-// Wrap: the grid's x halo is wrapped in the kernel (P.wrap bit 0); a separate instantiation,
-// so that the other grids run a kernel without that branch.
-template <typename R, bool Dev, int Lim, bool Wrap>
+template <typename R, bool Dev, int Lim>
 __global__ void __launch_bounds__(kTmaTX * TmaShape<R>::TT, TmaShape<R>::CTAS)
 k_step_tma(const __grid_constant__ Params P, const __grid_constant__ CUtensorMap tm, const R *__restrict__ fin,
            R *__restrict__ fout, int *err)
@@ -166,6 +164,8 @@ k_step_tma(const __grid_constant__ Params P, const __grid_constant__ CUtensorMap
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    grid_dependency_wait();
+    grid_launch_dependents();
     if (tid == 0) {
         // box origin: interior column x0 - HX = padded column x0 + OX - HX; interior row y0 - 2 =
         // padded row y0
@@ -190,6 +190,9 @@ k_step_tma(const __grid_constant__ Params P, const __grid_constant__ CUtensorMap
             }
         }
     }
+    GhostFill<R, S> ghost;
+    const bool edge = GhostFill<R, S>::edge_tile(P, x0, y0);
+    if (edge) ghost.load(P, P.edge, fin, x0, y0, tid);
     const bool ok = mbar_wait(bar_a, 0);
     if (!__syncthreads_and(ok)) {
         if (tid == 0) {
@@ -198,9 +201,8 @@ k_step_tma(const __grid_constant__ Params P, const __grid_constant__ CUtensorMap
         }
         return;
     }
-    // tiles whose staged box reaches past a periodic x edge (uniform per CTA)
-    if (Wrap && (x0 < S::HX || x0 + kTmaTX + S::HX > nx)) {
-        wrap_halo<R>(P, fin, tile, x0, y0, tid, kTmaTX * S::TT);
+    if (edge) {
+        ghost.store(tile);
         __syncthreads();
     }
     const Coef<R> &C = coef<R>(P);
@@ -311,12 +313,12 @@ k_step_tma(const __grid_constant__ Params P, const __grid_constant__ CUtensorMap
 // Batched form (float32): one CTA per tile of the launch's grids (TmaBatchArgs).  Thread 0
 // issues the tile copy with the grid's tensor map from the parameter block, then the CTA
 // copies the grid's TileGrid block into shared memory while the copy is in flight; the
-// arithmetic is that of k_step_tma.  The ghost cells come from the batched ghost fill, so no
-// x wrap.
+// arithmetic is that of k_step_tma.
 // ---------------------------------------------------------------------------
 template <int Lim>
 __global__ void __launch_bounds__(kTmaTX * TmaShape<float>::TT, TmaShape<float>::CTAS)
-k_step_tma_batch(const __grid_constant__ TmaBatchArgs A, const TileGrid<Coef<float>> *__restrict__ TG)
+k_step_tma_batch(const __grid_constant__ TmaBatchArgs A, const TileGrid<Coef<float>> *__restrict__ TG,
+                 const Params *__restrict__ Pall)
 {
     using S = TmaShape<float>;
     using T = TileGrid<Coef<float>>;
@@ -332,6 +334,8 @@ k_step_tma_batch(const __grid_constant__ TmaBatchArgs A, const TileGrid<Coef<flo
     int x0, y0;
     const int g = batch_tile(A, blockIdx.x, S::TR, x0, y0);
     const unsigned bar_a = (unsigned)__cvta_generic_to_shared(&bar);
+    grid_dependency_wait();
+    grid_launch_dependents();
     if (tid == 0)
         batch_issue<S::TR, S::HX>(A, g, x0, y0, (unsigned)__cvta_generic_to_shared(tile), bar_a,
                                   (unsigned)S::tile_bytes, S::CTAS);
@@ -342,6 +346,9 @@ k_step_tma_batch(const __grid_constant__ TmaBatchArgs A, const TileGrid<Coef<flo
         for (int k = tid; k < (int)(sizeof(T) / sizeof(int4)); k += kThreads) dst[k] = src[k];
     }
     __syncthreads();                            // the barrier is initialised
+    GhostFill<float, S> ghost;
+    const bool edge = GhostFill<float, S>::edge_tile(Ts, x0, y0);
+    if (edge) ghost.load(Ts, Pall[Ts.member].edge, static_cast<const float *>(A.in[g]), x0, y0, tid);
     const bool ok = mbar_wait(bar_a, 0);
     if (!__syncthreads_and(ok)) {
         if (tid == 0) {
@@ -350,23 +357,24 @@ k_step_tma_batch(const __grid_constant__ TmaBatchArgs A, const TileGrid<Coef<flo
         }
         return;
     }
+    if (edge) {
+        ghost.store(tile);
+        __syncthreads();
+    }
     flow_phase<float, true>(Ts.cf, tile, su, nullptr, nullptr, tid);
     __syncthreads();
     phase2_packed<true, Lim>(Ts, reinterpret_cast<const float2 *>(tile), reinterpret_cast<const float2 *>(su), lane,
                              ty, x0, y0, static_cast<float *>(A.out[g]));
 }
 
-cudaError_t launch_step_tma_batch(const TmaBatchArgs &A, const TileGrid<Coef<float>> *tg, int limiter,
-                                  cudaStream_t st)
+cudaError_t launch_step_tma_batch(const TmaBatchArgs &A, const TileGrid<Coef<float>> *tg, const Params *Pall,
+                                  int limiter, cudaStream_t st)
 {
     using S = TmaShape<float>;
     const int ntiles = A.first[A.n];
     if (ntiles <= 0) return cudaSuccess;
-    const dim3 block(kTmaTX, S::TT);
-    if (limiter == 0) k_step_tma_batch<0><<<ntiles, block, S::smem_bytes, st>>>(A, tg);
-    else if (limiter == 1) k_step_tma_batch<1><<<ntiles, block, S::smem_bytes, st>>>(A, tg);
-    else k_step_tma_batch<2><<<ntiles, block, S::smem_bytes, st>>>(A, tg);
-    return cudaGetLastError();
+    const auto fn = limiter == 0 ? k_step_tma_batch<0> : limiter == 1 ? k_step_tma_batch<1> : k_step_tma_batch<2>;
+    return launch_chained(fn, dim3(ntiles), dim3(kTmaTX, S::TT), S::smem_bytes, st, A, tg, Pall);
 }
 
 // ---------------------------------------------------------------------------
@@ -536,34 +544,22 @@ bool tma_supported(const Params &P, int prec)
     return P.pitch >= TmaShape<float>::SW && P.ny + 4 >= sh && P.nx >= kTmaTX;
 }
 
-template <typename R, bool Dev, bool Wrap>
-static void launch_tma_lim(const Params &P, const CUtensorMap &tm, const R *a, R *b, int *err, cudaStream_t st)
+template <typename R, bool Dev>
+static cudaError_t launch_tma_lim(const Params &P, const CUtensorMap &tm, const R *a, R *b, int *err, cudaStream_t st)
 {
     using S = TmaShape<R>;
     const dim3 block(kTmaTX, S::TT);
     const dim3 grid((P.nx + kTmaTX - 1) / kTmaTX, (P.ny + S::TR - 1) / S::TR);
-    if (P.limiter == 0) k_step_tma<R, Dev, 0, Wrap><<<grid, block, S::smem_bytes, st>>>(P, tm, a, b, err);
-    else if (P.limiter == 1) k_step_tma<R, Dev, 1, Wrap><<<grid, block, S::smem_bytes, st>>>(P, tm, a, b, err);
-    else k_step_tma<R, Dev, 2, Wrap><<<grid, block, S::smem_bytes, st>>>(P, tm, a, b, err);
+    const auto fn = P.limiter == 0 ? k_step_tma<R, Dev, 0> : P.limiter == 1 ? k_step_tma<R, Dev, 1> : k_step_tma<R, Dev, 2>;
+    return launch_chained(fn, grid, block, S::smem_bytes, st, P, tm, a, b, err);
 }
 
 cudaError_t launch_step_tma(const Params &P, int prec, const void *tmap, const void *fin, void *fout, int *err,
                             cudaStream_t st)
 {
     const CUtensorMap &tm = *reinterpret_cast<const CUtensorMap *>(tmap);
-    const bool wrap = (P.wrap & 1) != 0;
-    if (prec == 0) {
-        const double *a = (const double *)fin;
-        double *b = (double *)fout;
-        if (wrap) launch_tma_lim<double, false, true>(P, tm, a, b, err, st);
-        else launch_tma_lim<double, false, false>(P, tm, a, b, err, st);
-    } else {
-        const float *a = (const float *)fin;
-        float *b = (float *)fout;
-        if (wrap) launch_tma_lim<float, true, true>(P, tm, a, b, err, st);
-        else launch_tma_lim<float, true, false>(P, tm, a, b, err, st);
-    }
-    return cudaGetLastError();
+    return prec == 0 ? launch_tma_lim<double, false>(P, tm, (const double *)fin, (double *)fout, err, st)
+                     : launch_tma_lim<float, true>(P, tm, (const float *)fin, (float *)fout, err, st);
 }
 
 cudaError_t tma_prepare()
@@ -572,18 +568,12 @@ cudaError_t tma_prepare()
     auto set = [&](const void *fn, size_t bytes) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     };
-    set((const void *)k_step_tma<double, false, 0, false>, TmaShape<double>::smem_bytes);
-    set((const void *)k_step_tma<double, false, 1, false>, TmaShape<double>::smem_bytes);
-    set((const void *)k_step_tma<double, false, 2, false>, TmaShape<double>::smem_bytes);
-    set((const void *)k_step_tma<double, false, 0, true>, TmaShape<double>::smem_bytes);
-    set((const void *)k_step_tma<double, false, 1, true>, TmaShape<double>::smem_bytes);
-    set((const void *)k_step_tma<double, false, 2, true>, TmaShape<double>::smem_bytes);
-    set((const void *)k_step_tma<float, true, 0, false>, TmaShape<float>::smem_bytes);
-    set((const void *)k_step_tma<float, true, 1, false>, TmaShape<float>::smem_bytes);
-    set((const void *)k_step_tma<float, true, 2, false>, TmaShape<float>::smem_bytes);
-    set((const void *)k_step_tma<float, true, 0, true>, TmaShape<float>::smem_bytes);
-    set((const void *)k_step_tma<float, true, 1, true>, TmaShape<float>::smem_bytes);
-    set((const void *)k_step_tma<float, true, 2, true>, TmaShape<float>::smem_bytes);
+    set((const void *)k_step_tma<double, false, 0>, TmaShape<double>::smem_bytes);
+    set((const void *)k_step_tma<double, false, 1>, TmaShape<double>::smem_bytes);
+    set((const void *)k_step_tma<double, false, 2>, TmaShape<double>::smem_bytes);
+    set((const void *)k_step_tma<float, true, 0>, TmaShape<float>::smem_bytes);
+    set((const void *)k_step_tma<float, true, 1>, TmaShape<float>::smem_bytes);
+    set((const void *)k_step_tma<float, true, 2>, TmaShape<float>::smem_bytes);
     set((const void *)k_step_tma_batch<0>, TmaShape<float>::smem_bytes);
     set((const void *)k_step_tma_batch<1>, TmaShape<float>::smem_bytes);
     set((const void *)k_step_tma_batch<2>, TmaShape<float>::smem_bytes);
