@@ -58,18 +58,18 @@ TOTALS_EVERY = 100
 # of the kernel sources it was captured from.  bench reports the traffic only while the sources
 # still hash to that value, else null.
 TRAFFIC_PER_CELL = {
-    "f32": {"bytes": 125.68, "sources": ("lbm_step_tma.cu", "lbm_device.cuh", "lbm_tma_util.cuh"),
-            "sha": "47657e46462e9076"},
-    "f64": {"bytes": 251.45, "sources": ("lbm_step_stream.cu", "lbm_device.cuh", "lbm_tma_util.cuh"),
-            "sha": "aebba609368ceed7"},
-    "dd": {"bytes": 248.23, "sources": ("lbm_step_dd.cu", "lbm_dd.cuh", "lbm_device.cuh", "lbm_tma_util.cuh"),
-           "sha": "bfccad890b1bf1cf"},
+    "f32": {"bytes": 125.70, "sources": ("lbm_step_tma.cu", "lbm_device.cuh", "lbm_tma_util.cuh"),
+            "sha": "4437e33d9d1d1cc0"},
+    "f64": {"bytes": 251.48, "sources": ("lbm_step_stream.cu", "lbm_device.cuh", "lbm_tma_util.cuh"),
+            "sha": "d54b8a6059b7b053"},
+    "dd": {"bytes": 248.27, "sources": ("lbm_step_dd.cu", "lbm_dd.cuh", "lbm_device.cuh", "lbm_tma_util.cuh"),
+           "sha": "b4d1b2d9de8aaa66"},
 }
 # float32-pipe lane operations per cell of one launch of the double-float float64 kernel on wide
 # tiles: ncu's FMA-pipe busy fraction x cycles x 128 lanes (its counters of float32 instructions do
 # not see the packed f32x2 ones), on the same sources (profiles/k_step_dd_f64_shear_layer.md); None
 # when the sources changed since.
-DD_FP32_OPS = {"ops": 3543.9, "sha": "bfccad890b1bf1cf"}
+DD_FP32_OPS = {"ops": 3543.9, "sha": "b4d1b2d9de8aaa66"}
 FP32_LANES_PER_SM = 128           # float32 FMA lanes per SM per cycle (GB300)
 
 

@@ -309,14 +309,19 @@ bool tma_ready(lbm_ctx *c)
     return lbm::tma_supported(c->P, c->prec) && lbm::tma_prepare() == cudaSuccess && make_tile_maps(c);
 }
 
-// Edges whose ghost cells the ghost launch fills before a step of context c: walls only where the
-// step's tiles fill the others themselves, else every edge.
+int edges_of_kind(const lbm_ctx *c, int kind)
+{
+    int m = 0;
+    for (int e = 0; e < 4; e++) m |= (c->P.edge[e].kind == kind) << e;
+    return m;
+}
+
+// Edges whose ghost cells the ghost launch fills before a step of context c: every edge for the
+// streaming and the double-buffered kernel, else walls only (the other kernels read periodic and
+// zero-gradient neighbours in place; fixed-equilibrium ghost cells are filled at create time).
 int ghost_edges(const lbm_ctx *c)
 {
-    if (!(c->use_tma || c->use_dd || c->use_ddn)) return lbm::kAllEdges;
-    int m = 0;
-    for (int e = 0; e < 4; e++) m |= (c->P.edge[e].kind == LBM_BC_NEQ_WALL) << e;
-    return m;
+    return c->use_stream || c->use_pipe ? lbm::kAllEdges : edges_of_kind(c, LBM_BC_NEQ_WALL);
 }
 
 // The double-float float64 kernel: the float64 tile maps and the CoefDD of the context.
@@ -333,6 +338,14 @@ bool ddn_ready(lbm_ctx *c)
     if (c->prec != LBM_FP64 || !lbm::dd_narrow_supported(c->P) || lbm::dd_prepare() != cudaSuccess) return false;
     lbm::coef_dd(c->P, &c->cdd);
     return make_narrow_maps(c);
+}
+
+// The ghost launch that precedes a step of context c from buffer `in`, if it needs one.
+cudaError_t launch_step_ghosts(lbm_ctx *c, int in, cudaStream_t st)
+{
+    const bool plain = !(c->use_dd || c->use_ddn || c->use_pipe || c->use_stream || c->use_tma);
+    return lbm::launch_ghost(c->P, c->prec, c->f[in], st, ghost_edges(c),
+                             plain && lbm::lane_step(c->P, c->prec, c->plain_ty));
 }
 
 // One fused step of context c from buffer `in` into buffer in ^ 1, on stream st.
@@ -360,7 +373,7 @@ cudaError_t step_pair_graph(lbm_ctx *c, int in)
     if (ce != cudaSuccess) return ce;
     cudaError_t le = cudaSuccess;
     for (int k = 0; k < 2 && le == cudaSuccess; k++) {
-        le = lbm::launch_ghost(c->P, c->prec, c->f[in ^ k], c->cap, ghost_edges(c));
+        le = launch_step_ghosts(c, in ^ k, c->cap);
         if (le == cudaSuccess) le = launch_fused_step(c, in ^ k, c->cap);
     }
     ce = cudaStreamEndCapture(c->cap, &graph);
@@ -607,6 +620,9 @@ int lbm_create_ex(int nx, int ny, double dx, double dt, double gamma, double Pr,
     cudaGetLastError();
     ce = cudaMemsetAsync(c->buf, 0, c->buf_bytes, c->stream);
     if (ce == cudaSuccess) ce = cudaMemsetAsync(c->aux, 0, c->aux_bytes, c->stream);
+    // the ghost cells of fixed-equilibrium edges, which no step changes, in both buffers
+    for (int k = 0; k < 2 && ce == cudaSuccess; k++)
+        ce = lbm::launch_ghost(c->P, c->prec, c->f[k], c->stream, edges_of_kind(c, LBM_BC_EQUILIBRIUM));
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(c->stream);
     if (ce != cudaSuccess) {
         lbm_destroy(c);
@@ -727,7 +743,7 @@ int lbm_step(lbm_ctx *c, int n)
         cudaEvent_t *ev = nullptr;
         if (c->prof && c->prof_used < c->prof_max) ev = &c->prof_ev[4 * c->prof_used++];
         if (ev) cudaEventRecord(ev[0], c->stream);
-        ce = lbm::launch_ghost(c->P, c->prec, c->f[c->cur], c->stream, ghost_edges(c));
+        ce = launch_step_ghosts(c, c->cur, c->stream);
         if (ce != cudaSuccess) return cuda_fail(c, ce, "ghost kernel");
         if (ev) { cudaEventRecord(ev[1], c->stream); cudaEventRecord(ev[2], c->stream); }
         ce = launch_fused_step(c, c->cur, c->stream);
@@ -1315,7 +1331,7 @@ int lbm_batch_create(lbm_ctx *const *ctxs, int n, lbm_batch **out)
         for (size_t k = 0; k < g.members.size(); k++) {
             const lbm_ctx *c = b->ctxs[g.members[k]];
             hp.push_back(c->P);
-            hp.back().ghost = g.tma[k] ? ghost_edges(c) : lbm::kAllEdges;
+            hp.back().ghost = ghost_edges(c);
             g.hG.push_back(lbm::BatchGrid{{c->f[0], c->f[1]}, c->tma_err, c->cur, 0});
             if (hp.back().ghost) g.max_ghost = std::max(g.max_ghost, 4 * (c->P.nx + c->P.ny));
             if (g.tma[k]) {

@@ -24,9 +24,12 @@ constexpr int kTotalsThreads = 256;
 // addresses of the first of those rows); a bad cell sets *bad.
 cudaError_t launch_init(const Params &P, int prec, void *f, const double *rho, const double *u, const double *v,
                         const double *T, int row0, int rows, int *bad, cudaStream_t st);
-// Ghost cells of the edges in `edges` (bit e: x-lo, x-hi, y-lo, y-hi).
+// Whether the plain step with tiles of 32 x ty cells takes 16 lanes per cell (small float64 grids).
+bool lane_step(const Params &P, int prec, int ty);
+// Ghost cells of the edges in `edges` (bit e: x-lo, x-hi, y-lo, y-hi); lanes: float64 walls with 16
+// lanes per cell.
 constexpr int kAllEdges = 15;
-cudaError_t launch_ghost(const Params &P, int prec, void *f, cudaStream_t st, int edges = kAllEdges);
+cudaError_t launch_ghost(const Params &P, int prec, void *f, cudaStream_t st, int edges = kAllEdges, bool lanes = false);
 
 // Launch of a kernel that calls grid_dependency_wait before it touches memory: its CTAs may start
 // (barrier initialisation, parameter fetches) while the stream's previous launch drains.

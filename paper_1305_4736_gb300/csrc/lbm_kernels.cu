@@ -1,6 +1,7 @@
 // lbm_kernels.cu -- CUDA kernels of the D2V16 MRT flux-limiter FDLBM step (sm_103a).
 //
 //   k_ghost    ghost cells of every edge (Sec. IV.A, IV.C, V)
+//   k_step_lanes  the fused step with 16 lanes per cell (small float64 grids); k_wall its walls
 //   k_step     fused step: local rho/u on the tile + 1 ring, central-difference
 //              grad u, MRT collision with the energy-flux correction (Eq. 3,
 //              Sec. II), flux-limited x and y convection and the forward-Euler
@@ -14,6 +15,7 @@
 // (x, y) at row y + 2, column x + 4.  R = double stores f in 16 planes; R = float
 // stores g = f - f^eq0 (deviation mode) in 8 planes of population pairs (pidx).
 #include "lbm_internal.h"
+#include "lbm_lanes.cuh"
 #include "lbm_tma_util.cuh"
 
 namespace lbm {
@@ -88,6 +90,11 @@ __device__ __forceinline__ void step_tile(const Params &P, const R *__restrict__
     const int nx = P.nx, ny = P.ny, pitch = P.pitch;
     const long long plane = P.plane;
     const bool inside = (ix < nx) && (iy < ny);
+    // cell a read at (x, y) goes to: past a periodic or zero-gradient edge its interior source, so
+    // that only wall edges need a ghost launch (those of a fixed-equilibrium edge never change)
+    const int kx0 = P.edge[0].kind, kx1 = P.edge[1].kind, ky0 = P.edge[2].kind, ky1 = P.edge[3].kind;
+    auto col = [&](int x) { return ghost_source(x, nx, kx0, kx1) + OX; };
+    auto row = [&](int y) { return (long long)(ghost_source(y, ny, ky0, ky1) + OY) * pitch; };
     const long long c0 = (long long)(iy + OY) * pitch + (ix + OX);
 
     R f[NQ];
@@ -103,7 +110,7 @@ __device__ __forceinline__ void step_tile(const Params &P, const R *__restrict__
         sv[(ty + 1) * W + tx + 1] = jy * ir;
     } else if (u_cell(ix, iy, nx, ny)) {
         R g[NQ];
-        load16(fin, plane, c0, g);
+        load16(fin, plane, row(iy) + col(ix), g);
         R a, b;
         velocity_of<R, Dev>(P, g, a, b);
         su[(ty + 1) * W + tx + 1] = a;
@@ -118,7 +125,7 @@ __device__ __forceinline__ void step_tile(const Params &P, const R *__restrict__
         else { rx = x0 + TX; ry = y0 + t - 2 * TX - TY; lx = TX + 1; ly = t - 2 * TX - TY + 1; }
         if (u_cell(rx, ry, nx, ny)) {
             R g[NQ];
-            load16(fin, plane, (long long)(ry + OY) * pitch + (rx + OX), g);
+            load16(fin, plane, row(ry) + col(rx), g);
             R a, b;
             velocity_of<R, Dev>(P, g, a, b);
             su[ly * W + lx] = a;
@@ -141,6 +148,13 @@ __device__ __forceinline__ void step_tile(const Params &P, const R *__restrict__
 
         // limited convection: x and y projections, both from f^n (Sec. III)
         const Coef<R> &C = coef<R>(P);
+        // the stencil's cells at offsets -2 .. 2 along each axis
+        long long cx[5], cy[5];
+#pragma unroll
+        for (int d = 0; d < 5; d++) {
+            cx[d] = c0 - (ix + OX) + col(ix + d - 2);
+            cy[d] = row(iy + d - 2) + (ix + OX);
+        }
 #pragma unroll
         for (int q = 0; q < NQ; q++) {
             const int sx = sgn_x(q), sy = sgn_y(q);
@@ -149,10 +163,9 @@ __device__ __forceinline__ void step_tile(const Params &P, const R *__restrict__
             // sum over the axes of c_alpha (F_out - F_in) (Courant number and h/2 per axis)
             R conv = R(0);
             if (sx != 0)
-                conv = C.cr[shell] * flux_diff<R, Lim>(at(c0 - 2 * sx), at(c0 - sx), f[q], at(c0 + sx), C.hh[shell]);
+                conv = C.cr[shell] * flux_diff<R, Lim>(at(cx[2 - 2 * sx]), at(cx[2 - sx]), f[q], at(cx[2 + sx]), C.hh[shell]);
             if (sy != 0) {
-                const long long sp = (long long)sy * pitch;
-                const R ty_ = flux_diff<R, Lim>(at(c0 - 2 * sp), at(c0 - sp), f[q], at(c0 + sp), C.hhy[shell]);
+                const R ty_ = flux_diff<R, Lim>(at(cy[2 - 2 * sy]), at(cy[2 - sy]), f[q], at(cy[2 + sy]), C.hhy[shell]);
                 conv = sx != 0 ? conv + C.cry[shell] * ty_ : C.cry[shell] * ty_;
             }
             fout[pidx<R>(q, plane, c0)] = acc[q] - conv;
@@ -171,6 +184,94 @@ k_step(const __grid_constant__ Params P, const R *__restrict__ fin, R *__restric
     R *su = reinterpret_cast<R *>(smem_plain);
     R *sv = su + (TX + 2) * (TY + 2);
     step_tile<R, Dev, Lim>(P, fin, fout, blockIdx.x * TX, blockIdx.y * TY, TX, log_tx, TY, su, sv);
+}
+
+// Fused step, float64, 16 lanes per cell: for grids of at most kLaneCells cells.  A CTA of 128 threads
+// takes 8 cells (TX x 8/TX); each lane forms its population's convection, the shells and moments go
+// between lanes, the flow velocities of the neighbours (for the energy-flux correction) through
+// shared memory.  About 60 float64 instructions a warp instead of 440, on as many partitions as the
+// grid has pairs of cells (see lbm_lanes.cuh).
+constexpr int kLaneTile = 8;          // cells per CTA
+template <int Lim, bool C9>
+__global__ void __launch_bounds__(kLaneTile * kCellLanes)
+k_step_lanes(const __grid_constant__ Params P, const double *__restrict__ fin, double *__restrict__ fout, int TX,
+             int log_tx)
+{
+    constexpr int kRingMax = 2 * (kLaneTile + 1);
+    __shared__ double2 su[kLaneTile + kRingMax];      // (u_x, u_y): the tile's cells, then the ring
+    const Coef<double> &C = P.cd;
+    const int tid = threadIdx.x, cell = tid / kCellLanes;
+    const Lane L = lane_of(C, tid & (kCellLanes - 1));
+    double kcol[4];
+    lane_collision(C, L, kcol);
+    const int nx = P.nx, ny = P.ny, pitch = P.pitch, q = L.q;
+    const int TY = kLaneTile >> log_tx, tx = cell & (TX - 1), ty = cell >> log_tx;
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
+    // the tile's cells past the grid give the velocity of the first ghost layer (a corner of it, which
+    // no difference reads, that of an edge) and are not stored
+    const int ix = min(x0 + tx, nx), iy = min(y0 + ty, ix == nx ? ny - 1 : ny);
+    const bool store = ix < nx && iy < ny;
+    const int kx0 = P.edge[0].kind, kx1 = P.edge[1].kind, ky0 = P.edge[2].kind, ky1 = P.edge[3].kind;
+    const long long base = q * P.plane;
+    auto at = [&](int x, int y) {
+        return base + (long long)(ghost_source(y, ny, ky0, ky1) + OY) * pitch + (ghost_source(x, nx, kx0, kx1) + OX);
+    };
+    const int sx = store ? sgn_x(q) : 0, sy = store ? sgn_y(q) : 0;
+    grid_dependency_wait();
+    grid_launch_dependents();
+    // the populations of the two stencils, upwind first (a lane that does not move along an axis
+    // reads its own cell: its differences are zero)
+    const double f = fin[at(ix, iy)];
+    const double xmm = fin[at(ix - 2 * sx, iy)], xm = fin[at(ix - sx, iy)], xp = fin[at(ix + sx, iy)];
+    const double ymm = fin[at(ix, iy - 2 * sy)], ym = fin[at(ix, iy - sy)], yp = fin[at(ix, iy + sy)];
+    double jx, jy;
+    const double m = lane_block(L, L.row, lane_butterfly(L, f));
+    const LaneState s = lane_state(C, m, jx, jy);
+    double D = m - lane_feq(L, s);
+    if (C9) {
+        const int W = 2 * (TX + TY);
+        if (q == 0) su[cell] = make_double2(s.ux, s.uy);
+        for (int r = cell; r < W; r += kLaneTile) {
+            // ring: below, above, left, right of the tile
+            int rx, ry;
+            if (r < 2 * TX) {
+                rx = x0 + (r & (TX - 1));
+                ry = r < TX ? y0 - 1 : y0 + TY;
+            } else {
+                const int k = r - 2 * TX;
+                rx = k < TY ? x0 - 1 : x0 + TX;
+                ry = y0 + (k < TY ? k : k - TY);
+            }
+            // a cell that no stored cell's difference reads stands in for one past the ghost layer
+            rx = min(rx, nx);
+            ry = min(ry, ny);
+            if ((rx < 0 || rx == nx) && (ry < 0 || ry == ny)) ry = ny - 1;
+            double a, b;
+            const LaneState t = lane_state(C, lane_block(L, L.row, lane_butterfly(L, fin[at(rx, ry)])), a, b);
+            if (q == 0) su[kLaneTile + r] = make_double2(t.ux, t.uy);
+        }
+        __syncthreads();
+        const double2 l = tx > 0 ? su[cell - 1] : su[kLaneTile + 2 * TX + ty];
+        const double2 r = tx < TX - 1 ? su[cell + 1] : su[kLaneTile + 2 * TX + TY + ty];
+        const double2 d = ty > 0 ? su[cell - TX] : su[kLaneTile + tx];
+        const double2 u = ty < TY - 1 ? su[cell + TX] : su[kLaneTile + TX + tx];
+        const double dxux = r.x - l.x, dxuy = r.y - l.y, dyux = u.x - d.x, dyuy = u.y - d.y;
+        // rows m8 (lane 6) and m9 (lane 7); y differences weighted by ry = dx/dy
+        const bool row8 = q == 6;
+        const double div = fma(C.ry, dyuy, dxux), shr = fma(C.ry, dyux, dxuy);
+        const double g = row8 ? 4.0 * dxux : C.g4[1] * dyuy;
+        const double A = row8 ? s.ux : s.uy, B = row8 ? s.uy : s.ux;
+        const double h = fma(A, fma(-C.four_inv_b, div, g), (2.0 * B) * shr);
+        const double k = row8 ? C.q8 : (q == 7 ? C.q9 : 0.0);
+        D = fma(k * s.P, h, D);
+    }
+    const double acc = lane_unbutterfly(L, lane_block(L, kcol, D));
+    const double tX = flux_diff<double, Lim>(xmm, xm, f, xp, C.hh[L.shell]);
+    const double tY = flux_diff<double, Lim>(ymm, ym, f, yp, C.hhy[L.shell]);
+    double out = f - acc;
+    if (sy != 0) out = fma(-C.cry[L.shell], tY, out);
+    if (sx != 0) out = fma(-C.cr[L.shell], tX, out);
+    if (store) fout[base + (long long)(iy + OY) * pitch + (ix + OX)] = out;
 }
 
 static_assert(sizeof(Params) % sizeof(int4) == 0, "Params is copied to shared memory as int4 words");
@@ -335,6 +436,46 @@ __device__ __forceinline__ void ghost_cell(const Params &P, R *__restrict__ f, i
 #pragma unroll
         for (int q = 0; q < NQ; q++) f[pidx<R>(q, plane, cg)] = g[q] + fd[q];
     }
+}
+
+// Ghost cell of a float64 wall, 16 lanes per cell: idx over the edge's two layers.  rho_g = rho_m,
+// j_g = 2 rho_m u_w - j_m, P_g = rho_m (2 T_w - T_m); f_g = f_m + M^-1 (f_hat^eq(g) - f_hat^eq(m)).
+__device__ __forceinline__ void wall_cell(const Params &P, double *__restrict__ f, int edge, int idx, const Lane &L,
+                                          const double *inv)
+{
+    const int n = edge < 2 ? P.ny : P.nx, m = edge < 2 ? P.nx : P.ny;
+    const bool ok = idx < 2 * n;
+    const int layer = idx >= n && ok ? 2 : 1, along = ok ? (layer == 2 ? idx - n : idx) : 0;
+    const int g = (edge & 1) ? m - 1 + layer : -layer;
+    int mir = (edge & 1) ? m - layer : layer - 1;
+    mir = mir < 0 ? 0 : (mir >= m ? m - 1 : mir);
+    auto at = [&](int v) {
+        return (long long)((edge < 2 ? along : v) + OY) * P.pitch + ((edge < 2 ? v : along) + OX);
+    };
+    const EdgeDev &E = P.edge[edge];
+    const Coef<double> &C = P.cd;
+    const double fm = f[L.q * P.plane + at(mir)];
+    double jx, jy;
+    const LaneState s = lane_state(C, lane_block(L, L.row, lane_butterfly(L, fm)), jx, jy);
+    LaneState w = s;
+    const double r2 = 2.0 * s.rho;
+    lane_kinetic(w, fma(r2, E.uw, -jx), fma(r2, E.vw, -jy));
+    w.P = fma(r2, E.Tw, -s.P);
+    const double d = lane_feq(L, w) - lane_feq(L, s);
+    const double fg = fm + lane_unbutterfly(L, lane_block(L, inv, d));
+    if (ok) f[L.q * P.plane + at(g)] = fg;
+}
+
+constexpr int kWallThreads = 32;     // two cells a block: one warp per partition of as many SMs as there are
+
+__global__ void __launch_bounds__(kWallThreads) k_wall(const __grid_constant__ Params P, double *__restrict__ f, int edge)
+{
+    const Lane L = lane_of(P.cd, threadIdx.x & (kCellLanes - 1));
+    double inv[4];
+    lane_inverse(P.cd, L, inv);
+    grid_dependency_wait();
+    grid_launch_dependents();
+    wall_cell(P, f, edge + blockIdx.y, (int)((blockIdx.x * kWallThreads + threadIdx.x) / kCellLanes), L, inv);
 }
 
 // first: index of the first ghost cell handled; edges: those to fill (bit e)
@@ -660,12 +801,28 @@ cudaError_t launch_init(const Params &P, int prec, void *f, const double *rho, c
     return cudaGetLastError();
 }
 
-// Threads per block of the ghost launches: float64 walls form two equilibria a cell on the float64
-// pipe, so their warps go to as many SMs as there are.
+// Threads per block of the ghost launches: a float64 wall cell is some 225 float64 instructions, which
+// a partition of an SM takes 78 cycles each for, so one-warp blocks reach every partition.
 static int ghost_threads(int prec) { return prec == 0 ? 32 : 128; }
 
-cudaError_t launch_ghost(const Params &P, int prec, void *f, cudaStream_t st, int edges)
+// Grids whose step takes 16 lanes per cell (lane_step) have their float64 walls formed that way too (55
+// instructions for two cells in a warp instead of 225 for 32).  The others keep one thread per wall
+// cell, with which a grid gives the same bits alone and in a batch.
+cudaError_t launch_ghost(const Params &P, int prec, void *f, cudaStream_t st, int edges, bool lanes)
 {
+    if (lanes) {
+        for (int axis = 0; axis < 2; axis++) {             // opposite walls in one launch
+            const bool lo = (edges >> (2 * axis) & 1) && P.edge[2 * axis].kind == 3;
+            const bool hi = (edges >> (2 * axis + 1) & 1) && P.edge[2 * axis + 1].kind == 3;
+            if (!lo && !hi) continue;
+            const dim3 grid(blocks_for(2LL * kCellLanes * (axis ? P.nx : P.ny), kWallThreads), lo && hi ? 2 : 1);
+            const cudaError_t ce =
+                launch_chained(k_wall, grid, dim3(kWallThreads), 0, st, P, (double *)f, 2 * axis + (lo ? 0 : 1));
+            if (ce != cudaSuccess) return ce;
+        }
+        for (int e = 0; e < 4; e++)
+            if (P.edge[e].kind == 3) edges &= ~(1 << e);
+    }
     if (edges == 0) return cudaSuccess;
     const int bound[5] = {0, 2 * P.ny, 4 * P.ny, 4 * P.ny + 2 * P.nx, 4 * (P.ny + P.nx)};
     int lo = 0, hi = 4;
@@ -686,6 +843,16 @@ int plain_log_tx(int nx)
     return l;
 }
 
+// The float64 kernel on 64-cell tiles gives way to 16 lanes per cell on grids of at most 7296 cells:
+// pairs of cells over 608 partitions, 60 float64 instructions of 78 cycles each, against one wave of
+// 440.  Measured, us per step, 64-cell tiles and lanes: 4 x 200 with walls 28.7 and 11.3, 8 x 400 28.7
+// and 15.4, 16 x 380 28.7 and 21.5, 16 x 450 24.6 and (extrapolated) 24.1; without walls or energy-flux
+// correction 4 x 200 27.7 and 5.9, 16 x 380 27.7 and 14.3, 16 x 600 20.5.
+bool lane_step(const Params &P, int prec, int ty)
+{
+    return prec == 0 && ty == 2 && (long long)P.nx * P.ny <= 7296;
+}
+
 template <typename R, bool Dev, int NT>
 static cudaError_t step_launch_nt(const Params &P, const R *a, R *b, cudaStream_t st)
 {
@@ -699,6 +866,17 @@ static cudaError_t step_launch_nt(const Params &P, const R *a, R *b, cudaStream_
 
 cudaError_t launch_step(const Params &P, int prec, const void *fin, void *fout, cudaStream_t st, int ty)
 {
+    if (lane_step(P, prec, ty)) {
+        int log_tx = plain_log_tx(P.nx);
+        if (log_tx > 2) log_tx = 2;                         // 4 x 2 cells, or 2 x 4, 1 x 8
+        const int TX = 1 << log_tx, TY = kLaneTile >> log_tx;
+        const dim3 grid((P.nx + TX - 1) / TX, (P.ny + TY - 1) / TY);
+        const auto fn = P.limiter == 0   ? (P.has_c9 ? k_step_lanes<0, true> : k_step_lanes<0, false>)
+                        : P.limiter == 1 ? (P.has_c9 ? k_step_lanes<1, true> : k_step_lanes<1, false>)
+                                         : (P.has_c9 ? k_step_lanes<2, true> : k_step_lanes<2, false>);
+        return launch_chained(fn, grid, dim3(kLaneTile * kCellLanes), 0, st, P, (const double *)fin, (double *)fout, TX,
+                              log_tx);
+    }
     // ty: rows of a 32-column tile (2, 4, 8 or 16: 64 .. 512 threads); grids narrower than
     // 32 columns keep the thread count with TX = the smallest power of two >= nx
     if (prec == 0) {

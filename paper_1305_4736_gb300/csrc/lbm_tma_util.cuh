@@ -73,10 +73,20 @@ __device__ __forceinline__ R slope2(R a, R b)
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// Ghost cells of the tiles at an edge of the grid: periodic, zero-gradient and fixed-equilibrium
-// edges are filled in the staged tile, with the values the ghost launch would have written, so
-// that no ghost launch precedes the step (wall edges keep theirs: they need the mirror cell's
-// moments).  One thread per ghost cell of the cross: the tile's columns in up to four ghost rows,
+// Coordinate a read at v goes to along an axis of n cells: the wrapped cell past a periodic edge
+// (kind 0), the edge cell past a zero-gradient one (1), else v itself.
+__device__ __forceinline__ int ghost_source(int v, int n, int kind_lo, int kind_hi)
+{
+    if (v >= 0 && v < n) return v;
+    const int kind = v < 0 ? kind_lo : kind_hi;
+    if (kind == 1) return v < 0 ? 0 : n - 1;
+    return kind == 0 ? ((v % n) + n) % n : v;
+}
+
+// Ghost cells of the tiles at an edge of the grid: periodic and zero-gradient edges are filled in
+// the staged tile, with the values the ghost launch would have written; those of a
+// fixed-equilibrium edge never change (lbm_create_ex fills them).  So no ghost launch precedes the
+// step, but for wall edges, which need the mirror cell's moments.  One thread per ghost cell of the cross: the tile's columns in up to four ghost rows,
 // its rows in up to four ghost columns.  The sources are interior cells, read from global memory
 // while the tile copy is in flight; they replace the tile's ghost cells once it has landed.
 // Measured per step, with the launches chained (launch_chained): 200 x 4 float64 20.5 -> 9.3 us,
@@ -119,25 +129,13 @@ struct GhostFill {
             const bool in = k < kSlots && at >= 0 && at < (row ? S::SH : S::SW) && along < (row ? P.nx : P.ny);
             if (!in) continue;
             const EdgeDev &D = edges[(row ? 2 : 0) + (layer >> 1)];
-            if (D.kind > 2) continue;
+            if (D.kind > 1) continue;
             c[n] = row ? at * S::SW + (along - x0 + S::HX) : (along - y0 + 2) * S::SW + at;
-            if (D.kind == 2) {
-                if constexpr (sizeof(R) == sizeof(float)) {
+            const int s = ghost_source(g, size, D.kind, D.kind);
+            const long long cell = (long long)((row ? s : along) + OY) * P.pitch + ((row ? along : s) + OX);
+            const E *src = reinterpret_cast<const E *>(fin) + cell;
 #pragma unroll
-                    for (int pr = 0; pr < N; pr++) v[n][pr] = f2(D.feqf[pair_q(pr)], D.feqf[pair_q(pr) + 4]);
-                } else {
-#pragma unroll
-                    for (int q = 0; q < N; q++) v[n][q] = D.feq[q];
-                }
-            } else {
-                // periodic: two layers wrap at most once unless the grid has a single cell there
-                int s = D.kind == 1 ? (layer < 2 ? 0 : size - 1) : (layer < 2 ? g + size : g - size);
-                if (D.kind == 0 && (s < 0 || s >= size)) s = 0;
-                const long long cell = (long long)((row ? s : along) + OY) * P.pitch + ((row ? along : s) + OX);
-                const E *src = reinterpret_cast<const E *>(fin) + cell;
-#pragma unroll
-                for (int q = 0; q < N; q++) v[n][q] = src[q * P.plane];
-            }
+            for (int q = 0; q < N; q++) v[n][q] = src[q * P.plane];
         }
     }
 
