@@ -114,10 +114,11 @@ typedef struct {
                                       with a thread per population), 8 = LBM_FP64 only: TMA-staged tiles
                                       with the step's arithmetic in double-float form (pairs of
                                       float32, about 2^-47 rounding per operation) on the float32
-                                      pipe, 32 x 16 tiles, populations still stored and returned in float64
-                                      (grids of at least 32 x 32), 9 = LBM_FP64 only: the same
-                                      arithmetic on 32 x 4 tiles, two CTAs per SM (grids of at
-                                      least 32 columns and 4 rows); all agree to round-off of
+                                      pipe, populations still stored and returned in float64
+                                      (grids of at least 32 x 32; tiles of 32 x 16 or 32 x 8 by
+                                      the grid's size), 9 = LBM_FP64 only: the same arithmetic on
+                                      32 x 8 or 32 x 4 tiles (grids of at least 32 columns and 4
+                                      rows); all agree to round-off of
                                       their arithmetic (see lbm_autotune) */
     double dy;                     /* grid spacing along y; <= 0 means dy = dx.  The y projection
                                       of the convection uses the Courant numbers |v_iy| dt / dy and
@@ -222,10 +223,11 @@ int lbm_autotune(lbm_ctx *ctx, int reps, int *choice);
    grids whose step kernel needs one) and fused-step launches over the tiles of the group's grids:
    - contexts whose step kernel is the TMA-staged tile kernel (float32) or a double-float
      kernel (float64), i.e. the automatic choice on grids of at least 32 x 16 (float32) or
-     32 x 4 (float64), have their tiles in one launch of that kernel's batched form per 128
-     such grids (float64: one for the 32 x 16 tiles, one for the 32 x 4 tiles) (one CTA per tile; the launch's parameters hold each grid's tensor map,
-     output buffer and tile count, and the CTA stages its grid's coefficients in shared
-     memory), with the arithmetic of the single-grid kernel, bit for bit;
+     32 x 4 (float64), have their tiles in launches of that kernel's batched form, one per 128
+     such grids (float64: one per tile shape, 32 x 16, 32 x 8 and 32 x 4; one CTA per tile; the
+     launch's parameters hold each grid's tensor map, buffers and tile count, and the CTA stages
+     its grid's coefficients in shared memory), with the arithmetic of the single-grid kernel, bit
+     for bit;
    - the other grids share the packed plain kernel, whose persistent CTAs walk a tile list
      (float32: 256-cell tiles, float64: 64-cell tiles, which spread small float64 grids over
      more SMs; 32 columns wide, or TX = the smallest power of two >= nx for narrower grids)
@@ -237,6 +239,7 @@ int lbm_autotune(lbm_ctx *ctx, int reps, int *choice);
    Pairs of steps are replayed from a CUDA graph captured on the first call with n >= 2
    (recaptured when a context was stepped alone an odd number of times since).  Tiles are independent, so a grid's result does not depend on the other members
    of its batch (bit for bit).
+   The launches of one step do not wait for each other: each starts as the one before drains.
    Contexts may also be stepped alone between batch steps.  Errors: LBM_ERR_ARG (NULL, empty, mixed device or stream, a
    context listed twice), LBM_ERR_STATE (uninitialised context, n <= 0), LBM_ERR_OOM,
    LBM_ERR_CUDA. */

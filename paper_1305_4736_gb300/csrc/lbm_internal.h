@@ -68,9 +68,9 @@ struct BatchGrid {
 // Batched ghost fill (grid index = blockIdx.y) and batched fused step over a tile list
 // (int4 {grid, x0, y0, 0}); `phase` = 0 reads buf[cur], 1 reads buf[cur ^ 1].
 cudaError_t launch_ghost_batch(const Params *Pall, const BatchGrid *G, int ngrids, int max_ghost, int prec,
-                               int phase, cudaStream_t st);
+                               int phase, int late, cudaStream_t st);
 cudaError_t launch_step_batch(const Params *Pall, const BatchGrid *G, const int4 *tiles, int ntiles, int prec,
-                              int limiter, int nt, int ctas, int phase, cudaStream_t st);
+                              int limiter, int nt, int ctas, int phase, int late, cudaStream_t st);
 cudaError_t launch_moments(const Params &P, int prec, const void *f, int row0, int rows,
                            double *rho, double *u, double *v, double *T, double *delta,
                            double *dstar, int *flag, cudaStream_t st);
@@ -104,12 +104,13 @@ struct TmaShape {
     static constexpr size_t smem_bytes = tile_bytes + sizeof(R) * (sizeof(R) == sizeof(float) ? 2 : 3) * UW * UH;
 };
 bool tma_supported(const Params &P, int prec);
-// Tiles of the double-float float64 kernels: 32 columns by TT * KR rows, TT warps, KR rows per
-// thread, CTAS CTAs per SM.
-template <int TT_, int KR_, int CTAS_>
+// Tiles of the double-float float64 kernels: 32 columns by TR rows, TT warps, KR rows per thread,
+// CTAS CTAs per SM.  ROLES: two warps per row, one for the collision and one for the convection.
+template <int TT_, int KR_, int CTAS_, bool ROLES_ = false>
 struct DdShape {
     static constexpr int TT = TT_, KR = KR_, CTAS = CTAS_;
-    static constexpr int TR = TT * KR;
+    static constexpr bool ROLES = ROLES_;
+    static constexpr int TR = ROLES ? TT / 2 : TT * KR;
     static constexpr int HX = 2;                       // x halo (8-byte elements: 16-byte TMA origin)
     static constexpr int SW = kTmaTX + 2 * HX;
     static constexpr int SH = TR + 4;
@@ -120,12 +121,22 @@ struct DdShape {
     // of its rows
     static constexpr size_t uv_off = tile_bytes;
     static constexpr size_t edge_off = uv_off + 16 * UW * UH;
-    static constexpr size_t smem_bytes = edge_off + 2 * 16 * 6 * TR;
+    static constexpr size_t acc_off = edge_off + 2 * 16 * 6 * TR;            // ROLES: the collision terms
+    static constexpr size_t smem_bytes = acc_off + (ROLES ? 16 * 8 * kTmaTX * TR : 0);
 };
-using DdWideShape = DdShape<8, 2, 2>;
-// Narrow tiles (step_kernel 9): 32 x 4, for grids of 4 to 31 rows (and 32 columns or more) and for
-// small grids.
-using DdNarrowShape = DdShape<4, 1, 2>;
+using DdWideShape = DdShape<8, 2, 2>;            // 32 x 16: the fewest instructions per cell
+using DdMidShape = DdShape<8, 1, 2>;             // 32 x 8
+using DdNarrowShape = DdShape<8, 1, 2, true>;    // 32 x 4: the shortest step of a tile
+enum { kDdWide = 0, kDdMid = 1, kDdNarrow = 2, kDdShapes = 3 };
+constexpr int kDdRows[kDdShapes] = {DdWideShape::TR, DdMidShape::TR, DdNarrowShape::TR};
+// Whether a grid's staged boxes of a shape fit its buffers.
+bool dd_shape_supported(const Params &P, int shape);
+// Estimated duration (us) of `tiles` tiles of a shape on sms SMs, for choosing between shapes: whole
+// waves of two CTAs per SM, then the remainder at one or two per SM.  Measured on grids of 26 to 160
+// thousand cells (MC, Pr != 1), us per step, 32 x 4 / 32 x 8 / 32 x 16 tiles: 161 x 97 9.2 / 12.3 / 19.5,
+// 300 x 100 12.3 / 12.3 / 19.5, 256^2 20.1 / 16.4 / 17.4, 320^2 27.8 / 22.5 / 27.5, 380^2 38.0 / 29.4 /
+// 30.5, 400^2 44.1 / 34.8 / 39.0.
+double dd_shape_time(int shape, long long tiles, int sms);
 static_assert(DdWideShape::CTAS * (DdWideShape::smem_bytes + 2048) <= 228 * 1024, "wide tiles per SM");
 // Coefficients of the double-float kernels in the order of the population pairs (lane e of pair
 // p belongs to shell 2p + e); the column of row 13 in pEy is negated, as the kernel forms that
@@ -137,7 +148,6 @@ struct CoefDD {
     dd b, inv_b, two_b2, six_b, b4, four_inv_b, ry, pad_;
 };
 static_assert(sizeof(CoefDD) % 16 == 0, "CoefDD is copied in 16-byte words");
-bool dd_narrow_supported(const Params &P);
 // Batched TMA-staged steps over the tiles of up to kTmaBatchGrids grids of a batch group, one
 // CTA per tile of kTmaTX x TmaShape<R>::TR cells: grid k owns the launch's tiles first[k] ..
 // first[k+1] - 1, row by row from row y0[k], ntx[k] to a row.  A CTA finds its grid and tile from blockIdx
@@ -154,7 +164,13 @@ struct TmaBatchArgs {
     int ntx[kTmaBatchGrids];            // tiles per row of grid k
     int y0[kTmaBatchGrids];             // first row of grid k's tiles in this launch
     int n;                              // grids of the launch
+    int late;                           // see launch order below
 };
+// Launch order: the step launches of one batch step are independent of each other.  The first of them
+// waits for the launches before it (grid_dependency_wait) when it starts; a `late` one, chained behind
+// it, starts once all CTAs of the one before have passed their own wait or start, so that everything
+// before the step is complete, and has one thread wait for that launch at its end, so that its own
+// completion stands for both.
 // Per-grid block of a batched launch (global memory, one per grid in launch order): the
 // geometry and the coefficients that the tile kernels read (C = Coef<float> or CoefDD); each
 // CTA copies its grid's block to shared memory while its tile copy is in flight.
@@ -167,8 +183,8 @@ struct TileGrid {
 };
 cudaError_t launch_step_tma_batch(const TmaBatchArgs &A, const TileGrid<Coef<float>> *tg, const Params *Pall, int limiter,
                                   cudaStream_t st);
-// narrow: tiles of DdNarrowShape (the grids' maps have its box), else of TmaShape<double>.
-cudaError_t launch_step_dd_batch(const TmaBatchArgs &A, const TileGrid<CoefDD> *tg, const Params *Pall, int limiter, bool narrow,
+// shape: kDdWide, kDdMid or kDdNarrow (the grids' maps have its box).
+cudaError_t launch_step_dd_batch(const TmaBatchArgs &A, const TileGrid<CoefDD> *tg, const Params *Pall, int limiter, int shape,
                                  cudaStream_t st);
 // Failure-path check of the bounded mbarrier waits (lbm_wait_selftest): *flag = 1 when the
 // wait on a phase that nothing completes gave up at its limit; *ms = the kernel's duration.
@@ -218,13 +234,13 @@ cudaError_t stream_prepare();
 // `tmap` points to the CUtensorMap of the input buffer with box BW x 1 x 16.
 cudaError_t launch_step_stream(const Params &P, int prec, const void *tmap, void *fout, int *err, cudaStream_t st);
 
-// Float64-mode step in double-float arithmetic on the float32 pipe (step_kernel 8), on tiles of
-// DdWideShape, or (narrow, step_kernel 9) of DdNarrowShape, `tmap` with their box; `coef` is the
-// CoefDD of the context (coef_dd).  Ghost cells as in launch_step_tma.
+// Float64-mode step in double-float arithmetic on the float32 pipe (step_kernel 8, 9), on tiles of
+// `shape`, `tmap` with its box; `coef` is the CoefDD of the context (coef_dd).  Ghost cells as in
+// launch_step_tma.
 void coef_dd(const Params &P, CoefDD *out);
 cudaError_t dd_prepare();
 cudaError_t launch_step_dd(const Params &P, const void *coef, const void *tmap, const void *fin, void *fout,
-                           int *err, cudaStream_t st, bool narrow = false);
+                           int *err, cudaStream_t st, int shape);
 
 // Sustained float64 FMA rate of the current device in FLOP/s (FMA = 2).
 cudaError_t measure_fp64_fma(double *flops);

@@ -1,7 +1,6 @@
 // lbm_kernels.cu -- CUDA kernels of the D2V16 MRT flux-limiter FDLBM step (sm_103a).
 //
 //   k_ghost    ghost cells of every edge (Sec. IV.A, IV.C, V)
-//   k_step_lanes  the fused step with 16 lanes per cell (small float64 grids); k_wall its walls
 //   k_step     fused step: local rho/u on the tile + 1 ring, central-difference
 //              grad u, MRT collision with the energy-flux correction (Eq. 3,
 //              Sec. II), flux-limited x and y convection and the forward-Euler
@@ -286,8 +285,9 @@ static_assert(sizeof(Params) % sizeof(int4) == 0, "Params is copied to shared me
 template <typename R, bool Dev, int Lim, int NT>
 __global__ void __launch_bounds__(NT)
 k_step_batch(const Params *__restrict__ Pall, const BatchGrid *__restrict__ G, const int4 *__restrict__ tiles,
-             int ntiles, int phase)
+             int ntiles, int phase, int late)
 {
+    batch_begin(late);
     constexpr int kSmem = 3 * (NT + 2);            // max over TX of (TX + 2)(TY + 2), at TX = 1
     __shared__ R su[kSmem];
     __shared__ R sv[kSmem];
@@ -314,6 +314,7 @@ k_step_batch(const Params *__restrict__ Pall, const BatchGrid *__restrict__ G, c
         step_tile<R, Dev, Lim>(Ps, (const R *)g.buf[in], (R *)g.buf[in ^ 1], tl.y, tl.z, TX, tl.w, NT / TX, su,
                                sv);
     }
+    batch_end(late, tid);
 }
 
 // ---------------------------------------------------------------------------
@@ -489,17 +490,18 @@ __global__ void k_ghost(const __grid_constant__ Params P, R *__restrict__ f, int
 
 // Batched ghost fill: blockIdx.y selects the grid of the batch, P.ghost its edges.
 template <typename R, bool Dev>
-__global__ void k_ghost_batch(const Params *__restrict__ Pall, const BatchGrid *__restrict__ G, int phase)
+__global__ void k_ghost_batch(const Params *__restrict__ Pall, const BatchGrid *__restrict__ G, int phase, int late)
 {
-    grid_dependency_wait();
-    grid_launch_dependents();
+    batch_begin(late);
     const int gi = blockIdx.y;
     const Params &P = Pall[gi];
-    if (P.ghost == 0) return;
-    const int n_all = 4 * (P.nx + P.ny);
-    const BatchGrid g = G[gi];
-    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n_all; idx += gridDim.x * blockDim.x)
-        ghost_cell<R, Dev>(P, (R *)g.buf[g.cur ^ phase], idx, P.ghost);
+    if (P.ghost != 0) {
+        const int n_all = 4 * (P.nx + P.ny);
+        const BatchGrid g = G[gi];
+        for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n_all; idx += gridDim.x * blockDim.x)
+            ghost_cell<R, Dev>(P, (R *)g.buf[g.cur ^ phase], idx, P.ghost);
+    }
+    batch_end(late, threadIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -896,36 +898,34 @@ cudaError_t launch_step(const Params &P, int prec, const void *fin, void *fout, 
 }
 
 cudaError_t launch_ghost_batch(const Params *Pall, const BatchGrid *G, int ngrids, int max_ghost, int prec,
-                               int phase, cudaStream_t st)
+                               int phase, int late, cudaStream_t st)
 {
     if (ngrids == 0 || max_ghost == 0) return cudaSuccess;
     const int nt = ghost_threads(prec), most = 64 * 128 / nt;
     const int bx = (max_ghost + nt - 1) / nt;
     const dim3 grid(bx > most ? most : bx, ngrids);
-    return prec == 0 ? launch_chained(k_ghost_batch<double, false>, grid, dim3(nt), 0, st, Pall, G, phase)
-                     : launch_chained(k_ghost_batch<float, true>, grid, dim3(nt), 0, st, Pall, G, phase);
+    return prec == 0 ? launch_chained(k_ghost_batch<double, false>, grid, dim3(nt), 0, st, Pall, G, phase, late)
+                     : launch_chained(k_ghost_batch<float, true>, grid, dim3(nt), 0, st, Pall, G, phase, late);
 }
 
 cudaError_t launch_step_batch(const Params *Pall, const BatchGrid *G, const int4 *tiles, int ntiles, int prec,
-                              int limiter, int nt, int ctas, int phase, cudaStream_t st)
+                              int limiter, int nt, int ctas, int phase, int late, cudaStream_t st)
 {
     if (ntiles == 0) return cudaSuccess;
-    const int grid = ntiles < ctas ? ntiles : ctas;
+    const dim3 grid(ntiles < ctas ? ntiles : ctas);
     constexpr int N64 = kBatchThreadsFp64, N32 = kBatchThreads;
-    if (prec == 0 && nt == N64) {
-        if (limiter == 0) k_step_batch<double, false, 0, N64><<<grid, N64, 0, st>>>(Pall, G, tiles, ntiles, phase);
-        else if (limiter == 1) k_step_batch<double, false, 1, N64><<<grid, N64, 0, st>>>(Pall, G, tiles, ntiles, phase);
-        else k_step_batch<double, false, 2, N64><<<grid, N64, 0, st>>>(Pall, G, tiles, ntiles, phase);
-    } else if (prec == 0) {
-        if (limiter == 0) k_step_batch<double, false, 0, N32><<<grid, N32, 0, st>>>(Pall, G, tiles, ntiles, phase);
-        else if (limiter == 1) k_step_batch<double, false, 1, N32><<<grid, N32, 0, st>>>(Pall, G, tiles, ntiles, phase);
-        else k_step_batch<double, false, 2, N32><<<grid, N32, 0, st>>>(Pall, G, tiles, ntiles, phase);
-    } else {
-        if (limiter == 0) k_step_batch<float, true, 0, N32><<<grid, N32, 0, st>>>(Pall, G, tiles, ntiles, phase);
-        else if (limiter == 1) k_step_batch<float, true, 1, N32><<<grid, N32, 0, st>>>(Pall, G, tiles, ntiles, phase);
-        else k_step_batch<float, true, 2, N32><<<grid, N32, 0, st>>>(Pall, G, tiles, ntiles, phase);
-    }
-    return cudaGetLastError();
+    auto pick = [&](auto *a, auto *b, auto *c) { return limiter == 0 ? a : limiter == 1 ? b : c; };
+    if (prec == 0 && nt == N64)
+        return launch_chained(pick(k_step_batch<double, false, 0, N64>, k_step_batch<double, false, 1, N64>,
+                                   k_step_batch<double, false, 2, N64>),
+                              grid, dim3(N64), 0, st, Pall, G, tiles, ntiles, phase, late);
+    if (prec == 0)
+        return launch_chained(pick(k_step_batch<double, false, 0, N32>, k_step_batch<double, false, 1, N32>,
+                                   k_step_batch<double, false, 2, N32>),
+                              grid, dim3(N32), 0, st, Pall, G, tiles, ntiles, phase, late);
+    return launch_chained(pick(k_step_batch<float, true, 0, N32>, k_step_batch<float, true, 1, N32>,
+                               k_step_batch<float, true, 2, N32>),
+                          grid, dim3(N32), 0, st, Pall, G, tiles, ntiles, phase, late);
 }
 
 cudaError_t launch_moments(const Params &P, int prec, const void *f, int row0, int rows, double *rho,

@@ -250,43 +250,68 @@ __device__ __forceinline__ dd2 slope_dd(dd2 a, dd2 b)
 __device__ __forceinline__ constexpr int xpair(int e) { return e < 2 ? 2 * e : e + 2; }
 __device__ __forceinline__ constexpr int xpair_index(int pr) { return pr < 4 ? pr >> 1 : pr - 2; }
 
-}  // namespace
-
-// ---------------------------------------------------------------------------
-// The tile body shared by the single-grid and the batched kernel: the staged float64 tile in
-// shared memory (smraw) is split, then phases 1 and 2 produce the tile's new float64 values.
-// ---------------------------------------------------------------------------
-// P: the context's Params, or the TileGrid block of a batched launch (nx, ny, pitch, plane).
-// S: the tile shape (DdWideShape or DdNarrowShape).
-// C9: whether the energy-flux correction runs (0, 1), or 2 to ask P.has_c9.
-template <int Lim, int C9, typename S, typename PP>
-__device__ __forceinline__ void dd_tile(const PP &P, const CoefDD &C, unsigned char *smraw,
-                                        double *__restrict__ fout, int x0, int y0)
+// Limited flux differences (F_out - F_in) of pair pr along y, for KR cells of a column (the first at
+// smem offset c, values f): emit(k, t).  The slopes come from a window sliding along the motion: last
+// value, face difference, slope; downward pairs carry differences and slopes, and t, negated.
+template <int Lim, typename S, typename F>
+__device__ __forceinline__ void y_flux_dd(const CoefDD &C, const float2 *tile, int pr, int c, const dd2 *f, F &&emit)
 {
-    double *tile64 = reinterpret_cast<double *>(smraw);
-    float2 *tile = reinterpret_cast<float2 *>(smraw);
-    float4 *suv = reinterpret_cast<float4 *>(smraw + S::uv_off);        // (u_x, u_y), tile + ring
-    float4 *sedge = reinterpret_cast<float4 *>(smraw + S::edge_off);    // x edge values per row and pair
-    const bool c9 = C9 == 2 ? P.has_c9 != 0 : C9 != 0;
-    const int lane = threadIdx.x, ty = threadIdx.y, tid = ty * kTmaTX + lane;
-    constexpr int kThreads = kTmaTX * S::TT;
-    const int nx = P.nx, ny = P.ny;
-    // ---- split: float64 -> hi + lo in place, population pairs (q, q + 4)
-#pragma unroll 4
-    for (int k = tid; k < 8 * S::PL; k += kThreads) {
-        const int a = k < 4 * S::PL ? k : k + 4 * S::PL, b = a + 4 * S::PL;
-        const dd2 v = dd_split2(tile64[a], tile64[b]);
-        tile[a] = v.hi;
-        tile[b] = v.lo;
+    const int sy = tsgn_y(pair_q(pr)), sp = pr >> 2;
+    const int first_row = sy > 0 ? -2 : -1;
+    dd2 w = tile_pair<S>(tile, pr, c + first_row * S::SW);
+    dd2 d = dd2{f2(0.0f, 0.0f), f2(0.0f, 0.0f)}, m = d;
+#pragma unroll
+    for (int i = 1; i < S::KR + 3; i++) {
+        const int row = first_row + i;
+        const dd2 wn = row >= 0 && row < S::KR ? f[row] : tile_pair<S>(tile, pr, c + row * S::SW);
+        const dd2 dn = norm_lim<Lim>(wn - w);
+        if (i >= 2) {
+            const dd2 mn = sy > 0 ? slope_dd<Lim>(d, dn) : slope_dd<Lim>(dn, d);
+            if (i >= 3) {
+                const dd2 dm = sy > 0 ? mn - m : m - mn;
+                // Lim 0: both slopes have the sign of d and at most 4 |d|, and hhy <= 1/4
+                emit(i - 3, Lim == 2 ? d : Lim == 0 ? add_smaller(d, C.hhy[sp] * dm) : d + C.hhy[sp] * dm);
+            }
+            m = mn;
+        }
+        w = wn;
+        d = dn;
     }
-    __syncthreads();
+}
 
-    // ---- phase 1: flow velocity of the ring (for grad u), then the values one column outside the
-    // tile for the x stencils: per row and x-moving pair D(x0 + 32) for lane 31, and the slope
-    // beyond the upwind end, S(x0 - 1) = mc2(D(x0 - 1), D(x0)) for pairs moving right, S(x0 + 32) =
-    // mc2(D(x0 + 32), D(x0 + 33)) for those moving left
+// The same along x for the cell of value f at smem offset c: the lane's face difference
+// D(x) = f(x) - f(x-1) and slope S(x) = mc2(D(x), D(x+1)); the neighbours' values by shuffles, those
+// one column outside the tile from the edge table at ea.  Negated for pairs moving left.
+template <int Lim, typename S>
+__device__ __forceinline__ dd2 x_flux_dd(const CoefDD &C, const float2 *tile, int pr, int c, dd2 f, unsigned ea,
+                                         int lane)
+{
+    const int sx = tsgn_x(pair_q(pr)), sp = pr >> 2;
+    const dd2 D = norm_lim<Lim>(f - tile_pair<S>(tile, pr, c - 1));
+    dd2 Dr = shfl_down_dd(D);
+    take_edge(Dr, ea, lane == kTmaTX - 1);
+    const dd2 t = sx > 0 ? D : Dr;
+    if (Lim == 2) return t;
+    if (Lim == 1) return t + scale2(C.hh[sp], 2.0f) * (sx > 0 ? Dr - D : D - Dr);
+    const dd2 Sx = mc2n(D, Dr);
+    // upwind slope: S(x - 1) for pairs moving right; moving left, d1 = -D(x+1) with slopes -S(x) and
+    // -S(x+1) (mc2n is odd and symmetric, up to the choice between candidates within 2^-47 of each
+    // other)
+    dd2 Su = sx > 0 ? shfl_up_dd(Sx) : shfl_down_dd(Sx);
+    take_edge(Su, ea + 16u, lane == (sx > 0 ? 0 : kTmaTX - 1));
+    return add_smaller(t, C.hh[sp] * (Sx - Su));   // as along y
+}
+
+// Flow velocity of the tile's ring (for grad u, where c9), and the values one column outside the tile
+// for the x stencils: per row and x-moving pair D(x0 + 32) for lane 31, and the slope beyond the
+// upwind end, S(x0 - 1) = mc2(D(x0 - 1), D(x0)) for pairs moving right, S(x0 + 32) =
+// mc2(D(x0 + 32), D(x0 + 33)) for those moving left.  Shared by threads tid of `threads`.
+template <int Lim, typename S>
+__device__ __forceinline__ void ring_and_edges(const float2 *tile, float4 *suv, float4 *sedge, int tid, int threads,
+                                               bool c9)
+{
     constexpr int kRing = 2 * (kTmaTX + S::TR), kEdges = 6 * S::TR;
-    for (int k = tid; k < kRing + kEdges; k += kThreads) {
+    for (int k = tid; k < kRing + kEdges; k += threads) {
         if (k < kRing) {
             if (!c9) continue;
             int i, j;                                                 // column, row in the tile + ring
@@ -310,8 +335,106 @@ __device__ __forceinline__ void dd_tile(const PP &P, const CoefDD &C, unsigned c
             }
         }
     }
-    // the residuals of rows ty*KR .. ty*KR+KR-1 of the tile, column `lane`
+}
+
+}  // namespace
+
+// ---------------------------------------------------------------------------
+// The tile body shared by the single-grid and the batched kernel: the staged float64 tile in
+// shared memory (smraw) is split, then phases 1 and 2 produce the tile's new float64 values.
+// ---------------------------------------------------------------------------
+// P: the context's Params, or the TileGrid block of a batched launch (nx, ny, pitch, plane).
+// S: the tile shape.
+// C9: whether the energy-flux correction runs (0, 1), or 2 to ask P.has_c9.
+template <int Lim, int C9, typename S, typename PP>
+__device__ __forceinline__ void dd_tile(const PP &P, const CoefDD &C, unsigned char *smraw,
+                                        double *__restrict__ fout, int x0, int y0)
+{
+    double *tile64 = reinterpret_cast<double *>(smraw);
+    float2 *tile = reinterpret_cast<float2 *>(smraw);
+    float4 *suv = reinterpret_cast<float4 *>(smraw + S::uv_off);        // (u_x, u_y), tile + ring
+    float4 *sedge = reinterpret_cast<float4 *>(smraw + S::edge_off);    // x edge values per row and pair
+    const bool c9 = C9 == 2 ? P.has_c9 != 0 : C9 != 0;
+    const int lane = threadIdx.x, ty = threadIdx.y, tid = ty * kTmaTX + lane;
+    constexpr int kThreads = kTmaTX * S::TT;
+    const int nx = P.nx, ny = P.ny;
+    // ---- split: float64 -> hi + lo in place, population pairs (q, q + 4)
+#pragma unroll 4
+    for (int k = tid; k < 8 * S::PL; k += kThreads) {
+        const int a = k < 4 * S::PL ? k : k + 4 * S::PL, b = a + 4 * S::PL;
+        const dd2 v = dd_split2(tile64[a], tile64[b]);
+        tile[a] = v.hi;
+        tile[b] = v.lo;
+    }
+    __syncthreads();
+
+    const unsigned edge_a = (unsigned)__cvta_generic_to_shared(sedge);
     const int gx = x0 + lane;
+    if constexpr (S::ROLES) {
+        // ---- warps 0 .. TR-1: residual and relaxation of their row; warps TR .. 2 TR-1: ring, edge
+        // values and convection of theirs.  A small grid has one CTA of these per SM: a warp's chain
+        // of instructions is what its step lasts, and each half is about half of it.
+        float4 *sacc = reinterpret_cast<float4 *>(smraw + S::acc_off);
+        const bool convect = ty >= S::TR;
+        const int r = convect ? ty - S::TR : ty;
+        const int c0 = (r + 2) * S::SW + lane + S::HX;
+        sacc += r * 8 * kTmaTX + lane;
+        dd2 py[8], px[8];                                   // c_y and c_x times the flux differences
+        ResidualDD res;
+        if (convect) {
+            ring_and_edges<Lim, S>(tile, suv, sedge, tid - S::TR * kTmaTX, S::TR * kTmaTX, c9);
+#pragma unroll
+            for (int pr = 0; pr < 8; pr++) {
+                if (tsgn_y(pair_q(pr)) == 0) continue;
+                const dd2 f = tile_pair<S>(tile, pr, c0);
+                y_flux_dd<Lim, S>(C, tile, pr, c0, &f, [&](int, dd2 t) { py[pr] = C.cry[pr >> 2] * t; });
+            }
+        } else {
+            dd2 fp[8];
+#pragma unroll
+            for (int pr = 0; pr < 8; pr++) fp[pr] = tile_pair<S>(tile, pr, c0);
+            res = residual_dd(C, fp);
+            if (c9) suv[(r + 1) * S::UW + (lane + 1)] = quad(res.u);
+        }
+        __syncthreads();
+        if (convect) {
+#pragma unroll
+            for (int pr = 0; pr < 8; pr++) {
+                if (tsgn_x(pair_q(pr)) == 0) continue;
+                px[pr] = C.cr[pr >> 2] * x_flux_dd<Lim, S>(C, tile, pr, c0, tile_pair<S>(tile, pr, c0),
+                                                         edge_a + 32u * (unsigned)(6 * r + xpair_index(pr)), lane);
+            }
+        } else {
+            if (c9) {
+                const int ui = (r + 1) * S::UW + (lane + 1);
+                correct_dd(C, res, unquad(suv[ui + 1]) - unquad(suv[ui - 1]),
+                           unquad(suv[ui + S::UW]) - unquad(suv[ui - S::UW]));
+            }
+            dd2 acc[8];
+            relax_dd(C, res, acc);
+#pragma unroll
+            for (int pr = 0; pr < 8; pr++) sacc[pr * kTmaTX] = quad(acc[pr]);
+        }
+        __syncthreads();
+        if (!convect) return;
+        const int gy = y0 + r;
+        if (gx >= nx || gy >= ny) return;
+        double *o = fout + (long long)(gy + OY) * P.pitch + (gx + OX);
+#pragma unroll
+        for (int pr = 0; pr < 8; pr++) {
+            const int qa = pair_q(pr), sx = tsgn_x(qa), sy = tsgn_y(qa);
+            // f - C - c_x (F_out - F_in)_x - c_y (F_out - F_in)_y
+            dd2 out = tile_pair<S>(tile, pr, c0) - unquad(sacc[pr * kTmaTX]);
+            if (sy != 0) out = sy > 0 ? out - py[pr] : out + py[pr];
+            if (sx != 0) out = sx > 0 ? out - px[pr] : out + px[pr];
+            o[qa * P.plane] = dd_to_double(first(out));
+            o[(qa + 4) * P.plane] = dd_to_double(second(out));
+        }
+        return;
+    } else {
+    // ---- phase 1: the ring, the edge values, and the residuals of rows ty*KR .. ty*KR+KR-1 of the
+    // tile, column `lane`
+    ring_and_edges<Lim, S>(tile, suv, sedge, tid, kThreads, c9);
     const int r0 = ty * S::KR;
     const int c0 = (r0 + 2) * S::SW + lane + S::HX;
     ResidualDD res[S::KR];
@@ -341,7 +464,6 @@ __device__ __forceinline__ void dd_tile(const PP &P, const CoefDD &C, unsigned c
     // compiler does for loads from equal addresses) they would be spilled
     int c1 = c0;
     asm volatile("" : "+r"(c1));
-    const unsigned edge_a = (unsigned)__cvta_generic_to_shared(sedge) + 32u * 6u * (unsigned)r0;
     // f - C - c_x (F_out - F_in)_x - c_y (F_out - F_in)_y
 #pragma unroll
     for (int pr = 0; pr < 8; pr++) {
@@ -354,55 +476,15 @@ __device__ __forceinline__ void dd_tile(const PP &P, const CoefDD &C, unsigned c
             f[k] = tile_pair<S>(tile, pr, c1 + k * S::SW);
             out[k] = f[k] - acc[k][pr];
         }
-        if (sy != 0) {
-            // y slopes from a window sliding along the motion: last value, face difference, slope;
-            // downward pairs carry differences and slopes negated
-            const int first_row = sy > 0 ? -2 : -1;
-            dd2 w = tile_pair<S>(tile, pr, c1 + first_row * S::SW);
-            dd2 d = dd2{f2(0.0f, 0.0f), f2(0.0f, 0.0f)}, m = d;
-#pragma unroll
-            for (int i = 1; i < S::KR + 3; i++) {
-                const int row = first_row + i;
-                const dd2 wn = row >= 0 && row < S::KR ? f[row] : tile_pair<S>(tile, pr, c1 + row * S::SW);
-                const dd2 dn = norm_lim<Lim>(wn - w);
-                if (i >= 2) {
-                    const dd2 mn = sy > 0 ? slope_dd<Lim>(d, dn) : slope_dd<Lim>(dn, d);
-                    if (i >= 3) {
-                        const int k = i - 3;
-                        const dd2 dm = sy > 0 ? mn - m : m - mn;
-                        // Lim 0: both slopes have the sign of d and at most 4 |d|, and hhy <= 1/4
-                        const dd2 t = Lim == 2   ? d
-                                      : Lim == 0 ? add_smaller(d, C.hhy[sp] * dm)
-                                                 : d + C.hhy[sp] * dm;
-                        out[k] = sy > 0 ? out[k] - C.cry[sp] * t : out[k] + C.cry[sp] * t;
-                    }
-                    m = mn;
-                }
-                w = wn;
-                d = dn;
-            }
-        }
+        if (sy != 0)
+            y_flux_dd<Lim, S>(C, tile, pr, c1, f, [&](int k, dd2 t) {
+                out[k] = sy > 0 ? out[k] - C.cry[sp] * t : out[k] + C.cry[sp] * t;
+            });
 #pragma unroll
         for (int k = 0; k < S::KR; k++) {
             if (sx != 0) {
-                // this lane's face difference D(x) = f(x) - f(x-1) and slope S(x) =
-                // mc2(D(x), D(x+1)); the neighbours' values by shuffles, those one column
-                // outside the tile from the edge table
-                const unsigned ea = edge_a + 32u * (unsigned)(6 * k + xpair_index(pr));
-                const dd2 D = norm_lim<Lim>(f[k] - tile_pair<S>(tile, pr, c1 + k * S::SW - 1));
-                dd2 Dr = shfl_down_dd(D);
-                take_edge(Dr, ea, lane == kTmaTX - 1);
-                dd2 t = sx > 0 ? D : Dr;
-                if (Lim == 1) t = t + scale2(C.hh[sp], 2.0f) * (sx > 0 ? Dr - D : D - Dr);
-                if (Lim == 0) {
-                    const dd2 Sx = mc2n(D, Dr);
-                    // upwind slope: S(x - 1) for pairs moving right; moving left, d1 = -D(x+1) with
-                    // slopes -S(x) and -S(x+1) (mc2n is odd and symmetric, up to the choice between
-                    // candidates within 2^-47 of each other)
-                    dd2 Su = sx > 0 ? shfl_up_dd(Sx) : shfl_down_dd(Sx);
-                    take_edge(Su, ea + 16u, lane == (sx > 0 ? 0 : kTmaTX - 1));
-                    t = add_smaller(t, C.hh[sp] * (Sx - Su));   // as for y
-                }
+                const dd2 t = x_flux_dd<Lim, S>(C, tile, pr, c1 + k * S::SW, f[k],
+                                                edge_a + 32u * (unsigned)(6 * (r0 + k) + xpair_index(pr)), lane);
                 out[k] = sx > 0 ? out[k] - C.cr[sp] * t : out[k] + C.cr[sp] * t;
             }
             const int gy = y0 + r0 + k;
@@ -412,6 +494,7 @@ __device__ __forceinline__ void dd_tile(const PP &P, const CoefDD &C, unsigned c
                 o[(qa + 4) * P.plane] = dd_to_double(second(out[k]));
             }
         }
+    }
     }
 }
 
@@ -497,8 +580,7 @@ k_step_dd_batch(const __grid_constant__ TmaBatchArgs A, const TileGrid<CoefDD> *
     int x0, y0;
     const int g = batch_tile(A, blockIdx.x, S::TR, x0, y0);
     const unsigned bar_a = (unsigned)__cvta_generic_to_shared(&bar);
-    grid_dependency_wait();
-    grid_launch_dependents();
+    batch_begin(A.late);
     if (tid == 0)
         batch_issue<S::TR, S::HX>(A, g, x0, y0, (unsigned)__cvta_generic_to_shared(smraw), bar_a,
                                   (unsigned)S::tile_bytes, S::CTAS);
@@ -518,13 +600,14 @@ k_step_dd_batch(const __grid_constant__ TmaBatchArgs A, const TileGrid<CoefDD> *
             atomicExch(A.err[g], 1);
             mbar_wait(bar_a, 0);               // let a late copy land before the CTA exits (bounded)
         }
-        return;
+    } else {
+        if (edge) {
+            ghost.store(reinterpret_cast<double *>(smraw));
+            __syncthreads();
+        }
+        dd_tile<Lim, 2, S>(Ts, Ts.cf, smraw, static_cast<double *>(A.out[g]), x0, y0);
     }
-    if (edge) {
-        ghost.store(reinterpret_cast<double *>(smraw));
-        __syncthreads();
-    }
-    dd_tile<Lim, 2, S>(Ts, Ts.cf, smraw, static_cast<double *>(A.out[g]), x0, y0);
+    batch_end(A.late, tid);
 }
 
 // Coefficients in double-float from the float64 tables (host).
@@ -573,21 +656,29 @@ static cudaError_t launch_dd_shape(const Params &P, const CoefDD &C, const CUten
     return launch_chained(fn, grid, block, S::smem_bytes, st, P, C, tm, a, b, err);
 }
 
-bool dd_narrow_supported(const Params &P)
+bool dd_shape_supported(const Params &P, int shape)
 {
-    using S = DdNarrowShape;
-    return P.pitch >= S::SW && P.ny + 4 >= S::SH && P.nx >= kTmaTX;
+    return P.pitch >= DdWideShape::SW && P.nx >= kTmaTX && P.ny >= kDdRows[shape];
+}
+
+double dd_shape_time(int shape, long long tiles, int sms)
+{
+    constexpr double whole[kDdShapes] = {23.5, 13.0, 8.3}, one[kDdShapes] = {15.5, 10.5, 8.2},
+                     two[kDdShapes] = {27.0, 16.4, 12.3};
+    const long long slots = 2LL * sms, rest = tiles % slots;
+    return (double)(tiles / slots) * whole[shape] + (rest == 0 ? 0.0 : (rest <= sms ? one[shape] : two[shape]));
 }
 
 cudaError_t launch_step_dd(const Params &P, const void *coef, const void *tmap, const void *fin, void *fout,
-                           int *err, cudaStream_t st, bool narrow)
+                           int *err, cudaStream_t st, int shape)
 {
     const CUtensorMap &tm = *reinterpret_cast<const CUtensorMap *>(tmap);
     const CoefDD &C = *reinterpret_cast<const CoefDD *>(coef);
     const double *a = (const double *)fin;
     double *b = (double *)fout;
-    return narrow ? launch_dd_shape<DdNarrowShape>(P, C, tm, a, b, err, st)
-                  : launch_dd_shape<DdWideShape>(P, C, tm, a, b, err, st);
+    return shape == kDdNarrow ? launch_dd_shape<DdNarrowShape>(P, C, tm, a, b, err, st)
+           : shape == kDdMid  ? launch_dd_shape<DdMidShape>(P, C, tm, a, b, err, st)
+                              : launch_dd_shape<DdWideShape>(P, C, tm, a, b, err, st);
 }
 
 template <typename S>
@@ -600,32 +691,34 @@ static cudaError_t launch_dd_batch_shape(const TmaBatchArgs &A, const TileGrid<C
 }
 
 cudaError_t launch_step_dd_batch(const TmaBatchArgs &A, const TileGrid<CoefDD> *tg, const Params *Pall, int limiter,
-                                 bool narrow, cudaStream_t st)
+                                 int shape, cudaStream_t st)
 {
     const int ntiles = A.first[A.n];
     if (ntiles <= 0) return cudaSuccess;
-    return narrow ? launch_dd_batch_shape<DdNarrowShape>(A, tg, Pall, limiter, ntiles, st)
-                  : launch_dd_batch_shape<DdWideShape>(A, tg, Pall, limiter, ntiles, st);
+    return shape == kDdNarrow ? launch_dd_batch_shape<DdNarrowShape>(A, tg, Pall, limiter, ntiles, st)
+           : shape == kDdMid  ? launch_dd_batch_shape<DdMidShape>(A, tg, Pall, limiter, ntiles, st)
+                              : launch_dd_batch_shape<DdWideShape>(A, tg, Pall, limiter, ntiles, st);
+}
+
+template <typename S>
+static cudaError_t dd_prepare_shape()
+{
+    cudaError_t e = cudaSuccess;
+    for (const void *fn : {(const void *)k_step_dd<0, false, S>, (const void *)k_step_dd<0, true, S>,
+                           (const void *)k_step_dd<1, false, S>, (const void *)k_step_dd<1, true, S>,
+                           (const void *)k_step_dd<2, false, S>, (const void *)k_step_dd<2, true, S>,
+                           (const void *)k_step_dd_batch<0, S>, (const void *)k_step_dd_batch<1, S>,
+                           (const void *)k_step_dd_batch<2, S>})
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem_bytes);
+    return e;
 }
 
 cudaError_t dd_prepare()
 {
-    cudaError_t e = cudaSuccess;
-    auto set = [&](const void *fn) {
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DdWideShape::smem_bytes);
-    };
-    set((const void *)k_step_dd<0, false>);
-    set((const void *)k_step_dd<0, true>);
-    set((const void *)k_step_dd<1, false>);
-    set((const void *)k_step_dd<1, true>);
-    set((const void *)k_step_dd<2, false>);
-    set((const void *)k_step_dd<2, true>);
-    set((const void *)k_step_dd_batch<0>);
-    set((const void *)k_step_dd_batch<1>);
-    set((const void *)k_step_dd_batch<2>);
-    // narrow tiles: within the default 48 KB of dynamic shared memory
-    static_assert(DdNarrowShape::smem_bytes <= 48 * 1024, "narrow tile within the default shared memory");
+    cudaError_t e = dd_prepare_shape<DdWideShape>();
+    if (e == cudaSuccess) e = dd_prepare_shape<DdMidShape>();
+    if (e == cudaSuccess) e = dd_prepare_shape<DdNarrowShape>();
     return e;
 }
 

@@ -334,8 +334,7 @@ k_step_tma_batch(const __grid_constant__ TmaBatchArgs A, const TileGrid<Coef<flo
     int x0, y0;
     const int g = batch_tile(A, blockIdx.x, S::TR, x0, y0);
     const unsigned bar_a = (unsigned)__cvta_generic_to_shared(&bar);
-    grid_dependency_wait();
-    grid_launch_dependents();
+    batch_begin(A.late);
     if (tid == 0)
         batch_issue<S::TR, S::HX>(A, g, x0, y0, (unsigned)__cvta_generic_to_shared(tile), bar_a,
                                   (unsigned)S::tile_bytes, S::CTAS);
@@ -355,16 +354,17 @@ k_step_tma_batch(const __grid_constant__ TmaBatchArgs A, const TileGrid<Coef<flo
             atomicExch(A.err[g], 1);
             mbar_wait(bar_a, 0);               // let a late copy land before the CTA exits (bounded)
         }
-        return;
-    }
-    if (edge) {
-        ghost.store(tile);
+    } else {
+        if (edge) {
+            ghost.store(tile);
+            __syncthreads();
+        }
+        flow_phase<float, true>(Ts.cf, tile, su, nullptr, nullptr, tid);
         __syncthreads();
+        phase2_packed<true, Lim>(Ts, reinterpret_cast<const float2 *>(tile), reinterpret_cast<const float2 *>(su),
+                                 lane, ty, x0, y0, static_cast<float *>(A.out[g]));
     }
-    flow_phase<float, true>(Ts.cf, tile, su, nullptr, nullptr, tid);
-    __syncthreads();
-    phase2_packed<true, Lim>(Ts, reinterpret_cast<const float2 *>(tile), reinterpret_cast<const float2 *>(su), lane,
-                             ty, x0, y0, static_cast<float *>(A.out[g]));
+    batch_end(A.late, tid);
 }
 
 cudaError_t launch_step_tma_batch(const TmaBatchArgs &A, const TileGrid<Coef<float>> *tg, const Params *Pall,

@@ -73,6 +73,17 @@ __device__ __forceinline__ R slope2(R a, R b)
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Start and end of a batched launch (`late`: TmaBatchArgs).
+__device__ __forceinline__ void batch_begin(int late)
+{
+    if (!late) grid_dependency_wait();
+    grid_launch_dependents();
+}
+__device__ __forceinline__ void batch_end(int late, int tid)
+{
+    if (late && tid == 0 && blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1) grid_dependency_wait();
+}
+
 // Coordinate a read at v goes to along an axis of n cells: the wrapped cell past a periodic edge
 // (kind 0), the edge cell past a zero-gradient one (1), else v itself.
 __device__ __forceinline__ int ghost_source(int v, int n, int kind_lo, int kind_hi)
