@@ -694,16 +694,24 @@ k_totals_partial(const __grid_constant__ Params P, const R *__restrict__ f, doub
         for (int x = threadIdx.x; x < P.nx; x += blockDim.x) {
             R g[NQ];
             load16(f, P.plane, row + x, g);
+            if constexpr (sizeof(R) == sizeof(double)) {
+                // straight into the accumulators: 16 float64 additions a cell, which bound this pass
 #pragma unroll
-            for (int q = 0; q < NQ; q++) run[q] += g[q];
-            if (sizeof(R) == sizeof(double) || ++cnt == 32) {
+                for (int q = 0; q < NQ; q++) a[q] += g[q];
+            } else {
 #pragma unroll
-                for (int q = 0; q < NQ; q++) { a[q] += (double)run[q]; run[q] = R(0); }
-                cnt = 0;
+                for (int q = 0; q < NQ; q++) run[q] += g[q];
+                if (++cnt == 32) {
+#pragma unroll
+                    for (int q = 0; q < NQ; q++) { a[q] += (double)run[q]; run[q] = R(0); }
+                    cnt = 0;
+                }
             }
         }
+        if constexpr (sizeof(R) == sizeof(float)) {
 #pragma unroll
-        for (int q = 0; q < NQ; q++) a[q] += (double)run[q];
+            for (int q = 0; q < NQ; q++) a[q] += (double)run[q];
+        }
     }
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
