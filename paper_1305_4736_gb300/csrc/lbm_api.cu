@@ -55,9 +55,9 @@ struct lbm_ctx {
     CUtensorMap smap[2];          // row-copy descriptors (streaming kernel)
     CUtensorMap pmap[2];          // tile-copy descriptors of the double-buffered kernel
     CUtensorMap dmap[lbm::kDdShapes][2];   // tile-copy descriptors of the double-float tile shapes
-    // lbm_step replays pairs of steps (ghost fill + fused step, twice) from a CUDA graph per
-    // starting buffer, captured on a private stream at first use; lbm_autotune drops them
-    cudaGraphExec_t pair[2] = {nullptr, nullptr};
+    // lbm_step replays pairs or runs of kRunSteps steps from a CUDA graph per starting buffer,
+    // captured on a private stream at first use; lbm_autotune drops them
+    cudaGraphExec_t pair[2] = {nullptr, nullptr}, run[2] = {nullptr, nullptr};
     cudaStream_t cap = nullptr;
     bool initialized = false;
     long long steps = 0;
@@ -325,7 +325,7 @@ bool stream_ready(lbm_ctx *c)
 
 bool tma_ready(lbm_ctx *c)
 {
-    return lbm::tma_supported(c->P, c->prec) && lbm::tma_prepare() == cudaSuccess && make_tile_maps(c);
+    return lbm::tma_supported(c->P, c->prec) && lbm::tma_prepare(c->prec, c->P.limiter) == cudaSuccess && make_tile_maps(c);
 }
 
 int edges_of_kind(const lbm_ctx *c, int kind)
@@ -347,7 +347,7 @@ int ghost_edges(const lbm_ctx *c)
 // maps and the CoefDD of the context.
 bool dd_ready(lbm_ctx *c)
 {
-    if (c->prec != LBM_FP64 || !lbm::tma_supported(c->P, LBM_FP64) || lbm::dd_prepare() != cudaSuccess) return false;
+    if (c->prec != LBM_FP64 || !lbm::tma_supported(c->P, LBM_FP64) || lbm::dd_prepare(c->P) != cudaSuccess) return false;
     lbm::coef_dd(c->P, &c->cdd);
     c->dd8 = dd_pick(c, lbm::kDdMid, lbm::kDdWide);
     return make_dd_maps(c, c->dd8);
@@ -356,7 +356,7 @@ bool dd_ready(lbm_ctx *c)
 // The same on the tiles for small grids, 32 x 8 or 32 x 4 (grids of at least 32 x 4).
 bool ddn_ready(lbm_ctx *c)
 {
-    if (c->prec != LBM_FP64 || !lbm::dd_shape_supported(c->P, lbm::kDdNarrow) || lbm::dd_prepare() != cudaSuccess)
+    if (c->prec != LBM_FP64 || !lbm::dd_shape_supported(c->P, lbm::kDdNarrow) || lbm::dd_prepare(c->P) != cudaSuccess)
         return false;
     lbm::coef_dd(c->P, &c->cdd);
     c->dd9 = dd_pick(c, lbm::kDdMid, lbm::kDdNarrow);
@@ -384,35 +384,38 @@ cudaError_t launch_fused_step(lbm_ctx *c, int in, cudaStream_t st)
     return lbm::launch_step(c->P, c->prec, c->f[in], c->f[in ^ 1], st, c->plain_ty);
 }
 
-constexpr int kGraphSteps = 16;
+// Calls of at least kGraphSteps steps replay graphs of two steps, calls of at least kRunMin graphs of
+// kRunSteps: consecutive graphs do not overlap as the chained launches inside one do (200 x 4 float32:
+// 5.1 us a step in pairs, 4.2 in runs of 16), but a longer one takes longer to build.
+constexpr int kGraphSteps = 16, kRunSteps = 16, kRunMin = 64;
 
-// The pair graph of context c starting from buffer `in` (two ghost fills and fused steps), captured
-// on the context's private stream at first use.
-cudaError_t step_pair_graph(lbm_ctx *c, int in)
+// Graph of `steps` steps (even) of context c starting from buffer `in` (a ghost launch where needed and
+// the fused step, each), captured on the context's private stream at first use.
+cudaError_t step_graph(lbm_ctx *c, cudaGraphExec_t *exec, int in, int steps)
 {
-    if (c->pair[in]) return cudaSuccess;
+    if (*exec) return cudaSuccess;
     cudaError_t ce = c->cap ? cudaSuccess : cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking);
     cudaGraph_t graph = nullptr;
     if (ce == cudaSuccess) ce = cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal);
     if (ce != cudaSuccess) return ce;
     cudaError_t le = cudaSuccess;
-    for (int k = 0; k < 2 && le == cudaSuccess; k++) {
-        le = launch_step_ghosts(c, in ^ k, c->cap);
-        if (le == cudaSuccess) le = launch_fused_step(c, in ^ k, c->cap);
+    for (int k = 0; k < steps && le == cudaSuccess; k++) {
+        le = launch_step_ghosts(c, in ^ (k & 1), c->cap);
+        if (le == cudaSuccess) le = launch_fused_step(c, in ^ (k & 1), c->cap);
     }
     ce = cudaStreamEndCapture(c->cap, &graph);
     if (ce == cudaSuccess) ce = le;
-    if (ce == cudaSuccess) ce = cudaGraphInstantiate(&c->pair[in], graph, 0);
+    if (ce == cudaSuccess) ce = cudaGraphInstantiate(exec, graph, 0);
     if (graph) cudaGraphDestroy(graph);
-    if (ce != cudaSuccess) c->pair[in] = nullptr;
+    if (ce != cudaSuccess) *exec = nullptr;
     return ce;
 }
 
 void drop_step_graphs(lbm_ctx *c)
 {
-    for (cudaGraphExec_t &g : c->pair) {
-        if (g) cudaGraphExecDestroy(g);
-        g = nullptr;
+    for (cudaGraphExec_t *g : {&c->pair[0], &c->pair[1], &c->run[0], &c->run[1]}) {
+        if (*g) cudaGraphExecDestroy(*g);
+        *g = nullptr;
     }
 }
 
@@ -751,17 +754,17 @@ int lbm_step(lbm_ctx *c, int n)
     if (!c->initialized) return fail(c, LBM_ERR_STATE, "lbm_step before lbm_init / lbm_set_state");
     cudaError_t ce = cudaSetDevice(c->device);
     if (ce != cudaSuccess) return cuda_fail(c, ce, "cudaSetDevice");
-    // runs of at least kGraphSteps steps outside profiling: pairs of steps from a graph (one
-    // launch instead of four; on small grids the launches, not the kernels, set the pace)
+    // outside profiling, graphs (one launch for many; on small grids the launches set the pace)
     if (!c->prof && n >= kGraphSteps) {
-        ce = step_pair_graph(c, c->cur);
+        const int unit = n >= kRunMin ? kRunSteps : 2;
+        cudaGraphExec_t *exec = unit == 2 ? &c->pair[c->cur] : &c->run[c->cur];
+        ce = step_graph(c, exec, c->cur, unit);
         if (ce != cudaSuccess) return cuda_fail(c, ce, "step graph");
-        for (; n >= 2; n -= 2) {
-            ce = cudaGraphLaunch(c->pair[c->cur], c->stream);
+        for (; n >= unit; n -= unit) {
+            ce = cudaGraphLaunch(*exec, c->stream);
             if (ce != cudaSuccess) return cuda_fail(c, ce, "step graph launch");
-            c->steps += 2;
+            c->steps += unit;
         }
-        if (n == 0) return LBM_OK;
     }
     for (int s = 0; s < n; s++) {
         cudaEvent_t *ev = nullptr;
@@ -1150,6 +1153,7 @@ struct lbm_batch {
             int k, y0, rows;
         };
         std::vector<Span> tk[lbm::kDdShapes];    // float32: [0]
+        std::vector<Span> alone;                 // spans from row 0 with a launch of their own
         void *tblock = nullptr;
         size_t tbytes = 0;
         int ntt = 0;                             // tiles per step
@@ -1165,9 +1169,10 @@ struct lbm_batch {
     cudaStream_t fork[kForks] = {};
     cudaEvent_t ev_fork = nullptr, ev_join[kForks] = {};
     cudaStream_t stream = nullptr, cap = nullptr;
-    cudaGraphExec_t exec2 = nullptr;
+    cudaGraphExec_t exec2 = nullptr, run = nullptr;   // graphs of 2 and of kRunSteps steps
     lbm_allocator alloc{};
     int device = 0, ctas = 0;
+    int launches = 0;                           // kernels per step
 };
 
 namespace {
@@ -1227,6 +1232,15 @@ cudaError_t batch_launch_tma(lbm_batch *b, const lbm_batch::Group &g, int phase,
 {
     const char *tg = (const char *)g.tblock;
     cudaError_t ce = cudaSuccess;
+    for (size_t j = 0; j < g.alone.size() && ce == cudaSuccess; j++) {
+        lbm_ctx *c = b->ctxs[g.members[g.alone[j].k]];
+        const int in = c->cur ^ phase;
+        ce = g.prec == LBM_FP64
+                 ? lbm::launch_step_dd(c->P, &c->cdd, &c->dmap[lbm::kDdWide][in], c->f[in], c->f[in ^ 1], c->tma_err, st,
+                                       lbm::kDdWide, *late, g.alone[j].rows)
+                 : lbm::launch_step_tma(c->P, c->prec, &c->tmap[in], c->f[in], c->f[in ^ 1], c->tma_err, st, *late);
+        *late = 1;
+    }
     for (int k = 0; k < lbm::kDdShapes && ce == cudaSuccess; k++) {
         ce = batch_launch_tma_list(b, g, k, tg, phase, late, st);
         tg += g.tk[k].size() * sizeof(lbm::TileGrid<lbm::CoefDD>);
@@ -1282,6 +1296,31 @@ bool batch_tma(const lbm_ctx *c)
     return (c->prec == LBM_FP32_DEV && c->use_tma) || (c->prec == LBM_FP64 && (c->use_dd || c->use_ddn));
 }
 
+// Tiles of 32 x 16 cells of a grid.
+long long wide_tiles(const lbm_ctx *c)
+{
+    const int tr = lbm::DdWideShape::TR;
+    static_assert(tr == lbm::TmaShape<float>::TR, "one rule for both precisions");
+    return (long long)((c->P.nx + lbm::kTmaTX - 1) / lbm::kTmaTX) * (c->P.ny / tr);
+}
+
+// Members of a batched TMA-staged launch with at least kAloneTiles tiles (of 32 x 16 cells) get a launch of
+// their own, whose coefficients are operands from the constant bank and not in shared memory, in groups
+// whose members have kAloneMean tiles on average: between short launches slots stay empty.  Measured, us
+// per batch step, all batched and with the rule: 24 float32 grids of 0.58 M cells on average 347 and 315,
+// of 0.14 M 94.2 and 87.7; float64, 2070 and 1906, 550 and 514.  Without the condition on the average, 21
+// float64 serving grids of 38 thousand cells 174 and 195, 57 406 and 420, 255 float32 ones 487 and 483.
+constexpr int kAloneTiles = 64, kAloneMean = 256;
+
+// Rows (from row 0) of member c that such a launch covers: the whole float32 grid; of a float64 one the
+// rows of full tiles, or all where the last tile row is more than 3/4 full.
+int alone_rows(const lbm_ctx *c, bool allowed)
+{
+    const int tr = lbm::DdWideShape::TR, ny = c->P.ny;
+    if (!allowed || wide_tiles(c) < kAloneTiles) return 0;
+    return c->prec == LBM_FP32_DEV || 4 * (ny % tr) > 3 * tr ? ny : ny - ny % tr;
+}
+
 bool batch_solo(const lbm_ctx *c, int sms)
 {
     return (c->use_stream || c->use_pipe) && (long long)c->P.nx * c->P.ny >= 512LL * sms;
@@ -1333,6 +1372,8 @@ int lbm_batch_create(lbm_ctx *const *ctxs, int n, lbm_batch **out)
         g->tma.push_back(tma ? 1 : 0);
     }
     for (auto &g : b->groups) {
+        ce = g.prec == LBM_FP64 ? lbm::dd_batch_prepare(g.limiter) : lbm::tma_batch_prepare(g.limiter);
+        if (ce != cudaSuccess) { lbm_batch_destroy(b); return cuda_fail(nullptr, ce, "batch kernels"); }
         // float64 groups too small to give every SM four 256-cell tiles take 64-cell tiles,
         // which spread their float64 work over more SMs
         if (g.prec == LBM_FP64) {
@@ -1345,6 +1386,13 @@ int lbm_batch_create(lbm_ctx *const *ctxs, int n, lbm_batch **out)
         std::vector<lbm::Params> hp;
         std::vector<lbm::TileGrid<lbm::Coef<float>>> htf;
         std::vector<lbm::TileGrid<lbm::CoefDD>> htd[lbm::kDdShapes];
+        long long mean = 0, count = 0;
+        for (size_t k = 0; k < g.members.size(); k++)
+            if (g.tma[k]) {
+                mean += wide_tiles(b->ctxs[g.members[k]]);
+                count++;
+            }
+        const bool allowed = mean >= kAloneMean * count;
         // The double-float members' rows go to the shape that the group's tiles together last shortest
         // on, those left over to smaller shapes (the shapes run the same operations on every value: the
         // same bits).
@@ -1355,7 +1403,7 @@ int lbm_batch_create(lbm_ctx *const *ctxs, int n, lbm_batch **out)
                 const lbm_ctx *c = b->ctxs[g.members[k]];
                 for (int sh = 0; sh < lbm::kDdShapes && g.tma[k]; sh++)
                     tiles[sh] += (long long)((c->P.nx + lbm::kTmaTX - 1) / lbm::kTmaTX) *
-                                 ((c->P.ny + lbm::kDdRows[sh] - 1) / lbm::kDdRows[sh]);
+                                 ((c->P.ny - alone_rows(c, allowed) + lbm::kDdRows[sh] - 1) / lbm::kDdRows[sh]);
             }
             for (int sh = 1; sh < lbm::kDdShapes; sh++)
                 if (lbm::dd_shape_time(sh, tiles[sh], sms) < lbm::dd_shape_time(dd_shape, tiles[dd_shape], sms))
@@ -1369,12 +1417,18 @@ int lbm_batch_create(lbm_ctx *const *ctxs, int n, lbm_batch **out)
             if (hp.back().ghost) g.max_ghost = std::max(g.max_ghost, 4 * (c->P.nx + c->P.ny));
             if (g.tma[k]) {
                 const int ntx = (c->P.nx + lbm::kTmaTX - 1) / lbm::kTmaTX;
+                // a large member has its own launch of the single-grid kernel
+                int y = alone_rows(c, allowed);
+                if (y > 0) {
+                    g.alone.push_back({(int)k, 0, y});
+                    g.ntt += ntx * ((y + lbm::DdWideShape::TR - 1) / lbm::DdWideShape::TR);
+                }
+                if (y == c->P.ny) continue;
                 if (g.prec == LBM_FP64) {
                     const lbm::TileGrid<lbm::CoefDD> blk{c->P.nx, c->P.ny, c->P.pitch, c->P.has_c9,
                                                                 c->P.plane, (long long)k, c->cdd};
                     // rows by shape, from dd_shape down: a part-filled last tile row stays with a shape
                     // where it holds more than 3/4 of its rows (a tile costs 23.5 : 13 : 8.3)
-                    int y = 0;
                     for (int sh = dd_shape; sh < lbm::kDdShapes && y < c->P.ny; sh++) {
                         if (!lbm::dd_shape_supported(c->P, sh)) continue;
                         const int tr = lbm::kDdRows[sh], left = c->P.ny - y;
@@ -1403,6 +1457,8 @@ int lbm_batch_create(lbm_ctx *const *ctxs, int n, lbm_batch **out)
                 for (int x = 0; x < c->P.nx; x += tw) tiles.push_back(make_int4((int)k, x, y, lt));
         }
         g.ntiles = (int)tiles.size();
+        b->launches += (int)g.alone.size() + (g.ntiles > 0) + (g.max_ghost > 0);
+        for (const auto &list : g.tk) b->launches += !list.empty();
         // sections start on 256-byte boundaries (the tile list is read as int4)
         auto up = [](size_t v) { return (v + 255) / 256 * 256; };
         const size_t np = up(hp.size() * sizeof(lbm::Params)), ng = up(g.hG.size() * sizeof(lbm::BatchGrid));
@@ -1430,6 +1486,7 @@ int lbm_batch_create(lbm_ctx *const *ctxs, int n, lbm_batch **out)
         if (ce == cudaSuccess) ce = cudaStreamSynchronize(b->stream);
         if (ce != cudaSuccess) { lbm_batch_destroy(b); return cuda_fail(nullptr, ce, "batch tables"); }
     }
+    b->launches += (int)b->solo.size();
     ce = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
     if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming);
     for (int k = 0; k < lbm_batch::kForks && ce == cudaSuccess; k++) {
@@ -1451,43 +1508,52 @@ int lbm_batch_step(lbm_batch *b, int n)
     cudaError_t ce = cudaSetDevice(b->device);
     if (ce == cudaSuccess) ce = batch_upload_cur(b);
     if (ce != cudaSuccess) return cuda_fail(c0, ce, "batch");
-    if (b->exec2) {
-        // the graph's own-kernel and batched TMA-staged launches name their buffers: recapture
+    if (b->exec2 || b->run) {
+        // the graphs' own-kernel and batched TMA-staged launches name their buffers: recapture
         // if a context was stepped alone an odd number of times since the capture
         bool same = true;
         for (size_t k = 0; k < b->ctxs.size(); k++) same = same && b->ctxs[k]->cur == b->cap_cur[k];
         if (!same) {
             ce = cudaStreamSynchronize(b->stream);
-            if (ce == cudaSuccess) ce = cudaGraphExecDestroy(b->exec2);
-            b->exec2 = nullptr;
+            for (cudaGraphExec_t *g : {&b->exec2, &b->run}) {
+                if (*g && ce == cudaSuccess) ce = cudaGraphExecDestroy(*g);
+                *g = nullptr;
+            }
             if (ce != cudaSuccess) return cuda_fail(c0, ce, "batch graph");
         }
     }
-    if (n >= 2 && !b->exec2) {
+    // whole units from a graph captured once (the tables' current contents are read at replay), the
+    // steps left over launched directly
+    // (runs of kRunSteps where a step is a launch or two: there the gap between graphs shows, and the
+    // graph is quickly built)
+    const int unit = n >= kRunMin && b->launches <= 2 ? kRunSteps : 2;
+    cudaGraphExec_t *exec = unit == 2 ? &b->exec2 : &b->run;
+    if (n >= unit && !*exec) {
         b->cap_cur.clear();
         for (lbm_ctx *c : b->ctxs) b->cap_cur.push_back(c->cur);
-        // capture two steps (both buffer parities) once; replays read the tables' current contents
         cudaGraph_t graph = nullptr;
         ce = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal);
         if (ce == cudaSuccess) {
-            cudaError_t le = batch_launch_step(b, 0, b->cap);
-            if (le == cudaSuccess) le = batch_launch_step(b, 1, b->cap);
+            cudaError_t le = cudaSuccess;
+            for (int k = 0; k < unit && le == cudaSuccess; k++) le = batch_launch_step(b, k & 1, b->cap);
             ce = cudaStreamEndCapture(b->cap, &graph);
             if (ce == cudaSuccess) ce = le;
         }
-        if (ce == cudaSuccess) ce = cudaGraphInstantiate(&b->exec2, graph, 0);
+        if (ce == cudaSuccess) ce = cudaGraphInstantiate(exec, graph, 0);
         if (graph) cudaGraphDestroy(graph);
-        if (ce != cudaSuccess) { b->exec2 = nullptr; return cuda_fail(c0, ce, "batch graph"); }
+        if (ce != cudaSuccess) { *exec = nullptr; return cuda_fail(c0, ce, "batch graph"); }
     }
-    for (int k = 0; k + 1 < n; k += 2) {
-        ce = cudaGraphLaunch(b->exec2, b->stream);
+    int left = n;
+    for (; left >= unit; left -= unit) {
+        ce = cudaGraphLaunch(*exec, b->stream);
         if (ce != cudaSuccess) return cuda_fail(c0, ce, "batch graph launch");
     }
-    if (n & 1) {
-        ce = batch_launch_step(b, 0, b->stream);
+    for (int k = 0; k < left; k++) {
+        ce = batch_launch_step(b, k & 1, b->stream);
         if (ce != cudaSuccess) return cuda_fail(c0, ce, "batch step");
-        for (lbm_ctx *c : b->ctxs) c->cur ^= 1;
     }
+    if (n & 1)
+        for (lbm_ctx *c : b->ctxs) c->cur ^= 1;
     for (lbm_ctx *c : b->ctxs) c->steps += n;
     return LBM_OK;
 }
@@ -1498,6 +1564,7 @@ void lbm_batch_destroy(lbm_batch *b)
     cudaSetDevice(b->device);
     cudaStreamSynchronize(b->stream);
     if (b->exec2) cudaGraphExecDestroy(b->exec2);
+    if (b->run) cudaGraphExecDestroy(b->run);
     if (b->cap) cudaStreamDestroy(b->cap);
     for (int k = 0; k < lbm_batch::kForks; k++) {
         if (b->fork[k]) cudaStreamDestroy(b->fork[k]);

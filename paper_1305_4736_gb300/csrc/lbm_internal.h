@@ -189,11 +189,14 @@ cudaError_t launch_step_dd_batch(const TmaBatchArgs &A, const TileGrid<CoefDD> *
 // Failure-path check of the bounded mbarrier waits (lbm_wait_selftest): *flag = 1 when the
 // wait on a phase that nothing completes gave up at its limit; *ms = the kernel's duration.
 cudaError_t wait_selftest(int *flag, float *ms);
-cudaError_t tma_prepare();   // opt the kernels in to their dynamic shared memory (once per device)
+// Opt the kernels that a context (a batch's groups of a limiter) launches in to their dynamic shared
+// memory.
+cudaError_t tma_prepare(int prec, int limiter);
+cudaError_t tma_batch_prepare(int limiter);
 // `tmap` points to the CUtensorMap of the input buffer fin (3-D: pitch x (ny+4) x 16).  The tiles fill
 // the ghost cells of every edge but walls themselves, from the interior of fin.
 cudaError_t launch_step_tma(const Params &P, int prec, const void *tmap, const void *fin, void *fout, int *err,
-                            cudaStream_t st);
+                            cudaStream_t st, int late = 0);
 
 // Persistent double-buffered TMA-staged kernel (float32): CTAs walk tiles of kTmaTX columns
 // by TR rows round-robin with two tile buffers, so that the copy of the next tile overlaps
@@ -236,11 +239,13 @@ cudaError_t launch_step_stream(const Params &P, int prec, const void *tmap, void
 
 // Float64-mode step in double-float arithmetic on the float32 pipe (step_kernel 8, 9), on tiles of
 // `shape`, `tmap` with its box; `coef` is the CoefDD of the context (coef_dd).  Ghost cells as in
-// launch_step_tma.
+// launch_step_tma.  late: as in TmaBatchArgs; rows: the first rows only (0: all), a multiple of the
+// shape's.
 void coef_dd(const Params &P, CoefDD *out);
-cudaError_t dd_prepare();
+cudaError_t dd_prepare(const Params &P);
+cudaError_t dd_batch_prepare(int limiter);
 cudaError_t launch_step_dd(const Params &P, const void *coef, const void *tmap, const void *fin, void *fout,
-                           int *err, cudaStream_t st, int shape);
+                           int *err, cudaStream_t st, int shape, int late = 0, int rows = 0);
 
 // Sustained float64 FMA rate of the current device in FLOP/s (FMA = 2).
 cudaError_t measure_fp64_fma(double *flops);

@@ -38,6 +38,7 @@
 //   0.587     the residuals formed in phase 1 and kept in registers, so that no cell's shells are
 //             formed twice, nothing spills, and the ring is left out where s8 = s5 (3501 -> 3188
 //             thread instructions a cell)
+//   0.559     the pairs that move along both axes first; results stored evict-first
 // Other shapes (warps x rows per thread, CTAs per SM), same code: 16 x 2, one CTA 0.807 ms; 12 x 2,
 // one CTA 0.843; 5 x 3, two CTAs 1.09; 4 x 4, two CTAs 1.31 (the unrolled rows spill), against 0.643;
 // 6 x 2, two CTAs 0.677; 7 x 2, two CTAs 0.665; 10 x 2, one CTA 0.885, against 0.587.  The results are bit for bit those of the scalar kernel.
@@ -466,7 +467,8 @@ __device__ __forceinline__ void dd_tile(const PP &P, const CoefDD &C, unsigned c
     asm volatile("" : "+r"(c1));
     // f - C - c_x (F_out - F_in)_x - c_y (F_out - F_in)_y
 #pragma unroll
-    for (int pr = 0; pr < 8; pr++) {
+    for (int n = 0; n < 8; n++) {
+        const int pr = n ^ 4;                               // the diagonal pairs first
         const int qa = pair_q(pr);
         const int sx = tsgn_x(qa), sy = tsgn_y(qa);
         const int sp = pr >> 2;                             // shell pair
@@ -490,8 +492,8 @@ __device__ __forceinline__ void dd_tile(const PP &P, const CoefDD &C, unsigned c
             const int gy = y0 + r0 + k;
             if (gx < nx && gy < ny) {
                 double *o = fout + (long long)(gy + OY) * P.pitch + (gx + OX);
-                o[qa * P.plane] = dd_to_double(first(out[k]));
-                o[(qa + 4) * P.plane] = dd_to_double(second(out[k]));
+                __stcs(o + qa * P.plane, dd_to_double(first(out[k])));
+                __stcs(o + (qa + 4) * P.plane, dd_to_double(second(out[k])));
             }
         }
     }
@@ -504,7 +506,7 @@ __device__ __forceinline__ void dd_tile(const PP &P, const CoefDD &C, unsigned c
 template <int Lim, bool C9, typename S = DdWideShape>
 __global__ void __launch_bounds__(kTmaTX * S::TT, S::CTAS)
 k_step_dd(const __grid_constant__ Params P, const __grid_constant__ CoefDD C, const __grid_constant__ CUtensorMap tm,
-          const double *__restrict__ fin, double *__restrict__ fout, int *err)
+          const double *__restrict__ fin, double *__restrict__ fout, int *err, int late)
 {
     extern __shared__ __align__(128) unsigned char smraw[];
     double *tile64 = reinterpret_cast<double *>(smraw);
@@ -518,8 +520,7 @@ k_step_dd(const __grid_constant__ Params P, const __grid_constant__ CoefDD C, co
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
-    grid_dependency_wait();
-    grid_launch_dependents();
+    batch_begin(late);
     if (tid == 0) {
         // box origin: interior column x0 - HX = padded column x0 + OX - HX; interior row y0 - 2 =
         // padded row y0
@@ -549,13 +550,14 @@ k_step_dd(const __grid_constant__ Params P, const __grid_constant__ CoefDD C, co
             atomicExch(err, 1);
             mbar_wait(bar_a, 0);               // let a late copy land before the CTA exits (bounded)
         }
-        return;
+    } else {
+        if (edge) {
+            ghost.store(tile64);
+            __syncthreads();
+        }
+        dd_tile<Lim, C9, S>(P, C, smraw, fout, x0, y0);
     }
-    if (edge) {
-        ghost.store(tile64);
-        __syncthreads();
-    }
-    dd_tile<Lim, C9, S>(P, C, smraw, fout, x0, y0);
+    batch_end(late, tid);
 }
 
 // ---------------------------------------------------------------------------
@@ -645,15 +647,21 @@ void coef_dd(const Params &P, CoefDD *out)
 }
 
 template <typename S>
+static auto dd_kernel(const Params &P)
+{
+    return P.limiter == 0   ? (P.has_c9 ? k_step_dd<0, true, S> : k_step_dd<0, false, S>)
+           : P.limiter == 1 ? (P.has_c9 ? k_step_dd<1, true, S> : k_step_dd<1, false, S>)
+                            : (P.has_c9 ? k_step_dd<2, true, S> : k_step_dd<2, false, S>);
+}
+
+template <typename S>
 static cudaError_t launch_dd_shape(const Params &P, const CoefDD &C, const CUtensorMap &tm, const double *a, double *b,
-                                   int *err, cudaStream_t st)
+                                   int *err, int late, int rows, cudaStream_t st)
 {
     const dim3 block(kTmaTX, S::TT);
-    const dim3 grid((P.nx + kTmaTX - 1) / kTmaTX, (P.ny + S::TR - 1) / S::TR);
-    const auto fn = P.limiter == 0   ? (P.has_c9 ? k_step_dd<0, true, S> : k_step_dd<0, false, S>)
-                    : P.limiter == 1 ? (P.has_c9 ? k_step_dd<1, true, S> : k_step_dd<1, false, S>)
-                                     : (P.has_c9 ? k_step_dd<2, true, S> : k_step_dd<2, false, S>);
-    return launch_chained(fn, grid, block, S::smem_bytes, st, P, C, tm, a, b, err);
+    const dim3 grid((P.nx + kTmaTX - 1) / kTmaTX, (rows + S::TR - 1) / S::TR);
+    const auto fn = dd_kernel<S>(P);
+    return launch_chained(fn, grid, block, S::smem_bytes, st, P, C, tm, a, b, err, late);
 }
 
 bool dd_shape_supported(const Params &P, int shape)
@@ -670,15 +678,22 @@ double dd_shape_time(int shape, long long tiles, int sms)
 }
 
 cudaError_t launch_step_dd(const Params &P, const void *coef, const void *tmap, const void *fin, void *fout,
-                           int *err, cudaStream_t st, int shape)
+                           int *err, cudaStream_t st, int shape, int late, int rows)
 {
     const CUtensorMap &tm = *reinterpret_cast<const CUtensorMap *>(tmap);
     const CoefDD &C = *reinterpret_cast<const CoefDD *>(coef);
     const double *a = (const double *)fin;
     double *b = (double *)fout;
-    return shape == kDdNarrow ? launch_dd_shape<DdNarrowShape>(P, C, tm, a, b, err, st)
-           : shape == kDdMid  ? launch_dd_shape<DdMidShape>(P, C, tm, a, b, err, st)
-                              : launch_dd_shape<DdWideShape>(P, C, tm, a, b, err, st);
+    if (rows == 0) rows = P.ny;
+    return shape == kDdNarrow ? launch_dd_shape<DdNarrowShape>(P, C, tm, a, b, err, late, rows, st)
+           : shape == kDdMid  ? launch_dd_shape<DdMidShape>(P, C, tm, a, b, err, late, rows, st)
+                              : launch_dd_shape<DdWideShape>(P, C, tm, a, b, err, late, rows, st);
+}
+
+template <typename S>
+static auto dd_batch_kernel(int limiter)
+{
+    return limiter == 0 ? k_step_dd_batch<0, S> : limiter == 1 ? k_step_dd_batch<1, S> : k_step_dd_batch<2, S>;
 }
 
 template <typename S>
@@ -686,8 +701,7 @@ static cudaError_t launch_dd_batch_shape(const TmaBatchArgs &A, const TileGrid<C
                                          int limiter, int ntiles, cudaStream_t st)
 {
     const dim3 block(kTmaTX, S::TT);
-    const auto fn = limiter == 0 ? k_step_dd_batch<0, S> : limiter == 1 ? k_step_dd_batch<1, S> : k_step_dd_batch<2, S>;
-    return launch_chained(fn, dim3(ntiles), block, S::smem_bytes, st, A, tg, Pall);
+    return launch_chained(dd_batch_kernel<S>(limiter), dim3(ntiles), block, S::smem_bytes, st, A, tg, Pall);
 }
 
 cudaError_t launch_step_dd_batch(const TmaBatchArgs &A, const TileGrid<CoefDD> *tg, const Params *Pall, int limiter,
@@ -700,25 +714,25 @@ cudaError_t launch_step_dd_batch(const TmaBatchArgs &A, const TileGrid<CoefDD> *
                               : launch_dd_batch_shape<DdWideShape>(A, tg, Pall, limiter, ntiles, st);
 }
 
-template <typename S>
-static cudaError_t dd_prepare_shape()
+template <typename S, typename K>
+static cudaError_t dd_allow(K *kernel)
 {
-    cudaError_t e = cudaSuccess;
-    for (const void *fn : {(const void *)k_step_dd<0, false, S>, (const void *)k_step_dd<0, true, S>,
-                           (const void *)k_step_dd<1, false, S>, (const void *)k_step_dd<1, true, S>,
-                           (const void *)k_step_dd<2, false, S>, (const void *)k_step_dd<2, true, S>,
-                           (const void *)k_step_dd_batch<0, S>, (const void *)k_step_dd_batch<1, S>,
-                           (const void *)k_step_dd_batch<2, S>})
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem_bytes);
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem_bytes);
+}
+
+cudaError_t dd_prepare(const Params &P)
+{
+    cudaError_t e = dd_allow<DdWideShape>(dd_kernel<DdWideShape>(P));
+    if (e == cudaSuccess) e = dd_allow<DdMidShape>(dd_kernel<DdMidShape>(P));
+    if (e == cudaSuccess) e = dd_allow<DdNarrowShape>(dd_kernel<DdNarrowShape>(P));
     return e;
 }
 
-cudaError_t dd_prepare()
+cudaError_t dd_batch_prepare(int limiter)
 {
-    cudaError_t e = dd_prepare_shape<DdWideShape>();
-    if (e == cudaSuccess) e = dd_prepare_shape<DdMidShape>();
-    if (e == cudaSuccess) e = dd_prepare_shape<DdNarrowShape>();
+    cudaError_t e = dd_allow<DdWideShape>(dd_batch_kernel<DdWideShape>(limiter));
+    if (e == cudaSuccess) e = dd_allow<DdMidShape>(dd_batch_kernel<DdMidShape>(limiter));
+    if (e == cudaSuccess) e = dd_allow<DdNarrowShape>(dd_batch_kernel<DdNarrowShape>(limiter));
     return e;
 }
 

@@ -142,7 +142,9 @@ __device__ __forceinline__ void flow_phase(const Coef<R> &C, const R *tile, R *s
     }
 }
 
-template <typename R, bool Dev, int Lim>
+// Late: as in TmaBatchArgs, a member of a batch with its own launch (an instantiation of its own: as a
+// run-time argument it made the step 2% slower).
+template <typename R, bool Dev, int Lim, bool Late>
 __global__ void __launch_bounds__(kTmaTX * TmaShape<R>::TT, TmaShape<R>::CTAS)
 k_step_tma(const __grid_constant__ Params P, const __grid_constant__ CUtensorMap tm, const R *__restrict__ fin,
            R *__restrict__ fout, int *err)
@@ -164,8 +166,7 @@ k_step_tma(const __grid_constant__ Params P, const __grid_constant__ CUtensorMap
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
-    grid_dependency_wait();
-    grid_launch_dependents();
+    batch_begin(Late);
     if (tid == 0) {
         // box origin: interior column x0 - HX = padded column x0 + OX - HX; interior row y0 - 2 =
         // padded row y0
@@ -199,6 +200,7 @@ k_step_tma(const __grid_constant__ Params P, const __grid_constant__ CUtensorMap
             atomicExch(err, 1);
             mbar_wait(bar_a, 0);               // let a late copy land before the CTA exits (bounded)
         }
+        if (Late) batch_end(1, tid);
         return;
     }
     if (edge) {
@@ -307,6 +309,7 @@ k_step_tma(const __grid_constant__ Params P, const __grid_constant__ CUtensorMap
         }
 
     }
+    if (Late) batch_end(1, tid);
 }
 
 // ---------------------------------------------------------------------------
@@ -367,14 +370,18 @@ k_step_tma_batch(const __grid_constant__ TmaBatchArgs A, const TileGrid<Coef<flo
     batch_end(A.late, tid);
 }
 
+static auto tma_batch_kernel(int limiter)
+{
+    return limiter == 0 ? k_step_tma_batch<0> : limiter == 1 ? k_step_tma_batch<1> : k_step_tma_batch<2>;
+}
+
 cudaError_t launch_step_tma_batch(const TmaBatchArgs &A, const TileGrid<Coef<float>> *tg, const Params *Pall,
                                   int limiter, cudaStream_t st)
 {
     using S = TmaShape<float>;
     const int ntiles = A.first[A.n];
     if (ntiles <= 0) return cudaSuccess;
-    const auto fn = limiter == 0 ? k_step_tma_batch<0> : limiter == 1 ? k_step_tma_batch<1> : k_step_tma_batch<2>;
-    return launch_chained(fn, dim3(ntiles), dim3(kTmaTX, S::TT), S::smem_bytes, st, A, tg, Pall);
+    return launch_chained(tma_batch_kernel(limiter), dim3(ntiles), dim3(kTmaTX, S::TT), S::smem_bytes, st, A, tg, Pall);
 }
 
 // ---------------------------------------------------------------------------
@@ -544,40 +551,50 @@ bool tma_supported(const Params &P, int prec)
     return P.pitch >= TmaShape<float>::SW && P.ny + 4 >= sh && P.nx >= kTmaTX;
 }
 
-template <typename R, bool Dev>
-static cudaError_t launch_tma_lim(const Params &P, const CUtensorMap &tm, const R *a, R *b, int *err, cudaStream_t st)
+template <typename R, bool Dev, bool Late>
+static auto tma_kernel(int limiter)
+{
+    return limiter == 0   ? k_step_tma<R, Dev, 0, Late>
+           : limiter == 1 ? k_step_tma<R, Dev, 1, Late>
+                          : k_step_tma<R, Dev, 2, Late>;
+}
+
+template <typename R, bool Dev, bool Late>
+static cudaError_t launch_tma_lim(const Params &P, const CUtensorMap &tm, const void *a, void *b, int *err,
+                                  cudaStream_t st)
 {
     using S = TmaShape<R>;
     const dim3 block(kTmaTX, S::TT);
     const dim3 grid((P.nx + kTmaTX - 1) / kTmaTX, (P.ny + S::TR - 1) / S::TR);
-    const auto fn = P.limiter == 0 ? k_step_tma<R, Dev, 0> : P.limiter == 1 ? k_step_tma<R, Dev, 1> : k_step_tma<R, Dev, 2>;
-    return launch_chained(fn, grid, block, S::smem_bytes, st, P, tm, a, b, err);
+    return launch_chained(tma_kernel<R, Dev, Late>(P.limiter), grid, block, S::smem_bytes, st, P, tm, (const R *)a, (R *)b,
+                          err);
 }
 
 cudaError_t launch_step_tma(const Params &P, int prec, const void *tmap, const void *fin, void *fout, int *err,
-                            cudaStream_t st)
+                            cudaStream_t st, int late)
 {
     const CUtensorMap &tm = *reinterpret_cast<const CUtensorMap *>(tmap);
-    return prec == 0 ? launch_tma_lim<double, false>(P, tm, (const double *)fin, (double *)fout, err, st)
-                     : launch_tma_lim<float, true>(P, tm, (const float *)fin, (float *)fout, err, st);
+    if (prec == 0) return launch_tma_lim<double, false, false>(P, tm, fin, fout, err, st);   // never late
+    return late ? launch_tma_lim<float, true, true>(P, tm, fin, fout, err, st)
+                : launch_tma_lim<float, true, false>(P, tm, fin, fout, err, st);
 }
 
-cudaError_t tma_prepare()
+template <typename S, typename K>
+static cudaError_t tma_allow(K *kernel)
 {
-    cudaError_t e = cudaSuccess;
-    auto set = [&](const void *fn, size_t bytes) {
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    };
-    set((const void *)k_step_tma<double, false, 0>, TmaShape<double>::smem_bytes);
-    set((const void *)k_step_tma<double, false, 1>, TmaShape<double>::smem_bytes);
-    set((const void *)k_step_tma<double, false, 2>, TmaShape<double>::smem_bytes);
-    set((const void *)k_step_tma<float, true, 0>, TmaShape<float>::smem_bytes);
-    set((const void *)k_step_tma<float, true, 1>, TmaShape<float>::smem_bytes);
-    set((const void *)k_step_tma<float, true, 2>, TmaShape<float>::smem_bytes);
-    set((const void *)k_step_tma_batch<0>, TmaShape<float>::smem_bytes);
-    set((const void *)k_step_tma_batch<1>, TmaShape<float>::smem_bytes);
-    set((const void *)k_step_tma_batch<2>, TmaShape<float>::smem_bytes);
-    return e;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem_bytes);
+}
+
+cudaError_t tma_prepare(int prec, int limiter)
+{
+    return prec == 0 ? tma_allow<TmaShape<double>>(tma_kernel<double, false, false>(limiter))
+                     : tma_allow<TmaShape<float>>(tma_kernel<float, true, false>(limiter));
+}
+
+cudaError_t tma_batch_prepare(int limiter)
+{
+    const cudaError_t e = tma_allow<TmaShape<float>>(tma_kernel<float, true, true>(limiter));
+    return e == cudaSuccess ? tma_allow<TmaShape<float>>(tma_batch_kernel(limiter)) : e;
 }
 
 }  // namespace lbm
