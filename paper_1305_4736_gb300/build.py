@@ -16,8 +16,10 @@ CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "liblbm.so")
 SOURCES = ["lbm_api.cu", "lbm_kernels.cu", "lbm_step_tma.cu", "lbm_step_stream.cu", "lbm_step_dd.cu",
+           "lbm_step_dd_wide.cu", "lbm_step_dd_mid.cu", "lbm_step_dd_narrow.cu",
            "lbm_peak.cu", "lbm_noalloc.cu"]
-HEADERS = ["lbm_dd.cuh", "lbm_device.cuh", "lbm_internal.h", "lbm_lanes.cuh", "lbm_tma_util.cuh"]
+HEADERS = ["lbm_dd.cuh", "lbm_device.cuh", "lbm_internal.h", "lbm_lanes.cuh", "lbm_step_dd.cuh",
+           "lbm_tma_util.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xptxas", "-v",
          f"-I{os.path.join(ROOT, 'include')}"]

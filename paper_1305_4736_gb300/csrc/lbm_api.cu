@@ -336,10 +336,12 @@ int edges_of_kind(const lbm_ctx *c, int kind)
 }
 
 // Edges whose ghost cells the ghost launch fills before a step of context c: every edge for the
-// streaming and the double-buffered kernel, else walls only (the other kernels read periodic and
-// zero-gradient neighbours in place; fixed-equilibrium ghost cells are filled at create time).
+// streaming and the double-buffered kernel, none for the double-float kernels, else walls only (the
+// other kernels read periodic and zero-gradient neighbours in place; fixed-equilibrium ghost cells are
+// filled at create time).
 int ghost_edges(const lbm_ctx *c)
 {
+    if (c->use_dd || c->use_ddn) return 0;
     return c->use_stream || c->use_pipe ? lbm::kAllEdges : edges_of_kind(c, LBM_BC_NEQ_WALL);
 }
 
@@ -600,15 +602,15 @@ int lbm_create_ex(int nx, int ny, double dx, double dt, double gamma, double Pr,
     if (want == 4) c->plain_ty = 16;
     if (want == 7) c->plain_ty = 2;
     // automatic, float64: the double-float kernels (on GB300 the float32 pipe runs their
-    // arithmetic 2.5x faster than the float64 kernels run theirs) wherever their tiles fit; on
+    // arithmetic 5x faster than the float64 kernels run theirs) wherever their tiles fit; on
     // grids narrower than 32 columns or lower than 4 rows the float64 pipe (about 1.6 lane
     // operations per cycle per SM): the streaming kernel when the grid gives every SM at least
     // 32 rows of a 256-column strip; else the plain kernel, on 256-cell tiles when they still
     // give every SM four tiles (their flow-velocity ring costs less), on 64-cell tiles below
-    // that, which spread a small grid's float64 work over more SMs.  The double-float kernel
-    // runs on 32 x 16 tiles (two CTAs per SM) where the grid has at least two thirds of an SM's
-    // count of 32 x 32 cells; on smaller grids, and on grids of 4 to 31 rows, on 32 x 4 tiles: a
-    // small grid finishes sooner in more, shorter tiles
+    // that, which spread a small grid's float64 work over more SMs.  Grids of at
+    // least two thirds of the SM count in 32 x 32 cells take kernel 8 (tiles of 32 x 16 or 32 x 8),
+    // smaller ones and those of 4 to 31 rows kernel 9 (32 x 8 or 32 x 4), each the shape whose
+    // waves last shortest (dd_shape_time has the times)
     if (want == 0 && prec == LBM_FP64) {
         int sms = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
@@ -1153,6 +1155,7 @@ struct lbm_batch {
             int k, y0, rows;
         };
         std::vector<Span> tk[lbm::kDdShapes];    // float32: [0]
+        bool walls = false;                      // some double-float member has a wall
         std::vector<Span> alone;                 // spans from row 0 with a launch of their own
         void *tblock = nullptr;
         size_t tbytes = 0;
@@ -1221,7 +1224,7 @@ cudaError_t batch_launch_tma_list(lbm_batch *b, const lbm_batch::Group &g, int s
         *late = 1;
         const char *tg = tg0 + c0 * tgb;
         const cudaError_t ce =
-            f64 ? lbm::launch_step_dd_batch(A, (const lbm::TileGrid<lbm::CoefDD> *)tg, g.dP, g.limiter, shape, st)
+            f64 ? lbm::launch_step_dd_batch(A, (const lbm::TileGrid<lbm::CoefDD> *)tg, g.dP, g.limiter, shape, g.walls, st)
                 : lbm::launch_step_tma_batch(A, (const lbm::TileGrid<lbm::Coef<float>> *)tg, g.dP, g.limiter, st);
         if (ce != cudaSuccess) return ce;
     }
@@ -1372,7 +1375,9 @@ int lbm_batch_create(lbm_ctx *const *ctxs, int n, lbm_batch **out)
         g->tma.push_back(tma ? 1 : 0);
     }
     for (auto &g : b->groups) {
-        ce = g.prec == LBM_FP64 ? lbm::dd_batch_prepare(g.limiter) : lbm::tma_batch_prepare(g.limiter);
+        for (size_t k = 0; k < g.members.size(); k++)
+            g.walls = g.walls || (g.tma[k] && edges_of_kind(b->ctxs[g.members[k]], LBM_BC_NEQ_WALL) != 0);
+        ce = g.prec == LBM_FP64 ? lbm::dd_batch_prepare(g.limiter, g.walls) : lbm::tma_batch_prepare(g.limiter);
         if (ce != cudaSuccess) { lbm_batch_destroy(b); return cuda_fail(nullptr, ce, "batch kernels"); }
         // float64 groups too small to give every SM four 256-cell tiles take 64-cell tiles,
         // which spread their float64 work over more SMs

@@ -145,6 +145,7 @@ struct CoefDD {
     dd2 hh[2], hhy[2], cr[2], cry[2];
     dd2 pA[2][2], pEx[2][3], pEy[2][3], pB1[2], pB2[2];
     dd2 q89, g4;
+    dd2 wA[2][3], wEx[2][4], wEy[2][4], wB1[2], wB2[2];   // full inverse blocks (walls), without the density row
     dd b, inv_b, two_b2, six_b, b4, four_inv_b, ry, pad_;
 };
 static_assert(sizeof(CoefDD) % 16 == 0, "CoefDD is copied in 16-byte words");
@@ -183,8 +184,8 @@ struct TileGrid {
 };
 cudaError_t launch_step_tma_batch(const TmaBatchArgs &A, const TileGrid<Coef<float>> *tg, const Params *Pall, int limiter,
                                   cudaStream_t st);
-// shape: kDdWide, kDdMid or kDdNarrow (the grids' maps have its box).
-cudaError_t launch_step_dd_batch(const TmaBatchArgs &A, const TileGrid<CoefDD> *tg, const Params *Pall, int limiter, int shape,
+// shape: kDdWide, kDdMid or kDdNarrow (the grids' maps have its box); walls: some grid has one.
+cudaError_t launch_step_dd_batch(const TmaBatchArgs &A, const TileGrid<CoefDD> *tg, const Params *Pall, int limiter, int shape, bool walls,
                                  cudaStream_t st);
 // Failure-path check of the bounded mbarrier waits (lbm_wait_selftest): *flag = 1 when the
 // wait on a phase that nothing completes gave up at its limit; *ms = the kernel's duration.
@@ -242,8 +243,21 @@ cudaError_t launch_step_stream(const Params &P, int prec, const void *tmap, void
 // launch_step_tma.  late: as in TmaBatchArgs; rows: the first rows only (0: all), a multiple of the
 // shape's.
 void coef_dd(const Params &P, CoefDD *out);
+// The kernels of one shape (lbm_step_dd.cuh).
+template <typename S>
+struct DdOps {
+    static cudaError_t launch(const Params &P, const CoefDD &C, const CUtensorMap &tm, const double *a, double *b, int *err,
+                              int late, int rows, cudaStream_t st);
+    static cudaError_t launch_batch(const TmaBatchArgs &A, const TileGrid<CoefDD> *tg, const Params *Pall, int limiter,
+                                    bool walls, cudaStream_t st);
+    static cudaError_t prepare(const Params &P);
+    static cudaError_t prepare_batch(int limiter, bool walls);
+};
+extern template struct DdOps<DdWideShape>;
+extern template struct DdOps<DdMidShape>;
+extern template struct DdOps<DdNarrowShape>;
 cudaError_t dd_prepare(const Params &P);
-cudaError_t dd_batch_prepare(int limiter);
+cudaError_t dd_batch_prepare(int limiter, bool walls);
 cudaError_t launch_step_dd(const Params &P, const void *coef, const void *tmap, const void *fin, void *fout,
                            int *err, cudaStream_t st, int shape, int late = 0, int rows = 0);
 

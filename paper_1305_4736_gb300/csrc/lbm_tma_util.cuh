@@ -107,12 +107,38 @@ struct TileElem { using T = double; static constexpr int N = NQ; };            /
 template <>
 struct TileElem<float> { using T = float2; static constexpr int N = NQ / 2; };
 
+// Ghost cell k of a tile's cross: k < 128 in the ghost rows of the tile's columns, then in the ghost
+// columns of its rows.
+template <typename S>
+struct GhostSlot {
+    static constexpr int kSlots = 4 * kTmaTX + 4 * S::TR;
+    bool row, in;              // in a ghost row (else column); within the staged tile and the grid
+    int layer, edge;           // 0, 1: -1, -2; 2, 3: n, n + 1; x-lo, x-hi, y-lo, y-hi
+    int along, g, at, fix;     // coordinate along the edge, across it; staged row or column; the other one
+    template <typename PP>
+    __device__ __forceinline__ GhostSlot(const PP &P, int k, int x0, int y0)
+    {
+        row = k < 4 * kTmaTX;
+        const int j = row ? k : k - 4 * kTmaTX;
+        layer = row ? j / kTmaTX : j / S::TR;
+        along = row ? x0 + j % kTmaTX : y0 + j % S::TR;
+        const int size = row ? P.ny : P.nx, first = row ? y0 : x0;
+        g = layer < 2 ? -1 - layer : size + layer - 2;
+        at = g - first + 2;
+        fix = row ? along - x0 + S::HX : along - y0 + 2;
+        edge = (row ? 2 : 0) + (layer >> 1);
+        in = k < kSlots && at >= 0 && at < (row ? S::SH : S::SW) && along < (row ? P.nx : P.ny);
+    }
+    // offset in a staged plane of the cell at staged row (column) v across the edge
+    __device__ __forceinline__ int offset(int v) const { return row ? v * S::SW + fix : fix * S::SW + v; }
+};
+
 template <typename R, typename S>
 struct GhostFill {
     using E = typename TileElem<R>::T;
     static constexpr int N = TileElem<R>::N;
-    static constexpr int kSlots = 4 * kTmaTX + 4 * S::TR, kThreads = kTmaTX * S::TT;
-    static constexpr int kRounds = (kSlots + kThreads - 1) / kThreads;
+    static constexpr int kThreads = kTmaTX * S::TT;
+    static constexpr int kRounds = (GhostSlot<S>::kSlots + kThreads - 1) / kThreads;
     E v[kRounds][N];
     int c[kRounds];            // cell of the staged tile, or -1
 
@@ -128,22 +154,15 @@ struct GhostFill {
     {
 #pragma unroll
         for (int n = 0; n < kRounds; n++) {
-            const int k = tid + n * kThreads;
+            const GhostSlot<S> slot(P, tid + n * kThreads, x0, y0);
             c[n] = -1;
-            const bool row = k < 4 * kTmaTX;                 // a ghost row's cell, or a ghost column's
-            const int j = row ? k : k - 4 * kTmaTX;
-            const int layer = row ? j / kTmaTX : j / S::TR;  // 0, 1: -1, -2; 2, 3: n, n + 1
-            const int along = row ? x0 + j % kTmaTX : y0 + j % S::TR;
-            const int size = row ? P.ny : P.nx, first = row ? y0 : x0;
-            const int g = layer < 2 ? -1 - layer : size + layer - 2;
-            const int at = g - first + 2;                    // staged row or column
-            const bool in = k < kSlots && at >= 0 && at < (row ? S::SH : S::SW) && along < (row ? P.nx : P.ny);
-            if (!in) continue;
-            const EdgeDev &D = edges[(row ? 2 : 0) + (layer >> 1)];
+            if (!slot.in) continue;
+            const EdgeDev &D = edges[slot.edge];
             if (D.kind > 1) continue;
-            c[n] = row ? at * S::SW + (along - x0 + S::HX) : (along - y0 + 2) * S::SW + at;
-            const int s = ghost_source(g, size, D.kind, D.kind);
-            const long long cell = (long long)((row ? s : along) + OY) * P.pitch + ((row ? along : s) + OX);
+            c[n] = slot.offset(slot.at);
+            const int s = ghost_source(slot.g, slot.row ? P.ny : P.nx, D.kind, D.kind);
+            const long long cell =
+                (long long)((slot.row ? s : slot.along) + OY) * P.pitch + ((slot.row ? slot.along : s) + OX);
             const E *src = reinterpret_cast<const E *>(fin) + cell;
 #pragma unroll
             for (int q = 0; q < N; q++) v[n][q] = src[q * P.plane];
