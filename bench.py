@@ -63,13 +63,13 @@ TRAFFIC_PER_CELL = {
     "f64": {"bytes": 251.37, "sources": ("lbm_step_stream.cu", "lbm_device.cuh", "lbm_tma_util.cuh"),
             "sha": "605189e5c16eda2a"},
     "dd": {"bytes": 246.34, "sources": ("lbm_step_dd.cuh", "lbm_dd.cuh", "lbm_device.cuh", "lbm_tma_util.cuh"),
-           "sha": "1ea6a139482c403e"},
+           "sha": "486023eea404501d"},
 }
 # float32-pipe lane operations per cell of one launch of the double-float float64 kernel on wide
 # tiles: ncu's FMA-pipe busy fraction x cycles x 128 lanes (its counters of float32 instructions do
 # not see the packed f32x2 ones), on the same sources (profiles/k_step_dd_f64_shear_layer.md); None
 # when the sources changed since.
-DD_FP32_OPS = {"ops": 3537.8, "sha": "1ea6a139482c403e"}
+DD_FP32_OPS = {"ops": 3537.8, "sha": "486023eea404501d"}
 FP32_LANES_PER_SM = 128           # float32 FMA lanes per SM per cycle (GB300)
 
 
