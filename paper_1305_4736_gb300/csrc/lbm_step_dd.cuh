@@ -595,7 +595,7 @@ __device__ __forceinline__ void dd_tile(const PP &P, const CoefDD &C, unsigned c
 template <int Lim, bool C9, bool Walls, typename S>
 __global__ void __launch_bounds__(kTmaTX * S::TT, S::CTAS)
 k_step_dd(const __grid_constant__ Params P, const __grid_constant__ CoefDD C, const __grid_constant__ CUtensorMap tm,
-          const double *__restrict__ fin, double *__restrict__ fout, int *err, int late)
+          const double *fin, double *fout, int *err, int late)
 {
     extern __shared__ __align__(128) unsigned char smraw[];
     double *tile64 = reinterpret_cast<double *>(smraw);

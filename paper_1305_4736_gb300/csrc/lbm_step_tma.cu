@@ -146,8 +146,8 @@ __device__ __forceinline__ void flow_phase(const Coef<R> &C, const R *tile, R *s
 // run-time argument it made the step 2% slower).
 template <typename R, bool Dev, int Lim, bool Late>
 __global__ void __launch_bounds__(kTmaTX * TmaShape<R>::TT, TmaShape<R>::CTAS)
-k_step_tma(const __grid_constant__ Params P, const __grid_constant__ CUtensorMap tm, const R *__restrict__ fin,
-           R *__restrict__ fout, int *err)
+k_step_tma(const __grid_constant__ Params P, const __grid_constant__ CUtensorMap tm, const R *fin,
+           R *fout, int *err)
 {
     using S = TmaShape<R>;
     extern __shared__ __align__(128) unsigned char smraw[];

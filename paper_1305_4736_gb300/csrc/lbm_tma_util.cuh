@@ -69,7 +69,10 @@ __device__ __forceinline__ R slope2(R a, R b)
 }
 
 // Programmatic dependent launch: a step kernel's CTAs may start while the previous launch of the
-// stream drains, and wait here before they touch its results.
+// stream drains, and wait here before they touch its results.  A kernel that is launched so does not
+// take its populations as __restrict__: until the wait is over the launch before it still writes them,
+// and the qualifier would let the compiler read them through the non-coherent path, or above the wait.
+// Functions called after the wait may (until the kernel ends nothing else writes what they read).
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
