@@ -374,16 +374,16 @@ cudaError_t launch_step_ghosts(lbm_ctx *c, int in, cudaStream_t st)
 }
 
 // One fused step of context c from buffer `in` into buffer in ^ 1, on stream st.
-cudaError_t launch_fused_step(lbm_ctx *c, int in, cudaStream_t st)
+cudaError_t launch_fused_step(lbm_ctx *c, int in, cudaStream_t st, bool chain = true)
 {
     if (c->use_dd || c->use_ddn) {
         const int k = c->use_dd ? c->dd8 : c->dd9;
-        return lbm::launch_step_dd(c->P, &c->cdd, &c->dmap[k][in], c->f[in], c->f[in ^ 1], c->tma_err, st, k);
+        return lbm::launch_step_dd(c->P, &c->cdd, &c->dmap[k][in], c->f[in], c->f[in ^ 1], c->tma_err, st, k, chain);
     }
     if (c->use_pipe) return lbm::launch_step_tma_pipe(c->P, &c->pmap[in], c->f[in ^ 1], c->tma_err, st);
     if (c->use_stream) return lbm::launch_step_stream(c->P, c->prec, &c->smap[in], c->f[in ^ 1], c->tma_err, st);
-    if (c->use_tma) return lbm::launch_step_tma(c->P, c->prec, &c->tmap[in], c->f[in], c->f[in ^ 1], c->tma_err, st);
-    return lbm::launch_step(c->P, c->prec, c->f[in], c->f[in ^ 1], st, c->plain_ty);
+    if (c->use_tma) return lbm::launch_step_tma(c->P, c->prec, &c->tmap[in], c->f[in], c->f[in ^ 1], c->tma_err, st, chain);
+    return lbm::launch_step(c->P, c->prec, c->f[in], c->f[in ^ 1], st, c->plain_ty, chain);
 }
 
 // Calls of at least kGraphSteps steps replay graphs of two steps, calls of at least kRunMin graphs of
@@ -1165,8 +1165,8 @@ struct lbm_batch {
     std::vector<Group> groups;
     // contexts on the streaming or the double-buffered kernel with at least a quarter wave of
     // its work: their ghost cells come from their group's batched ghost launch, their step from
-    // that kernel, launched on kForks forked streams so that the grids' kernels overlap
-    static constexpr int kForks = 8;
+    // that kernel, on a branch of its own (BatchBranches)
+    static constexpr int kForks = 3;
     std::vector<int> solo;
     std::vector<int> cap_cur;                   // every context's buffer parity at graph capture
     cudaStream_t fork[kForks] = {};
@@ -1175,7 +1175,7 @@ struct lbm_batch {
     cudaGraphExec_t exec2 = nullptr, run = nullptr;   // graphs of 2 and of kRunSteps steps
     lbm_allocator alloc{};
     int device = 0, ctas = 0;
-    int launches = 0;                           // kernels per step
+    int ghost_launches = 0, step_launches = 0;  // kernels per step
 };
 
 namespace {
@@ -1191,11 +1191,54 @@ cudaError_t batch_upload_cur(lbm_batch *b)
     return cudaSuccess;
 }
 
+// The ghost or the step launches of one batch step, which are independent of each other, side by side: on
+// the batch's stream and up to kForks streams of its own, each of which starts when everything before in
+// the batch's stream is complete and is joined to it at the end.  So every launch has a full dependency on
+// the whole previous step (and waits for it before it reads, as all of them do), while the launches of one
+// step fill the slots that the others leave empty.  A batch with one launch a step needs no branches, and
+// its steps are chained as those of lbm_step.
+// Three more branches (us per batch step of 24 float32 grids of 0.58 M and 0.14 M cells on average, and of
+// as many float64 ones): 307, 88.7, 1910, 527; one: 311, 123.8, 1911, 565; eight: 316, 90.4, 1937, 540.
+struct BatchBranches {
+    struct Next {
+        cudaStream_t st;
+        bool chain;
+    };
+    lbm_batch *b;
+    cudaStream_t st;
+    int n, j = 0;
+    BatchBranches(lbm_batch *batch, cudaStream_t stream, int launches)
+        : b(batch), st(stream), n(std::max(1, std::min(launches, 1 + lbm_batch::kForks))) {}
+    cudaError_t fork()
+    {
+        cudaError_t ce = n > 1 ? cudaEventRecord(b->ev_fork, st) : cudaSuccess;
+        for (int k = 0; k < n - 1 && ce == cudaSuccess; k++) ce = cudaStreamWaitEvent(b->fork[k], b->ev_fork, 0);
+        return ce;
+    }
+    // Where the next launch goes; chained only behind another launch in the same stream.
+    Next next()
+    {
+        const int k = j % n;
+        const bool chain = j >= n || std::max(b->ghost_launches, b->step_launches) <= 1;
+        j++;
+        return {k == 0 ? st : b->fork[k - 1], chain};
+    }
+    cudaError_t join()
+    {
+        cudaError_t ce = cudaSuccess;
+        for (int k = 0; k < n - 1 && ce == cudaSuccess; k++) {
+            ce = cudaEventRecord(b->ev_join[k], b->fork[k]);
+            if (ce == cudaSuccess) ce = cudaStreamWaitEvent(st, b->ev_join[k], 0);
+        }
+        return ce;
+    }
+};
+
 // The group's batched TMA-staged launches (kTmaBatchGrids grids each) over the spans of one shape
 // (float32: the tile kernel's), with every member's buffers, input map and flag resolved for this step's
-// parity; tg0: the shape's TileGrid blocks.  `late`: whether a step launch of this batch step precedes.
+// parity; tg0: the shape's TileGrid blocks.
 cudaError_t batch_launch_tma_list(lbm_batch *b, const lbm_batch::Group &g, int shape, const char *tg0, int phase,
-                                  int *late, cudaStream_t st)
+                                  BatchBranches &br)
 {
     static thread_local lbm::TmaBatchArgs A;
     const bool f64 = g.prec == LBM_FP64;
@@ -1220,32 +1263,33 @@ cudaError_t batch_launch_tma_list(lbm_batch *b, const lbm_batch::Group &g, int s
         }
         A.first[n] = tiles;
         A.n = n;
-        A.late = *late;
-        *late = 1;
         const char *tg = tg0 + c0 * tgb;
+        const BatchBranches::Next at = br.next();
         const cudaError_t ce =
-            f64 ? lbm::launch_step_dd_batch(A, (const lbm::TileGrid<lbm::CoefDD> *)tg, g.dP, g.limiter, shape, g.walls, st)
-                : lbm::launch_step_tma_batch(A, (const lbm::TileGrid<lbm::Coef<float>> *)tg, g.dP, g.limiter, st);
+            f64 ? lbm::launch_step_dd_batch(A, (const lbm::TileGrid<lbm::CoefDD> *)tg, g.dP, g.limiter, shape, g.walls,
+                                            at.chain, at.st)
+                : lbm::launch_step_tma_batch(A, (const lbm::TileGrid<lbm::Coef<float>> *)tg, g.dP, g.limiter, at.chain,
+                                             at.st);
         if (ce != cudaSuccess) return ce;
     }
     return cudaSuccess;
 }
 
-cudaError_t batch_launch_tma(lbm_batch *b, const lbm_batch::Group &g, int phase, int *late, cudaStream_t st)
+cudaError_t batch_launch_tma(lbm_batch *b, const lbm_batch::Group &g, int phase, BatchBranches &br)
 {
     const char *tg = (const char *)g.tblock;
     cudaError_t ce = cudaSuccess;
     for (size_t j = 0; j < g.alone.size() && ce == cudaSuccess; j++) {
         lbm_ctx *c = b->ctxs[g.members[g.alone[j].k]];
         const int in = c->cur ^ phase;
+        const BatchBranches::Next at = br.next();
         ce = g.prec == LBM_FP64
-                 ? lbm::launch_step_dd(c->P, &c->cdd, &c->dmap[lbm::kDdWide][in], c->f[in], c->f[in ^ 1], c->tma_err, st,
-                                       lbm::kDdWide, *late, g.alone[j].rows)
-                 : lbm::launch_step_tma(c->P, c->prec, &c->tmap[in], c->f[in], c->f[in ^ 1], c->tma_err, st, *late);
-        *late = 1;
+                 ? lbm::launch_step_dd(c->P, &c->cdd, &c->dmap[lbm::kDdWide][in], c->f[in], c->f[in ^ 1], c->tma_err,
+                                       at.st, lbm::kDdWide, at.chain, g.alone[j].rows)
+                 : lbm::launch_step_tma(c->P, c->prec, &c->tmap[in], c->f[in], c->f[in ^ 1], c->tma_err, at.st, at.chain);
     }
     for (int k = 0; k < lbm::kDdShapes && ce == cudaSuccess; k++) {
-        ce = batch_launch_tma_list(b, g, k, tg, phase, late, st);
+        ce = batch_launch_tma_list(b, g, k, tg, phase, br);
         tg += g.tk[k].size() * sizeof(lbm::TileGrid<lbm::CoefDD>);
     }
     return ce;
@@ -1253,40 +1297,31 @@ cudaError_t batch_launch_tma(lbm_batch *b, const lbm_batch::Group &g, int phase,
 
 cudaError_t batch_launch_step(lbm_batch *b, int phase, cudaStream_t st)
 {
-    cudaError_t ce = cudaSuccess;
-    int late = 0;                                // the groups' ghost fills do not depend on each other
+    BatchBranches ghosts(b, st, b->ghost_launches);
+    cudaError_t ce = ghosts.fork();
     for (auto &g : b->groups) {
+        if (ce != cudaSuccess) return ce;
         if (g.max_ghost == 0) continue;
-        ce = lbm::launch_ghost_batch(g.dP, g.dG, (int)g.members.size(), g.max_ghost, g.prec, phase, late, st);
-        if (ce != cudaSuccess) return ce;
-        late = 1;
+        const BatchBranches::Next at = ghosts.next();
+        ce = lbm::launch_ghost_batch(g.dP, g.dG, (int)g.members.size(), g.max_ghost, g.prec, phase, at.chain, at.st);
     }
-    const int nf = std::min<int>(lbm_batch::kForks, (int)b->solo.size());
-    if (nf > 0) {
-        ce = cudaEventRecord(b->ev_fork, st);
-        for (int k = 0; k < nf && ce == cudaSuccess; k++) ce = cudaStreamWaitEvent(b->fork[k], b->ev_fork, 0);
-        if (ce != cudaSuccess) return ce;
-    }
-    late = 0;                                    // nor do the step launches
+    if (ce == cudaSuccess) ce = ghosts.join();
+    BatchBranches steps(b, st, b->step_launches);
+    if (ce == cudaSuccess) ce = steps.fork();
     for (auto &g : b->groups) {
-        ce = batch_launch_tma(b, g, phase, &late, st);
-        if (ce == cudaSuccess && g.ntiles > 0) {
-            ce = lbm::launch_step_batch(g.dP, g.dG, g.dT, g.ntiles, g.prec, g.limiter, g.nt,
-                                        g.nt == lbm::kBatchThreadsFp64 ? 2 * b->ctas : b->ctas, phase, late, st);
-            late = 1;
-        }
+        if (ce == cudaSuccess) ce = batch_launch_tma(b, g, phase, steps);
         if (ce != cudaSuccess) return ce;
+        if (g.ntiles == 0) continue;
+        const BatchBranches::Next at = steps.next();
+        ce = lbm::launch_step_batch(g.dP, g.dG, g.dT, g.ntiles, g.prec, g.limiter, g.nt,
+                                    g.nt == lbm::kBatchThreadsFp64 ? 2 * b->ctas : b->ctas, phase, at.chain, at.st);
     }
-    for (size_t j = 0; j < b->solo.size(); j++) {
+    for (size_t j = 0; j < b->solo.size() && ce == cudaSuccess; j++) {
         lbm_ctx *c = b->ctxs[b->solo[j]];
-        ce = launch_fused_step(c, c->cur ^ phase, b->fork[j % lbm_batch::kForks]);
-        if (ce != cudaSuccess) return ce;
+        const BatchBranches::Next at = steps.next();
+        ce = launch_fused_step(c, c->cur ^ phase, at.st, at.chain);
     }
-    for (int k = 0; k < nf && ce == cudaSuccess; k++) {
-        ce = cudaEventRecord(b->ev_join[k], b->fork[k]);
-        if (ce == cudaSuccess) ce = cudaStreamWaitEvent(st, b->ev_join[k], 0);
-    }
-    return ce;
+    return ce == cudaSuccess ? steps.join() : ce;
 }
 
 // Inside a batch, a context whose kernel is the TMA-staged tile kernel (float32) or the
@@ -1310,9 +1345,8 @@ long long wide_tiles(const lbm_ctx *c)
 // Members of a batched TMA-staged launch with at least kAloneTiles tiles (of 32 x 16 cells) get a launch of
 // their own, whose coefficients are operands from the constant bank and not in shared memory, in groups
 // whose members have kAloneMean tiles on average: between short launches slots stay empty.  Measured, us
-// per batch step, all batched and with the rule: 24 float32 grids of 0.58 M cells on average 347 and 315,
-// of 0.14 M 94.2 and 87.7; float64, 2070 and 1906, 550 and 514.  Without the condition on the average, 21
-// float64 serving grids of 38 thousand cells 174 and 195, 57 406 and 420, 255 float32 ones 487 and 483.
+// per batch step, all batched and with the rule: 24 float32 grids of 0.58 M cells on average 343 and 307,
+// of 0.14 M 93.4 and 88.7; float64, 2092 and 1910, 580 and 527.
 constexpr int kAloneTiles = 64, kAloneMean = 256;
 
 // Rows (from row 0) of member c that such a launch covers: the whole float32 grid; of a float64 one the
@@ -1462,8 +1496,9 @@ int lbm_batch_create(lbm_ctx *const *ctxs, int n, lbm_batch **out)
                 for (int x = 0; x < c->P.nx; x += tw) tiles.push_back(make_int4((int)k, x, y, lt));
         }
         g.ntiles = (int)tiles.size();
-        b->launches += (int)g.alone.size() + (g.ntiles > 0) + (g.max_ghost > 0);
-        for (const auto &list : g.tk) b->launches += !list.empty();
+        b->ghost_launches += g.max_ghost > 0;
+        b->step_launches += (int)g.alone.size() + (g.ntiles > 0);
+        for (const auto &list : g.tk) b->step_launches += (int)((list.size() + lbm::kTmaBatchGrids - 1) / lbm::kTmaBatchGrids);
         // sections start on 256-byte boundaries (the tile list is read as int4)
         auto up = [](size_t v) { return (v + 255) / 256 * 256; };
         const size_t np = up(hp.size() * sizeof(lbm::Params)), ng = up(g.hG.size() * sizeof(lbm::BatchGrid));
@@ -1491,7 +1526,7 @@ int lbm_batch_create(lbm_ctx *const *ctxs, int n, lbm_batch **out)
         if (ce == cudaSuccess) ce = cudaStreamSynchronize(b->stream);
         if (ce != cudaSuccess) { lbm_batch_destroy(b); return cuda_fail(nullptr, ce, "batch tables"); }
     }
-    b->launches += (int)b->solo.size();
+    b->step_launches += (int)b->solo.size();
     ce = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
     if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming);
     for (int k = 0; k < lbm_batch::kForks && ce == cudaSuccess; k++) {
@@ -1531,7 +1566,7 @@ int lbm_batch_step(lbm_batch *b, int n)
     // steps left over launched directly
     // (runs of kRunSteps where a step is a launch or two: there the gap between graphs shows, and the
     // graph is quickly built)
-    const int unit = n >= kRunMin && b->launches <= 2 ? kRunSteps : 2;
+    const int unit = n >= kRunMin && b->ghost_launches + b->step_launches <= 2 ? kRunSteps : 2;
     cudaGraphExec_t *exec = unit == 2 ? &b->exec2 : &b->run;
     if (n >= unit && !*exec) {
         b->cap_cur.clear();

@@ -31,10 +31,12 @@ bool lane_step(const Params &P, int prec, int ty);
 constexpr int kAllEdges = 15;
 cudaError_t launch_ghost(const Params &P, int prec, void *f, cudaStream_t st, int edges = kAllEdges, bool lanes = false);
 
-// Launch of a kernel that calls grid_dependency_wait before it touches memory: its CTAs may start
-// (barrier initialisation, parameter fetches) while the stream's previous launch drains.
+// Launch of a kernel that calls grid_dependency_wait before it touches memory.  chain: its CTAs may start
+// (barrier initialisation, parameter fetches) while the stream's previous launch drains; else once
+// everything before it in the stream is complete.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args)
+cudaError_t launch_kernel(bool chain, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                          Args &&...args)
 {
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -45,11 +47,17 @@ cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = chain ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
+template <typename... KArgs, typename... Args>
+cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args)
+{
+    return launch_kernel(true, kernel, grid, block, smem, st, std::forward<Args>(args)...);
+}
 // Plain fused step with tiles of 32 x ty cells (ty = 4, 8 or 16).
-cudaError_t launch_step(const Params &P, int prec, const void *fin, void *fout, cudaStream_t st, int ty = kTY);
+cudaError_t launch_step(const Params &P, int prec, const void *fin, void *fout, cudaStream_t st, int ty = kTY,
+                        bool chain = true);
 // log2 of the plain kernels' tile width for a grid nx columns wide (5 for nx >= 32, else the
 // smallest power of two >= nx); the tile has (kTX * kTY) >> log rows.
 int plain_log_tx(int nx);
@@ -68,9 +76,9 @@ struct BatchGrid {
 // Batched ghost fill (grid index = blockIdx.y) and batched fused step over a tile list
 // (int4 {grid, x0, y0, 0}); `phase` = 0 reads buf[cur], 1 reads buf[cur ^ 1].
 cudaError_t launch_ghost_batch(const Params *Pall, const BatchGrid *G, int ngrids, int max_ghost, int prec,
-                               int phase, int late, cudaStream_t st);
+                               int phase, bool chain, cudaStream_t st);
 cudaError_t launch_step_batch(const Params *Pall, const BatchGrid *G, const int4 *tiles, int ntiles, int prec,
-                              int limiter, int nt, int ctas, int phase, int late, cudaStream_t st);
+                              int limiter, int nt, int ctas, int phase, bool chain, cudaStream_t st);
 cudaError_t launch_moments(const Params &P, int prec, const void *f, int row0, int rows,
                            double *rho, double *u, double *v, double *T, double *delta,
                            double *dstar, int *flag, cudaStream_t st);
@@ -165,13 +173,7 @@ struct TmaBatchArgs {
     int ntx[kTmaBatchGrids];            // tiles per row of grid k
     int y0[kTmaBatchGrids];             // first row of grid k's tiles in this launch
     int n;                              // grids of the launch
-    int late;                           // see launch order below
 };
-// Launch order: the step launches of one batch step are independent of each other.  The first of them
-// waits for the launches before it (grid_dependency_wait) when it starts; a `late` one, chained behind
-// it, starts once all CTAs of the one before have passed their own wait or start, so that everything
-// before the step is complete, and has one thread wait for that launch at its end, so that its own
-// completion stands for both.
 // Per-grid block of a batched launch (global memory, one per grid in launch order): the
 // geometry and the coefficients that the tile kernels read (C = Coef<float> or CoefDD); each
 // CTA copies its grid's block to shared memory while its tile copy is in flight.
@@ -183,10 +185,10 @@ struct TileGrid {
     C cf;
 };
 cudaError_t launch_step_tma_batch(const TmaBatchArgs &A, const TileGrid<Coef<float>> *tg, const Params *Pall, int limiter,
-                                  cudaStream_t st);
+                                  bool chain, cudaStream_t st);
 // shape: kDdWide, kDdMid or kDdNarrow (the grids' maps have its box); walls: some grid has one.
 cudaError_t launch_step_dd_batch(const TmaBatchArgs &A, const TileGrid<CoefDD> *tg, const Params *Pall, int limiter, int shape, bool walls,
-                                 cudaStream_t st);
+                                 bool chain, cudaStream_t st);
 // Failure-path check of the bounded mbarrier waits (lbm_wait_selftest): *flag = 1 when the
 // wait on a phase that nothing completes gave up at its limit; *ms = the kernel's duration.
 cudaError_t wait_selftest(int *flag, float *ms);
@@ -197,7 +199,7 @@ cudaError_t tma_batch_prepare(int limiter);
 // `tmap` points to the CUtensorMap of the input buffer fin (3-D: pitch x (ny+4) x 16).  The tiles fill
 // the ghost cells of every edge but walls themselves, from the interior of fin.
 cudaError_t launch_step_tma(const Params &P, int prec, const void *tmap, const void *fin, void *fout, int *err,
-                            cudaStream_t st, int late = 0);
+                            cudaStream_t st, bool chain = true);
 
 // Persistent double-buffered TMA-staged kernel (float32): CTAs walk tiles of kTmaTX columns
 // by TR rows round-robin with two tile buffers, so that the copy of the next tile overlaps
@@ -240,16 +242,16 @@ cudaError_t launch_step_stream(const Params &P, int prec, const void *tmap, void
 
 // Float64-mode step in double-float arithmetic on the float32 pipe (step_kernel 8, 9), on tiles of
 // `shape`, `tmap` with its box; `coef` is the CoefDD of the context (coef_dd).  Ghost cells as in
-// launch_step_tma.  late: as in TmaBatchArgs; rows: the first rows only (0: all), a multiple of the
+// launch_step_tma.  chain: as in launch_kernel; rows: the first rows only (0: all), a multiple of the
 // shape's.
 void coef_dd(const Params &P, CoefDD *out);
 // The kernels of one shape (lbm_step_dd.cuh).
 template <typename S>
 struct DdOps {
     static cudaError_t launch(const Params &P, const CoefDD &C, const CUtensorMap &tm, const double *a, double *b, int *err,
-                              int late, int rows, cudaStream_t st);
+                              bool chain, int rows, cudaStream_t st);
     static cudaError_t launch_batch(const TmaBatchArgs &A, const TileGrid<CoefDD> *tg, const Params *Pall, int limiter,
-                                    bool walls, cudaStream_t st);
+                                    bool walls, bool chain, cudaStream_t st);
     static cudaError_t prepare(const Params &P);
     static cudaError_t prepare_batch(int limiter, bool walls);
 };
@@ -259,7 +261,7 @@ extern template struct DdOps<DdNarrowShape>;
 cudaError_t dd_prepare(const Params &P);
 cudaError_t dd_batch_prepare(int limiter, bool walls);
 cudaError_t launch_step_dd(const Params &P, const void *coef, const void *tmap, const void *fin, void *fout,
-                           int *err, cudaStream_t st, int shape, int late = 0, int rows = 0);
+                           int *err, cudaStream_t st, int shape, bool chain = true, int rows = 0);
 
 // Sustained float64 FMA rate of the current device in FLOP/s (FMA = 2).
 cudaError_t measure_fp64_fma(double *flops);

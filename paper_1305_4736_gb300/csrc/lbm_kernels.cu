@@ -288,9 +288,10 @@ static_assert(sizeof(Params) % sizeof(int4) == 0, "Params is copied to shared me
 template <typename R, bool Dev, int Lim, int NT>
 __global__ void __launch_bounds__(NT)
 k_step_batch(const Params *__restrict__ Pall, const BatchGrid *__restrict__ G, const int4 *__restrict__ tiles,
-             int ntiles, int phase, int late)
+             int ntiles, int phase)
 {
-    batch_begin(late);
+    grid_dependency_wait();
+    grid_launch_dependents();
     constexpr int kSmem = 3 * (NT + 2);            // max over TX of (TX + 2)(TY + 2), at TX = 1
     __shared__ R su[kSmem];
     __shared__ R sv[kSmem];
@@ -317,7 +318,6 @@ k_step_batch(const Params *__restrict__ Pall, const BatchGrid *__restrict__ G, c
         step_tile<R, Dev, Lim>(Ps, (const R *)g.buf[in], (R *)g.buf[in ^ 1], tl.y, tl.z, TX, tl.w, NT / TX, su,
                                sv);
     }
-    batch_end(late, tid);
 }
 
 // ---------------------------------------------------------------------------
@@ -493,9 +493,10 @@ __global__ void k_ghost(const __grid_constant__ Params P, R *f, int first, int e
 
 // Batched ghost fill: blockIdx.y selects the grid of the batch, P.ghost its edges.
 template <typename R, bool Dev>
-__global__ void k_ghost_batch(const Params *__restrict__ Pall, const BatchGrid *__restrict__ G, int phase, int late)
+__global__ void k_ghost_batch(const Params *__restrict__ Pall, const BatchGrid *__restrict__ G, int phase)
 {
-    batch_begin(late);
+    grid_dependency_wait();
+    grid_launch_dependents();
     const int gi = blockIdx.y;
     const Params &P = Pall[gi];
     if (P.ghost != 0) {
@@ -504,7 +505,6 @@ __global__ void k_ghost_batch(const Params *__restrict__ Pall, const BatchGrid *
         for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n_all; idx += gridDim.x * blockDim.x)
             ghost_cell<R, Dev>(P, (R *)g.buf[g.cur ^ phase], idx, P.ghost);
     }
-    batch_end(late, threadIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -867,17 +867,17 @@ bool lane_step(const Params &P, int prec, int ty)
 }
 
 template <typename R, bool Dev, int NT>
-static cudaError_t step_launch_nt(const Params &P, const R *a, R *b, cudaStream_t st)
+static cudaError_t step_launch_nt(const Params &P, const R *a, R *b, cudaStream_t st, bool chain)
 {
     const int log_tx = plain_log_tx(P.nx);
     const int TX = 1 << log_tx, TY = NT / TX;
     const dim3 grid((P.nx + TX - 1) / TX, (P.ny + TY - 1) / TY);
     const size_t smem = 2 * sizeof(R) * (TX + 2) * (TY + 2);
     const auto fn = P.limiter == 0 ? k_step<R, Dev, 0, NT> : P.limiter == 1 ? k_step<R, Dev, 1, NT> : k_step<R, Dev, 2, NT>;
-    return launch_chained(fn, grid, dim3(NT), smem, st, P, a, b, TX, log_tx);
+    return launch_kernel(chain, fn, grid, dim3(NT), smem, st, P, a, b, TX, log_tx);
 }
 
-cudaError_t launch_step(const Params &P, int prec, const void *fin, void *fout, cudaStream_t st, int ty)
+cudaError_t launch_step(const Params &P, int prec, const void *fin, void *fout, cudaStream_t st, int ty, bool chain)
 {
     if (lane_step(P, prec, ty)) {
         int log_tx = plain_log_tx(P.nx);
@@ -887,56 +887,56 @@ cudaError_t launch_step(const Params &P, int prec, const void *fin, void *fout, 
         const auto fn = P.limiter == 0   ? (P.has_c9 ? k_step_lanes<0, true> : k_step_lanes<0, false>)
                         : P.limiter == 1 ? (P.has_c9 ? k_step_lanes<1, true> : k_step_lanes<1, false>)
                                          : (P.has_c9 ? k_step_lanes<2, true> : k_step_lanes<2, false>);
-        return launch_chained(fn, grid, dim3(kLaneTile * kCellLanes), 0, st, P, (const double *)fin, (double *)fout, TX,
-                              log_tx);
+        return launch_kernel(chain, fn, grid, dim3(kLaneTile * kCellLanes), 0, st, P, (const double *)fin, (double *)fout, TX,
+                             log_tx);
     }
     // ty: rows of a 32-column tile (2, 4, 8 or 16: 64 .. 512 threads); grids narrower than
     // 32 columns keep the thread count with TX = the smallest power of two >= nx
     if (prec == 0) {
         const double *a = (const double *)fin;
         double *b = (double *)fout;
-        if (ty == 2) return step_launch_nt<double, false, kTX * 2>(P, a, b, st);
-        if (ty == 4) return step_launch_nt<double, false, kTX * 4>(P, a, b, st);
-        if (ty == 16) return step_launch_nt<double, false, kTX * 16>(P, a, b, st);
-        return step_launch_nt<double, false, kTX * 8>(P, a, b, st);
+        if (ty == 2) return step_launch_nt<double, false, kTX * 2>(P, a, b, st, chain);
+        if (ty == 4) return step_launch_nt<double, false, kTX * 4>(P, a, b, st, chain);
+        if (ty == 16) return step_launch_nt<double, false, kTX * 16>(P, a, b, st, chain);
+        return step_launch_nt<double, false, kTX * 8>(P, a, b, st, chain);
     }
     const float *a = (const float *)fin;
     float *b = (float *)fout;
-    if (ty == 2) return step_launch_nt<float, true, kTX * 2>(P, a, b, st);
-    if (ty == 4) return step_launch_nt<float, true, kTX * 4>(P, a, b, st);
-    if (ty == 16) return step_launch_nt<float, true, kTX * 16>(P, a, b, st);
-    return step_launch_nt<float, true, kTX * 8>(P, a, b, st);
+    if (ty == 2) return step_launch_nt<float, true, kTX * 2>(P, a, b, st, chain);
+    if (ty == 4) return step_launch_nt<float, true, kTX * 4>(P, a, b, st, chain);
+    if (ty == 16) return step_launch_nt<float, true, kTX * 16>(P, a, b, st, chain);
+    return step_launch_nt<float, true, kTX * 8>(P, a, b, st, chain);
 }
 
 cudaError_t launch_ghost_batch(const Params *Pall, const BatchGrid *G, int ngrids, int max_ghost, int prec,
-                               int phase, int late, cudaStream_t st)
+                               int phase, bool chain, cudaStream_t st)
 {
     if (ngrids == 0 || max_ghost == 0) return cudaSuccess;
     const int nt = ghost_threads(prec), most = 64 * 128 / nt;
     const int bx = (max_ghost + nt - 1) / nt;
     const dim3 grid(bx > most ? most : bx, ngrids);
-    return prec == 0 ? launch_chained(k_ghost_batch<double, false>, grid, dim3(nt), 0, st, Pall, G, phase, late)
-                     : launch_chained(k_ghost_batch<float, true>, grid, dim3(nt), 0, st, Pall, G, phase, late);
+    return prec == 0 ? launch_kernel(chain, k_ghost_batch<double, false>, grid, dim3(nt), 0, st, Pall, G, phase)
+                     : launch_kernel(chain, k_ghost_batch<float, true>, grid, dim3(nt), 0, st, Pall, G, phase);
 }
 
 cudaError_t launch_step_batch(const Params *Pall, const BatchGrid *G, const int4 *tiles, int ntiles, int prec,
-                              int limiter, int nt, int ctas, int phase, int late, cudaStream_t st)
+                              int limiter, int nt, int ctas, int phase, bool chain, cudaStream_t st)
 {
     if (ntiles == 0) return cudaSuccess;
     const dim3 grid(ntiles < ctas ? ntiles : ctas);
     constexpr int N64 = kBatchThreadsFp64, N32 = kBatchThreads;
     auto pick = [&](auto *a, auto *b, auto *c) { return limiter == 0 ? a : limiter == 1 ? b : c; };
     if (prec == 0 && nt == N64)
-        return launch_chained(pick(k_step_batch<double, false, 0, N64>, k_step_batch<double, false, 1, N64>,
-                                   k_step_batch<double, false, 2, N64>),
-                              grid, dim3(N64), 0, st, Pall, G, tiles, ntiles, phase, late);
+        return launch_kernel(chain, pick(k_step_batch<double, false, 0, N64>, k_step_batch<double, false, 1, N64>,
+                                         k_step_batch<double, false, 2, N64>),
+                             grid, dim3(N64), 0, st, Pall, G, tiles, ntiles, phase);
     if (prec == 0)
-        return launch_chained(pick(k_step_batch<double, false, 0, N32>, k_step_batch<double, false, 1, N32>,
-                                   k_step_batch<double, false, 2, N32>),
-                              grid, dim3(N32), 0, st, Pall, G, tiles, ntiles, phase, late);
-    return launch_chained(pick(k_step_batch<float, true, 0, N32>, k_step_batch<float, true, 1, N32>,
-                               k_step_batch<float, true, 2, N32>),
-                          grid, dim3(N32), 0, st, Pall, G, tiles, ntiles, phase, late);
+        return launch_kernel(chain, pick(k_step_batch<double, false, 0, N32>, k_step_batch<double, false, 1, N32>,
+                                         k_step_batch<double, false, 2, N32>),
+                             grid, dim3(N32), 0, st, Pall, G, tiles, ntiles, phase);
+    return launch_kernel(chain, pick(k_step_batch<float, true, 0, N32>, k_step_batch<float, true, 1, N32>,
+                                     k_step_batch<float, true, 2, N32>),
+                         grid, dim3(N32), 0, st, Pall, G, tiles, ntiles, phase);
 }
 
 cudaError_t launch_moments(const Params &P, int prec, const void *f, int row0, int rows, double *rho,

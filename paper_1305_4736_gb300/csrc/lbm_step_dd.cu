@@ -63,25 +63,25 @@ double dd_shape_time(int shape, long long tiles, int sms)
 }
 
 cudaError_t launch_step_dd(const Params &P, const void *coef, const void *tmap, const void *fin, void *fout,
-                           int *err, cudaStream_t st, int shape, int late, int rows)
+                           int *err, cudaStream_t st, int shape, bool chain, int rows)
 {
     const CUtensorMap &tm = *reinterpret_cast<const CUtensorMap *>(tmap);
     const CoefDD &C = *reinterpret_cast<const CoefDD *>(coef);
     const double *a = (const double *)fin;
     double *b = (double *)fout;
     if (rows == 0) rows = P.ny;
-    return shape == kDdNarrow ? DdOps<DdNarrowShape>::launch(P, C, tm, a, b, err, late, rows, st)
-           : shape == kDdMid  ? DdOps<DdMidShape>::launch(P, C, tm, a, b, err, late, rows, st)
-                              : DdOps<DdWideShape>::launch(P, C, tm, a, b, err, late, rows, st);
+    return shape == kDdNarrow ? DdOps<DdNarrowShape>::launch(P, C, tm, a, b, err, chain, rows, st)
+           : shape == kDdMid  ? DdOps<DdMidShape>::launch(P, C, tm, a, b, err, chain, rows, st)
+                              : DdOps<DdWideShape>::launch(P, C, tm, a, b, err, chain, rows, st);
 }
 
 cudaError_t launch_step_dd_batch(const TmaBatchArgs &A, const TileGrid<CoefDD> *tg, const Params *Pall, int limiter,
-                                 int shape, bool walls, cudaStream_t st)
+                                 int shape, bool walls, bool chain, cudaStream_t st)
 {
     if (A.first[A.n] <= 0) return cudaSuccess;
-    return shape == kDdNarrow ? DdOps<DdNarrowShape>::launch_batch(A, tg, Pall, limiter, walls, st)
-           : shape == kDdMid  ? DdOps<DdMidShape>::launch_batch(A, tg, Pall, limiter, walls, st)
-                              : DdOps<DdWideShape>::launch_batch(A, tg, Pall, limiter, walls, st);
+    return shape == kDdNarrow ? DdOps<DdNarrowShape>::launch_batch(A, tg, Pall, limiter, walls, chain, st)
+           : shape == kDdMid  ? DdOps<DdMidShape>::launch_batch(A, tg, Pall, limiter, walls, chain, st)
+                              : DdOps<DdWideShape>::launch_batch(A, tg, Pall, limiter, walls, chain, st);
 }
 
 cudaError_t dd_prepare(const Params &P)

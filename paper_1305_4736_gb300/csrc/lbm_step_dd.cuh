@@ -595,7 +595,7 @@ __device__ __forceinline__ void dd_tile(const PP &P, const CoefDD &C, unsigned c
 template <int Lim, bool C9, bool Walls, typename S>
 __global__ void __launch_bounds__(kTmaTX * S::TT, S::CTAS)
 k_step_dd(const __grid_constant__ Params P, const __grid_constant__ CoefDD C, const __grid_constant__ CUtensorMap tm,
-          const double *fin, double *fout, int *err, int late)
+          const double *fin, double *fout, int *err)
 {
     extern __shared__ __align__(128) unsigned char smraw[];
     double *tile64 = reinterpret_cast<double *>(smraw);
@@ -609,7 +609,8 @@ k_step_dd(const __grid_constant__ Params P, const __grid_constant__ CoefDD C, co
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
-    batch_begin(late);
+    grid_dependency_wait();
+    grid_launch_dependents();
     if (tid == 0) {
         // box origin: interior column x0 - HX = padded column x0 + OX - HX; interior row y0 - 2 =
         // padded row y0
@@ -646,7 +647,6 @@ k_step_dd(const __grid_constant__ Params P, const __grid_constant__ CoefDD C, co
         }
         dd_tile<Lim, C9, Walls, S>(P, C, smraw, fout, x0, y0, edge ? P.edge : nullptr);
     }
-    batch_end(late, tid);
 }
 
 // ---------------------------------------------------------------------------
@@ -671,7 +671,8 @@ k_step_dd_batch(const __grid_constant__ TmaBatchArgs A, const TileGrid<CoefDD> *
     int x0, y0;
     const int g = batch_tile(A, blockIdx.x, S::TR, x0, y0);
     const unsigned bar_a = (unsigned)__cvta_generic_to_shared(&bar);
-    batch_begin(A.late);
+    grid_dependency_wait();
+    grid_launch_dependents();
     if (tid == 0)
         batch_issue<S::TR, S::HX>(A, g, x0, y0, (unsigned)__cvta_generic_to_shared(smraw), bar_a,
                                   (unsigned)S::tile_bytes, S::CTAS);
@@ -700,7 +701,6 @@ k_step_dd_batch(const __grid_constant__ TmaBatchArgs A, const TileGrid<CoefDD> *
         dd_tile<Lim, 2, Walls, S>(Ts, Ts.cf, smraw, static_cast<double *>(A.out[g]), x0, y0,
                            edge ? edges : nullptr);
     }
-    batch_end(A.late, tid);
 }
 
 static bool has_walls(const Params &P)
@@ -742,19 +742,19 @@ static cudaError_t dd_allow(K *kernel)
 
 template <typename S>
 cudaError_t DdOps<S>::launch(const Params &P, const CoefDD &C, const CUtensorMap &tm, const double *a, double *b, int *err,
-                             int late, int rows, cudaStream_t st)
+                             bool chain, int rows, cudaStream_t st)
 {
     const dim3 block(kTmaTX, S::TT);
     const dim3 grid((P.nx + kTmaTX - 1) / kTmaTX, (rows + S::TR - 1) / S::TR);
-    return launch_chained(dd_kernel<S>(P), grid, block, S::smem_bytes, st, P, C, tm, a, b, err, late);
+    return launch_kernel(chain, dd_kernel<S>(P), grid, block, S::smem_bytes, st, P, C, tm, a, b, err);
 }
 
 template <typename S>
 cudaError_t DdOps<S>::launch_batch(const TmaBatchArgs &A, const TileGrid<CoefDD> *tg, const Params *Pall, int limiter,
-                                   bool walls, cudaStream_t st)
+                                   bool walls, bool chain, cudaStream_t st)
 {
-    return launch_chained(dd_batch_kernel<S>(limiter, walls), dim3(A.first[A.n]), dim3(kTmaTX, S::TT), S::smem_bytes, st, A,
-                          tg, Pall);
+    return launch_kernel(chain, dd_batch_kernel<S>(limiter, walls), dim3(A.first[A.n]), dim3(kTmaTX, S::TT), S::smem_bytes,
+                         st, A, tg, Pall);
 }
 
 template <typename S>

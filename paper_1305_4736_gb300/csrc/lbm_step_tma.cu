@@ -142,9 +142,7 @@ __device__ __forceinline__ void flow_phase(const Coef<R> &C, const R *tile, R *s
     }
 }
 
-// Late: as in TmaBatchArgs, a member of a batch with its own launch (an instantiation of its own: as a
-// run-time argument it made the step 2% slower).
-template <typename R, bool Dev, int Lim, bool Late>
+template <typename R, bool Dev, int Lim>
 __global__ void __launch_bounds__(kTmaTX * TmaShape<R>::TT, TmaShape<R>::CTAS)
 k_step_tma(const __grid_constant__ Params P, const __grid_constant__ CUtensorMap tm, const R *fin,
            R *fout, int *err)
@@ -166,7 +164,8 @@ k_step_tma(const __grid_constant__ Params P, const __grid_constant__ CUtensorMap
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
-    batch_begin(Late);
+    grid_dependency_wait();
+    grid_launch_dependents();
     if (tid == 0) {
         // box origin: interior column x0 - HX = padded column x0 + OX - HX; interior row y0 - 2 =
         // padded row y0
@@ -200,7 +199,6 @@ k_step_tma(const __grid_constant__ Params P, const __grid_constant__ CUtensorMap
             atomicExch(err, 1);
             mbar_wait(bar_a, 0);               // let a late copy land before the CTA exits (bounded)
         }
-        if (Late) batch_end(1, tid);
         return;
     }
     if (edge) {
@@ -309,7 +307,6 @@ k_step_tma(const __grid_constant__ Params P, const __grid_constant__ CUtensorMap
         }
 
     }
-    if (Late) batch_end(1, tid);
 }
 
 // ---------------------------------------------------------------------------
@@ -337,7 +334,8 @@ k_step_tma_batch(const __grid_constant__ TmaBatchArgs A, const TileGrid<Coef<flo
     int x0, y0;
     const int g = batch_tile(A, blockIdx.x, S::TR, x0, y0);
     const unsigned bar_a = (unsigned)__cvta_generic_to_shared(&bar);
-    batch_begin(A.late);
+    grid_dependency_wait();
+    grid_launch_dependents();
     if (tid == 0)
         batch_issue<S::TR, S::HX>(A, g, x0, y0, (unsigned)__cvta_generic_to_shared(tile), bar_a,
                                   (unsigned)S::tile_bytes, S::CTAS);
@@ -367,7 +365,6 @@ k_step_tma_batch(const __grid_constant__ TmaBatchArgs A, const TileGrid<Coef<flo
         phase2_packed<true, Lim>(Ts, reinterpret_cast<const float2 *>(tile), reinterpret_cast<const float2 *>(su),
                                  lane, ty, x0, y0, static_cast<float *>(A.out[g]));
     }
-    batch_end(A.late, tid);
 }
 
 static auto tma_batch_kernel(int limiter)
@@ -376,12 +373,13 @@ static auto tma_batch_kernel(int limiter)
 }
 
 cudaError_t launch_step_tma_batch(const TmaBatchArgs &A, const TileGrid<Coef<float>> *tg, const Params *Pall,
-                                  int limiter, cudaStream_t st)
+                                  int limiter, bool chain, cudaStream_t st)
 {
     using S = TmaShape<float>;
     const int ntiles = A.first[A.n];
     if (ntiles <= 0) return cudaSuccess;
-    return launch_chained(tma_batch_kernel(limiter), dim3(ntiles), dim3(kTmaTX, S::TT), S::smem_bytes, st, A, tg, Pall);
+    return launch_kernel(chain, tma_batch_kernel(limiter), dim3(ntiles), dim3(kTmaTX, S::TT), S::smem_bytes, st, A, tg,
+                         Pall);
 }
 
 // ---------------------------------------------------------------------------
@@ -551,32 +549,29 @@ bool tma_supported(const Params &P, int prec)
     return P.pitch >= TmaShape<float>::SW && P.ny + 4 >= sh && P.nx >= kTmaTX;
 }
 
-template <typename R, bool Dev, bool Late>
+template <typename R, bool Dev>
 static auto tma_kernel(int limiter)
 {
-    return limiter == 0   ? k_step_tma<R, Dev, 0, Late>
-           : limiter == 1 ? k_step_tma<R, Dev, 1, Late>
-                          : k_step_tma<R, Dev, 2, Late>;
+    return limiter == 0 ? k_step_tma<R, Dev, 0> : limiter == 1 ? k_step_tma<R, Dev, 1> : k_step_tma<R, Dev, 2>;
 }
 
-template <typename R, bool Dev, bool Late>
+template <typename R, bool Dev>
 static cudaError_t launch_tma_lim(const Params &P, const CUtensorMap &tm, const void *a, void *b, int *err,
-                                  cudaStream_t st)
+                                  cudaStream_t st, bool chain)
 {
     using S = TmaShape<R>;
     const dim3 block(kTmaTX, S::TT);
     const dim3 grid((P.nx + kTmaTX - 1) / kTmaTX, (P.ny + S::TR - 1) / S::TR);
-    return launch_chained(tma_kernel<R, Dev, Late>(P.limiter), grid, block, S::smem_bytes, st, P, tm, (const R *)a, (R *)b,
-                          err);
+    return launch_kernel(chain, tma_kernel<R, Dev>(P.limiter), grid, block, S::smem_bytes, st, P, tm, (const R *)a, (R *)b,
+                         err);
 }
 
 cudaError_t launch_step_tma(const Params &P, int prec, const void *tmap, const void *fin, void *fout, int *err,
-                            cudaStream_t st, int late)
+                            cudaStream_t st, bool chain)
 {
     const CUtensorMap &tm = *reinterpret_cast<const CUtensorMap *>(tmap);
-    if (prec == 0) return launch_tma_lim<double, false, false>(P, tm, fin, fout, err, st);   // never late
-    return late ? launch_tma_lim<float, true, true>(P, tm, fin, fout, err, st)
-                : launch_tma_lim<float, true, false>(P, tm, fin, fout, err, st);
+    return prec == 0 ? launch_tma_lim<double, false>(P, tm, fin, fout, err, st, chain)
+                     : launch_tma_lim<float, true>(P, tm, fin, fout, err, st, chain);
 }
 
 template <typename S, typename K>
@@ -587,14 +582,13 @@ static cudaError_t tma_allow(K *kernel)
 
 cudaError_t tma_prepare(int prec, int limiter)
 {
-    return prec == 0 ? tma_allow<TmaShape<double>>(tma_kernel<double, false, false>(limiter))
-                     : tma_allow<TmaShape<float>>(tma_kernel<float, true, false>(limiter));
+    return prec == 0 ? tma_allow<TmaShape<double>>(tma_kernel<double, false>(limiter))
+                     : tma_allow<TmaShape<float>>(tma_kernel<float, true>(limiter));
 }
 
 cudaError_t tma_batch_prepare(int limiter)
 {
-    const cudaError_t e = tma_allow<TmaShape<float>>(tma_kernel<float, true, true>(limiter));
-    return e == cudaSuccess ? tma_allow<TmaShape<float>>(tma_batch_kernel(limiter)) : e;
+    return tma_allow<TmaShape<float>>(tma_batch_kernel(limiter));
 }
 
 }  // namespace lbm

@@ -69,23 +69,14 @@ __device__ __forceinline__ R slope2(R a, R b)
 }
 
 // Programmatic dependent launch: a step kernel's CTAs may start while the previous launch of the
-// stream drains, and wait here before they touch its results.  A kernel that is launched so does not
+// stream drains, and wait here before they touch its results.  Every kernel of a chained launch waits,
+// also one that reads nothing of the launch before it: the wait is what makes the results of all earlier
+// launches visible to it, and its completion then stands for theirs.  A kernel that is launched so does not
 // take its populations as __restrict__: until the wait is over the launch before it still writes them,
 // and the qualifier would let the compiler read them through the non-coherent path, or above the wait.
 // Functions called after the wait may (until the kernel ends nothing else writes what they read).
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
-// Start and end of a batched launch (`late`: TmaBatchArgs).
-__device__ __forceinline__ void batch_begin(int late)
-{
-    if (!late) grid_dependency_wait();
-    grid_launch_dependents();
-}
-__device__ __forceinline__ void batch_end(int late, int tid)
-{
-    if (late && tid == 0 && blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1) grid_dependency_wait();
-}
 
 // Coordinate a read at v goes to along an axis of n cells: the wrapped cell past a periodic edge
 // (kind 0), the edge cell past a zero-gradient one (1), else v itself.

@@ -22,7 +22,7 @@ def _kernels():
 
 
 def _chained():
-    out = [k for k in _kernels() if re.search(r"\b(grid_dependency_wait|batch_begin)\(", k[2])]
+    out = [k for k in _kernels() if re.search(r"griddepcontrol|\b(grid_dependency_wait|grid_launch_dependents|batch_begin)\(", k[2])]
     assert {"k_step", "k_step_lanes", "k_step_tma", "k_step_dd", "k_ghost", "k_wall", "k_step_batch"} <= {k[0] for k in out}
     return out
 
@@ -30,3 +30,14 @@ def _chained():
 def test_chained_kernels_do_not_promise_that_nobody_writes_their_populations():
     for name, params, _ in _chained():
         assert not re.search(r"\b(R|double|float) \*__restrict__", params), name
+
+
+def test_chained_kernels_wait_before_anything_else_of_their_grid():
+    """A grid reads the results of earlier launches only behind its own griddepcontrol.wait: every kernel that
+    is launched so waits, whatever its arguments, and before it reads populations or tables."""
+    for name, _, body in _chained():
+        at = body.find("grid_dependency_wait();")
+        assert at >= 0, name
+        before = body[:at]
+        assert not re.search(r"\bif\s*\([^)]*$", before), name                    # not conditional
+        assert not re.search(r"\b(fin|f|Pall|G|TG|tiles)\s*\[|->|\bload\(|cp\.async", before), name
