@@ -60,16 +60,16 @@ TOTALS_EVERY = 100
 TRAFFIC_PER_CELL = {
     "f32": {"bytes": 125.70, "sources": ("lbm_step_tma.cu", "lbm_device.cuh", "lbm_tma_util.cuh"),
             "sha": "f57fd1118d25abec"},
-    "f64": {"bytes": 251.33, "sources": ("lbm_step_stream.cu", "lbm_device.cuh", "lbm_tma_util.cuh"),
+    "f64": {"bytes": 251.50, "sources": ("lbm_step_stream.cu", "lbm_device.cuh", "lbm_tma_util.cuh"),
             "sha": "26f4c99f86763e64"},
-    "dd": {"bytes": 246.42, "sources": ("lbm_step_dd.cuh", "lbm_dd.cuh", "lbm_device.cuh", "lbm_tma_util.cuh"),
-           "sha": "8f11fe86e2ce9475"},
+    "dd": {"bytes": 246.72, "sources": ("lbm_step_dd.cuh", "lbm_dd.cuh", "lbm_device.cuh", "lbm_tma_util.cuh"),
+           "sha": "17adc38de3cc6a8a"},
 }
 # float32-pipe lane operations per cell of one launch of the double-float float64 kernel on wide
 # tiles: ncu's FMA-pipe busy fraction x cycles x 128 lanes (its counters of float32 instructions do
 # not see the packed f32x2 ones), on the same sources (profiles/k_step_dd_f64_shear_layer.md); None
 # when the sources changed since.
-DD_FP32_OPS = {"ops": 3537.6, "sha": "8f11fe86e2ce9475"}
+DD_FP32_OPS = {"ops": 3537.7, "sha": "17adc38de3cc6a8a"}
 FP32_LANES_PER_SM = 128           # float32 FMA lanes per SM per cycle (GB300)
 
 

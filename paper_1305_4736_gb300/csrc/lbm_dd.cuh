@@ -231,8 +231,10 @@ __device__ __forceinline__ dd2 add_smaller(dd2 a, dd2 b)
 // mc2n for both lanes: the sums, products and differences packed, the selects per lane.  The
 // order tests read the sign of a difference relative to that of a (or of s, equal to it where the
 // differences agree) from their product: below 2^-149, where it reads as zero, the candidates
-// differ by less than 2^-74, the flush threshold of the split.  Where a and b disagree in sign
-// the candidate m is scaled by 0 instead of 4, and |m| < |s| selects it.
+// differ by less than 2^-74, the flush threshold of the split.  Where a and b disagree in sign the result
+// is set to zero last: s is not normalised, so where the high parts cancel the sign of s.hi is not that of
+// s, and no test against s can tell (at an extremum symmetric to 2^-24, s would be taken for the slope).
+// Scaling the candidates by 0 there instead is 1% of the step less, and gives NaN for infinities and NaN.
 __device__ __forceinline__ dd2 mc2n(dd2 a, dd2 b)
 {
     const dd2 s = a + b;
@@ -243,14 +245,17 @@ __device__ __forceinline__ dd2 mc2n(dd2 a, dd2 b)
     m.lo.x = tab.x < 0.0f ? a.lo.x : b.lo.x;
     m.hi.y = tab.y < 0.0f ? a.hi.y : b.hi.y;
     m.lo.y = tab.y < 0.0f ? a.lo.y : b.lo.y;
-    const float2 w = f2(ab.x > 0.0f ? 4.0f : 0.0f, ab.y > 0.0f ? 4.0f : 0.0f);
-    const dd2 m4 = dd2{mul2(m.hi, w), mul2(m.lo, w)};
+    const dd2 m4 = scale2(m, 4.0f);
     const float2 tms = mul2(add2(sub2(m4.hi, s.hi), sub2(m4.lo, s.lo)), s.hi);
     dd2 r;
     r.hi.x = tms.x < 0.0f ? m4.hi.x : s.hi.x;
     r.lo.x = tms.x < 0.0f ? m4.lo.x : s.lo.x;
     r.hi.y = tms.y < 0.0f ? m4.hi.y : s.hi.y;
     r.lo.y = tms.y < 0.0f ? m4.lo.y : s.lo.y;
+    r.hi.x = ab.x > 0.0f ? r.hi.x : 0.0f;
+    r.lo.x = ab.x > 0.0f ? r.lo.x : 0.0f;
+    r.hi.y = ab.y > 0.0f ? r.hi.y : 0.0f;
+    r.lo.y = ab.y > 0.0f ? r.lo.y : 0.0f;
     return r;
 }
 
