@@ -379,6 +379,35 @@ __device__ __forceinline__ R flux_diff(R fmm, R fm, R f0, R fp, R hh)
     return d1 + hh * (mc2(d1, d2) - mc2(d0, d1));
 }
 
+// Non-equilibrium extrapolation wall: f_g - f_m of a ghost cell and its mirror cell m, of populations g.
+template <typename R>
+__device__ __forceinline__ R pick(double d, float f);
+template <> __device__ __forceinline__ double pick<double>(double d, float) { return d; }
+template <> __device__ __forceinline__ float pick<float>(double, float f) { return f; }
+template <typename R, bool Dev>
+__device__ __forceinline__ void wall_change(const Coef<R> &C, const EdgeDev &E, const R *g, R *fd)
+{
+    const Shells<R> s = shells_of(g);
+    R drho, jx, jy, de;
+    conserved_of(s, drho, jx, jy, de);
+    const R rho = Dev ? C.rho0 + drho : drho;
+    const R ir = recip(rho);
+    const R J2 = (jx * jx + jy * jy) * ir;
+    const R dP = (de - J2) * C.inv_b;
+    // ghost state: rho_g = rho_m, j_g = 2 rho_m u_w - j_m, P_g = rho_m (2 T_w - T_m)
+    const R uw = pick<R>(E.uw, E.uwf), vw = pick<R>(E.vw, E.vwf), Tw = pick<R>(E.Tw, E.Twf);
+    const R jgx = R(2.0) * rho * uw - jx;
+    const R jgy = R(2.0) * rho * vw - jy;
+    const R dPg = Dev ? pick<R>(E.two_rho0_dTw, E.two_rho0_dTwf) + R(2.0) * drho * Tw - dP
+                      : R(2.0) * rho * Tw - dP;
+    R qm[NQ], qg[NQ], d[NQ];
+    feq_hat_dev<R, Dev>(C, drho, jx, jy, dP, ir, qm);
+    feq_hat_dev<R, Dev>(C, drho, jgx, jgy, dPg, ir, qg);
+#pragma unroll
+    for (int q = 0; q < NQ; q++) d[q] = qg[q] - qm[q];
+    pop_from_moments(C, d, fd);
+}
+
 // ---------------------------------------------------------------------------
 // Collision (Eq. 3 with the energy-flux correction of Sec. II):
 //   out = dt M^-1 S (f_hat - f_hat^eq), residuals of rows 1..4 are zero.

@@ -153,7 +153,6 @@ struct CoefDD {
     dd2 hh[2], hhy[2], cr[2], cry[2];
     dd2 pA[2][2], pEx[2][3], pEy[2][3], pB1[2], pB2[2];
     dd2 q89, g4;
-    dd2 wA[2][3], wEx[2][4], wEy[2][4], wB1[2], wB2[2];   // full inverse blocks (walls), without the density row
     dd b, inv_b, two_b2, six_b, b4, four_inv_b, ry, pad_;
 };
 static_assert(sizeof(CoefDD) % 16 == 0, "CoefDD is copied in 16-byte words");

@@ -35,11 +35,6 @@ __device__ __forceinline__ bool u_cell(int x, int y, int nx, int ny)
     return (x >= -1 && x <= nx && y >= 0 && y < ny) || (y >= -1 && y <= ny && x >= 0 && x < nx);
 }
 
-template <typename R>
-__device__ __forceinline__ R pick(double d, float f);
-template <> __device__ __forceinline__ double pick<double>(double d, float) { return d; }
-template <> __device__ __forceinline__ float pick<float>(double, float f) { return f; }
-
 __device__ __forceinline__ void load16(const double *__restrict__ f, long long plane, long long c, double *out)
 {
 #pragma unroll
@@ -418,25 +413,8 @@ __device__ __forceinline__ void ghost_cell(const Params &P, R *__restrict__ f, i
         const long long cm = (long long)(my + OY) * P.pitch + (mx + OX);
         R g[NQ];
         load16(f, plane, cm, g);
-        const Shells<R> s = shells_of(g);
-        R drho, jx, jy, de;
-        conserved_of(s, drho, jx, jy, de);
-        const R rho = Dev ? C.rho0 + drho : drho;
-        const R ir = recip(rho);
-        const R J2 = (jx * jx + jy * jy) * ir;
-        const R dP = (de - J2) * C.inv_b;
-        // ghost state: rho_g = rho_m, j_g = 2 rho_m u_w - j_m, P_g = rho_m (2 T_w - T_m)
-        const R uw = pick<R>(E.uw, E.uwf), vw = pick<R>(E.vw, E.vwf), Tw = pick<R>(E.Tw, E.Twf);
-        const R jgx = R(2.0) * rho * uw - jx;
-        const R jgy = R(2.0) * rho * vw - jy;
-        const R dPg = Dev ? pick<R>(E.two_rho0_dTw, E.two_rho0_dTwf) + R(2.0) * drho * Tw - dP
-                          : R(2.0) * rho * Tw - dP;
-        R qm[NQ], qg[NQ], d[NQ], fd[NQ];
-        feq_hat_dev<R, Dev>(C, drho, jx, jy, dP, ir, qm);
-        feq_hat_dev<R, Dev>(C, drho, jgx, jgy, dPg, ir, qg);
-#pragma unroll
-        for (int q = 0; q < NQ; q++) d[q] = qg[q] - qm[q];
-        pop_from_moments(C, d, fd);
+        R fd[NQ];
+        wall_change<R, Dev>(C, E, g, fd);
 #pragma unroll
         for (int q = 0; q < NQ; q++) f[pidx<R>(q, plane, cg)] = g[q] + fd[q];
     }

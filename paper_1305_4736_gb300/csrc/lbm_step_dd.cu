@@ -27,16 +27,6 @@ void coef_dd(const Params &P, CoefDD *out)
         out->pB1[p] = pair(C.cB1[0][p], C.cB1[1][p]);
         out->pB2[p] = pair(C.cB2[0][p], C.cB2[1][p]);
     }
-    for (int p = 0; p < 2; p++) {
-        for (int j = 0; j < 3; j++) out->wA[p][j] = pair(C.iA[2 * p][j + 1], C.iA[2 * p + 1][j + 1]);
-        for (int j = 0; j < 4; j++) {
-            const double sg = j == 3 ? -1.0 : 1.0;
-            out->wEx[p][j] = pair(C.iEx[2 * p][j], C.iEx[2 * p + 1][j]);
-            out->wEy[p][j] = pair(sg * C.iEy[2 * p][j], sg * C.iEy[2 * p + 1][j]);
-        }
-        out->wB1[p] = pair(C.iB1[0][p], C.iB1[1][p]);
-        out->wB2[p] = pair(C.iB2[0][p], C.iB2[1][p]);
-    }
     out->q89 = pair(C.q8, C.q9);
     out->g4 = pair(C.g4[0], C.g4[1]);
     out->b = dd_host(C.b);

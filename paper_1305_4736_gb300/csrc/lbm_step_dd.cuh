@@ -341,83 +341,35 @@ __device__ __forceinline__ void ring_and_edges(const float2 *tile, float4 *suv, 
     }
 }
 
-// Rows of f_hat^eq (Appendix A closed forms) but the density, in the pairs the inverse blocks take; the
-// row of m13 negated.
-struct RowsDD { dd m4; dd2 j, d513, d78, d910, d1112, d515, d614; };
-
-__device__ __forceinline__ RowsDD equilibrium_dd(const CoefDD &C, dd2 j, dd2 u, dd ir, dd P)
+// One ghost cell of a wall in the staged tile (before its split) from its mirror cell, in float64 as the
+// ghost launch of the other kernels forms it: the two warps of a tile's wall cells take some 225 float64
+// instructions each, 4.5 us, while the other warps wait (161 x 97 channel 14.8 us a step, 18.8 with a
+// launch before the step, 512 x 512 52 and 53, 1023 x 517 94 and 114).  In double-float it was 10.3 us on
+// 161 x 97, with three to four times the error of a step at the wall cells.  A function of its own: every tile shape,
+// alone and in a batch, runs the same code and has the same bits.
+__device__ __noinline__ void wall_cell64(const Coef<double> &C, const EdgeDev &E, const double *mirror, double *ghost,
+                                         int plane)
 {
-    RowsDD r;
-    const dd2 jj = j * u;
-    const dd J2 = sum_lanes(jj), dxy = first(jj) - second(jj);
-    const dd P2 = scale2(P, 2.0f), k = fma_dd(C.b4, P, J2);
-    const dd q6 = first(j) * second(u);
-    r.j = j;
-    r.m4 = fma_dd(C.b, P, J2);
-    r.d513 = pack(P2 + J2, ir * (P * fma_dd(C.two_b2, P, C.six_b * J2) + J2 * J2));
-    r.d78 = bcast(r.m4 + P2) * u;
-    r.d910 = bcast(scale2(P, 4.0f) + J2) * u;
-    r.d1112 = pack(P2 + dxy, P2 - dxy) * u;
-    const dd2 q1415 = bcast(k) * pack(first(u), dxy) * pack(second(u), ir);
-    r.d515 = pack(dxy, second(q1415));
-    r.d614 = pack(q6, first(q1415));
-    return r;
+    double g[NQ], fd[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; q++) g[q] = mirror[q * plane];
+    wall_change<double, false>(C, E, g, fd);
+#pragma unroll
+    for (int q = 0; q < NQ; q++) ghost[q * plane] = g[q] + fd[q];
 }
 
-// Ghost cells of the walls at an edge tile, in the split staged tile: rho_g = rho_m, j_g = 2 rho_m u_w -
-// j_m, P_g = rho_m (2 T_w - T_m) of the mirror cell m, f_g = f_m + M^-1 (f_hat^eq(g) - f_hat^eq(m)).  One
-// thread per ghost cell.  In double-float, as the step: on the float64 pipe, in a launch before the
-// step's, they made a step of a 161 x 97 channel 18.9 us, here 10.3.  Error against 64 bits, over
-// that with float64 walls (68 runs of 16 channels, 150 to 1000 steps, geometric means and their standard
-// errors): rho 1.015 +- 0.011 (of 1e-14), velocity 0.996 +- 0.010 (of 1e-12), T 0.998 +- 0.009, all three 1.003
-// +- 0.006: the staged tile holds 48 bits of a ghost cell in either case.
+// Ghost cells of the walls at an edge tile, one thread per cell.  G: the grid's extents; P: its
+// coefficients and edges.
 template <typename S, typename PP>
-__device__ __noinline__ void wall_fill(const PP &P, const CoefDD &C, const EdgeDev *edges, float2 *tile, int x0, int y0,
-                                       int tid)
+__device__ __forceinline__ void wall_fill(const PP &G, const Params &P, double *tile, int x0, int y0, int tid)
 {
-    constexpr int kSlots = 4 * kTmaTX + 4 * S::TR;
-    for (int k = tid; k < kSlots; k += kTmaTX * S::TT) {
-        const GhostSlot<S> g(P, k, x0, y0);
-        if (!g.in) continue;
-        const EdgeDev &E = edges[g.edge];
-        if (E.kind != 3) continue;
-        const int n = g.row ? P.ny : P.nx, depth = g.layer & 1;
+    for (int k = tid; k < GhostSlot<S>::kSlots; k += kTmaTX * S::TT) {
+        const GhostSlot<S> g(G, k, x0, y0);
+        if (!g.in || P.edge[g.edge].kind != 3) continue;
+        const int n = g.row ? G.ny : G.nx, depth = g.layer & 1;
         const int m = min(max(g.layer < 2 ? depth : n - 1 - depth, 0), n - 1);
-        const int c = g.offset(g.row ? m - y0 + 2 : m - x0 + S::HX);
-        dd2 fp[8];
-#pragma unroll
-        for (int pr = 0; pr < 8; pr++) fp[pr] = tile_pair<S>(tile, pr, c);
-        const ShellsDD s = shells_dd(fp);
-        const dd rho = sum_lanes(s.S[0]) + sum_lanes(s.S[1]);
-        const dd ir = recip(rho);
-        const dd2 j = flux_dd(s.X[0], s.X[1], s.Y[0], s.Y[1]);
-        const dd2 e0 = s.S[0] * f2(7.25f, 36.0f), e1 = s.S[1] * f2(4.0f, 9.0f);
-        const dd e = (sum_lanes(e0) + first(e1)) + second(e1);
-        const dd2 u = j * bcast(ir);
-        const dd Pm = (e - sum_lanes(j * u)) * C.inv_b;
-        const dd r2 = scale2(rho, 2.0f);
-        const dd2 jg = bcast(r2) * pack(dd_split(E.uw), dd_split(E.vw)) - j;
-        const RowsDD a = equilibrium_dd(C, jg, jg * bcast(ir), ir, r2 * dd_split(E.Tw) - Pm);
-        const RowsDD b = equilibrium_dd(C, j, u, ir, Pm);
-        const dd2 dj = a.j - b.j, d513 = a.d513 - b.d513, d78 = a.d78 - b.d78, d910 = a.d910 - b.d910;
-        const dd2 d1112 = a.d1112 - b.d1112, d515 = a.d515 - b.d515, d614 = a.d614 - b.d614;
-        const dd2 d4 = bcast(a.m4 - b.m4), d5 = bcast(first(d513)), d14 = bcast(second(d513));
-        dd2 fd[8];
-        auto iso = [&](int p) { return (C.wA[p][0] * d4 + C.wA[p][1] * d5) + C.wA[p][2] * d14; };
-        auto odd = [&](const dd2 *w, dd a0, dd a1, dd a2, dd a3) {
-            return ((w[0] * bcast(a0) + w[1] * bcast(a1)) + w[2] * bcast(a2)) + w[3] * bcast(a3);
-        };
-        auto X = [&](int p) { return odd(C.wEx[p], first(dj), first(d78), first(d910), first(d1112)); };
-        auto Y = [&](int p) { return odd(C.wEy[p], second(dj), second(d78), second(d910), second(d1112)); };
-        unbutterfly_dd_axis(iso(0), X(0), Y(0), C.wB1[0] * bcast(first(d515)) + C.wB1[1] * bcast(second(d515)), fd);
-        unbutterfly_dd_diag(iso(1), X(1), Y(1), C.wB2[0] * bcast(first(d614)) + C.wB2[1] * bcast(second(d614)), fd + 4);
-        const int to = g.offset(g.at);
-#pragma unroll
-        for (int pr = 0; pr < 8; pr++) {
-            const dd2 v = norm(fp[pr] + fd[pr]);
-            tile[pair_q(pr) * S::PL + to] = v.hi;
-            tile[(pair_q(pr) + 4) * S::PL + to] = v.lo;
-        }
+        wall_cell64(P.cd, P.edge[g.edge], tile + g.offset(g.row ? m - y0 + 2 : m - x0 + S::HX), tile + g.offset(g.at),
+                    S::PL);
     }
 }
 
@@ -430,11 +382,9 @@ __device__ __noinline__ void wall_fill(const PP &P, const CoefDD &C, const EdgeD
 // P: the context's Params, or the TileGrid block of a batched launch (nx, ny, pitch, plane).
 // S: the tile shape.
 // C9: whether the energy-flux correction runs (0, 1), or 2 to ask P.has_c9.
-// Walls: a grid with walls (an instantiation of its own: the call of wall_fill made the step of grids
-// without any 1.5% slower); walls: its edges, where the tile holds ghost cells, else null.
-template <int Lim, int C9, bool Walls, typename S, typename PP>
+template <int Lim, int C9, typename S, typename PP>
 __device__ __forceinline__ void dd_tile(const PP &P, const CoefDD &C, unsigned char *smraw,
-                                        double *__restrict__ fout, int x0, int y0, const EdgeDev *walls)
+                                        double *__restrict__ fout, int x0, int y0)
 {
     double *tile64 = reinterpret_cast<double *>(smraw);
     float2 *tile = reinterpret_cast<float2 *>(smraw);
@@ -453,10 +403,6 @@ __device__ __forceinline__ void dd_tile(const PP &P, const CoefDD &C, unsigned c
         tile[b] = v.lo;
     }
     __syncthreads();
-    if (Walls && walls) {
-        wall_fill<S>(P, C, walls, tile, x0, y0, tid);
-        __syncthreads();
-    }
 
     const unsigned edge_a = (unsigned)__cvta_generic_to_shared(sedge);
     const int gx = x0 + lane;
@@ -590,7 +536,8 @@ __device__ __forceinline__ void dd_tile(const PP &P, const CoefDD &C, unsigned c
 }
 
 // ---------------------------------------------------------------------------
-// The single-grid kernel.
+// The single-grid kernel.  Walls: a grid with walls (an instantiation of its own: with the call of
+// wall_fill the step of grids without any takes 1.5% longer).
 // ---------------------------------------------------------------------------
 template <int Lim, bool C9, bool Walls, typename S>
 __global__ void __launch_bounds__(kTmaTX * S::TT, S::CTAS)
@@ -643,9 +590,10 @@ k_step_dd(const __grid_constant__ Params P, const __grid_constant__ CoefDD C, co
     } else {
         if (edge) {
             ghost.store(tile64);
+            if (Walls) wall_fill<S>(P, P, tile64, x0, y0, tid);
             __syncthreads();
         }
-        dd_tile<Lim, C9, Walls, S>(P, C, smraw, fout, x0, y0, edge ? P.edge : nullptr);
+        dd_tile<Lim, C9, S>(P, C, smraw, fout, x0, y0);
     }
 }
 
@@ -695,11 +643,10 @@ k_step_dd_batch(const __grid_constant__ TmaBatchArgs A, const TileGrid<CoefDD> *
     } else {
         if (edge) {
             ghost.store(reinterpret_cast<double *>(smraw));
+            if (Walls) wall_fill<S>(Ts, Pall[Ts.member], reinterpret_cast<double *>(smraw), x0, y0, tid);
             __syncthreads();
         }
-        const EdgeDev *edges = Pall[Ts.member].edge;
-        dd_tile<Lim, 2, Walls, S>(Ts, Ts.cf, smraw, static_cast<double *>(A.out[g]), x0, y0,
-                           edge ? edges : nullptr);
+        dd_tile<Lim, 2, S>(Ts, Ts.cf, smraw, static_cast<double *>(A.out[g]), x0, y0);
     }
 }
 
