@@ -1347,14 +1347,15 @@ long long wide_tiles(const lbm_ctx *c)
 // whose members have kAloneMean tiles on average: between short launches slots stay empty.  Measured, us
 // per batch step, all batched and with the rule: 24 float32 grids of 0.58 M cells on average 343 and 307,
 // of 0.14 M 93.4 and 88.7; float64, 2092 and 1910, 580 and 527.
-constexpr int kAloneTiles = 64, kAloneMean = 256;
+// Members of more tile rows than a launch has in y keep to the batched launch, which numbers its tiles in x.
+constexpr int kAloneTiles = 64, kAloneMean = 256, kAloneRows = lbm::kMaxGridY * lbm::DdWideShape::TR;
 
 // Rows (from row 0) of member c that such a launch covers: the whole float32 grid; of a float64 one the
 // rows of full tiles, or all where the last tile row is more than 3/4 full.
 int alone_rows(const lbm_ctx *c, bool allowed)
 {
     const int tr = lbm::DdWideShape::TR, ny = c->P.ny;
-    if (!allowed || wide_tiles(c) < kAloneTiles) return 0;
+    if (!allowed || wide_tiles(c) < kAloneTiles || ny > kAloneRows) return 0;
     return c->prec == LBM_FP32_DEV || 4 * (ny % tr) > 3 * tr ? ny : ny - ny % tr;
 }
 

@@ -111,6 +111,7 @@ struct TmaShape {
     static constexpr size_t tile_bytes = sizeof(R) * NQ * PL;
     static constexpr size_t smem_bytes = tile_bytes + sizeof(R) * (sizeof(R) == sizeof(float) ? 2 : 3) * UW * UH;
 };
+constexpr int kMaxGridY = 65535;        // a launch's limit on gridDim.y and z
 bool tma_supported(const Params &P, int prec);
 // Tiles of the double-float float64 kernels: 32 columns by TR rows, TT warps, KR rows per thread,
 // CTAS CTAs per SM.  ROLES: two warps per row, one for the collision and one for the convection.

@@ -549,7 +549,9 @@ k_step_dd(const __grid_constant__ Params P, const __grid_constant__ CoefDD C, co
     __shared__ __align__(8) unsigned long long bar;
 
     const int tid = threadIdx.y * kTmaTX + threadIdx.x;
-    const int x0 = blockIdx.x * kTmaTX, y0 = blockIdx.y * S::TR;
+    // tile rows past 65535, the grid dimension's limit, go on along z (DdOps::launch)
+    const int x0 = blockIdx.x * kTmaTX, row = blockIdx.z * gridDim.y + blockIdx.y, y0 = row * S::TR;
+    if (y0 >= P.ny) return;
     const unsigned bar_a = (unsigned)__cvta_generic_to_shared(&bar);
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar_a) : "memory");
@@ -571,9 +573,9 @@ k_step_dd(const __grid_constant__ Params P, const __grid_constant__ CoefDD C, co
         // bring the tile of the CTA half a resident wave later into L2
         unsigned nsm;
         asm("mov.u32 %0, %%nsmid;" : "=r"(nsm));
-        const long long bn = (long long)blockIdx.y * gridDim.x + blockIdx.x + (long long)S::CTAS * nsm / 2;
-        if (bn < (long long)gridDim.x * gridDim.y) {
-            const int xn = (int)(bn % gridDim.x) * kTmaTX + OX - S::HX, yn = (int)(bn / gridDim.x) * S::TR;
+        const long long bn = (long long)row * gridDim.x + blockIdx.x + (long long)S::CTAS * nsm / 2;
+        const int xn = (int)(bn % gridDim.x) * kTmaTX + OX - S::HX, yn = (int)(bn / gridDim.x) * S::TR;
+        if (yn < P.ny) {
             asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];"
                          ::"l"(reinterpret_cast<unsigned long long>(&tm)), "r"(xn), "r"(yn), "r"(0) : "memory");
         }
@@ -692,7 +694,9 @@ cudaError_t DdOps<S>::launch(const Params &P, const CoefDD &C, const CUtensorMap
                              bool chain, int rows, cudaStream_t st)
 {
     const dim3 block(kTmaTX, S::TT);
-    const dim3 grid((P.nx + kTmaTX - 1) / kTmaTX, (rows + S::TR - 1) / S::TR);
+    // tile rows in y, and in z by as few as y holds
+    const int trows = (rows + S::TR - 1) / S::TR, z = (trows + kMaxGridY - 1) / kMaxGridY;
+    const dim3 grid((P.nx + kTmaTX - 1) / kTmaTX, (trows + z - 1) / z, z);
     return launch_kernel(chain, dd_kernel<S>(P), grid, block, S::smem_bytes, st, P, C, tm, a, b, err);
 }
 
