@@ -365,12 +365,18 @@ bool ddn_ready(lbm_ctx *c)
     return make_dd_maps(c, c->dd9);
 }
 
-// The ghost launch that precedes a step of context c from buffer `in`, if it needs one.
+// The ghost launch that precedes a step of context c from buffer `in`, if it needs one.  Chained behind the
+// step before only on grids of at most kGhostChain cells: there it saves the gap (64 x 64 float32 with walls, one
+// step a call, 10.4 us and 8.3 chained).  On larger ones its CTAs take slots between those of the step
+// before, and the next step's are placed unevenly (us a step, not chained and chained: 600 x 300 float32
+// 14.2 and 16.5, 1000 x 700 22.3 and 24.3, 4000 x 3000 252 and 259).
+constexpr long long kGhostChain = 40000;
 cudaError_t launch_step_ghosts(lbm_ctx *c, int in, cudaStream_t st)
 {
     const bool plain = !(c->use_dd || c->use_ddn || c->use_pipe || c->use_stream || c->use_tma);
     return lbm::launch_ghost(c->P, c->prec, c->f[in], st, ghost_edges(c),
-                             plain && lbm::lane_step(c->P, c->prec, c->plain_ty));
+                             plain && lbm::lane_step(c->P, c->prec, c->plain_ty),
+                             (long long)c->P.nx * c->P.ny <= kGhostChain);
 }
 
 // One fused step of context c from buffer `in` into buffer in ^ 1, on stream st.

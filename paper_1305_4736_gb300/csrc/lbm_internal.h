@@ -27,9 +27,10 @@ cudaError_t launch_init(const Params &P, int prec, void *f, const double *rho, c
 // Whether the plain step with tiles of 32 x ty cells takes 16 lanes per cell (small float64 grids).
 bool lane_step(const Params &P, int prec, int ty);
 // Ghost cells of the edges in `edges` (bit e: x-lo, x-hi, y-lo, y-hi); lanes: float64 walls with 16
-// lanes per cell.
+// lanes per cell.  chain: as in launch_kernel (k_wall is always chained).
 constexpr int kAllEdges = 15;
-cudaError_t launch_ghost(const Params &P, int prec, void *f, cudaStream_t st, int edges = kAllEdges, bool lanes = false);
+cudaError_t launch_ghost(const Params &P, int prec, void *f, cudaStream_t st, int edges = kAllEdges, bool lanes = false,
+                         bool chain = true);
 
 // Launch of a kernel that calls grid_dependency_wait before it touches memory.  chain: its CTAs may start
 // (barrier initialisation, parameter fetches) while the stream's previous launch drains; else once

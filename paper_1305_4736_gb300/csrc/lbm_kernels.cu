@@ -815,7 +815,7 @@ static int ghost_threads(int prec) { return prec == 0 ? 32 : 128; }
 // Grids whose step takes 16 lanes per cell (lane_step) have their float64 walls formed that way too (55
 // instructions for two cells in a warp instead of 225 for 32).  The others keep one thread per wall
 // cell, with which a grid gives the same bits alone and in a batch.
-cudaError_t launch_ghost(const Params &P, int prec, void *f, cudaStream_t st, int edges, bool lanes)
+cudaError_t launch_ghost(const Params &P, int prec, void *f, cudaStream_t st, int edges, bool lanes, bool chain)
 {
     if (lanes) {
         for (int axis = 0; axis < 2; axis++) {             // opposite walls in one launch
@@ -837,8 +837,8 @@ cudaError_t launch_ghost(const Params &P, int prec, void *f, cudaStream_t st, in
     while (!(edges >> (hi - 1) & 1)) hi--;
     const int first = bound[lo], nt = ghost_threads(prec);
     const dim3 grid(blocks_for(bound[hi] - first, nt));
-    return prec == 0 ? launch_chained(k_ghost<double, false>, grid, dim3(nt), 0, st, P, (double *)f, first, edges)
-                     : launch_chained(k_ghost<float, true>, grid, dim3(nt), 0, st, P, (float *)f, first, edges);
+    return prec == 0 ? launch_kernel(chain, k_ghost<double, false>, grid, dim3(nt), 0, st, P, (double *)f, first, edges)
+                     : launch_kernel(chain, k_ghost<float, true>, grid, dim3(nt), 0, st, P, (float *)f, first, edges);
 }
 
 // Tile width of the plain kernels for a grid nx columns wide: 32, or the smallest power of
