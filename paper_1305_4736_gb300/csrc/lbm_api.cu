@@ -1202,7 +1202,8 @@ cudaError_t batch_upload_cur(lbm_batch *b)
 // the batch's stream is complete and is joined to it at the end.  So every launch has a full dependency on
 // the whole previous step (and waits for it before it reads, as all of them do), while the launches of one
 // step fill the slots that the others leave empty.  A batch with one launch a step needs no branches, and
-// its steps are chained as those of lbm_step.
+// its steps are chained as those of lbm_step; not so behind a ghost launch, whose CTAs hold slots when the
+// step's are placed (four narrow float64 grids with walls, one 64-cell tile per SM: 33 us a step, chained 46).
 // Three more branches (us per batch step of 24 float32 grids of 0.58 M and 0.14 M cells on average, and of
 // as many float64 ones): 307, 88.7, 1910, 527; one: 311, 123.8, 1911, 565; eight: 316, 90.4, 1937, 540.
 struct BatchBranches {
@@ -1221,11 +1222,11 @@ struct BatchBranches {
         for (int k = 0; k < n - 1 && ce == cudaSuccess; k++) ce = cudaStreamWaitEvent(b->fork[k], b->ev_fork, 0);
         return ce;
     }
-    // Where the next launch goes; chained only behind another launch in the same stream.
+    // Where the next launch goes; chained only behind a launch of the same kind in the same stream.
     Next next()
     {
         const int k = j % n;
-        const bool chain = j >= n || std::max(b->ghost_launches, b->step_launches) <= 1;
+        const bool chain = j >= n || (b->ghost_launches == 0 && b->step_launches <= 1);
         j++;
         return {k == 0 ? st : b->fork[k - 1], chain};
     }
