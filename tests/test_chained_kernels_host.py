@@ -13,7 +13,8 @@ def _kernels():
     """(name, parameters, body) of every __global__ function."""
     for path in sorted(glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cuh"))):
         text = re.sub(r"//[^\n]*", "", open(path).read())
-        for m in re.finditer(r"__global__\s+void\s+(?:__launch_bounds__\([^()]*\)\s*)?(\w+)\(([^{;]*?)\)\s*\{", text):
+        text = re.sub(r"__launch_bounds__(\((?:[^()]|\((?:[^()]|\([^()]*\))*\))*\))", "", text)
+        for m in re.finditer(r"__global__\s+void\s+(\w+)\(([^{;]*?)\)\s*\{", text):
             depth, end = 1, m.end()
             while depth:
                 depth += {"{": 1, "}": -1}.get(text[end], 0)
