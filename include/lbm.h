@@ -206,12 +206,12 @@ int lbm_profile_end(lbm_ctx *ctx, double out[4]);
    The roofline of the float64 mode, which is bound by the float64 pipe, uses it. */
 int lbm_peak_fp64(int device, double *flops);
 
-/* Pick the fastest fused-step kernel for this context's grid: times `reps` launches of
-   each candidate (plain 32 x 4, 32 x 8, 32 x 16 and 64-cell tiles; TMA-staged tiles, the
-   streaming kernel, the double-buffered TMA-staged kernel and the double-float kernels 8
-   and 9, when the grid and precision allow) on the context's current state, writing the
-   spare buffer without advancing the state, and keeps the fastest for later lbm_step calls.
-   *choice (may be NULL) receives the lbm_options.step_kernel code of the winner.
+/* Pick the fastest fused-step kernel for this context's grid: times `reps` complete steps of
+   each candidate, with the ghost launch that it needs (plain 32 x 4, 32 x 8, 32 x 16 and 64-cell
+   tiles; TMA-staged tiles, the streaming kernel, the double-buffered TMA-staged kernel and the
+   double-float kernels 8 and 9, when the grid and precision allow) on the context's current
+   state, writing the spare buffer without advancing the state, and keeps the fastest for later
+   lbm_step calls.  *choice (may be NULL) receives the lbm_options.step_kernel code of the winner.
    Synchronous.  Not part of the paper's method: a throughput tool. */
 int lbm_autotune(lbm_ctx *ctx, int reps, int *choice);
 

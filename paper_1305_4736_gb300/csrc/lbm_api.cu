@@ -392,6 +392,17 @@ cudaError_t launch_fused_step(lbm_ctx *c, int in, cudaStream_t st, bool chain = 
     return lbm::launch_step(c->P, c->prec, c->f[in], c->f[in ^ 1], st, c->plain_ty, chain);
 }
 
+// Takes the step kernel of lbm_options.step_kernel code `code`, which is ready (tma_ready and the like).
+void select_kernel(lbm_ctx *c, int code)
+{
+    c->use_tma = code == 2;
+    c->use_stream = code == 5;
+    c->use_pipe = code == 6;
+    c->use_dd = code == 8;
+    c->use_ddn = code == 9;
+    c->plain_ty = code == 3 ? 4 : (code == 4 ? 16 : (code == 7 ? 2 : 8));
+}
+
 // Calls of at least kGraphSteps steps replay graphs of two steps, calls of at least kRunMin graphs of
 // kRunSteps: consecutive graphs do not overlap as the chained launches inside one do (200 x 4 float32:
 // 5.1 us a step in pairs, 4.2 in runs of 16), but a longer one takes longer to build.
@@ -1057,7 +1068,7 @@ int lbm_autotune(lbm_ctx *c, int reps, int *choice)
     if (ce != cudaSuccess) return cuda_fail(c, ce, "cudaSetDevice");
     // candidates: 1 = plain 32x8, 3 = plain 32x4, 4 = plain 32x16, 7 = plain 64-cell tiles,
     // 2 = TMA-staged, 5 = streaming, 6 = double-buffered TMA-staged 32x16 (float32),
-    // 8 = double-float TMA-staged (float64), 9 = the same on 32 x 4 tiles
+    // 8, 9 = double-float TMA-staged (float64), larger and smaller tiles
     int cands[10] = {1, 3, 4, 7, 0, 0, 0, 0, 0, 0};
     int ncand = 4;
     const bool tma_ok = c->use_tma || tma_ready(c);
@@ -1078,28 +1089,17 @@ int lbm_autotune(lbm_ctx *c, int reps, int *choice)
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
         return cuda_fail(c, cudaGetLastError(), "cudaEventCreate");
-    // the candidates write the other buffer without flipping it: the state does not advance
-    ce = lbm::launch_ghost(c->P, c->prec, c->f[c->cur], c->stream);
+    // the candidates write the other buffer without flipping it: the state does not advance.  Each is timed
+    // over complete steps, with the ghost launch that it needs: on small grids and grids with walls that
+    // is a large part of the step, and some kernels form those cells themselves
+    const int before = lbm_step_kernel(c);
     float best = 1e30f;
     int best_c = 1;
     for (int k = 0; k < ncand && ce == cudaSuccess; k++) {
+        select_kernel(c, cands[k]);
         auto run = [&]() {
-            const int cd = cands[k];
-            if (cd == 8 || cd == 9) {
-                const int sh = cd == 8 ? c->dd8 : c->dd9;
-                return lbm::launch_step_dd(c->P, &c->cdd, &c->dmap[sh][c->cur], c->f[c->cur], c->f[c->cur ^ 1],
-                                           c->tma_err, c->stream, sh);
-            }
-            if (cd == 6)
-                return lbm::launch_step_tma_pipe(c->P, &c->pmap[c->cur], c->f[c->cur ^ 1], c->tma_err, c->stream);
-            if (cd == 5)
-                return lbm::launch_step_stream(c->P, c->prec, &c->smap[c->cur], c->f[c->cur ^ 1], c->tma_err,
-                                               c->stream);
-            if (cd == 2)
-                return lbm::launch_step_tma(c->P, c->prec, &c->tmap[c->cur], c->f[c->cur], c->f[c->cur ^ 1], c->tma_err,
-                                            c->stream);
-            return lbm::launch_step(c->P, c->prec, c->f[c->cur], c->f[c->cur ^ 1], c->stream,
-                                    cd == 3 ? 4 : (cd == 4 ? 16 : (cd == 7 ? 2 : 8)));
+            const cudaError_t e = launch_step_ghosts(c, c->cur, c->stream);
+            return e == cudaSuccess ? launch_fused_step(c, c->cur, c->stream) : e;
         };
         ce = run();
         if (ce != cudaSuccess) break;
@@ -1113,14 +1113,9 @@ int lbm_autotune(lbm_ctx *c, int reps, int *choice)
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
+    select_kernel(c, ce == cudaSuccess ? best_c : before);
     if (ce != cudaSuccess) return cuda_fail(c, ce, "autotune");
-    c->use_tma = best_c == 2;
-    c->use_stream = best_c == 5;
-    c->use_pipe = best_c == 6;
     drop_step_graphs(c);
-    c->use_dd = best_c == 8;
-    c->use_ddn = best_c == 9;
-    c->plain_ty = best_c == 3 ? 4 : (best_c == 4 ? 16 : (best_c == 7 ? 2 : 8));
     if (choice) *choice = best_c;
     return LBM_OK;
 }
