@@ -1470,7 +1470,7 @@ int lbm_batch_create(lbm_ctx *const *ctxs, int n, lbm_batch **out)
                     const lbm::TileGrid<lbm::CoefDD> blk{c->P.nx, c->P.ny, c->P.pitch, c->P.has_c9,
                                                                 c->P.plane, (long long)k, c->cdd};
                     // rows by shape, from dd_shape down: a part-filled last tile row stays with a shape
-                    // where it holds more than 3/4 of its rows (a tile costs 23.5 : 13 : 8.3)
+                    // where it holds more than 3/4 of its rows (a wave costs 22.4 : 12.3 : 8.6)
                     for (int sh = dd_shape; sh < lbm::kDdShapes && y < c->P.ny; sh++) {
                         if (!lbm::dd_shape_supported(c->P, sh)) continue;
                         const int tr = lbm::kDdRows[sh], left = c->P.ny - y;

@@ -141,11 +141,13 @@ enum { kDdWide = 0, kDdMid = 1, kDdNarrow = 2, kDdShapes = 3 };
 constexpr int kDdRows[kDdShapes] = {DdWideShape::TR, DdMidShape::TR, DdNarrowShape::TR};
 // Whether a grid's staged boxes of a shape fit its buffers.
 bool dd_shape_supported(const Params &P, int shape);
-// Estimated duration (us) of `tiles` tiles of a shape on sms SMs, for choosing between shapes: whole
-// waves of two CTAs per SM, then the remainder at one or two per SM.  Measured on grids of 26 to 160
-// thousand cells (MC, Pr != 1), us per step, 32 x 4 / 32 x 8 / 32 x 16 tiles: 161 x 97 9.2 / 12.3 / 19.5,
-// 300 x 100 12.3 / 12.3 / 19.5, 256^2 20.1 / 16.4 / 17.4, 320^2 27.8 / 22.5 / 27.5, 380^2 38.0 / 29.4 /
-// 30.5, 400^2 44.1 / 34.8 / 39.0.
+// Estimated duration (us) of a step of `tiles` tiles of a shape on sms SMs, for choosing between shapes: a
+// fixed part, whole waves of two CTAs per SM, then the remainder at one or two per SM (which overlaps the
+// whole waves' tail).  Fitted to periodic grids on 152 SMs (MC, Pr != 1; graph runs), measured us per step on
+// 32 x 16 / 32 x 8 / 32 x 4 tiles: 161 x 97 18.9 / 11.1 / 8.1, 608 x 64 16.8 / 10.4 / 10.5, 256^2 16.8 / 15.5 /
+// 19.0, 320^2 26.4 / 21.5 / 27.0, 380^2 29.4 / 28.3 / 37.1, 400^2 38.7 / 33.9 / 43.2, 608 x 256 27.3 / 27.7 /
+// 36.5, 608 x 448 47.3 / 45.9 / 62.2, 608 x 512 50.1 / 52.1 / 71.7, 1023 x 517 82.8 / 86.9 / 121, 608 x 1280
+// 117 / 124 / 172.  The choice is the fastest on each of the 27 grids measured.
 double dd_shape_time(int shape, long long tiles, int sms);
 static_assert(DdWideShape::CTAS * (DdWideShape::smem_bytes + 2048) <= 228 * 1024, "wide tiles per SM");
 // Coefficients of the double-float kernels in the order of the population pairs (lane e of pair

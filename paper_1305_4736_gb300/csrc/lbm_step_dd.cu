@@ -46,10 +46,11 @@ bool dd_shape_supported(const Params &P, int shape)
 
 double dd_shape_time(int shape, long long tiles, int sms)
 {
-    constexpr double whole[kDdShapes] = {23.5, 13.0, 8.3}, one[kDdShapes] = {15.5, 10.5, 8.2},
-                     two[kDdShapes] = {27.0, 16.4, 12.3};
+    constexpr double fixed[kDdShapes] = {4.9, 3.1, 2.0}, whole[kDdShapes] = {22.4, 12.3, 8.6},
+                     one[kDdShapes] = {11.5, 6.7, 5.2}, two[kDdShapes] = {22.0, 11.0, 9.0};
     const long long slots = 2LL * sms, rest = tiles % slots;
-    return (double)(tiles / slots) * whole[shape] + (rest == 0 ? 0.0 : (rest <= sms ? one[shape] : two[shape]));
+    return fixed[shape] + (double)(tiles / slots) * whole[shape] +
+           (rest == 0 ? 0.0 : (rest <= sms ? one[shape] : two[shape]));
 }
 
 cudaError_t launch_step_dd(const Params &P, const void *coef, const void *tmap, const void *fin, void *fout,
