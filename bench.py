@@ -59,17 +59,17 @@ TOTALS_EVERY = 100
 # still hash to that value, else null.
 TRAFFIC_PER_CELL = {
     "f32": {"bytes": 125.70, "sources": ("lbm_step_tma.cu", "lbm_device.cuh", "lbm_tma_util.cuh"),
-            "sha": "6c8f927357f114a7"},
-    "f64": {"bytes": 251.29, "sources": ("lbm_step_stream.cu", "lbm_device.cuh", "lbm_tma_util.cuh"),
-            "sha": "96b8d4d555711f4f"},
-    "dd": {"bytes": 246.77, "sources": ("lbm_step_dd.cuh", "lbm_dd.cuh", "lbm_device.cuh", "lbm_tma_util.cuh"),
-           "sha": "c7788a8fb6be68e3"},
+            "sha": "e82818c6d7b51d14"},
+    "f64": {"bytes": 251.58, "sources": ("lbm_step_stream.cu", "lbm_device.cuh", "lbm_tma_util.cuh"),
+            "sha": "03d137c0a7392ddd"},
+    "dd": {"bytes": 246.71, "sources": ("lbm_step_dd.cuh", "lbm_dd.cuh", "lbm_device.cuh", "lbm_tma_util.cuh"),
+           "sha": "df3b840a957b1139"},
 }
 # float32-pipe lane operations per cell of one launch of the double-float float64 kernel on wide
 # tiles: ncu's FMA-pipe busy fraction x cycles x 128 lanes (its counters of float32 instructions do
 # not see the packed f32x2 ones), on the same sources (profiles/k_step_dd_f64_shear_layer.md); None
 # when the sources changed since.
-DD_FP32_OPS = {"ops": 3537.4, "sha": "c7788a8fb6be68e3"}
+DD_FP32_OPS = {"ops": 3537.5, "sha": "df3b840a957b1139"}
 FP32_LANES_PER_SM = 128           # float32 FMA lanes per SM per cycle (GB300)
 
 
@@ -485,8 +485,8 @@ def serving_measure(count, steps, max_nx, max_ny, device, seed=1305):
 
 
 def batch_measure(device, steps=20, warmup=3, seed=1305):
-    """Batched stepping (one lbm_batch: one batched tile-kernel launch per
-    step over the tiles of all grids) of 24 uneven float32 shear-layer grids whose buffers
+    """Batched stepping (one lbm_batch; grids of this size have a launch of the tile kernel
+    each, side by side on the batch's streams) of 24 uneven float32 shear-layer grids whose buffers
     exceed L2, against stepping the same grids one at a time on their automatic kernels."""
     import numpy as np
     import torch
@@ -531,8 +531,8 @@ def batch_measure(device, steps=20, warmup=3, seed=1305):
             "ms_per_step": ms, "cell_updates_per_s": cells / (ms * 1e-3),
             "roofline": {"bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm,
                          "peak_source": f"{peak_src} hbm_gbs", "traffic": None,
-                         "kernel": "k_step_tma_batch<MC> over the tiles of all 24 grids "
-                                   "(one CTA per 32 x 16 tile), in one CUDA graph"},
+                         "kernel": "k_step_tma<float,dev,MC>, one launch per large grid side by side (smaller "
+                                   "ones in k_step_tma_batch<MC>), in one CUDA graph"},
             "one_at_a_time_ms_per_step": ms_solo, "speedup_vs_one_at_a_time": ms_solo / ms}
 
 

@@ -1160,7 +1160,6 @@ struct lbm_batch {
         std::vector<Span> alone;                 // spans from row 0 with a launch of their own
         void *tblock = nullptr;
         size_t tbytes = 0;
-        int ntt = 0;                             // tiles per step
     };
     std::vector<lbm_ctx *> ctxs;
     std::vector<Group> groups;
@@ -1458,13 +1457,9 @@ int lbm_batch_create(lbm_ctx *const *ctxs, int n, lbm_batch **out)
             g.hG.push_back(lbm::BatchGrid{{c->f[0], c->f[1]}, c->tma_err, c->cur, 0});
             if (hp.back().ghost) g.max_ghost = std::max(g.max_ghost, 4 * (c->P.nx + c->P.ny));
             if (g.tma[k]) {
-                const int ntx = (c->P.nx + lbm::kTmaTX - 1) / lbm::kTmaTX;
                 // a large member has its own launch of the single-grid kernel
                 int y = alone_rows(c, allowed);
-                if (y > 0) {
-                    g.alone.push_back({(int)k, 0, y});
-                    g.ntt += ntx * ((y + lbm::DdWideShape::TR - 1) / lbm::DdWideShape::TR);
-                }
+                if (y > 0) g.alone.push_back({(int)k, 0, y});
                 if (y == c->P.ny) continue;
                 if (g.prec == LBM_FP64) {
                     const lbm::TileGrid<lbm::CoefDD> blk{c->P.nx, c->P.ny, c->P.pitch, c->P.has_c9,
@@ -1479,14 +1474,12 @@ int lbm_batch_create(lbm_ctx *const *ctxs, int n, lbm_batch **out)
                         if (last || 4 * (left % tr) > 3 * tr) rows = left;
                         if (rows == 0) continue;
                         g.tk[sh].push_back({(int)k, y, rows});
-                        g.ntt += ntx * ((rows + tr - 1) / tr);
                         htd[sh].push_back(blk);
                         y += rows;
                     }
                     continue;
                 }
                 g.tk[0].push_back({(int)k, 0, c->P.ny});
-                g.ntt += ntx * ((c->P.ny + lbm::TmaShape<float>::TR - 1) / lbm::TmaShape<float>::TR);
                 htf.push_back(lbm::TileGrid<lbm::Coef<float>>{c->P.nx, c->P.ny, c->P.pitch, c->P.has_c9,
                                                               c->P.plane, (long long)k, c->P.cf});
                 continue;

@@ -90,9 +90,6 @@ __device__ __forceinline__ dd operator*(float c, dd a) { return a * c; }
 // a * 2^k (exact).
 __device__ __forceinline__ dd scale2(dd a, float p2) { return dd{__fmul_rn(a.hi, p2), __fmul_rn(a.lo, p2)}; }
 
-__device__ __forceinline__ dd &operator+=(dd &a, dd b) { return a = a + b; }
-__device__ __forceinline__ dd &operator-=(dd &a, dd b) { return a = a - b; }
-
 // a * b + c (12).
 __device__ __forceinline__ dd fma_dd(dd a, dd b, dd c)
 {
@@ -117,40 +114,6 @@ __device__ __forceinline__ dd recip(dd x)
     const dd r = ddf(1.0f) - x * y;
     return fast2sum(y, __fmul_rn(y, __fadd_rn(r.hi, r.lo)));
 }
-
-// The pair renormalised: |lo| <= ulp(hi) / 2 (Fast2Sum; with a low part larger than the high
-// part, after a cancellation, it still returns the pair's value to within 2^-24 of that low part,
-// far below the pair's own accuracy).
-__device__ __forceinline__ dd norm(dd a) { return fast2sum(a.hi, a.lo); }
-
-// Twice the MC slope, 2 minmod(2a, (a + b)/2, 2b) = sign(a) min(4|a|, 4|b|, |a + b|) when a and
-// b agree in sign and 0 otherwise (Sec. III, reading A6); as mc2 of lbm_device.cuh.  a and b
-// must be normalised (norm), so that their high parts carry their signs; they agree when
-// a.hi b.hi > 0 (a product below 2^-149 counts as disagreement: then the smaller difference
-// is below 2^-74, so the slope, at most 4 times it, is below 2^-72, far below the populations'
-// 2^-47 resolution, and is taken as 0).  Two
-// candidates x, y of the sign of a are ordered by the float32 value
-// (x.hi - y.hi) + (x.lo - y.lo), whose sign is that of x - y (zero only for x = y or x, y within
-// a few units of 2^-47 of each other, where either is the slope to the pairs' accuracy); the
-// smaller magnitude is the lower value for a > 0 and the higher for a < 0.  The sum a + b is
-// left unnormalised (its low part stays within a few units of its high part's last place,
-// which the ordering tolerates).  Three float32 operations and a predicate per comparison;
-// flipping the three pairs to magnitudes and comparing lexicographically took 4% more of the
-// step.
-__device__ __forceinline__ dd mc2n(dd a, dd b)
-{
-    const dd s = a + b;
-    const bool agree = __fmul_rn(a.hi, b.hi) > 0.0f;
-    const bool neg = a.hi < 0.0f;
-    const float dab = __fadd_rn(__fsub_rn(a.hi, b.hi), __fsub_rn(a.lo, b.lo));
-    const dd m = ((dab < 0.0f) != neg) ? a : b;
-    const dd m4 = scale2(m, 4.0f);
-    const float dms = __fadd_rn(__fsub_rn(m4.hi, s.hi), __fsub_rn(m4.lo, s.lo));
-    return agree ? (((dms < 0.0f) != neg) ? m4 : s) : dd{0.0f, 0.0f};
-}
-
-// As mc2n, for pairs not yet normalised.
-__device__ __forceinline__ dd mc2(dd a, dd b) { return mc2n(norm(a), norm(b)); }
 
 // ---------------------------------------------------------------------------
 // Pairs of double-float values, (q, q + 4) of the population pairs: hi and lo parts as float2
@@ -205,7 +168,9 @@ __device__ __forceinline__ dd2 operator*(dd2 a, float2 c)
 
 __device__ __forceinline__ dd2 scale2(dd2 a, float p2) { return dd2{mul2(a.hi, f2(p2, p2)), mul2(a.lo, f2(p2, p2))}; }
 
-// The pairs renormalised (as norm below).
+// The pairs renormalised: |lo| <= ulp(hi) / 2 (Fast2Sum; with a low part larger than the high
+// part, after a cancellation, it still returns the pair's value to within 2^-24 of that low part,
+// far below the pair's own accuracy).
 __device__ __forceinline__ dd2 norm(dd2 a)
 {
     const float2 s = add2(a.hi, a.lo);
@@ -228,13 +193,22 @@ __device__ __forceinline__ dd2 add_smaller(dd2 a, dd2 b)
     return dd2{s, add2(sub2(b.hi, sub2(s, a.hi)), add2(a.lo, b.lo))};
 }
 
-// mc2n for both lanes: the sums, products and differences packed, the selects per lane.  The
-// order tests read the sign of a difference relative to that of a (or of s, equal to it where the
-// differences agree) from their product: below 2^-149, where it reads as zero, the candidates
-// differ by less than 2^-74, the flush threshold of the split.  Where a and b disagree in sign the result
-// is set to zero last: s is not normalised, so where the high parts cancel the sign of s.hi is not that of
-// s, and no test against s can tell (at an extremum symmetric to 2^-24, s would be taken for the slope).
-// Scaling the candidates by 0 there instead is 1% of the step less, and gives NaN for infinities and NaN.
+// Twice the MC slope, 2 minmod(2a, (a + b)/2, 2b) = sign(a) min(4|a|, 4|b|, |a + b|) when a and
+// b agree in sign and 0 otherwise (Sec. III, reading A6); as mc2 of lbm_device.cuh.  a and b
+// must be normalised (norm), so that their high parts carry their signs; they agree when
+// a.hi b.hi > 0 (a product below 2^-149 counts as disagreement: then the smaller difference
+// is below 2^-74, so the slope, at most 4 times it, is below 2^-72, far below the populations'
+// 2^-47 resolution, and is taken as 0).  Two candidates x, y of the sign of a are ordered by the float32
+// value (x.hi - y.hi) + (x.lo - y.lo), whose sign is that of x - y (zero only for x = y or x, y within
+// a few units of 2^-47 of each other, where either is the slope to the pairs' accuracy); the
+// smaller magnitude is the lower value for a > 0 and the higher for a < 0, read from the sign of that
+// value times a.hi (or s.hi): below 2^-149, where the product reads as zero, the candidates differ by
+// less than 2^-74, the flush threshold of the split.  The sum s = a + b is left unnormalised (its low
+// part stays within a few units of its high part's last place, which the ordering tolerates where a and b
+// agree).  Where they disagree the result is set to zero last: if the high parts cancel, the sign of s.hi
+// is not that of s, and no test against s can tell (at an extremum symmetric to 2^-24, s would be taken
+// for the slope).  Scaling the candidates by 0 there instead is 1% of the step less, and gives NaN for
+// infinities and NaN.
 __device__ __forceinline__ dd2 mc2n(dd2 a, dd2 b)
 {
     const dd2 s = a + b;
@@ -317,7 +291,8 @@ __device__ __forceinline__ dd2 dd_split2(double x, double y)
 
 // hi + lo rounded to float64 (to nearest, ties to even): both parts in float64 exactly, then one
 // float64 addition rounds their sum.  hi is converted on the float64 pipe (1.9 lanes per cycle per
-// SM; so infinities and NaN carry over), lo by moving its fields with integer operations: three
+// SM; so infinities and NaN in hi carry over; next to an infinite hi a lo that is not finite reads as a
+// finite number), lo by moving its fields with integer operations: three
 // float64-pipe operations a value kept that pipe 55% busy over the step and more in the update,
 // which waits for it (2048 x 2048: 0.588 ms, against 0.564 ms with two;
 // rounding by integer additions instead took 0.591 ms for half of the values and 0.619 for all).

@@ -36,13 +36,15 @@
 //             read again after the collision instead of kept
 //   0.643     the split in half the integer operations, Fast2Sum where the order is known
 //   0.587     the residuals formed in phase 1 and kept in registers, so that no cell's shells are
-//             formed twice, nothing spills, and the ring is left out where s8 = s5 (3501 -> 3188
+//             formed twice and the ring is left out where s8 = s5 (3501 -> 3188
 //             thread instructions a cell)
-//   0.559     the pairs that move along both axes first; results stored evict-first
+//   0.557     the pairs that move along both axes first; results stored evict-first
+//   0.562     the slope set to zero where differences disagree in sign (mc2n)
 // Other shapes (warps x rows per thread, CTAs per SM), same code: 16 x 2, one CTA 0.807 ms; 12 x 2,
 // one CTA 0.843; 5 x 3, two CTAs 1.09; 4 x 4, two CTAs 1.31 (the unrolled rows spill), against 0.643;
 // 6 x 2, two CTAs 0.677; 7 x 2, two CTAs 0.665; 10 x 2, one CTA 0.885, against 0.587.
-// The results are bit for bit those of the scalar kernel.
+// At their 128 registers the MC kernels on 32 x 16 tiles spill 8 to 24 bytes a thread, the batched ones on
+// those tiles (coefficients in shared memory) 88 to 190.  The results are bit for bit those of scalar operations.
 #pragma once
 
 #include <cuda.h>

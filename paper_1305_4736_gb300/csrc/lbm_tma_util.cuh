@@ -91,9 +91,11 @@ __device__ __forceinline__ int ghost_source(int v, int n, int kind_lo, int kind_
 // Ghost cells of the tiles at an edge of the grid: periodic and zero-gradient edges are filled in
 // the staged tile, with the values the ghost launch would have written; those of a
 // fixed-equilibrium edge never change (lbm_create_ex fills them).  So no ghost launch precedes the
-// step, but for wall edges, which need the mirror cell's moments.  One thread per ghost cell of the cross: the tile's columns in up to four ghost rows,
-// its rows in up to four ghost columns.  The sources are interior cells, read from global memory
-// while the tile copy is in flight; they replace the tile's ghost cells once it has landed.
+// step, but for walls in the float32 kernel and the float64 one of step_kernel 2 (the double-float
+// kernels form them in the tile too: wall_fill).  One thread per ghost cell of the cross: the tile's
+// columns in up to four ghost rows, its rows in up to four ghost columns.  The sources are interior
+// cells, read from global memory while the tile copy is in flight; they replace the tile's ghost
+// cells once it has landed.
 // Measured per step, with the launches chained (launch_chained): 200 x 4 float64 20.5 -> 9.3 us,
 // 256^2 float32 10.3 -> 6.2 us, 8192^2 float32 1.382 ms with its ghost launch -> 1.353 ms.
 template <typename R>
