@@ -200,11 +200,11 @@ k_step(const __grid_constant__ Params P, const R *fin, R *fout, int TX, int log_
     step_tile<R, Dev, Lim>(P, fin, fout, blockIdx.x * TX, blockIdx.y * TY, TX, log_tx, TY, su, sv);
 }
 
-// Fused step, float64, 16 lanes per cell: for grids of at most kLaneCells cells.  A CTA of 128 threads
+// Fused step, float64, 16 lanes per cell: for grids of at most kLaneCells cells (lane_step).  A CTA of 128 threads
 // takes 8 cells (TX x 8/TX); each lane forms its population's convection, the shells and moments go
 // between lanes, the flow velocities of the neighbours (for the energy-flux correction) through
-// shared memory.  About 60 float64 instructions a warp instead of 440, on as many partitions as the
-// grid has pairs of cells (see lbm_lanes.cuh).
+// shared memory.  79 float64 instructions a warp (ncu; 47 without the energy-flux correction) instead of
+// some 400, on as many partitions as the grid has pairs of cells (see lbm_lanes.cuh).
 constexpr int kLaneTile = 8;          // cells per CTA
 template <int Lim, bool C9>
 __global__ void __launch_bounds__(kLaneTile * kCellLanes)
@@ -808,12 +808,12 @@ cudaError_t launch_init(const Params &P, int prec, void *f, const double *rho, c
     return cudaGetLastError();
 }
 
-// Threads per block of the ghost launches: a float64 wall cell is some 225 float64 instructions, which
+// Threads per block of the ghost launches: a float64 wall cell is 213 float64 instructions, which
 // a partition of an SM takes 78 cycles each for, so one-warp blocks reach every partition.
 static int ghost_threads(int prec) { return prec == 0 ? 32 : 128; }
 
-// Grids whose step takes 16 lanes per cell (lane_step) have their float64 walls formed that way too (55
-// instructions for two cells in a warp instead of 225 for 32).  The others keep one thread per wall
+// Grids whose step takes 16 lanes per cell (lane_step) have their float64 walls formed that way too (46
+// instructions for two cells in a warp instead of 213 for 32).  The others keep one thread per wall
 // cell, with which a grid gives the same bits alone and in a batch.
 cudaError_t launch_ghost(const Params &P, int prec, void *f, cudaStream_t st, int edges, bool lanes, bool chain)
 {
@@ -850,14 +850,21 @@ int plain_log_tx(int nx)
     return l;
 }
 
-// The float64 kernel on 64-cell tiles gives way to 16 lanes per cell on grids of at most 7296 cells:
-// pairs of cells over 608 partitions, 60 float64 instructions of 78 cycles each, against one wave of
-// 440.  Measured, us per step, 64-cell tiles and lanes: 4 x 200 with walls 28.7 and 11.3, 8 x 400 28.7
-// and 15.4, 16 x 380 28.7 and 21.5, 16 x 450 24.6 and (extrapolated) 24.1; without walls or energy-flux
-// correction 4 x 200 27.7 and 5.9, 16 x 380 27.7 and 14.3, 16 x 600 20.5.
+// The float64 kernel on 64-cell tiles gives way to 16 lanes per cell on grids of at most kLaneCells cells:
+// a warp takes two cells, 79 float64 instructions (47 without the energy-flux correction; ncu) of 78 cycles each on
+// one of the 608 partitions of 152 SMs, and up to six warps share a partition, against one wave of some
+// 400.  With the correction the walls' ghost cells count too.  Measured, us per step, 64-cell tiles and lanes (MC;
+// with the correction / without): periodic 4 x 200 20.9 and 6.9 / 20.3 and 4.4, 8 x 900 20.7 and 20.1 / 20.1 and 16.5,
+// 16 x 520 20.7 and 26.2 / 20.1 and 17.0; two walls 4 x 200 28.8 and 9.5 / 28.2 and 7.1, 16 x 450 28.7 and 23.2 / 28.1
+// and 16.2; four walls 8 x 400 29.1 and 18.5 / 28.5 and 14.6, 16 x 380 28.9 and 35.9 / 28.4 and 17.8, 8 x 900 29.6 and
+// 37.0 / 29.0 and 29.8.
+constexpr int kLaneCells = 608 * 12;
 bool lane_step(const Params &P, int prec, int ty)
 {
-    return prec == 0 && ty == 2 && (long long)P.nx * P.ny <= 7296;
+    long long cells = (long long)P.nx * P.ny;
+    for (int e = 0; e < 4 && P.has_c9; e++)
+        if (P.edge[e].kind == 3) cells += 2 * (e < 2 ? P.ny : P.nx);
+    return prec == 0 && ty == 2 && cells <= kLaneCells;
 }
 
 template <typename R, bool Dev, int NT>

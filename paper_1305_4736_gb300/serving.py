@@ -5,9 +5,9 @@ precision) arrive over time.  The engine:
   - admits a waiting request as soon as its device footprint (lbm_footprint: both
     population buffers) fits the memory budget next to the solves already resident;
   - keeps every admitted solve's state resident on the GPU and advances all of them
-    together, a chunk of steps at a time, through one lbm_batch (one batched ghost-fill
-    and one batched fused-step launch per precision/limiter group per step, replayed from
-    a CUDA graph); the batch is rebuilt whenever its membership changes;
+    together, a chunk of steps at a time, through one lbm_batch (per step and group of one
+    precision and limiter a few batched launches over the tiles of its grids, replayed from a
+    CUDA graph); the batch is rebuilt whenever its membership changes;
   - retires a solve when its steps are done: its moments (rho, u, v, T) are read back,
     its memory is released, and its time to result (completion - arrival) is recorded.
 Requests that arrive while others run are admitted at the next chunk boundary, so their
