@@ -157,10 +157,12 @@ int lbm_create_ex(int nx, int ny, double dx, double dt, double gamma, double Pr,
 int lbm_init(lbm_ctx *ctx, const double *rho, const double *u, const double *v, const double *T);
 
 /* Enqueue n >= 1 time steps (fused collide/convect per step, preceded by a ghost-fill launch
-   where the step kernel does not read the boundary in place; Eq. (3) and the update of Sec. III).  Asynchronous on the context's stream.  Runs of 16 steps or more
-   (outside lbm_profile_begin / lbm_profile_end) replay pairs of steps from a CUDA graph that the
-   context captures on a private stream at first use, one per starting buffer (lbm_autotune
-   drops them): the same launches, one graph launch per pair.
+   where the step kernel does not form the boundary itself; Eq. (3) and the update of Sec. III).
+   Asynchronous on the context's stream.  Outside lbm_profile_begin / lbm_profile_end, calls of
+   16 steps or more replay CUDA graphs of two steps, calls of 64 or more graphs of 16, with the
+   steps left over by direct launches.  The context captures each graph on a private stream at
+   first use, one per length and starting buffer (lbm_autotune drops them); they hold the same
+   launches.
    LBM_ERR_STATE if n <= 0 or the context was never initialised. */
 int lbm_step(lbm_ctx *ctx, int n);
 
@@ -227,22 +229,25 @@ int lbm_autotune(lbm_ctx *ctx, int reps, int *choice);
      such grids (float64: one per tile shape, 32 x 16, 32 x 8 and 32 x 4; one CTA per tile; the
      launch's parameters hold each grid's tensor map, buffers and tile count, and the CTA stages
      its grid's coefficients in shared memory), with the arithmetic of the single-grid kernel, bit
-     for bit;
+     for bit.  In groups of large grids (256 tiles of 32 x 16 on average) those of at least 64 such
+     tiles have a launch of the single-grid kernel each: the same bits;
    - the other grids share the packed plain kernel, whose persistent CTAs walk a tile list
      (float32: 256-cell tiles, float64: 64-cell tiles, which spread small float64 grids over
      more SMs; 32 columns wide, or TX = the smallest power of two >= nx for narrower grids)
      with the arithmetic of the plain step kernel, to round-off (the compiler may contract
-     multiply-adds differently);
+     multiply-adds differently; the 16 lanes per cell that small float64 grids take alone add in
+     another order);
    - a context on the streaming or the double-buffered kernel with at least 512 cells per SM
-     takes part in its group's ghost launch only and steps with its own kernel, launched on
-     one of eight forked streams so that such grids overlap, bit for bit.
-   Pairs of steps are replayed from a CUDA graph captured on the first call with n >= 2
-   (recaptured when a context was stepped alone an odd number of times since).  Tiles are independent, so a grid's result does not depend on the other members
-   of its batch (bit for bit).
-   The launches of one step do not wait for each other: each starts as the one before drains.
-   Contexts may also be stepped alone between batch steps.  Errors: LBM_ERR_ARG (NULL, empty, mixed device or stream, a
-   context listed twice), LBM_ERR_STATE (uninitialised context, n <= 0), LBM_ERR_OOM,
-   LBM_ERR_CUDA. */
+     takes part in its group's ghost launch only and steps with its own kernel, bit for bit.
+   The ghost launches of a step, and then its step launches, run side by side on the batch's stream
+   and up to three streams of its own; each starts when the step before is complete.
+   Steps are replayed from CUDA graphs captured at first use: of two steps, or of 16 in calls of 64
+   steps or more where a step is at most two launches (recaptured when a context was stepped
+   alone an odd number of times since).  Tiles are independent, so a grid's result does not depend on
+   the other members of its batch (bit for bit).
+   Contexts may also be stepped alone between batch steps.  Errors: LBM_ERR_ARG (NULL, empty,
+   mixed device or stream, a context listed twice), LBM_ERR_STATE (uninitialised context, n <= 0),
+   LBM_ERR_OOM, LBM_ERR_CUDA. */
 typedef struct lbm_batch lbm_batch;
 int lbm_batch_create(lbm_ctx *const *ctxs, int n, lbm_batch **out);
 int lbm_batch_step(lbm_batch *batch, int n);        /* asynchronous on the shared stream */

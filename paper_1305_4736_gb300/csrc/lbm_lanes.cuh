@@ -5,8 +5,8 @@
 // populations.  Where a launch has few cells (walls; grids of a few thousand cells) the number of
 // float64 instructions in one warp is what it lasts, so here 16 lanes share a cell: the butterflies
 // of the shells take one instruction a stage, a block of the transformation four, an equilibrium
-// row six, about 60 instead of 440 for a whole step (30 against 14 per cell: the price where cells
-// abound).  Everything stays in float64.
+// row six, 79 instead of 398 for a whole step (47 without the energy-flux correction; 40 against 12 per
+// cell: the price where cells abound).  Everything stays in float64.
 //
 // Lane q of a cell holds population q = 4 shell + i, and in the shell basis the coefficient
 // `i` of its shell: 0 S, 1 Q, 2 X, 3 Y.  A moment row r of a component's block sits in the lane of

@@ -344,10 +344,10 @@ __device__ __forceinline__ void ring_and_edges(const float2 *tile, float4 *suv, 
 }
 
 // One ghost cell of a wall in the staged tile (before its split) from its mirror cell, in float64 as the
-// ghost launch of the other kernels forms it: the two warps of a tile's wall cells take some 225 float64
-// instructions each, 4.5 us, while the other warps wait (161 x 97 channel 14.8 us a step, 18.8 with a
-// launch before the step, 512 x 512 52 and 53, 1023 x 517 94 and 114).  In double-float it was 10.3 us on
-// 161 x 97, with three to four times the error of a step at the wall cells.  A function of its own: every tile shape,
+// ghost launch of the other kernels forms it: the two warps of a tile's wall cells take some 210 float64
+// instructions each while the other warps wait (161 x 97 channel 14.8 us a step, 18.8 with a launch before
+// the step, 512 x 512 52 and 53, 1023 x 517 94 and 114).  In double-float it was 10.3 us on 161 x 97, with
+// three to four times the error of a step at the wall cells.  A function of its own: every tile shape,
 // alone and in a batch, runs the same code and has the same bits.
 __device__ __noinline__ void wall_cell64(const Coef<double> &C, const EdgeDev &E, const double *mirror, double *ghost,
                                          int plane)
