@@ -110,8 +110,10 @@ typedef struct {
                                       128 columns), 6 = persistent TMA-staged 32 x 16 tiles with
                                       two tile buffers per CTA (LBM_FP32_DEV only), 7 = plain
                                       64-cell tiles (32 x 2; spreads small float64 grids over
-                                      every SM; float64 grids of at most 7296 cells: 8-cell tiles
-                                      with a thread per population), 8 = LBM_FP64 only: TMA-staged tiles
+                                      every SM; float64 grids of at most 7296 cells, with the
+                                      energy-flux correction counting their walls' ghost cells:
+                                      8-cell tiles with a thread per population), 8 = LBM_FP64
+                                      only: TMA-staged tiles
                                       with the step's arithmetic in double-float form (pairs of
                                       float32, about 2^-47 rounding per operation) on the float32
                                       pipe, populations still stored and returned in float64

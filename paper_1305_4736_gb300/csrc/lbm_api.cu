@@ -1224,14 +1224,16 @@ struct BatchBranches {
         j++;
         return {k == 0 ? st : b->fork[k - 1], chain};
     }
-    cudaError_t join()
+    // Joins the branches to st, also after a launch that failed: the batch's stream then stands for all that
+    // was launched.  Returns the first error.
+    cudaError_t join(cudaError_t first)
     {
-        cudaError_t ce = cudaSuccess;
-        for (int k = 0; k < n - 1 && ce == cudaSuccess; k++) {
-            ce = cudaEventRecord(b->ev_join[k], b->fork[k]);
+        for (int k = 0; k < n - 1; k++) {
+            cudaError_t ce = cudaEventRecord(b->ev_join[k], b->fork[k]);
             if (ce == cudaSuccess) ce = cudaStreamWaitEvent(st, b->ev_join[k], 0);
+            if (first == cudaSuccess) first = ce;
         }
-        return ce;
+        return first;
     }
 };
 
@@ -1300,19 +1302,20 @@ cudaError_t batch_launch_step(lbm_batch *b, int phase, cudaStream_t st)
 {
     BatchBranches ghosts(b, st, b->ghost_launches);
     cudaError_t ce = ghosts.fork();
-    for (auto &g : b->groups) {
-        if (ce != cudaSuccess) return ce;
+    for (size_t i = 0; i < b->groups.size() && ce == cudaSuccess; i++) {
+        const auto &g = b->groups[i];
         if (g.max_ghost == 0) continue;
         const BatchBranches::Next at = ghosts.next();
         ce = lbm::launch_ghost_batch(g.dP, g.dG, (int)g.members.size(), g.max_ghost, g.prec, phase, at.chain, at.st);
     }
-    if (ce == cudaSuccess) ce = ghosts.join();
+    ce = ghosts.join(ce);
+    if (ce != cudaSuccess) return ce;
     BatchBranches steps(b, st, b->step_launches);
-    if (ce == cudaSuccess) ce = steps.fork();
-    for (auto &g : b->groups) {
-        if (ce == cudaSuccess) ce = batch_launch_tma(b, g, phase, steps);
-        if (ce != cudaSuccess) return ce;
-        if (g.ntiles == 0) continue;
+    ce = steps.fork();
+    for (size_t i = 0; i < b->groups.size() && ce == cudaSuccess; i++) {
+        const auto &g = b->groups[i];
+        ce = batch_launch_tma(b, g, phase, steps);
+        if (ce != cudaSuccess || g.ntiles == 0) continue;
         const BatchBranches::Next at = steps.next();
         ce = lbm::launch_step_batch(g.dP, g.dG, g.dT, g.ntiles, g.prec, g.limiter, g.nt,
                                     g.nt == lbm::kBatchThreadsFp64 ? 2 * b->ctas : b->ctas, phase, at.chain, at.st);
@@ -1322,7 +1325,7 @@ cudaError_t batch_launch_step(lbm_batch *b, int phase, cudaStream_t st)
         const BatchBranches::Next at = steps.next();
         ce = launch_fused_step(c, c->cur ^ phase, at.st, at.chain);
     }
-    return ce == cudaSuccess ? steps.join() : ce;
+    return steps.join(ce);
 }
 
 // Inside a batch, a context whose kernel is the TMA-staged tile kernel (float32) or the
