@@ -60,16 +60,16 @@ TOTALS_EVERY = 100
 TRAFFIC_PER_CELL = {
     "f32": {"bytes": 125.71, "sources": ("lbm_step_tma.cu", "lbm_device.cuh", "lbm_tma_util.cuh"),
             "sha": "e82818c6d7b51d14"},
-    "f64": {"bytes": 251.35, "sources": ("lbm_step_stream.cu", "lbm_device.cuh", "lbm_tma_util.cuh"),
+    "f64": {"bytes": 251.36, "sources": ("lbm_step_stream.cu", "lbm_device.cuh", "lbm_tma_util.cuh"),
             "sha": "03d137c0a7392ddd"},
-    "dd": {"bytes": 246.67, "sources": ("lbm_step_dd.cuh", "lbm_dd.cuh", "lbm_device.cuh", "lbm_tma_util.cuh"),
-           "sha": "d22d3133056e38d7"},
+    "dd": {"bytes": 246.74, "sources": ("lbm_step_dd.cuh", "lbm_dd.cuh", "lbm_device.cuh", "lbm_tma_util.cuh"),
+           "sha": "72dfc07578c4cfff"},
 }
 # float32-pipe lane operations per cell of one launch of the double-float float64 kernel on wide
 # tiles: ncu's FMA-pipe busy fraction x cycles x 128 lanes (its counters of float32 instructions do
 # not see the packed f32x2 ones), on the same sources (profiles/k_step_dd_f64_shear_layer.md); None
 # when the sources changed since.
-DD_FP32_OPS = {"ops": 3537.4, "sha": "d22d3133056e38d7"}
+DD_FP32_OPS = {"ops": 3537.8, "sha": "72dfc07578c4cfff"}
 FP32_LANES_PER_SM = 128           # float32 FMA lanes per SM per cycle (GB300)
 
 

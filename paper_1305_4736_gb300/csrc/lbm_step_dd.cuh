@@ -192,7 +192,7 @@ __device__ __forceinline__ ResidualDD residual_dd(const CoefDD &C, const dd2 *fp
 __device__ __forceinline__ void correct_dd(const CoefDD &C, ResidualDD &r, dd2 gx, dd2 gy)
 {
     const dd div = first(gx) + C.ry * second(gy), shr = second(gx) + C.ry * first(gy);
-    const dd2 g = pack(first(gx), second(gy)) * C.g4 - bcast(C.four_inv_b * div);
+    const dd2 g = C.g4 * pack(first(gx), second(gy)) - bcast(C.four_inv_b * div);
     const dd2 h = r.u * g + scale2(pack(second(r.u), first(r.u)) * bcast(shr), 2.0f);
     r.d78 = r.d78 + C.q89 * bcast(r.P) * h;
 }
